@@ -42,7 +42,7 @@ import fsd_inputs as gi  # noqa: E402
 NOMINAL_HBM_GBS = 8000.0
 # DRAM bytes (read + written) of one pair-kernel launch on the headline workload, from the ncu
 # capture summarised under profiles/; None whenever that kernel has changed since the capture.
-PAIR_KERNEL_DRAM_BYTES = 311_813_120
+PAIR_KERNEL_DRAM_BYTES = None
 FALLBACK_HBM_GBS = 6650.0
 L2_BYTES = 126 * 1024 * 1024
 D_BAND = 1e-5          # |D_oracle - T| below this: the fp32 and fp64 decisions may differ
@@ -486,11 +486,11 @@ def main():
         pair_bytes = c.elem_size * B * P * 2 * V
     achieved = pair_bytes / (pair_ms * 1e-3) / 1e9
     call_achieved = ideal / (ms_per_step * 1e-3) / 1e9
-    kname = "fsd_pair_stream_kernel" if (V * c.elem_size) % 16 == 0 and V * c.elem_size >= 1024 else "fsd_pair_generic_kernel"
+    kname = "fsd_pair_stream_kernel" if -(-V * c.elem_size // 16) <= 40000 else "fsd_pair_generic_kernel"
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "traffic": PAIR_KERNEL_DRAM_BYTES if headline else None, "peak_kind": f"of {peak_kind}",
                 "frac_of_nominal_8000": achieved / NOMINAL_HBM_GBS,
-                "kernel": f"pair kernel ({kname}<{c.dtype}, {args.div.upper()}>; the interval includes the 64 KB "
+                "kernel": f"pair kernel ({kname}<{c.dtype}, {args.div.upper()}>; the interval includes the "
                           "memset of flags and exchange buffer in front of it)",
                 "algorithmic_bytes_per_launch": pair_bytes, "ms_per_launch": pair_ms,
                 "finish_kernel_ms": finish_ms,

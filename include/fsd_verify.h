@@ -27,8 +27,8 @@
  *     "host".  The library allocates no device memory: scratch space is the caller's
  *     `workspace`, sized by fsd_workspace_bytes().
  *   - Logit tensors are row-major and contiguous, both of the dtype named in the
- *     options.  Rows whose byte length is a multiple of 16 with 16-byte aligned bases
- *     take the vectorised kernels; any other shape takes a slower scalar kernel.
+ *     options.  Any vocabulary size and any element-aligned base is streamed; rows whose
+ *     byte length is a multiple of 16 with 16-byte aligned bases need no shifting on the way.
  *   - Calls are asynchronous on `stream` (a cudaStream_t passed as void*; NULL is the
  *     default stream).  Outputs are valid once the stream has been synchronised.
  *   - The return value is a host-side status: FSD_OK (0) or a negative FSD_ERR_*.
@@ -171,7 +171,7 @@ int fsd_verify_chain_host(const void *h_target_logits, const void *h_draft_logit
  * device budget is already handed out.  Such a caller has no buffer to pass as `workspace` and
  * cannot call cudaMalloc to get one.  This variant computes exactly what fsd_verify_chain
  * computes, with the same kernels, but keeps the per-position scratch (accept bits, status words
- * and the 592-byte record of each position) in a fixed array that is part of the library's device image, so the caller passes only inputs and
+ * and the 736-byte record of each position) in a fixed array that is part of the library's device image, so the caller passes only inputs and
  * outputs.  It calls no cudaMalloc, cudaFree or any other allocating routine.
  *
  * Limits and rules

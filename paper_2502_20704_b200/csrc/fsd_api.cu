@@ -18,8 +18,8 @@ namespace {
 using namespace fsd;
 
 constexpr size_t kAlign = 256;
-constexpr int kMaxVirtualCtas = 512;                                   // two per SM
-constexpr size_t kExchangeBytes = 2 * kMaxVirtualCtas * sizeof(GroupMsg);
+constexpr int kMaxBlocks = 256;                                        // of the streaming kernel (one per SM)
+constexpr size_t kExchangeBytes = 2 * kMaxBlocks * sizeof(GroupMsg);
 inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 inline bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 
@@ -85,68 +85,81 @@ std::atomic<int> g_group_size{0};            // see fsd_set_group_size
 // ---- streaming kernel launch -----------------------------------------------------------
 constexpr int kMaxDev = 64;
 
-// One CTA of two virtual CTAs per SM, all resident (cooperative launch).  Puts nothing on a stream.
-template <int DT, int DIV>
+// One block per SM, all resident (cooperative launch).  Puts nothing on a stream.
+template <int DT, int DIV, bool RAGGED>
 int prepare_stream(int dev) {
     static bool ready[kMaxDev] = {};
     static std::mutex mu;
-    auto kernel = fsd_pair_stream_kernel<DT, DIV>;
+    auto kernel = fsd_pair_stream_kernel<DT, DIV, RAGGED>;
     if (dev < 0 || dev >= kMaxDev) return FSD_ERR_CUDA;
     std::lock_guard<std::mutex> lock(mu);
     if (!ready[dev]) {
-        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(kStreamSmemBytes)) != cudaSuccess)
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kStreamSmemBytes)) != cudaSuccess)
             return FSD_ERR_CUDA;
-        int per = 0;                                 // one CTA must fit an SM, or the cooperative launch is refused
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, kStreamCtaThreads, kStreamSmemBytes) != cudaSuccess || per < 1)
+        int per = 0;                                 // one block must fit an SM, or the cooperative launch is refused
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, kStreamThreads, kStreamSmemBytes) != cudaSuccess || per < 1)
             return FSD_ERR_CUDA;
         ready[dev] = true;
     }
     return FSD_OK;
 }
 
-template <int DT, int DIV>
+template <int DT, int DIV, bool RAGGED>
 int launch_stream(const StreamParams& gp, int nsm, cudaStream_t s) {
-    // as many CTAs as give every pair a group, at most one per SM and what the exchange buffer holds
-    long long want = (static_cast<long long>(gp.n_items) * gp.C + kStreamHalves - 1) / kStreamHalves;
-    int grid = nsm;
-    if (grid > kMaxVirtualCtas / kStreamHalves) grid = kMaxVirtualCtas / kStreamHalves;
+    // as many blocks as give every pair a group, at most one per SM and what the exchange buffer holds
+    const long long want = static_cast<long long>(gp.n_items) * gp.C;
+    int grid = nsm < kMaxBlocks ? nsm : kMaxBlocks;
     if (want < grid) grid = static_cast<int>(want);
-    if (grid * kStreamHalves < gp.C) return FSD_ERR_CUDA;
+    if (grid < gp.C) return FSD_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(grid), 1, 1);
-    cfg.blockDim = dim3(kStreamCtaThreads, 1, 1);
+    cfg.blockDim = dim3(kStreamThreads, 1, 1);
     cfg.dynamicSmemBytes = kStreamSmemBytes;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;     // the groups' virtual CTAs wait for one another: all must be resident
+    attr[0].id = cudaLaunchAttributeCooperative;     // the groups' blocks wait for one another: all must be resident
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, fsd_pair_stream_kernel<DT, DIV>, gp) != cudaSuccess) return FSD_ERR_CUDA;
+    if (cudaLaunchKernelEx(&cfg, fsd_pair_stream_kernel<DT, DIV, RAGGED>, gp) != cudaSuccess) return FSD_ERR_CUDA;
     return FSD_OK;
 }
 
-// Virtual CTAs per pair for the streaming kernel; 0 if the shape is not eligible (the generic
-// kernel takes it).  Between the fewest whose slice fits on chip and kMaxGroupSize it is the size
-// with the lowest estimated time -- rounds * (fixed cost of a round +
-// cost of a ring stage * stages per slice), the two costs (3.4 and 1.07 us) measured on a B200.
-// Few pairs are spread over many virtual CTAs (short rounds); many pairs over few (fewer rounds).
-int group_size(int nvec_row, bool vec, int items, int nsm) {
-    if (!vec || nvec_row < 64) return 0;
-    const int cmin = (nvec_row + kMaxVecPerCta - 1) / kMaxVecPerCta;
+using PrepareFn = int (*)(int);
+using LaunchFn = int (*)(const StreamParams&, int, cudaStream_t);
+template <int DT> PrepareFn stream_prepare(int div, bool ragged) {
+    if (div == FSD_DIV_JS) return ragged ? prepare_stream<DT, FSD_DIV_JS, true> : prepare_stream<DT, FSD_DIV_JS, false>;
+    if (div == FSD_DIV_KL) return ragged ? prepare_stream<DT, FSD_DIV_KL, true> : prepare_stream<DT, FSD_DIV_KL, false>;
+    return ragged ? prepare_stream<DT, FSD_DIV_TV, true> : prepare_stream<DT, FSD_DIV_TV, false>;
+}
+template <int DT> LaunchFn stream_launch(int div, bool ragged) {
+    if (div == FSD_DIV_JS) return ragged ? launch_stream<DT, FSD_DIV_JS, true> : launch_stream<DT, FSD_DIV_JS, false>;
+    if (div == FSD_DIV_KL) return ragged ? launch_stream<DT, FSD_DIV_KL, true> : launch_stream<DT, FSD_DIV_KL, false>;
+    return ragged ? launch_stream<DT, FSD_DIV_TV, true> : launch_stream<DT, FSD_DIV_TV, false>;
+}
+
+// Blocks per pair for the streaming kernel; 0 if the row is too long for the largest group (the
+// generic kernel takes it).  Between the fewest whose slice fits on chip and kMaxGroupSize it is the
+// size with the lowest estimated time -- rounds * (fixed cost of a round + cost of a step * steps a
+// warp has), or half a round and half an exchange where that is longer (the totals are needed two
+// rounds on).  The constants (microseconds) are measured on a B200.
+template <int DT>
+int group_size(int nvec_row, int items, int nsm) {
+    using S = StreamShape<DT>;
+    const int cmin = (nvec_row + S::kBlockVecs - 1) / S::kBlockVecs;
     const int forced = g_group_size.load();
-    if (forced >= cmin && forced <= kMaxGroupSize && cmin <= kMaxGroupSize) return forced;
-    int vctas = kStreamHalves * nsm;
-    if (vctas > kMaxVirtualCtas) vctas = kMaxVirtualCtas;
+    const int blocks = nsm < kMaxBlocks ? nsm : kMaxBlocks;
+    if (forced >= cmin && forced <= kMaxGroupSize && forced <= blocks) return forced;
     int best = 0;
     double best_cost = 0.0;
-    for (int C = cmin; C <= kMaxGroupSize && C <= vctas; ++C) {
-        const int groups = vctas / C;
+    for (int C = cmin; C <= kMaxGroupSize && C <= blocks; ++C) {
+        const int groups = blocks / C;
         const int rounds = (items + groups - 1) / groups;
         const int slice = (nvec_row + C - 1) / C;
-        const int stages = (slice + kStageVecs - 1) / kStageVecs;
-        const double cost = rounds * (3.4 + 1.07 * stages);
+        const int warp_steps = (slice + 32 * S::kVecPerStep - 1) / (32 * S::kVecPerStep);     // of a block
+        double round = 0.3 + 0.4 * warp_steps / kComputeWarps;
+        if (round < 0.5 * (round + 1.6)) round = 0.5 * (round + 1.6);
+        const double cost = rounds * round;
         if (best == 0 || cost < best_cost) { best = C; best_cost = cost; }
     }
     return best;
@@ -155,34 +168,39 @@ int group_size(int nvec_row, bool vec, int items, int nsm) {
 template <int DT>
 int launch_all(const PairParams& pp, FinishParams fp, bool vec, int* flags, GroupMsg* exchange, PairRecord* records, cudaStream_t s) {
     const int items = pp.B * pp.G;
-    const int nvec_row = pp.V / Logit<DT>::kPerVec;
     int dev = 0, nsm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1)
         return FSD_ERR_CUDA;
-    const int C = group_size(nvec_row, vec, items, nsm);
+    const size_t row_bytes = static_cast<size_t>(pp.V) * Logit<DT>::kBytes;
+    // an unaligned row covers at most as many 16-byte granules as one that starts at a granule's last element
+    const size_t nvec_row = vec ? row_bytes / 16 : (row_bytes + 16 - Logit<DT>::kBytes + 15) / 16;
+    const int C = nvec_row <= static_cast<size_t>(kMaxGroupSize) * StreamShape<DT>::kBlockVecs ? group_size<DT>(static_cast<int>(nvec_row), items, nsm) : 0;
     if (C > 0) {
         StreamParams sp;
-        sp.target = pp.target; sp.draft = pp.draft; sp.parent = pp.parent; sp.B = pp.B; sp.G = pp.G;
-        sp.nvec_row = nvec_row; sp.n_items = items; sp.records = records; sp.timeout_flag = flags; sp.next_pair = flags + 1;
+        sp.target = pp.target; sp.draft = pp.draft; sp.parent = pp.parent; sp.G = pp.G;
+        sp.nvec_row = static_cast<int>(nvec_row); sp.row_bytes = row_bytes; sp.n_items = items; sp.records = records; sp.timeout_flag = flags;
         sp.C = C; sp.exchange = exchange;
-        // test aid: one virtual CTA keeps its first message to itself, so that its group's exchange
+        const int slice = static_cast<int>((nvec_row + C - 1) / C);
+        sp.slot_row_bytes = slot_row_bytes<DT>(slice); sp.slot_bytes = slot_bytes<DT>(slice, !vec);
+        sp.ring = kRingBytes / sp.slot_bytes < kMaxRing ? kRingBytes / sp.slot_bytes : kMaxRing;
+        // item / G by a multiplication: with 2^(l-1) < G <= 2^l, ceil(2^(31+l) / G) is exact for items below 2^31
+        int l = 0;
+        while ((1ll << l) < pp.G) ++l;
+        sp.g_magic = l == 0 ? 0u : static_cast<uint32_t>(((1ull << (31 + l)) + pp.G - 1) / pp.G);
+        sp.g_shift = l == 0 ? 0u : static_cast<uint32_t>(l - 1);
+        // test aid: one block keeps its first message to itself, so that its group's exchange
         // runs out (after a shorter limit: about a tenth of a second) and the kernel's own give-up path runs
         const bool silent = g_mark_timeout.load() == 2;
         sp.poll_limit = silent ? (1u << 17) : kSpinLimit;
         sp.silent_rank = silent ? C - 1 : -1;
         // everything that can fail without a launch (attributes, the occupancy query) comes before
         // the first thing put on the stream
-        int rc;
-        if (pp.div == FSD_DIV_JS)      rc = prepare_stream<DT, FSD_DIV_JS>(dev);
-        else if (pp.div == FSD_DIV_KL) rc = prepare_stream<DT, FSD_DIV_KL>(dev);
-        else                           rc = prepare_stream<DT, FSD_DIV_TV>(dev);
+        int rc = stream_prepare<DT>(pp.div, !vec)(dev);
         if (rc != FSD_OK) return rc;
-        // the flag block and the exchange buffer start every call at zero: flags [0] timeout, [1] pairs handed out
+        // the flag block and the exchange buffer start every call at zero: flags [0] timeout
         if (cudaMemsetAsync(flags, 0, kAlign + kExchangeBytes, s) != cudaSuccess) return FSD_ERR_CUDA;
-        if (pp.div == FSD_DIV_JS)      rc = launch_stream<DT, FSD_DIV_JS>(sp, nsm, s);
-        else if (pp.div == FSD_DIV_KL) rc = launch_stream<DT, FSD_DIV_KL>(sp, nsm, s);
-        else                           rc = launch_stream<DT, FSD_DIV_TV>(sp, nsm, s);
+        rc = stream_launch<DT>(pp.div, !vec)(sp, nsm, s);
         if (rc != FSD_OK) return rc;
         // test aid: behave as if a bounded wait of the streaming kernel had run out
         if (g_mark_timeout.load() == 1 && cudaMemsetAsync(flags, 1, sizeof(int), s) != cudaSuccess) return FSD_ERR_CUDA;
@@ -479,7 +497,7 @@ int fsd_set_timeout_injection(int mode) {
 }
 
 int fsd_set_group_size(int group_size) {
-    if (group_size < 0 || group_size > kMaxGroupSize) return FSD_ERR_SHAPE;
+    if (group_size < 0 || group_size > 16) return FSD_ERR_SHAPE;
     g_group_size.store(group_size);
     return FSD_OK;
 }

@@ -174,56 +174,40 @@ struct PairTotals {
 __device__ __forceinline__ double pow2_int_d(double d) {
     return d < -1022.0 ? 0.0 : __hiloint2double((1023 + static_cast<int>(d)) << 20, 0);
 }
-__device__ __forceinline__ double group_sum(double v) {       // over the kMaxGroupSize lanes of a record
-#pragma unroll
-    for (int m = kMaxGroupSize / 2; m > 0; m >>= 1) v += __shfl_xor_sync(0xffffffffu, v, m);
-    return v;
-}
-// Called by all 32 lanes: lane 16*q + r folds part r of the record `rec` of group q (null: no
-// record for this group); every lane of a group returns the group's totals.
+// Called by all 32 lanes: lane r folds part r of the record; every lane returns the totals.
 __device__ inline PairTotals fold_record(const PairRecord* rec, int div) {
-    const int r = threadIdx.x & (kMaxGroupSize - 1);
+    static_assert(kMaxGroupSize <= 32, "one lane per part");
+    const int r = threadIdx.x & 31;
     PairTotals t;
     t.state = 0;
     Stats c;
     c.ka = -INFINITY; c.kb = -INFINITY; c.za = 0.f; c.zb = 0.f; c.s0 = 0.f; c.sb = 0.f; c.x = 0.f; c.diff = 0;
     float x = 0.f;
-    if (rec != nullptr) {
-        // every lane fetches its part at once with the count (one trip to L2); parts beyond the count are stale
-        const Stats cr = rec->part[r];
-        const float xr = rec->x[r];
-        t.state = rec->state;
-        if (r < static_cast<int>(rec->ncta)) { c = cr; x = xr; }
-    }
-    float ka = c.ka, kb = c.kb;                          // NaN references win
-#pragma unroll
-    for (int m = kMaxGroupSize / 2; m > 0; m >>= 1) {
-        const float oa = __shfl_xor_sync(0xffffffffu, ka, m), ob = __shfl_xor_sync(0xffffffffu, kb, m);
-        ka = (oa != oa || ka != ka) ? __int_as_float(0x7fc00000) : fmaxf(ka, oa);
-        kb = (ob != ob || kb != kb) ? __int_as_float(0x7fc00000) : fmaxf(kb, ob);
-    }
+    // every lane fetches its part at once with the count (one trip to L2); parts beyond the count are stale
+    const int rr = r < kMaxGroupSize ? r : 0;
+    const Stats cr = rec->part[rr];
+    const float xr = rec->x[rr];
+    t.state = rec->state;
+    if (r < static_cast<int>(rec->ncta) && r < kMaxGroupSize) { c = cr; x = xr; }
+    const float ka = warp_redux_max_nan(c.ka), kb = warp_redux_max_nan(c.kb);      // NaN references win
     t.ka = ka; t.kb = kb;
     const double da = c.ka == -INFINITY ? 0.0 : static_cast<double>(c.ka) - ka;
     const double db = c.kb == -INFINITY ? 0.0 : static_cast<double>(c.kb) - kb;
     const double fa = (c.ka == -INFINITY || da != da) ? 0.0 : pow2_int_d(da);
     const double fb = (c.kb == -INFINITY || db != db) ? 0.0 : pow2_int_d(db);
-    t.Za = group_sum(fa * c.za); t.Zb = group_sum(fb * c.zb);
+    t.Za = warp_sum(fa * c.za); t.Zb = warp_sum(fb * c.zb);
     t.Sa = 0.0; t.Sb = 0.0; t.K = 0.0;
     if (div == FSD_DIV_KL) {
         const bool inf = c.s0 == INFINITY;
         const double k = inf ? 0.0 : fa * (static_cast<double>(c.s0) + (da - db) * c.za);
-        t.K = group_sum(k);
-        const unsigned any_inf = __ballot_sync(0xffffffffu, inf) >> (threadIdx.x & 16) & 0xffffu;
-        if (any_inf) t.K = static_cast<double>(INFINITY);
+        t.K = warp_sum(k);
+        if (__any_sync(0xffffffffu, inf)) t.K = static_cast<double>(INFINITY);
     } else {
-        t.Sa = group_sum(fa * (static_cast<double>(c.s0) + da * c.za));
-        t.Sb = group_sum(fb * (static_cast<double>(c.sb) + db * c.zb));
+        t.Sa = warp_sum(fa * (static_cast<double>(c.s0) + da * c.za));
+        t.Sb = warp_sum(fb * (static_cast<double>(c.sb) + db * c.zb));
     }
-    t.X = group_sum(static_cast<double>(x));
-    uint32_t df = c.diff;
-#pragma unroll
-    for (int m = kMaxGroupSize / 2; m > 0; m >>= 1) df |= __shfl_xor_sync(0xffffffffu, df, m);
-    t.differ = df;
+    t.X = warp_sum(static_cast<double>(x));
+    t.differ = __any_sync(0xffffffffu, c.diff != 0) ? 1u : 0u;
     return t;
 }
 
@@ -380,15 +364,14 @@ __global__ void __launch_bounds__(kFinishThreads, 2) fsd_finish_kernel(FinishPar
     int st = 0, first = G;
     if (tid == 0 && P.timeout_flag != nullptr && *reinterpret_cast<const volatile int*>(P.timeout_flag) != 0) st |= FSD_ROW_TIMEOUT;
     if (P.records != nullptr) {
-        // two pairs per warp: sixteen lanes fold a pair's record, the first of them judges it
-        for (int i0 = 2 * warp; i0 < G; i0 += 2 * (blockDim.x >> 5)) {
-            const int i = i0 + (lane >> 4);
+        // a pair per warp: its lanes fold the parts of the pair's record, the first of them judges it
+        for (int i = warp; i < G; i += blockDim.x >> 5) {
             const int item = b * G + i;
-            const PairTotals tot = fold_record(i < G ? P.records + item : nullptr, P.div);
+            const PairTotals tot = fold_record(P.records + item, P.div);
             // the two logarithms the judgement needs, by two lanes at once
-            const double lz = log((lane & 15) == 1 ? tot.Zb : tot.Za);
+            const double lz = log(lane == 1 ? tot.Zb : tot.Za);
             const double lnZa = lz, lnZb = __shfl_down_sync(0xffffffffu, lz, 1);
-            if (i < G && (lane & 15) == 0) {
+            if (lane == 0) {
                 int trow = i;
                 if (tree) {
                     const int par = P.parent[item];

@@ -1,60 +1,66 @@
 // Streaming per-(row, position) kernel: every logit is read from HBM once.
 //
-// A (row, position) pair is split along the vocabulary over a GROUP of C virtual CTAs (C <= 16,
-// chosen by the host from the slice that fits on chip and the number of pairs).  A CTA of 512
-// threads, one per SM, holds two virtual CTAs of 256 threads, each with its own half of the SM's
-// tensor memory, its own shared-memory ring and its own named barriers; the two belong to
-// different groups, so that one computes while the other waits for its group.  The launch is
-// cooperative (all CTAs resident: the virtual CTAs of a group wait for one another) and the groups
-// are persistent: they claim pairs from a shared counter.  Per pair, each virtual CTA
-//   1. receives its slice of both rows in shared memory through a ring of bulk asynchronous
-//      copies (cp.async.bulk + mbarrier).  A warp releases a slot as soon as its vectors are in
-//      registers; the slot is refilled one stage later by a rotating duty warp, so the next
-//      pair's slices stream in while this pair is finished and nobody waits for a slot to drain;
-//   2. sweeps each stage once as it lands: e = 2^(logit * log2e - k) with one MUFU ex2 per
-//      logit, the sums Z = sum e and S = sum e*y (or the KL sum), a bitwise "rows differ" flag,
-//      and parks the e values in tensor memory (128 per thread) and registers (32).  k is a
-//      per-thread integer reference in the log2 domain, taken from the thread's first finite
-//      logits and moved -- with an exact power-of-two rescale of what has been summed and parked
-//      -- only if a later logit exceeds it by more than 2^30, so no separate maximum pass over
-//      the slice is needed and every change of reference is exact;
-//   3. combines (k, Z, S) over threads and warps; one combiner warp per virtual CTA (rotating)
-//      folds the warps' statistics, leaves them as a tagged message in global memory, fetches the
-//      messages of the whole group (they live in L2), folds those and wakes the virtual CTA
-//      (named barriers: waiting warps issue nothing);
-//   4. sweeps the parked e values: p = e_a/Z_a, q = e_b/Z_b; JS needs sum (p+q) log2(p+q) (one
-//      MUFU lg2 per pair), TV needs sum |p - q|; KL needs no second sweep.
-// The group's rank-0 virtual CTA leaves all members' statistics in the pair's record; the finish
-// kernel folds them in double precision and turns them into divergences and accept bits, so no
-// double-precision arithmetic runs here.  HBM traffic is the algorithmic minimum.  The
-// special-function pipe (1 ex2 per logit + 1 lg2 per pair) and instruction issue are the
-// co-bottlenecks, which is why e values are kept rather than recomputed, and why a thread
-// owns two vectors per row and stage (independent work to overlap its own latencies) with 512
-// threads of 128 registers per SM.  Groups need no co-scheduling on neighbouring SMs, so every
-// SM is used whatever C is.
+// A (row, position) pair is split along the vocabulary over a GROUP of C thread blocks (C <= 20,
+// chosen by the host from what fits on chip and the number of pairs), one block of sixteen compute
+// warps and one helper warp per SM.  The launch is cooperative (all blocks resident: the blocks of a
+// group wait for one another) and the groups are persistent: group g takes pairs g, g + groups, ...
+//
+// A block's slice of a pair's two rows arrives in a ring of shared-memory slots (bulk asynchronous
+// copies started by the helper warp; the ring is as deep as the slices allow, three slots at least).
+// The compute warps are independent of one another: a warp owns a fixed run of the slice's 16-byte
+// vectors (at most four steps of eight entries a lane), and in round n it does, step by step,
+//   1. the first sweep of pair n: e = 2^(logit * log2e - k), the sums Z = sum e and S = sum e*y (or
+//      the KL sum), a bitwise "rows differ" flag.  The references k (integers in the log2 domain) come
+//      from the maxima of the part's first step, looked at a round earlier.  That is near enough for
+//      any ordinary logits; a warp whose sums say it was not (a later logit 2^30 above it, a -inf in
+//      the entropy sums) does the sweep over with exact maxima and clamped logits;
+//   2. interleaved with it, the SECOND sweep of pair n - 2 over the e values parked two rounds
+//      earlier: p = e_a/Z_a, q = e_b/Z_b, JS needs sum (p+q) log2(p+q), TV sum |p - q|, KL nothing.
+//      The new e values take the tensor-memory columns the old ones leave (64 values a lane and pair,
+//      two pairs in flight, 128 columns a warp: all of the SM's tensor memory);
+//   3. a fold of its five sums over its lanes, posted for the helper warp.
+// The helper warp folds the sixteen warps' sums, leaves them as a tagged message in global memory,
+// fetches the messages of the whole group (they live in L2), folds those and hands 1/Z_a, 1/Z_b to
+// its block.  That exchange has a whole round's time: the totals of pair n are needed in round n + 2.
+//
+// What bounds it.  JS takes three special-function results per vocabulary entry (two ex2, one lg2):
+// 512 pairs of 152064 entries are 50 us of that pipe on 148 SMs at 1965 MHz, and 48 us of HBM.  The
+// kernel takes 92 us there (3.4 TB/s; the form in which all warps of a block waited for the group's
+// totals between the two sweeps of a pair took 127 us): 40 rounds of 2.0 us, of which the sweeps are
+// two thirds, the wait for data and totals a sixth, the fold a seventh, plus 3.5 us until the first
+// slices have landed.  KL has no second sweep and no exchange and runs at 4.7 TB/s.  Of what was
+// tried on it: ex2 on the FMA pipe for a part of the entries (+8 %, the extra instructions cost more
+// than the special-function pipe gains), five and more pairs in flight in smaller parts (more rounds,
+// the fold weighs more), reading the references from a full pass over the part (+1 %).
+//
+// Rows that are not whole 16-byte vectors (or start off a 16-byte boundary) are streamed as the
+// aligned 16-byte granules that cover them; the draft row's granules are shifted onto the target
+// row's in registers and the entries in front of and behind the rows are read as -inf.  A granule
+// that holds at least one byte of a row never crosses into another page.
 #pragma once
+
+#include <climits>
+#include <cstddef>
+#include <type_traits>
 
 #include "fsd_device.cuh"
 
 namespace fsd {
 
-constexpr int kStreamThreads = 256;
-constexpr int kStreamWarps = kStreamThreads / 32;
-constexpr int kRing = 6;                                   // stages in the shared-memory ring
-constexpr int kVecPerThread = 2;                           // 16-byte vectors per thread, row and stage
-constexpr int kStageVecs = kStreamThreads * kVecPerThread; // vectors per row and stage
-constexpr int kStageRowBytes = kStageVecs * 16;
-constexpr int kStageBytes = 2 * kStageRowBytes;
-constexpr int kMaxStagesPerPair = kRing - 1;               // stages of e values a thread can park (4 in tensor memory, 1 in registers)
-constexpr int kTmemCols = 256;                             // per virtual CTA: 8 warps -> 2 per lane quarter x 128 columns
-constexpr int kTmemPerThread = 128;
-constexpr int kMaxVecPerCta = kMaxStagesPerPair * kStageVecs;
-constexpr int kMaxClusterSize = 8;                        // finish kernel (portable size)
-constexpr int kMaxGroupSize = 16;                      // most virtual CTAs in a group of the streaming kernel
+constexpr int kComputeWarps = 16;
+constexpr int kStreamThreads = 32 * (kComputeWarps + 1);   // and one helper warp
+constexpr int kMaxSteps = 4;                               // steps a warp parks per pair; two pairs in flight fill its 128 tensor-memory columns
+constexpr int kStepEntries = 8;                            // vocabulary entries a lane handles per step
+constexpr int kTmemCols = 512;                             // all of the SM's columns: warp w owns 32 lanes x 128 columns
+constexpr int kParkCols = 2 * kStepEntries;                // e values a lane parks per step (both rows)
+constexpr int kMaxClusterSize = 8;                         // finish kernel (portable size)
+constexpr int kMaxGroupSize = 20;                          // most blocks in a group of the streaming kernel
 constexpr uint32_t kSpinLimit = 1u << 24;                  // polls before a wait gives up
+constexpr uint64_t kWaitNs = 4000000000ull;                // and its limit in time
+constexpr uint32_t kSleepNs = 40;                          // sleep between two polls of a barrier in shared memory
 
-// Partial statistics of one (target row, draft row) pair: of a warp, of a virtual CTA, or -- in a
-// pair's record -- of each virtual CTA of the group that streamed the pair.
+// Partial statistics of one (target row, draft row) pair: of a warp, of a block, or -- in a pair's
+// record -- of each block of the group that streamed the pair.
 //   z = sum 2^y, s = sum 2^y * y with y = logit*log2e - k and k the integer reference (log2
 //   domain) the sums are relative to.  s0 is the target row's s for JS and the KL sum
 //   sum 2^ya (ya - yb) for KL.
@@ -62,9 +68,8 @@ struct alignas(16) Stats {
     float ka, kb;              // references; -inf: no finite logit seen; NaN: a NaN logit
     float za, zb;
     float s0, sb;
-    float x;                   // second-sweep sum of the PREVIOUS pair (in flight only)
-    uint32_t diff;             // 0: the two rows are bitwise identical so far (bit 0 once a virtual CTA has folded
-                               // it; rank 0's message carries the next claimed pair id in the bits above)
+    float x;                   // second-sweep sum (in flight only)
+    uint32_t diff;             // 0: the two rows are bitwise identical so far
 };
 static_assert(sizeof(Stats) == 32, "Stats travels as two 16-byte stores");
 
@@ -72,34 +77,35 @@ static_assert(sizeof(Stats) == 32, "Stats travels as two 16-byte stores");
 // double precision (second-sweep sums: JS sum s log2 s, TV sum |p - q|).
 struct alignas(16) PairRecord {
     Stats part[kMaxGroupSize];
-    float x[kMaxGroupSize];  // each virtual CTA's second-sweep sum of this pair
+    float x[kMaxGroupSize];    // each block's second-sweep sum of this pair
     uint32_t ncta;             // parts in use
     uint32_t state;            // kRecordStats | kRecordBadTree
     uint32_t pad[2];
 };
-static_assert(sizeof(PairRecord) == 592, "PairRecord layout");
+static_assert(sizeof(PairRecord) == 736, "PairRecord layout");
 constexpr uint32_t kRecordStats = 1, kRecordBadTree = 2;
 
-// One virtual CTA's statistics of a round as they cross global memory: three 16-byte units, each
-// stored whole and ending in the round's tag, so that a reader knows a unit is this round's
-// without any fence or flag (a unit whose tag is older is fetched again).
+// One block's statistics of a round as they cross global memory: 16-byte units, each stored whole
+// and ending in the round's tag, so that a reader knows a unit is this round's without any fence or
+// flag (a unit whose tag is older is fetched again).
 struct alignas(16) GroupMsg {
-    uint4 u[3];                // {ka, kb, za, tag}, {zb, s0, sb, tag}, {x, diff | next pair id << 1, 0, tag}
-    uint4 pad;
+    uint4 u[2];                // {ka, kb, za, tag}, {zb, 0, 0, tag}
 };
-static_assert(sizeof(GroupMsg) == 64, "GroupMsg layout");
+static_assert(sizeof(GroupMsg) == 32, "GroupMsg layout");
 
 struct StreamParams {
     const void* target;        // [B, G+1, V]
     const void* draft;         // [B, G,   V]
     const int32_t* parent;     // [B, G] (tree) or null (chain)
-    int B, G;
-    int nvec_row;              // 16-byte vectors per logit row
+    int G;
+    uint32_t g_magic, g_shift; // item / G == umulhi(item, g_magic) >> g_shift for items below 2^31
+    int nvec_row;              // 16-byte vectors (granules of an unaligned row, at most) per logit row
+    size_t row_bytes;
+    int slot_row_bytes, slot_bytes, ring;    // of the shared-memory ring (see slot_bytes())
     int n_items;               // B * G
     PairRecord* records;       // [B * G]
     int* timeout_flag;         // set to 1 if a bounded wait ran out; zero at launch
-    int* next_pair;            // pairs handed out beyond each group's fixed first ones; zero at launch
-    int C;                     // virtual CTAs per group (<= kMaxGroupSize)
+    int C;                     // blocks per group (<= kMaxGroupSize)
     uint32_t poll_limit;       // fetches of the group's messages before the exchange gives up (kSpinLimit normally)
     int silent_rank;           // test aid: this rank of group 0 keeps its first message to itself (-1: nobody)
     GroupMsg* exchange;        // [groups][2][C], zero at launch
@@ -126,63 +132,62 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
         : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
     return ok != 0;
 }
-// Bounded wait: returns false (and raises the flag) if the phase never completes.  Once a
-// wait of this thread has run out (`dead`), later waits return at once: the results are
-// already marked invalid and the kernel only has to reach its end.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* timeout_flag, bool& dead) {
-    if (dead) return false;
-#pragma unroll 1
-    for (uint32_t i = 0; i < kSpinLimit; ++i) {
-        if (mbar_try_wait(bar, parity)) return true;
-        // somebody has given up already: nothing this thread waits for is certain to come
-        if ((i & 1023u) == 1023u && *reinterpret_cast<volatile int*>(timeout_flag) != 0) break;
-    }
-    atomicExch(timeout_flag, 1);
-    dead = true;
-    return false;
-}
 __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
 }
 
-template <int N> __device__ __forceinline__ void tmem_st(uint32_t taddr, const float (&r)[N]);
-template <> __device__ __forceinline__ void tmem_st<16>(uint32_t taddr, const float (&r)[16]) {
+__device__ __forceinline__ uint64_t global_ns() {
+    uint64_t t;
+    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+    return t;
+}
+// Bounded wait of a whole warp for a phase of an mbarrier: kSpinLimit polls or kWaitNs, whatever is
+// first.  False (for every lane) and the flag raised if the phase never completes or somebody else's
+// wait has run out already.
+__device__ __noinline__ bool warp_wait_slow(uint64_t* bar, uint32_t parity, int* timeout_flag) {
+    uint64_t t0 = 0;
+#pragma unroll 1
+    for (uint32_t i = 0; i < kSpinLimit / 64; ++i) {
+#pragma unroll 1
+        for (int k = 0; k < 64; ++k) {
+            if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+            __nanosleep(kSleepNs);                   // (the warps that have work keep the issue slots)
+        }
+        // somebody has given up already: nothing this warp waits for is certain to come
+        const uint64_t t = global_ns();
+        if (t0 == 0) t0 = t;
+        if (__any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(timeout_flag) != 0 || t - t0 > kWaitNs)) break;
+    }
+    if ((threadIdx.x & 31) == 0) atomicExch(timeout_flag, 1);
+    return false;
+}
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, int* timeout_flag) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    return warp_wait_slow(bar, parity, timeout_flag);
+}
+
+// tensor memory: 16 columns of this warp's 32 lanes, one value a lane and column
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&r)[16]) {
     asm volatile(
         "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
         ::"r"(taddr), "f"(r[0]), "f"(r[1]), "f"(r[2]), "f"(r[3]), "f"(r[4]), "f"(r[5]), "f"(r[6]), "f"(r[7]),
-        "f"(r[8]), "f"(r[9]), "f"(r[10]), "f"(r[11]), "f"(r[12]), "f"(r[13]), "f"(r[14]), "f"(r[15]) : "memory");
+        "f"(r[8]), "f"(r[9]), "f"(r[10]), "f"(r[11]), "f"(r[12]), "f"(r[13]), "f"(r[14]), "f"(r[15]));
 }
-template <> __device__ __forceinline__ void tmem_st<8>(uint32_t taddr, const float (&r)[8]) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
-                 ::"r"(taddr), "f"(r[0]), "f"(r[1]), "f"(r[2]), "f"(r[3]), "f"(r[4]), "f"(r[5]), "f"(r[6]), "f"(r[7])
-                 : "memory");
-}
-template <int N> __device__ __forceinline__ void tmem_ld(uint32_t taddr, float (&r)[N]);
-template <> __device__ __forceinline__ void tmem_ld<16>(uint32_t taddr, float (&r)[16]) {
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&r)[16]) {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
         : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7]),
           "=f"(r[8]), "=f"(r[9]), "=f"(r[10]), "=f"(r[11]), "=f"(r[12]), "=f"(r[13]), "=f"(r[14]), "=f"(r[15])
-        : "r"(taddr) : "memory");
+        : "r"(taddr));
 }
-template <> __device__ __forceinline__ void tmem_ld<8>(uint32_t taddr, float (&r)[8]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7])
-                 : "r"(taddr) : "memory");
-}
-__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // NaN-propagating maxima: a NaN logit must reach the row maximum so that the row is flagged
 __device__ __forceinline__ uint32_t bf16x2_max_nan(uint32_t a, uint32_t b) {
     uint32_t d;
     asm("max.NaN.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
-    return d;
-}
-__device__ __forceinline__ uint32_t bf16x2_max(uint32_t a, uint32_t b) {
-    uint32_t d;
-    asm("max.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
     return d;
 }
 __device__ __forceinline__ float fmax_nan(float a, float b) {
@@ -231,55 +236,25 @@ __device__ __forceinline__ float pow2_int(float d) {
     return d < -126.f ? 0.f : __int_as_float((static_cast<int>(d) + 127) << 23);
 }
 
-// ---- in-stream references ---------------------------------------------------------------------
-// A thread keeps, per row, the largest logit its reference may meet without moving: bf16 rows
-// hold it as a packed pair so that one packed maximum tests a whole vector.  -1e30 is what -inf
-// logits are read as, so "nothing finite seen yet" is a limit of exactly that.
-template <int DT> __device__ __forceinline__ uint32_t unset_limit() {
-    return DT == FSD_BF16 ? 0xF149F149u : __float_as_uint(-1.0e30f);
+// 2^(k - K) for integer-valued k <= K, exact; 0 below the normal range, for k = -inf ("no reference"), and where
+// either is NaN (the sums it scales are NaN then)
+__device__ __forceinline__ float pow2_ref(float k, float K) {
+    return __int_as_float(__float_as_int(fmaxf(k - K, -127.f) + 12583039.f) << 23);      // 1.5 * 2^23 + 127: the low bits are the exponent field
 }
-// limit for a reference taken from maximum m: m + 30 ln 2, rounded to the row's type (rounding
-// can add at most another 30 ln 2 before it snaps back to m itself, so 2^y stays below 2^61)
-template <int DT> __device__ __forceinline__ uint32_t reference_limit(float m) {
-    const float lim = m + 20.7944f;
-    if constexpr (DT == FSD_BF16) {
-        uint32_t r;
-        asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(lim), "f"(lim));
-        return r;
-    } else {
-        return __float_as_uint(lim);
-    }
+__device__ __forceinline__ float rcp(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
 }
-// Multiplies the e values a warp has parked in tensor memory for stages 0..n-1 by fa (first
-// half of each stage: target row) and fb (second half: draft row).  Warp-collective.
-template <int EPT>
-__device__ __noinline__ void rescale_parked(uint32_t taddr, int n, float fa, float fb) {
-    tmem_wait_st();
-    for (int t = 0; t < n; ++t) {
-        float e[EPT];
-        tmem_ld<EPT>(taddr + t * EPT, e);
-        tmem_wait_ld();
-#pragma unroll
-        for (int j = 0; j < EPT / 2; ++j) { e[j] *= fa; e[EPT / 2 + j] *= fb; }
-        tmem_st<EPT>(taddr + t * EPT, e);
-    }
-    tmem_wait_st();
+// maximum over the warp, NaN if any lane holds one
+__device__ __forceinline__ float warp_redux_max_nan(float v) {
+    float d;
+    asm volatile("redux.sync.max.NaN.f32 %0, %1, 0xffffffff;" : "=f"(d) : "f"(v));
+    return d;
 }
-
 // A KL partial sum brought to another reference: +inf (a logit with p > 0 = q) stays +inf even
 // when the factor underflows to 0
 __device__ __forceinline__ float scale_kl(float f, float v) { return v == INFINITY ? v : f * v; }
-
-// Named barriers of one virtual CTA: waiting warps issue nothing.  `arrive` counts the warp in
-// without waiting; `sync` waits until kStreamThreads threads have arrived or synced.  The second
-// virtual CTA of a CTA uses ids two higher.
-__device__ __forceinline__ void named_arrive(int id) {
-    asm volatile("bar.arrive %0, %1;" ::"r"(id), "n"(kStreamThreads) : "memory");
-}
-__device__ __forceinline__ void named_sync(int id) {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(kStreamThreads) : "memory");
-}
-constexpr int kBarPosted = 1, kBarTotals = 2;
 
 // One unit is stored and fetched as a single 128-bit access (the .b128 forms: one access, not four
 // that happen to be adjacent), so a reader sees a unit either whole or not at all.
@@ -294,538 +269,597 @@ __device__ __forceinline__ uint4 ld_unit(const uint4* p) {
     return make_uint4(static_cast<uint32_t>(lo), static_cast<uint32_t>(lo >> 32), static_cast<uint32_t>(hi), static_cast<uint32_t>(hi >> 32));
 }
 
-// ---- shared-memory layout ---------------------------------------------------------------
-struct StreamShared {
-    uint64_t full[kRing];      // a ring stage has landed
-    uint64_t empty[kRing];     // every warp has finished reading the slot's current stage
-    uint32_t armed[kRing];     // copies started into each ring slot so far (the last one is waited for before leaving)
-    int items[8];              // pair ids of this group's rounds, indexed by round & 7
-    alignas(16) float tot[4];  // group totals of the current pair: Ka, Kb, Za, Zb
-    Stats ws[kStreamWarps];    // the warps' statistics of the current pair
-};
-constexpr int kStreamHalves = 2;                            // virtual CTAs per CTA
-constexpr int kStreamCtaThreads = kStreamHalves * kStreamThreads;
-constexpr size_t kStreamHalfBytes = kRing * kStageBytes + ((sizeof(StreamShared) + 127) / 128) * 128;
-constexpr size_t kStreamSmemBytes = kStreamHalves * kStreamHalfBytes + 128 + 16;
+// 16-byte accesses of shared memory by address
+__device__ __forceinline__ uint4 ld_shared16(uint32_t addr) {
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
+    return v;
+}
+__device__ __forceinline__ void st_shared16(uint32_t addr, const uint4& v) {
+    asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w));
+}
 
-template <int DT, int DIV>
-__global__ void __launch_bounds__(kStreamCtaThreads, 1) fsd_pair_stream_kernel(StreamParams P) {
+// ---- shared-memory layout ---------------------------------------------------------------
+// A ring of slots, each holding the block's slice of one pair: the target row's vectors (whole steps),
+// then the draft row's.  The draft part of an unaligned row is copied warp by warp, each part one granule longer
+// (its last vector straddles two), so there the parts lie a granule further apart.
+template <int DT> struct StreamShape {
+    static constexpr int kVecPerStep = kStepEntries / Logit<DT>::kPerVec;   // 16-byte vectors a lane handles per step and row
+    static constexpr int kSteps = DT == FSD_BF16 ? 4 : 2;                   // most steps of a warp's part: 2 KB of each row
+    static constexpr int kWarpVecs = 32 * kVecPerStep * kSteps;
+    static constexpr int kBlockVecs = kComputeWarps * kWarpVecs;
+    static constexpr int kStepVecs = 32 * kVecPerStep;
+};
+static_assert(StreamShape<FSD_BF16>::kSteps <= kMaxSteps && StreamShape<FSD_F32>::kSteps <= kMaxSteps, "two parts fit a warp's tensor memory");
+constexpr int kRingBytes = 224 * 1024;                     // shared memory for the ring (two slots are in use, the rest in flight)
+constexpr int kMaxRing = 8, kMinRing = 3;
+// bytes from a slot's start to its draft part, and of a whole slot, for slices of up to `slice` vectors
+template <int DT> constexpr int slot_row_bytes(int slice) {
+    return (slice + StreamShape<DT>::kStepVecs - 1) / StreamShape<DT>::kStepVecs * StreamShape<DT>::kStepVecs * 16;
+}
+template <int DT> constexpr int slot_bytes(int slice, bool ragged) { return 2 * slot_row_bytes<DT>(slice) + (ragged ? kComputeWarps * 16 : 0); }
+static_assert(kMinRing * slot_bytes<FSD_BF16>(StreamShape<FSD_BF16>::kBlockVecs, true) <= kRingBytes &&
+              kMinRing * slot_bytes<FSD_F32>(StreamShape<FSD_F32>::kBlockVecs, true) <= kRingBytes, "the largest slices have three slots");
+
+// A warp's part of the block's slice: whole steps, dealt out as evenly as they go.  The warps that share
+// a scheduler with the helper warp get a step more last.
+struct WarpPart { int pos, first, count, steps; };     // place in the slice's order; vectors from the slice's start; steps
+__device__ __forceinline__ WarpPart warp_part(int warp, int slice, int step_vecs) {
+    WarpPart p;
+    const int all = (slice + step_vecs - 1) / step_vecs, sb = all / kComputeWarps, sr = all % kComputeWarps;
+    p.pos = (warp & 3) == 0 ? 12 + (warp >> 2) : (warp >> 2) * 3 + (warp & 3) - 1;
+    p.steps = sb + (p.pos < sr ? 1 : 0);
+    p.first = (p.pos * sb + (p.pos < sr ? p.pos : sr)) * step_vecs;
+    p.count = p.steps == 0 ? 0 : slice - p.first < p.steps * step_vecs ? slice - p.first : p.steps * step_vecs;
+    return p;
+}
+
+struct alignas(16) WarpPost {              // what a compute warp hands the helper each round (its own lanes folded)
+    float z[4];                // za, zb, s0, sb of pair n
+    float ka, kb;
+    float x;                   // second-sweep sum of pair n - 2
+    uint32_t diff;
+};
+struct StreamShared {
+    uint64_t full[kMaxRing];                     // a slot's slices have landed
+    uint64_t posted[2];                        // all compute warps have posted round n (n & 1)
+    uint64_t totals[2];                        // the helper is done with the posts of round n: totals valid, slots free
+    WarpPost post[2][kComputeWarps];
+    alignas(16) float4 tot[2];                             // Ka, 1/Za, Kb, 1/Zb of the round's pair (0: not a valid distribution)
+    uint32_t meta[kMaxRing];                     // unaligned rows: byte offset of the target row's first granule << 8 | shift of the draft row
+    uint32_t tmem_base;
+};
+static_assert(sizeof(WarpPost) == 32 && offsetof(WarpPost, ka) == 16 && offsetof(StreamShared, post) % 16 == 0 && offsetof(StreamShared, tot) % 16 == 0, "16-byte accesses");
+static_assert(alignof(StreamShared) <= 16 && kRingBytes % 16 == 0, "16-byte copies");
+constexpr size_t kStreamSmemBytes = kRingBytes + sizeof(StreamShared) + 128;
+static_assert(kStreamSmemBytes <= 227 * 1024, "shared memory of an SM");
+
+// 16 bytes starting `sh` bytes into the 32 bytes (lo, hi); sh is the same for the whole warp
+template <int DT>
+__device__ __forceinline__ uint4 shifted(const uint4& lo, const uint4& hi, uint32_t sh) {
+    uint32_t w[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+    const bool two = (sh & 8) != 0, one = (sh & 4) != 0;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) w[i] = two ? w[i + 2] : w[i];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) w[i] = one ? w[i + 1] : w[i];
+    if constexpr (DT == FSD_BF16) {
+        const uint32_t bits = (sh & 2) * 8;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) w[i] = __funnelshift_r(w[i], w[i + 1], bits);
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// The vector's entries outside [0, V) read as -1e30 (2^y = 0); k0 is the index of its first entry
+template <int DT>
+__device__ __noinline__ uint4 masked_vector(uint4 v, int k0, int V) {
+    constexpr int EPV = Logit<DT>::kPerVec;
+    uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int j = 0; j < EPV; ++j) {
+        if (k0 + j >= 0 && k0 + j < V) continue;
+        if constexpr (DT == FSD_BF16) w[j >> 1] = (j & 1) ? ((w[j >> 1] & 0x0000ffffu) | 0xf1490000u) : ((w[j >> 1] & 0xffff0000u) | 0x0000f149u);
+        else w[j] = 0xf149f2cau;
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+template <int DT, int DIV, bool RAGGED>
+__global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(const __grid_constant__ StreamParams P) {
+    using S = StreamShape<DT>;
     constexpr int EPV = Logit<DT>::kPerVec;          // logits per 16-byte vector
-    constexpr int EPT = 2 * EPV;                     // e values per thread and vector position (both rows)
-    constexpr int VPT = kVecPerThread;
-    constexpr int EPS = VPT * EPT;                   // e values per thread and stage
-    constexpr int NT = (kTmemPerThread / EPS) < kMaxStagesPerPair ? (kTmemPerThread / EPS) : kMaxStagesPerPair;
-    constexpr int NR = kMaxStagesPerPair - NT;       // stages kept in registers
+    constexpr int VPS = S::kVecPerStep;
+    constexpr int SV = 32 * VPS;                     // vectors of a row a warp handles per step
     constexpr bool kSecondSweep = DIV != FSD_DIV_KL;
-    constexpr float kClamp = -1.0e30f;               // -inf logits are read as this: 2^y = 0 and 0 * y = 0 stay finite
+    [[maybe_unused]] constexpr float kClamp = -1.0e30f;
+    [[maybe_unused]] constexpr uint32_t kClamp2 = 0xF149F149u;       // the same as a pair of bf16
+    [[maybe_unused]] constexpr uint32_t kMinusInf2 = 0xFF80FF80u;
+    constexpr uint32_t kFill = DT == FSD_BF16 ? kClamp2 : 0xF149F2CAu;      // bits of kClamp
 
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
-    const int half = threadIdx.x / kStreamThreads;   // which virtual CTA of this CTA
-    unsigned char* ring = smem + half * kStreamHalfBytes;
-    StreamShared& sh = *reinterpret_cast<StreamShared*>(ring + kRing * kStageBytes);
-    uint32_t* tmem_base_slot = reinterpret_cast<uint32_t*>(smem + kStreamHalves * kStreamHalfBytes);
+    StreamShared& sh = *reinterpret_cast<StreamShared*>(smem + kRingBytes);
 
     const int C = P.C;
-    // numbered half by half, so that the two virtual CTAs of an SM belong to different groups: while one
-    // waits for its group's statistics the other has the SM to itself
-    const int vid = half * static_cast<int>(gridDim.x) + static_cast<int>(blockIdx.x);
-    const int n_groups = (kStreamHalves * static_cast<int>(gridDim.x)) / C;     // groups
-    const int group_id = vid / C, rank = vid - group_id * C;
-    const bool active = group_id < n_groups;     // the virtual CTAs left over form no group
-    const int tid = threadIdx.x % kStreamThreads, lane = tid & 31, warp = tid >> 5;
-    const int bar_posted = kBarPosted + 2 * half, bar_totals = kBarTotals + 2 * half;
+    const int n_groups = static_cast<int>(gridDim.x) / C;
+    const int group_id = static_cast<int>(blockIdx.x) / C, rank = static_cast<int>(blockIdx.x) - group_id * C;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // rounds of this group (the blocks left over form no group)
+    const int R = group_id < n_groups && group_id < P.n_items ? (P.n_items - group_id + n_groups - 1) / n_groups : 0;
 
-    // this virtual CTA's slice of every row, in vectors
+    // this block's slice of every row, in vectors, and a warp's part of it (the helper's lanes know a warp's each)
     const int base = P.nvec_row / C, rem = P.nvec_row % C;
-    const int vbeg = rank * base + (rank < rem ? rank : rem);
-    const int vcnt = base + (rank < rem ? 1 : 0);
-    const int ns = (vcnt + kStageVecs - 1) / kStageVecs;             // stages per pair (<= kMaxStagesPerPair)
-    const size_t row_bytes = static_cast<size_t>(P.nvec_row) * 16;
+    const int vbeg = rank * base + (rank < rem ? rank : rem), vcnt = base + (rank < rem ? 1 : 0);
+    const WarpPart mine = warp_part(warp < kComputeWarps ? warp : lane & (kComputeWarps - 1), vcnt, SV);
+    const int steps = mine.steps;
+    FSD_CHECK(P.timeout_flag + 2, steps <= S::kSteps && vbeg + vcnt <= P.nvec_row && mine.count >= 0 && mine.first + mine.count <= (steps == 0 ? INT_MAX : vcnt), kChkSlice);
 
-    // ---- set-up: barriers, tensor memory ----
-    // A group's first `ahead` pairs are fixed (group_id + round * n_groups): that is as far
-    // as the ring reads ahead.  Every later pair is the next one nobody has taken yet, claimed
-    // `ahead` rounds early by rank 0 and sent round with that round's statistics, so groups
-    // that happen to run faster take more pairs and all finish together.
-    // (from the smallest slice of the group, so that every member computes the same value
-    // whatever its own slice: the members must agree on which pairs are fixed and where a claimed
-    // id is kept; a member with one stage more per pair reads ahead less far, so the ids it needs
-    // are there even earlier)
-    const int ns_min = (base + kStageVecs - 1) / kStageVecs;
-    const int ahead = 2 + (kRing - 2) / (ns_min > 0 ? ns_min : 1);
-    if (tid == 0) {
-        for (int k = 0; k < ahead; ++k) sh.items[k] = group_id + k * n_groups;
-        for (int s = 0; s < kRing; ++s) { mbar_init(&sh.full[s], 1); mbar_init(&sh.empty[s], kStreamWarps); sh.armed[s] = 0; }
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    if (threadIdx.x < 32) {                          // one allocation for both virtual CTAs: all of the SM's columns
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     ::"r"(smem_u32(tmem_base_slot)), "r"(kStreamHalves * kTmemCols) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    // ---- the helper warp starts the copies ----
+    int in_slot = 0, in = 0, in_item = group_id, in_par = 0;      // the pair whose slices are asked for next: its number among the group's, its id, its parent node (trees)
+    auto issue_slices = [&]() {
+        if (in >= R) return;
+        const int slot = in_slot;
+        const int b = P.G == 1 ? in_item : static_cast<int>(__umulhi(static_cast<uint32_t>(in_item), P.g_magic) >> P.g_shift);
+        FSD_CHECK(P.timeout_flag + 2, in_item >= 0 && in_item < P.n_items && b == in_item / P.G, kChkItem);
+        int arow = in_item + b;                                      // chain: b * (G + 1) + i
+        if (P.parent != nullptr) {
+            const int i = in_item - b * P.G;
+            arow = b * (P.G + 1) + ((in_par >= -1 && in_par < i) ? in_par + 1 : 0);   // an invalid node still moves (ignored) data
+        }
+        FSD_CHECK(P.timeout_flag + 2, vcnt >= 0 && vcnt <= S::kBlockVecs && arow >= 0, kChkStage);
+        const char* arow_p = static_cast<const char*>(P.target) + static_cast<size_t>(arow) * P.row_bytes;
+        const char* brow_p = static_cast<const char*>(P.draft) + static_cast<size_t>(in_item) * P.row_bytes;
+        unsigned char* dst = smem + slot * P.slot_bytes;
+        if constexpr (!RAGGED) {
+            if (lane == 0) mbar_arrive_expect_tx(&sh.full[slot], static_cast<uint32_t>(vcnt) * 32);
+            if (lane < 2 && vcnt > 0)
+                bulk_g2s(dst + lane * P.slot_row_bytes, (lane == 0 ? arow_p : brow_p) + static_cast<size_t>(vbeg) * 16, static_cast<uint32_t>(vcnt) * 16, &sh.full[slot]);
+        } else {
+            // granules of 16 bytes from each row's rounded-down start; the draft row needs one more where it is shifted
+            const int oa = static_cast<int>(reinterpret_cast<uintptr_t>(arow_p) & 15), ob = static_cast<int>(reinterpret_cast<uintptr_t>(brow_p) & 15);
+            const int na = static_cast<int>((oa + P.row_bytes + 15) >> 4), nb = static_cast<int>((ob + P.row_bytes + 15) >> 4);
+            const int d = ob - oa;
+            const int ga1 = min(vbeg + vcnt, na);
+            const int wv0 = vbeg + mine.first;                       // lane w: warp w's part of the draft row
+            const int gb = wv0 + (d < 0 ? -1 : 0), gb0 = max(gb, 0), gb1 = min(gb + mine.count + (d != 0 ? 1 : 0), nb);
+            const uint32_t ba = ga1 > vbeg ? static_cast<uint32_t>(ga1 - vbeg) * 16 : 0;
+            const uint32_t bb = lane < kComputeWarps && mine.count > 0 && gb1 > gb0 ? static_cast<uint32_t>(gb1 - gb0) * 16 : 0;
+            // the warps moved the slot's last draft parts in place: those writes precede the copies
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            const uint32_t sum = ba + __reduce_add_sync(0xffffffffu, bb);
+            if (lane == 0) {
+                sh.meta[slot] = static_cast<uint32_t>(oa) << 8 | static_cast<uint32_t>(d & 15);
+                mbar_arrive_expect_tx(&sh.full[slot], sum);
+            }
+            __syncwarp();
+            if (lane == 0 && ba != 0) bulk_g2s(dst, arow_p - oa + static_cast<size_t>(vbeg) * 16, ba, &sh.full[slot]);
+            if (bb != 0) bulk_g2s(dst + P.slot_row_bytes + (mine.first + mine.pos + gb0 - gb) * 16, brow_p - ob + static_cast<size_t>(gb0) * 16, bb, &sh.full[slot]);
+        }
+        __syncwarp();
+        ++in; in_item += n_groups;
+        if (++in_slot == P.ring) in_slot = 0;
+        if (P.parent != nullptr && in < R) in_par = __ldg(P.parent + in_item);
+    };
+    if (warp == kComputeWarps) {
+        if (lane == 0) {
+            for (int k = 0; k < P.ring; ++k) mbar_init(&sh.full[k], 1);
+            for (int k = 0; k < 2; ++k) { mbar_init(&sh.posted[k], kComputeWarps); mbar_init(&sh.totals[k], 1); }
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        }
+        __syncwarp();
+        if (P.parent != nullptr && R > 0) in_par = __ldg(P.parent + in_item);
+        for (int q = 0; q < P.ring; ++q) issue_slices();
+        if constexpr (kSecondSweep) {
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh.tmem_base)), "n"(kTmemCols) : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        }
+    } else {
+        // lanes without a vector in the slice's last step read "-inf" there: no copy ever writes behind the slice
+        // (an unaligned draft row's vectors there are masked)
+        const int end = (vcnt + SV - 1) / SV * SV;
+        for (int v = vcnt + static_cast<int>(threadIdx.x); v < end; v += 32 * kComputeWarps) {
+            for (int q = 0; q < P.ring; ++q) {
+                *reinterpret_cast<uint4*>(smem + q * P.slot_bytes + v * 16) = make_uint4(kFill, kFill, kFill, kFill);
+                if constexpr (!RAGGED) *reinterpret_cast<uint4*>(smem + q * P.slot_bytes + P.slot_row_bytes + v * 16) = make_uint4(kFill, kFill, kFill, kFill);
+            }
+        }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    // warp w of a virtual CTA owns tensor-memory lanes 32*(w%4)..+31 and columns kTmemCols*half + kTmemPerThread*(w/4)..
-    const uint32_t taddr = *tmem_base_slot + (static_cast<uint32_t>(32 * (warp & 3)) << 16) +
-                           static_cast<uint32_t>(kTmemCols * half + kTmemPerThread * (warp >> 2));
-    // where this group's virtual CTAs exchange their statistics: [parity][rank] messages
-    GroupMsg* const xg = P.exchange + static_cast<size_t>(group_id < n_groups ? group_id : 0) * 2 * C;
 
-    bool dead = false;                               // a bounded wait of this thread ran out
+    // second sweep and totals lag two rounds behind; KL has neither
+    const int n_end = R == 0 ? 0 : (kSecondSweep ? R + 2 : R);
 
-    // ---- producer: stage number -> (pair, slice part); any thread may issue a stage ----
-    // Stage gg of this virtual CTA is part gg % ns of the (gg / ns)-th pair of its group (its id is in
-    // sh.items).  Stage gg + kRing is issued by the duty warp of stage gg + 1 (see the first sweep), so the
-    // copies go out early and the work is spread over the warps.
-    auto issue_stage = [&](uint32_t gg) {
-        const uint32_t k = gg / static_cast<uint32_t>(ns), s = gg - k * static_cast<uint32_t>(ns);
-        const int item = sh.items[k & 7];
-        if (item >= P.n_items) return;
-        FSD_CHECK(P.timeout_flag + 2, item >= 0, kChkItem);
-        const int b = item / P.G, i = item - b * P.G;
-        int trow = i;
-        if (P.parent != nullptr) {
-            const int par = __ldg(P.parent + item);
-            trow = (par >= -1 && par < i) ? par + 1 : 0;       // an invalid node still moves (ignored) data
-        }
-        const char* a_row = static_cast<const char*>(P.target) + (static_cast<size_t>(b) * (P.G + 1) + trow) * row_bytes;
-        const char* b_row = static_cast<const char*>(P.draft) + (static_cast<size_t>(b) * P.G + i) * row_bytes;
-        const uint32_t slot = gg % kRing;
-        const int v0 = static_cast<int>(s) * kStageVecs;
-        const int nv = (vcnt - v0) < kStageVecs ? (vcnt - v0) : kStageVecs;
-        const uint32_t bytes = static_cast<uint32_t>(nv) * 16;
-        FSD_CHECK(P.timeout_flag + 2, nv > 0 && vbeg + v0 + nv <= P.nvec_row && bytes <= kStageRowBytes, kChkSlice);
-        FSD_CHECK(P.timeout_flag + 2, s < static_cast<uint32_t>(ns) && ns <= kMaxStagesPerPair && trow >= 0 && trow <= P.G, kChkStage);
-        unsigned char* dst = ring + slot * kStageBytes;
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // earlier reads of the slot precede the async writes
-        sh.armed[slot] += 1;                         // one thread at a time starts copies into a slot
-        mbar_arrive_expect_tx(&sh.full[slot], 2 * bytes);
-        bulk_g2s(dst, a_row + (static_cast<size_t>(vbeg) + v0) * 16, bytes, &sh.full[slot]);
-        bulk_g2s(dst + kStageRowBytes, b_row + (static_cast<size_t>(vbeg) + v0) * 16, bytes, &sh.full[slot]);
-    };
-    if (tid == 0 && active) {
-        for (uint32_t gg = 0; gg < kRing; ++gg) issue_stage(gg);
-    }
-    __syncwarp();
+    if (warp < kComputeWarps) {
+        const uint32_t taddr = kSecondSweep ? sh.tmem_base + (static_cast<uint32_t>(32 * (warp & 3)) << 16) + static_cast<uint32_t>(128 * (warp >> 2)) : 0;
+        const uint64_t l2 = pack2(kLog2e, kLog2e);
+        bool dead = false;
+        float ka1 = -INFINITY, kb1 = -INFINITY, ka2 = -INFINITY, kb2 = -INFINITY;     // references of pairs n - 1 and n - 2
+        // shared-memory addresses of this lane's first vectors in slot 0
+        const uint32_t my_a = smem_u32(smem) + static_cast<uint32_t>(mine.first + lane) * 16;
+        const uint32_t my_b = smem_u32(smem) + static_cast<uint32_t>(P.slot_row_bytes) + static_cast<uint32_t>(mine.first + (RAGGED ? mine.pos : 0) + lane) * 16;
+        // Running maxima of the next pair's parts.  They fix its references, ceil(max * log2e).  Usually only the part's
+        // first step is looked at: the reference need not be the maximum, only near enough (see `near`).
+        float ma = -INFINITY, mb = -INFINITY;
+        uint32_t pa = kMinusInf2, pb = kMinusInf2;
+        auto maxima = [&](const uint4& wa, const uint4& wb) {
+            if constexpr (DT == FSD_BF16) {
+                pa = bf16x2_max_nan(pa, bf16x2_max_nan(bf16x2_max_nan(wa.x, wa.y), bf16x2_max_nan(wa.z, wa.w)));
+                pb = bf16x2_max_nan(pb, bf16x2_max_nan(bf16x2_max_nan(wb.x, wb.y), bf16x2_max_nan(wb.z, wb.w)));
+            } else {
+                ma = fmax_nan(ma, fmax_nan(fmax_nan(__uint_as_float(wa.x), __uint_as_float(wa.y)), fmax_nan(__uint_as_float(wa.z), __uint_as_float(wa.w))));
+                mb = fmax_nan(mb, fmax_nan(fmax_nan(__uint_as_float(wb.x), __uint_as_float(wb.y)), fmax_nan(__uint_as_float(wb.z), __uint_as_float(wb.w))));
+            }
+        };
+        // Vector v of an unaligned row's part in the slot at byte offset `o`: the draft's vector moves onto the target's
+        // entries, what lies outside the rows becomes -1e30, in place.
+        auto align_vector = [&](uint32_t o, uint32_t meta, int v) {
+            const uint32_t shift = meta & 255u;
+            uint4 wb = ld_shared16(my_b + o + v * 512);
+            if (shift != 0) wb = shifted<DT>(wb, ld_shared16(my_b + o + v * 512 + 16), shift);
+            const int g = vbeg + mine.first + v * 32 + lane;
+            if (g == 0 || g >= P.nvec_row - 2 || v * 32 + lane >= mine.count) {
+                const int V = static_cast<int>(P.row_bytes / Logit<DT>::kBytes);
+                const int k0 = v * 32 + lane < mine.count ? g * EPV - static_cast<int>(meta >> 8) / Logit<DT>::kBytes : V;
+                wb = masked_vector<DT>(wb, k0, V);
+                st_shared16(my_a + o + v * 512, masked_vector<DT>(ld_shared16(my_a + o + v * 512), k0, V));
+            }
+            __syncwarp();                            // the neighbours have read what is overwritten now
+            st_shared16(my_b + o + v * 512, wb);
+        };
+        // the references the maxima give; none (-inf) where no finite logit was seen
+        auto references = [&](float& ka, float& kb) {
+            if constexpr (DT == FSD_BF16) { ma = fmax_nan(bf16_lo(pa), bf16_hi(pa)); mb = fmax_nan(bf16_lo(pb), bf16_hi(pb)); pa = kMinusInf2; pb = kMinusInf2; }
+            __syncwarp();
+            const float ra = warp_redux_max_nan(ma), rb = warp_redux_max_nan(mb);
+            ma = -INFINITY; mb = -INFINITY;
+            ka = ra <= -9.9e29f ? -INFINITY : ceilf(ra * kLog2e);
+            kb = rb <= -9.9e29f ? -INFINITY : ceilf(rb * kLog2e);
+        };
 
-    float ereg[(NR > 0 ? NR : 1) * EPS];
-    uint32_t g = 0;                                  // first ring stage of the current pair
-    uint32_t li = 0;                                 // pairs this group has finished
-    float x_carry = 0.f;                             // previous pair's second-sweep sum of this warp
-    int prev_item = -1;                              // pair whose second-sweep sum is still to be published
-    int item = active ? group_id : P.n_items;
-    uint32_t claimed = 0;                            // rank 0, combiner lane 0: the pair id taken this round
-
-    for (;;) {
-        const bool live = item < P.n_items;          // one extra round publishes the last pair's second sweep
-        if (!live && prev_item < 0) break;
-        const int par = static_cast<int>(li & 1);
-        const uint32_t tag = li + 1;                 // what this round's messages carry (never 0, the buffer's initial state)
-        if (kSecondSweep && rank == 0 && lane == 0 && warp == static_cast<int>(li & (kStreamWarps - 1))) {
-            // asked now, needed only when the statistics go out
-            const long long id = static_cast<long long>(ahead) * n_groups + atomicAdd(P.next_pair, 1);
-            claimed = id < 0x3fffffffLL ? static_cast<uint32_t>(id) : 0x3fffffffu;
-        }
-        bool bad = false;
-        if (live && P.parent != nullptr) {
-            const int i = item % P.G;
-            const int pr = __ldg(P.parent + item);
-            bad = pr < -1 || pr >= i;
-        }
-
-        // ---- first sweep: exponentials, sums, park the e values; then this warp's statistics ----
-        float ka = -INFINITY, kb = -INFINITY;
-        Stats mine;
-        mine.ka = -INFINITY; mine.kb = -INFINITY; mine.za = 0.f; mine.zb = 0.f; mine.s0 = 0.f; mine.sb = 0.f;
-        mine.diff = 0;
-        if (live) {
-            float kk = 0.f;
-            uint32_t diff = 0;
-            uint64_t za2 = 0, zb2 = 0, sa2 = 0, sb2 = 0;     // packed (even, odd) partial sums
-            // Integer references in the log2 domain, y = logit*log2e - k.  A thread takes k from the
-            // first vector that holds a finite logit and keeps it while no later logit exceeds it by
-            // more than about 2^30 (2^60 at most); a larger one moves the reference and rescales what
-            // has been summed and parked, by an exact power of two.
-            uint32_t lima = unset_limit<DT>(), limb = unset_limit<DT>(); // a vector maximum above this moves the reference
-            uint64_t ca2 = 0, cb2 = 0;                       // packed -k (0 while no finite logit has been seen)
-            const uint64_t l2 = pack2(kLog2e, kLog2e);
+        // ---- first sweep of step s of the pair in the slot at byte offset `o` ----
+        struct Sums { uint64_t za2, zb2, sa2, sb2; float kk; uint32_t diff; };     // packed (even, odd) partial sums
+        const auto zero_sums = [] { return Sums{0, 0, 0, 0, 0.f, 0}; };
+        auto first_sweep = [&](auto careful_tag, int s, uint32_t o, uint64_t ca2, uint64_t cb2, Sums& t, float (&e)[kParkCols]) {
+            constexpr bool CAREFUL = decltype(careful_tag)::value;
 #pragma unroll
-            for (int s = 0; s < kMaxStagesPerPair; ++s) {
-                if (s < ns) {
-                    const uint32_t gs = g + s, slot = gs % kRing;
-                    mbar_wait(&sh.full[slot], (gs / kRing) & 1, P.timeout_flag, dead);
-                    // this thread's vectors of the stage: v * kStreamThreads + tid, v < VPT
-                    uint4 va[VPT], vb[VPT];
-                    bool has[VPT];
-                    float ma = 0.f, mb = 0.f;                // maxima of this thread's vectors of the stage
-                    bool fire_a = false, fire_b = false;
-                    {
-                        uint32_t pa = unset_limit<DT>(), pb = unset_limit<DT>();   // -1e30: below every clamped logit
+            for (int v = 0; v < VPS; ++v) {
+                uint4 wa = ld_shared16(my_a + o + (s * VPS + v) * 512);
+                uint4 wb = ld_shared16(my_b + o + (s * VPS + v) * 512);
+                if constexpr (CAREFUL && DIV == FSD_DIV_JS && DT == FSD_BF16) {
+                    // -inf becomes -1e30: 2^y = 0 and 0 * y = 0 stay finite (NaN passes through)
+                    wa.x = bf16x2_max_nan(wa.x, kClamp2); wa.y = bf16x2_max_nan(wa.y, kClamp2);
+                    wa.z = bf16x2_max_nan(wa.z, kClamp2); wa.w = bf16x2_max_nan(wa.w, kClamp2);
+                    wb.x = bf16x2_max_nan(wb.x, kClamp2); wb.y = bf16x2_max_nan(wb.y, kClamp2);
+                    wb.z = bf16x2_max_nan(wb.z, kClamp2); wb.w = bf16x2_max_nan(wb.w, kClamp2);
+                }
+                if constexpr (DIV != FSD_DIV_TV) t.diff |= (wa.x ^ wb.x) | (wa.y ^ wb.y) | (wa.z ^ wb.z) | (wa.w ^ wb.w);
+                float xa[EPV], xb[EPV];
+                unpack_vec<DT>(wa, xa);
+                unpack_vec<DT>(wb, xb);
 #pragma unroll
-                        for (int v = 0; v < VPT; ++v) {
-                            has[v] = s * kStageVecs + v * kStreamThreads + tid < vcnt;
-                            va[v] = make_uint4(0, 0, 0, 0); vb[v] = make_uint4(0, 0, 0, 0);
-                            if (has[v]) {
-                                const unsigned char* st = ring + slot * kStageBytes + (v * kStreamThreads + tid) * 16;
-                                va[v] = *reinterpret_cast<const uint4*>(st);
-                                vb[v] = *reinterpret_cast<const uint4*>(st + kStageRowBytes);
-                                diff |= (va[v].x ^ vb[v].x) | (va[v].y ^ vb[v].y) | (va[v].z ^ vb[v].z) | (va[v].w ^ vb[v].w);
-                                if constexpr (DT == FSD_BF16) {
-                                    constexpr uint32_t kClamp2 = 0xF149F149u;     // bf16x2 (-1e30, -1e30); NaN passes through
-                                    va[v].x = bf16x2_max_nan(va[v].x, kClamp2); va[v].y = bf16x2_max_nan(va[v].y, kClamp2);
-                                    va[v].z = bf16x2_max_nan(va[v].z, kClamp2); va[v].w = bf16x2_max_nan(va[v].w, kClamp2);
-                                    if constexpr (DIV != FSD_DIV_KL) {            // KL needs the draft's -inf: q = 0 < p gives +inf
-                                        vb[v].x = bf16x2_max_nan(vb[v].x, kClamp2); vb[v].y = bf16x2_max_nan(vb[v].y, kClamp2);
-                                        vb[v].z = bf16x2_max_nan(vb[v].z, kClamp2); vb[v].w = bf16x2_max_nan(vb[v].w, kClamp2);
-                                    }
-                                    pa = bf16x2_max_nan(pa, bf16x2_max_nan(bf16x2_max_nan(va[v].x, va[v].y), bf16x2_max_nan(va[v].z, va[v].w)));
-                                    pb = bf16x2_max_nan(pb, bf16x2_max_nan(bf16x2_max_nan(vb[v].x, vb[v].y), bf16x2_max_nan(vb[v].z, vb[v].w)));
-                                } else {
-                                    const float m1 = fmax_nan(fmax_nan(__uint_as_float(va[v].x), __uint_as_float(va[v].y)),
-                                                              fmax_nan(__uint_as_float(va[v].z), __uint_as_float(va[v].w)));
-                                    const float m2 = fmax_nan(fmax_nan(__uint_as_float(vb[v].x), __uint_as_float(vb[v].y)),
-                                                              fmax_nan(__uint_as_float(vb[v].z), __uint_as_float(vb[v].w)));
-                                    pa = __float_as_uint(fmax_nan(__uint_as_float(pa), m1));
-                                    pb = __float_as_uint(fmax_nan(__uint_as_float(pb), m2));
-                                }
+                for (int j = 0; j < EPV; j += 2) {
+                    float a0 = xa[j], a1 = xa[j + 1], b0 = xb[j], b1 = xb[j + 1];
+                    if constexpr (CAREFUL && DIV == FSD_DIV_JS && DT == FSD_F32) {
+                        a0 = fmax_nan(a0, kClamp); a1 = fmax_nan(a1, kClamp); b0 = fmax_nan(b0, kClamp); b1 = fmax_nan(b1, kClamp);
+                    }
+                    const uint64_t ya2 = fma2(pack2(a0, a1), l2, ca2), yb2 = fma2(pack2(b0, b1), l2, cb2);
+                    float ya0, ya1, yb0, yb1;
+                    unpack2(ya2, ya0, ya1);
+                    unpack2(yb2, yb0, yb1);
+                    const float ea0 = ex2(ya0), ea1 = ex2(ya1), eb0 = ex2(yb0), eb1 = ex2(yb1);
+                    const uint64_t ea2 = pack2(ea0, ea1), eb2 = pack2(eb0, eb1);
+                    t.za2 = add2(t.za2, ea2);
+                    t.zb2 = add2(t.zb2, eb2);
+                    if constexpr (DIV == FSD_DIV_JS) {
+                        t.sa2 = fma2(ea2, ya2, t.sa2);
+                        t.sb2 = fma2(eb2, yb2, t.sb2);
+                    }
+                    if constexpr (DIV == FSD_DIV_KL) {       // (q = 0 < p, a draft logit of -inf, gives +inf)
+                        if (ea0 > 0.f) t.kk = fmaf(ea0, ya0 - yb0, t.kk);
+                        if (ea1 > 0.f) t.kk = fmaf(ea1, ya1 - yb1, t.kk);
+                    }
+                    e[v * EPV + j] = ea0; e[v * EPV + j + 1] = ea1;
+                    e[kStepEntries + v * EPV + j] = eb0; e[kStepEntries + v * EPV + j + 1] = eb1;
+                }
+            }
+        };
+
+        float ka = -INFINITY, kb = -INFINITY;        // references of pair n
+        int slot = 0;
+        uint32_t so = 0;                             // its slot, and the slot's byte offset
+        uint32_t phase = 0;                          // of the next pair's slot
+        bool careful = false;                        // this warp has met logits that the quick form of the first sweep cannot take
+        if (R > 0) {
+            dead = !warp_wait(&sh.full[0], 0, P.timeout_flag);
+            if (!dead) {
+                if constexpr (RAGGED) {
+                    const uint32_t meta = sh.meta[0];
+                    for (int v = 0; v < steps * VPS; ++v) align_vector(0, meta, v);
+                }
+                if (steps > 0) {
+#pragma unroll
+                    for (int v = 0; v < VPS; ++v) maxima(ld_shared16(my_a + v * 512), ld_shared16(my_b + v * 512));
+                }
+                references(ka, kb);
+            }
+        }
+        // Both sweeps of a round, step by step.  FULL: a pair in every stage (this one's first sweep, the second sweep of
+        // n - 2, a look at the first step of n + 1), so that a step is one run of straight-line code whose strands cover one
+        // another's latencies; otherwise (the first and last rounds, and careful ones) each strand is looked at.
+        auto sweeps = [&](auto full_tag, const int n, const bool first, const uint32_t nso, [[maybe_unused]] const uint32_t meta,
+                          const float ia, const float ib, Sums& t, uint64_t& x2) {
+            constexpr bool FULL = decltype(full_tag)::value;
+            const bool live = FULL || first, next = FULL || n + 1 < R;
+            [[maybe_unused]] const bool old = FULL || n >= 2;
+            {
+                const float ca = ka == -INFINITY ? 0.f : -ka, cb = kb == -INFINITY ? 0.f : -kb;
+                const uint64_t ca2 = pack2(ca, ca), cb2 = pack2(cb, cb);
+                const uint64_t ia2 = pack2(ia, ia), ib2 = pack2(ib, ib);
+                // s = p + q + 1e-37 keeps lg2 finite where both terms vanish; the shift is below one ulp of any s that matters
+                const uint64_t tiny2 = pack2(1e-37f, 1e-37f);
+                __syncwarp();                        // converged from here to the fold
+                [[maybe_unused]] const uint32_t tslot = taddr + static_cast<uint32_t>((n & 1) * (kMaxSteps * kParkCols));
+#pragma unroll
+                for (int s = 0; s < S::kSteps; ++s) {
+                    if (s < steps) {
+                        [[maybe_unused]] float eo[kParkCols], e[kParkCols];
+                        if (next) {
+                            if constexpr (RAGGED) {
+#pragma unroll
+                                for (int v = 0; v < VPS; ++v) align_vector(nso, meta, s * VPS + v);
+                                __syncwarp();
+                            }
+                            if (s == 0) {
+#pragma unroll
+                                for (int v = 0; v < VPS; ++v) maxima(ld_shared16(my_a + nso + (s * VPS + v) * 512), ld_shared16(my_b + nso + (s * VPS + v) * 512));
                             }
                         }
-                        if constexpr (DT == FSD_BF16) {
-                            fire_a = bf16x2_max_nan(pa, lima) != lima;
-                            fire_b = bf16x2_max_nan(pb, limb) != limb;
-                            if (fire_a) ma = fmax_nan(bf16_lo(pa), bf16_hi(pa));
-                            if (fire_b) mb = fmax_nan(bf16_lo(pb), bf16_hi(pb));
-                        } else {
-                            ma = __uint_as_float(pa); mb = __uint_as_float(pb);
-                            fire_a = !(ma <= __uint_as_float(lima));      // NaN moves the reference too
-                            fire_b = !(mb <= __uint_as_float(limb));
-                        }
-                    }
-                    __syncwarp();
-                    if (__any_sync(0xffffffffu, fire_a || fire_b)) {
-                        // rare after a pair's first vector: lanes that did not fire scale by 1
-                        const float nka = fire_a ? ceilf(ma * kLog2e) : ka, nkb = fire_b ? ceilf(mb * kLog2e) : kb;
-                        const float da = ka == -INFINITY ? 0.f : ka - nka, db = kb == -INFINITY ? 0.f : kb - nkb;
-                        const float fa = ka == -INFINITY ? 0.f : pow2_int(da), fb = kb == -INFINITY ? 0.f : pow2_int(db);
-                        const uint64_t fa2 = pack2(fa, fa), fb2 = pack2(fb, fb);
-                        if constexpr (DIV == FSD_DIV_KL) kk = scale_kl(fa, fmaf(da - db, sum2(za2), kk));
-                        sa2 = mul2(fma2(za2, pack2(da, da), sa2), fa2); za2 = mul2(za2, fa2);
-                        sb2 = mul2(fma2(zb2, pack2(db, db), sb2), fb2); zb2 = mul2(zb2, fb2);
                         if constexpr (kSecondSweep) {
-                            if (s > 0) rescale_parked<EPT>(taddr, (s < NT ? s : NT) * VPT, fa, fb);
+                            if (old) tmem_ld16(tslot + s * kParkCols, eo);
+                        }
+                        if (live) first_sweep(std::false_type{}, s, so, ca2, cb2, t, e);
+                        if constexpr (kSecondSweep) {
+                            if (old) tmem_wait_ld();
+                            if (live) {
+                                FSD_CHECK(P.timeout_flag + 2, (s + 1) * kParkCols <= 64, kChkTmem);
+                                tmem_st16(tslot + s * kParkCols, e);
+                            }
+                            if (old) {
 #pragma unroll
-                            for (int t = NT; t < s; ++t) {
-#pragma unroll
-                                for (int v = 0; v < VPT; ++v) {
-#pragma unroll
-                                    for (int j = 0; j < EPV; ++j) {
-                                        ereg[(t - NT) * EPS + v * EPT + j] *= fa;
-                                        ereg[(t - NT) * EPS + v * EPT + EPV + j] *= fb;
+                                for (int j = 0; j < kStepEntries; j += 2) {
+                                    const uint64_t ea2 = pack2(eo[j], eo[j + 1]), eb2 = pack2(eo[kStepEntries + j], eo[kStepEntries + j + 1]);
+                                    if constexpr (DIV == FSD_DIV_JS) {
+                                        const uint64_t s2 = fma2(eb2, ib2, fma2(ea2, ia2, tiny2));
+                                        float s0, s1;
+                                        unpack2(s2, s0, s1);
+                                        x2 = fma2(s2, pack2(lg2(s0), lg2(s1)), x2);
+                                    } else {
+                                        // separately rounded products: a fused p - q would make TV(p, p) != 0
+                                        const uint64_t d2 = fma2(mul2(eb2, ib2), pack2(-1.f, -1.f), mul2(ea2, ia2));
+                                        float d0, d1;
+                                        unpack2(d2, d0, d1);
+                                        x2 = add2(x2, pack2(fabsf(d0), fabsf(d1)));
                                     }
                                 }
-                            }
-                        }
-                        if (fire_a) lima = reference_limit<DT>(ma);
-                        if (fire_b) limb = reference_limit<DT>(mb);
-                        ka = nka; kb = nkb;
-                        const float ca = ka == -INFINITY ? 0.f : -ka, cb = kb == -INFINITY ? 0.f : -kb;
-                        ca2 = pack2(ca, ca); cb2 = pack2(cb, cb);
-                    }
-                    // This warp is done with the slot: every lane's vectors are in registers (the vote
-                    // above consumed them).  Nobody waits for the slot to drain: one stage later, when
-                    // every warp has long left it, this stage's duty warp refills it.
-                    if (lane == 0) {
-                        mbar_arrive(&sh.empty[slot]);
-                        if (gs > 0 && warp == static_cast<int>(gs % kStreamWarps)) {
-                            const uint32_t ps = gs - 1;
-                            mbar_wait(&sh.empty[ps % kRing], (ps / kRing) & 1, P.timeout_flag, dead);
-                            if (!dead) issue_stage(ps + kRing);      // after a wait has run out nothing more is copied
-                        }
-                    }
-                    float e[VPT][EPT];
-#pragma unroll
-                    for (int v = 0; v < VPT; ++v) {
-                        if (has[v]) {
-                            float xa[EPV], xb[EPV];
-                            unpack_vec<DT>(va[v], xa);
-                            unpack_vec<DT>(vb[v], xb);
-#pragma unroll
-                            for (int j = 0; j < EPV; j += 2) {
-                                float a0 = xa[j], a1 = xa[j + 1], b0 = xb[j], b1 = xb[j + 1];
-                                if constexpr (DT == FSD_F32) {
-                                    a0 = fmaxf(a0, kClamp); a1 = fmaxf(a1, kClamp);
-                                    if constexpr (DIV != FSD_DIV_KL) { b0 = fmaxf(b0, kClamp); b1 = fmaxf(b1, kClamp); }
-                                }
-                                const uint64_t ya2 = fma2(pack2(a0, a1), l2, ca2), yb2 = fma2(pack2(b0, b1), l2, cb2);
-                                float ya0, ya1, yb0, yb1;
-                                unpack2(ya2, ya0, ya1);
-                                unpack2(yb2, yb0, yb1);
-                                const float ea0 = ex2(ya0), ea1 = ex2(ya1), eb0 = ex2(yb0), eb1 = ex2(yb1);
-                                const uint64_t ea2 = pack2(ea0, ea1), eb2 = pack2(eb0, eb1);
-                                za2 = add2(za2, ea2);
-                                zb2 = add2(zb2, eb2);
-                                if constexpr (DIV == FSD_DIV_JS) {
-                                    sa2 = fma2(ea2, ya2, sa2);
-                                    sb2 = fma2(eb2, yb2, sb2);
-                                }
-                                if constexpr (DIV == FSD_DIV_KL) {
-                                    if (ea0 > 0.f) kk = fmaf(ea0, ya0 - yb0, kk);
-                                    if (ea1 > 0.f) kk = fmaf(ea1, ya1 - yb1, kk);
-                                }
-                                e[v][j] = ea0; e[v][j + 1] = ea1;
-                                e[v][EPV + j] = eb0; e[v][EPV + j + 1] = eb1;
-                            }
-                        } else {
-#pragma unroll
-                            for (int j = 0; j < EPT; ++j) e[v][j] = 0.f;
-                        }
-                    }
-                    if constexpr (kSecondSweep) {
-#pragma unroll
-                        for (int v = 0; v < VPT; ++v) {
-                            if (s < NT) {
-                                FSD_CHECK(P.timeout_flag + 2, (s * VPT + v) * EPT + EPT <= kTmemPerThread, kChkTmem);
-                                tmem_st<EPT>(taddr + (s * VPT + v) * EPT, e[v]);
-                            } else {
-#pragma unroll
-                                for (int j = 0; j < EPT; ++j) ereg[(s - NT < 0 ? 0 : s - NT) * EPS + v * EPT + j] = e[v][j];
                             }
                         }
                     }
                 }
             }
-            if constexpr (kSecondSweep) tmem_wait_st();
+        };
 
-            // thread -> warp: bring the sums to the warp's reference (exact power-of-two factors)
-            const float za = sum2(za2), zb = sum2(zb2);
-            const float wka = warp_max_nan(ka), wkb = warp_max_nan(kb);
-            const float da = ka == -INFINITY ? 0.f : ka - wka, db = kb == -INFINITY ? 0.f : kb - wkb;
-            const float fa = ka == -INFINITY ? 0.f : pow2_int(da), fb = kb == -INFINITY ? 0.f : pow2_int(db);
-            float v_za = za * fa, v_zb = zb * fb;
-            float v_s0 = 0.f, v_sb = 0.f;
-            if constexpr (DIV == FSD_DIV_JS) { v_s0 = fa * fmaf(da, za, sum2(sa2)); v_sb = fb * fmaf(db, zb, sum2(sb2)); }
-            if constexpr (DIV == FSD_DIV_KL) v_s0 = scale_kl(fa, fmaf(da - db, za, kk));
-#pragma unroll
-            for (int m = 16; m > 0; m >>= 1) {
-                v_za += __shfl_xor_sync(0xffffffffu, v_za, m);
-                v_zb += __shfl_xor_sync(0xffffffffu, v_zb, m);
-                if constexpr (DIV != FSD_DIV_TV) v_s0 += __shfl_xor_sync(0xffffffffu, v_s0, m);
-                if constexpr (DIV == FSD_DIV_JS) v_sb += __shfl_xor_sync(0xffffffffu, v_sb, m);
+#pragma unroll 1
+        for (int n = 0; n < n_end && !dead; ++n) {
+            const bool live = n < R;
+            int nslot = slot + 1;
+            uint32_t nso = so + P.slot_bytes;
+            if (nslot == P.ring) { nslot = 0; nso = 0; phase ^= 1; }
+            uint32_t meta = 0;
+            if (n + 1 < R) {
+                if (!warp_wait(&sh.full[nslot], phase, P.timeout_flag)) { dead = true; break; }
+                if constexpr (RAGGED) meta = sh.meta[nslot];
             }
-            mine.ka = wka; mine.kb = wkb; mine.za = v_za; mine.zb = v_zb; mine.s0 = v_s0; mine.sb = v_sb;
-            mine.diff = __reduce_or_sync(0xffffffffu, diff);
-        }
-        mine.x = x_carry;
-
-        // ---- exchange.  Every warp leaves its statistics in shared memory and counts itself in
-        //      on a named barrier; this round's combiner warp waits there for the others, folds
-        //      the warps' statistics, stores the virtual CTA's message, fetches the group's messages
-        //      until all carry this round's tag, folds those and leaves the totals for the virtual
-        //      CTA.  Only the combiner polls; everyone else sleeps on a barrier. ----
-        if (lane == 0) sh.ws[warp] = mine;
-        __syncwarp();
-        if (warp != static_cast<int>(li & (kStreamWarps - 1))) {
-            __threadfence_block();
-            named_arrive(bar_posted);
-        } else {
-            named_sync(bar_posted);
-            Stats w;
-            w.ka = -INFINITY; w.kb = -INFINITY; w.za = 0.f; w.zb = 0.f; w.s0 = 0.f; w.sb = 0.f; w.x = 0.f; w.diff = 0;
-            if (lane < kStreamWarps) w = sh.ws[lane];
-            Stats c;
-            c.ka = warp_max_nan(w.ka); c.kb = warp_max_nan(w.kb);
+            // ---- the totals of pair n - 2 ----
+            float ia = 0.f, ib = 0.f;
+            if (n >= 2) {
+                if (!warp_wait(&sh.totals[n & 1], ((n - 2) >> 1) & 1, P.timeout_flag)) { dead = true; break; }
+                if constexpr (kSecondSweep) {
+                    const float4 t = sh.tot[n & 1];
+                    ia = pow2_ref(ka2, t.x) * t.y;
+                    ib = pow2_ref(kb2, t.z) * t.w;
+                }
+            }
+            Sums t = zero_sums();
+            uint64_t x2 = 0;
+            if (n >= 2 && n + 1 < R && !careful) sweeps(std::true_type{}, n, true, nso, meta, ia, ib, t, x2);
+            else sweeps(std::false_type{}, n, live && !careful, nso, meta, ia, ib, t, x2);
+            // Were the references near enough?  A lane's Z up to 4e10 (an entry may exceed 2^k by about 2^30, as the
+            // exponents' rounding allows), no NaN (-inf * 0 in the entropy sums), and a reference at all.  If not, the
+            // first sweep is done (over) with exact maxima and clamped logits, and this warp stays with that form.
+            if (live) {
+                const float z = sum2(t.za2) + sum2(t.zb2);
+                bool near = z < 4.0e10f && ((ka != -INFINITY && kb != -INFINITY) || steps == 0);
+                if constexpr (DIV == FSD_DIV_JS) near = near && fabsf(sum2(t.sa2)) + fabsf(sum2(t.sb2)) < 1.0e15f;
+                if (careful || __any_sync(0xffffffffu, !near)) {
+                    careful = true;
+                    float na = ma, nb = mb;          // (the next pair's maxima are in flight)
+                    const uint32_t npa = pa, npb = pb;
+                    ma = -INFINITY; mb = -INFINITY; pa = kMinusInf2; pb = kMinusInf2;
+                    for (int v = 0; v < steps * VPS; ++v) maxima(ld_shared16(my_a + so + v * 512), ld_shared16(my_b + so + v * 512));
+                    references(ka, kb);
+                    ma = na; mb = nb; pa = npa; pb = npb;
+                    const float ca = ka == -INFINITY ? 0.f : -ka, cb = kb == -INFINITY ? 0.f : -kb;
+                    t = zero_sums();
+                    __syncwarp();
+#pragma unroll 1
+                    for (int s = 0; s < steps; ++s) {
+                        float e[kParkCols];
+                        first_sweep(std::true_type{}, s, so, pack2(ca, ca), pack2(cb, cb), t, e);
+                        if constexpr (kSecondSweep) tmem_st16(taddr + static_cast<uint32_t>((n & 1) * (kMaxSteps * kParkCols) + s * kParkCols), e);
+                    }
+                }
+            }
+            // ---- fold over the lanes: four sums by halving (six shuffles), the second-sweep sum by a butterfly ----
             {
-                const float da = w.ka == -INFINITY ? 0.f : w.ka - c.ka, db = w.kb == -INFINITY ? 0.f : w.kb - c.kb;
-                const float fa = w.ka == -INFINITY ? 0.f : pow2_int(da), fb = w.kb == -INFINITY ? 0.f : pow2_int(db);
-                c.za = w.za * fa; c.zb = w.zb * fb;
-                c.s0 = DIV == FSD_DIV_KL ? scale_kl(fa, fmaf(da - db, w.za, w.s0)) : fa * fmaf(da, w.za, w.s0);
-                c.sb = fb * fmaf(db, w.zb, w.sb);
-                c.x = w.x;
-            }
+                const float v0 = sum2(t.za2), v1 = sum2(t.zb2), v2 = DIV == FSD_DIV_KL ? t.kk : sum2(t.sa2), v3 = sum2(t.sb2);
+                const bool hi = (lane & 16) != 0, up = (lane & 8) != 0;
+                float k0 = (hi ? v2 : v0) + __shfl_xor_sync(0xffffffffu, hi ? v0 : v2, 16);
+                float k1 = (hi ? v3 : v1) + __shfl_xor_sync(0xffffffffu, hi ? v1 : v3, 16);
+                float k = (up ? k1 : k0) + __shfl_xor_sync(0xffffffffu, up ? k0 : k1, 8);
+                float x = sum2(x2);
+                if constexpr (kSecondSweep) {
+                    x += __shfl_xor_sync(0xffffffffu, x, 16);
+                    x += __shfl_xor_sync(0xffffffffu, x, 8);
+                }
 #pragma unroll
-            for (int m = 8; m > 0; m >>= 1) {
-                c.za += __shfl_xor_sync(0xffffffffu, c.za, m); c.zb += __shfl_xor_sync(0xffffffffu, c.zb, m);
-                c.s0 += __shfl_xor_sync(0xffffffffu, c.s0, m); c.sb += __shfl_xor_sync(0xffffffffu, c.sb, m);
-                c.x += __shfl_xor_sync(0xffffffffu, c.x, m);
+                for (int m = 4; m > 0; m >>= 1) {
+                    k += __shfl_xor_sync(0xffffffffu, k, m);
+                    if constexpr (kSecondSweep) x += __shfl_xor_sync(0xffffffffu, x, m);
+                }
+                float kan, kbn;
+                references(kan, kbn);                // (of the next pair)
+                const bool differ = DIV == FSD_DIV_TV || __any_sync(0xffffffffu, t.diff != 0);
+                WarpPost& w = sh.post[n & 1][warp];
+                if ((lane & 7) == 0) w.z[lane >> 3] = k;
+                if (lane == 1) *reinterpret_cast<float4*>(&w.ka) = make_float4(ka, kb, x, __uint_as_float(differ ? 1u : 0u));
+                __syncwarp();                        // (every lane is through with the slot, too: it takes the pair after the next two)
+                if (lane == 0) mbar_arrive(&sh.posted[n & 1]);
+                ka2 = ka1; kb2 = kb1; ka1 = ka; kb1 = kb; ka = kan; kb = kbn;
             }
-            c.diff = __reduce_or_sync(0xffffffffu, w.diff) != 0 ? 1u : 0u;
-            if constexpr (!kSecondSweep) {
-                // KL has no second sweep, so nobody needs the group's totals: every member leaves its part
-                // straight in the pair's record and goes on.  Without messages there is no channel for
-                // claimed pair ids either: the group's pairs are group_id + round * n_groups throughout.
-                if (live && lane == 0) {
-                    FSD_CHECK(P.timeout_flag + 2, item >= 0 && item < P.n_items && rank < kMaxGroupSize, kChkRecord);
+            slot = nslot; so = nso;
+            if constexpr (kSecondSweep) {
+                __syncwarp();                        // tensor-memory instructions want the warp converged
+                tmem_wait_st();
+            }
+        }
+    } else {
+        // ---- helper warp: fold the warps' posts, exchange with the group, hand out the totals ----
+        // where this group exchanges its statistics: [parity][rank] messages
+        GroupMsg* const xg = P.exchange + static_cast<size_t>(group_id < n_groups ? group_id : 0) * 2 * C;
+        int item = group_id;
+#pragma unroll 1
+        for (int n = 0; n < n_end; ++n, item += n_groups) {
+            const int par = n & 1;
+            const uint32_t tag = static_cast<uint32_t>(n) + 1;       // what this round's messages carry (never 0, the buffer's initial state)
+            bool bad = false;
+            if (n < R && rank == 0 && P.parent != nullptr) {
+                const int pr = __ldg(P.parent + item);
+                bad = pr < -1 || pr >= item % P.G;
+            }
+            if (!warp_wait(&sh.posted[par], (n >> 1) & 1, P.timeout_flag)) break;
+            FSD_CHECK(P.timeout_flag + 2, n >= R || (item >= 0 && item < P.n_items && rank < kMaxGroupSize), kChkRecord);
+            // What the compute warps wait for comes first: Z and the references.  Lanes 0..15 take the
+            // target row's of one warp each, lanes 16..31 the draft row's.
+            __syncwarp();
+            const WarpPost& w = sh.post[par][lane & 15];
+            const bool b_side = lane >= 16;
+            const float wk = b_side ? w.kb : w.ka, wz = b_side ? w.z[1] : w.z[0];
+            float s = b_side ? w.z[3] : w.z[2], x = b_side ? 0.f : w.x;         // (read now: the slot is free once the totals are out)
+            const bool differ = __any_sync(0xffffffffu, w.diff != 0);
+            float Ka = -INFINITY, Kb = -INFINITY, f = 0.f;
+            if (n < R) {
+                Ka = warp_redux_max_nan(b_side ? -INFINITY : wk); Kb = warp_redux_max_nan(b_side ? wk : -INFINITY);
+                f = pow2_ref(wk, b_side ? Kb : Ka);
+                float z = wz * f;
+#pragma unroll
+                for (int m = 8; m > 0; m >>= 1) z += __shfl_xor_sync(0xffffffffu, z, m);
+                if constexpr (kSecondSweep) {
+                    // lanes 0 and 16 each store one 16-byte unit of this block's message; every unit ends in the round's tag
+                    if ((lane & 15) == 0 && !(n == 0 && group_id == 0 && rank == P.silent_rank))
+                        st_unit(&xg[par * C + rank].u[b_side], b_side ? Kb : Ka, z, 0.f, tag);
+                    // (while it travels: the slot all warps are through with takes the pair after the next two)
+                    __syncwarp();
+                    issue_slices();
+                    // group totals for the second sweep (float is enough there): lane r fetches the target
+                    // row's unit of block r, lane 16 + r the draft row's; a second fetch where C > 16
+                    const int r0 = lane & 15;
+                    float tk0 = -INFINITY, tz0 = 0.f, tk1 = -INFINITY, tz1 = 0.f;
+                    bool got = false;
+#pragma unroll 1
+                    for (uint32_t i = 0; i < P.poll_limit; ++i) {
+                        bool ok = true;
+                        if (r0 < C) {
+                            const uint4 u = ld_unit(&xg[par * C + r0].u[b_side]);
+                            ok = u.w == tag;
+                            tk0 = __uint_as_float(u.x); tz0 = __uint_as_float(u.y);
+                        }
+                        if (r0 + 16 < C) {
+                            const uint4 u = ld_unit(&xg[par * C + r0 + 16].u[b_side]);
+                            ok = ok && u.w == tag;
+                            tk1 = __uint_as_float(u.x); tz1 = __uint_as_float(u.y);
+                        }
+                        if (__all_sync(0xffffffffu, ok)) { got = true; break; }
+                        // has anybody's wait run out?  (then nothing this warp waits for is certain to come)
+                        if ((i & 255u) == 255u && __any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(P.timeout_flag) != 0)) break;
+                    }
+                    if (!got) {
+                        if (lane == 0) atomicExch(P.timeout_flag, 1);
+                        break;
+                    }
+                    const float tk = fmax_nan(tk0, tk1);
+                    const float Ga = warp_redux_max_nan(b_side ? -INFINITY : tk), Gb = warp_redux_max_nan(b_side ? tk : -INFINITY);
+                    const float G = b_side ? Gb : Ga;
+                    float tz = tz0 * pow2_ref(tk0, G);
+                    if (C > 16) tz = fmaf(tz1, pow2_ref(tk1, G), tz);
+#pragma unroll
+                    for (int m = 8; m > 0; m >>= 1) tz += __shfl_xor_sync(0xffffffffu, tz, m);
+                    // 1 / Z to the last bit or so; 0 where the row is not a valid distribution (NaN included)
+                    float iz = 0.f;
+                    if (tz > 1.0e-30f && tz < 1.0e30f) { const float r = rcp(tz); iz = fmaf(r, fmaf(-tz, r, 1.f), r); }
+                    if ((lane & 15) == 0) *reinterpret_cast<float2*>(reinterpret_cast<float*>(&sh.tot[par]) + 2 * b_side) = make_float2(G, iz);
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&sh.totals[par]);
+                }
+                // ---- what only the record needs ----
+                const float d = wk == -INFINITY ? 0.f : wk - (b_side ? Kb : Ka);
+                if constexpr (DIV == FSD_DIV_KL) {
+                    const float d_b = __shfl_down_sync(0xffffffffu, d, 16);
+                    s = b_side ? 0.f : scale_kl(f, fmaf(d - d_b, wz, s));
+                } else {
+                    s = f * fmaf(d, wz, s);
+                }
+#pragma unroll
+                for (int m = 8; m > 0; m >>= 1) s += __shfl_xor_sync(0xffffffffu, s, m);
+                const float z_b = __shfl_down_sync(0xffffffffu, z, 16), s_b = __shfl_down_sync(0xffffffffu, s, 16);
+                if (lane == 0) {
                     PairRecord* r = P.records + item;
+                    Stats c;
+                    c.ka = Ka; c.kb = Kb; c.za = z; c.zb = z_b; c.s0 = s; c.sb = s_b; c.x = 0.f; c.diff = differ ? 1u : 0u;
                     r->part[rank] = c;
                     if (rank == 0) { r->ncta = static_cast<uint32_t>(C); r->state = bad ? kRecordBadTree : kRecordStats; }
                 }
-                const long long id = static_cast<long long>(group_id) + static_cast<long long>(li + ahead) * n_groups;
-                const bool stop = __any_sync(0xffffffffu, dead);
-                if (lane == 0) {
-                    sh.items[(li + ahead) & 7] = (stop || id >= 0x3fffffffLL) ? 0x3fffffff : static_cast<int>(id);
-                    *reinterpret_cast<float4*>(sh.tot) = make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+            if constexpr (kSecondSweep) {
+                if (n >= 2) {
+#pragma unroll
+                    for (int m = 8; m > 0; m >>= 1) x += __shfl_xor_sync(0xffffffffu, x, m);
+                    if (lane == 0) P.records[item - 2 * n_groups].x[rank] = x;
                 }
-                named_sync(bar_totals);
             } else {
-            {
-                const uint32_t cl = __shfl_sync(0xffffffffu, claimed, 0);   // rank 0's message carries the pair id it took
-                if (rank == 0) c.diff |= cl << 1;
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&sh.totals[par]);
+                issue_slices();
             }
-            // lanes 0..2 each store one 16-byte unit of this virtual CTA's message; every unit ends in the round's tag
-            if (lane < 3 && !(li == 0 && group_id == 0 && rank == P.silent_rank)) {
-                const float m0 = lane == 0 ? c.ka : lane == 1 ? c.zb : c.x;
-                const float m1 = lane == 0 ? c.kb : lane == 1 ? c.s0 : __uint_as_float(c.diff);
-                const float m2 = lane == 0 ? c.za : lane == 1 ? c.sb : 0.f;
-                st_unit(&xg[par * C + rank].u[lane], m0, m1, m2, tag);
-            }
-            // group totals for the second sweep (float is enough there); lane r fetches virtual CTA r's message
-            Stats t;
-            t.ka = -INFINITY; t.kb = -INFINITY; t.za = 0.f; t.zb = 0.f; t.s0 = 0.f; t.sb = 0.f; t.x = 0.f; t.diff = 0;
-            if (!__any_sync(0xffffffffu, dead)) {          // (a lane's own earlier wait may have run out: decide as a warp)
-                bool got = false;
-#pragma unroll 1
-                for (uint32_t i = 0; i < P.poll_limit; ++i) {
-                    // with the first fetch and every 256th: has anybody's wait run out?  (then nothing
-                    // this warp waits for is certain to come, and the group takes no further pair)
-                    const bool look = (i & 255u) == 0;
-                    int gave_up = 0;
-                    if (look && lane == 0) gave_up = *reinterpret_cast<volatile int*>(P.timeout_flag);
-                    bool ok = true;
-                    if (lane < C) {
-                        const uint4 u0 = ld_unit(&xg[par * C + lane].u[0]), u1 = ld_unit(&xg[par * C + lane].u[1]),
-                                    u2 = ld_unit(&xg[par * C + lane].u[2]);
-                        ok = u0.w == tag && u1.w == tag && u2.w == tag;
-                        t.ka = __uint_as_float(u0.x); t.kb = __uint_as_float(u0.y); t.za = __uint_as_float(u0.z);
-                        t.zb = __uint_as_float(u1.x); t.s0 = __uint_as_float(u1.y); t.sb = __uint_as_float(u1.z);
-                        t.x = __uint_as_float(u2.x); t.diff = u2.y;
-                    }
-                    const bool all_ok = __all_sync(0xffffffffu, ok);
-                    if (look && __shfl_sync(0xffffffffu, gave_up, 0) != 0) break;
-                    if (all_ok) { got = true; break; }
-                }
-                if (!got) {
-                    if (lane == 0) atomicExch(P.timeout_flag, 1);
-                    dead = true;
-                    t.ka = __int_as_float(0x7fc00000);   // the totals of a round that never completed are invalid
-                }
-            }
-            {
-                // after a wait that ran out this group takes no further pair: every member reads the same
-                // "none" and leaves together once the pairs already in its ring are through
-                const uint32_t sent = __shfl_sync(0xffffffffu, t.diff, 0) >> 1;
-                const bool stop = __any_sync(0xffffffffu, dead);
-                const uint32_t nxt = stop ? 0x3fffffffu : sent;
-                t.diff &= 1u;
-                if (lane == 0) sh.items[(li + ahead) & 7] = static_cast<int>(nxt);
-            }
-            const float Ka = warp_max_nan(t.ka), Kb = warp_max_nan(t.kb);
-            float tza = t.ka == -INFINITY ? 0.f : t.za * pow2_int(t.ka - Ka);
-            float tzb = t.kb == -INFINITY ? 0.f : t.zb * pow2_int(t.kb - Kb);
-#pragma unroll
-            for (int m = 8; m > 0; m >>= 1) {
-                tza += __shfl_xor_sync(0xffffffffu, tza, m); tzb += __shfl_xor_sync(0xffffffffu, tzb, m);
-            }
-            if (lane == 0) *reinterpret_cast<float4*>(sh.tot) = make_float4(Ka, Kb, tza, tzb);
-            named_sync(bar_totals);
-            // rank 0 hands the parts to the finish kernel, which folds them in double; the
-            // previous pair gets its second-sweep sums
-            if (rank == 0 && lane < C) {
-                if (prev_item >= 0) P.records[prev_item].x[lane] = t.x;
-                if (live) {
-                    FSD_CHECK(P.timeout_flag + 2, item >= 0 && item < P.n_items && C <= kMaxGroupSize, kChkRecord);
-                    PairRecord* r = P.records + item;
-                    r->part[lane] = t;
-                    if (lane == 0) { r->ncta = static_cast<uint32_t>(C); r->state = bad ? kRecordBadTree : kRecordStats; }
-                }
-            }
-            }   // (the exchange that JS and TV need)
         }
-        if (warp != static_cast<int>(li & (kStreamWarps - 1))) named_sync(bar_totals);
-        const float4 tot = *reinterpret_cast<const float4*>(sh.tot);
-        const float Ka = tot.x, Kb = tot.y, tZa = tot.z, tZb = tot.w;
-        prev_item = -1;
-        x_carry = 0.f;
-        if (!live) break;
-        prev_item = kSecondSweep ? item : -1;        // (no second-sweep sum to publish a round later)
-
-        // ---- second sweep over the parked e values ----
-        if (kSecondSweep) {
-            const bool ok = tZa > 0.f && tZb > 0.f && tZa < 3.0e38f && tZb < 3.0e38f;   // false for NaN too
-            const float iza = ok ? 1.0f / tZa : 0.f, izb = ok ? 1.0f / tZb : 0.f;
-            const float ia = (ka == -INFINITY || !ok) ? 0.f : pow2_int(ka - Ka) * iza;
-            const float ib = (kb == -INFINITY || !ok) ? 0.f : pow2_int(kb - Kb) * izb;
-            uint64_t x2 = 0;
-            float xt = 0.f;
-            // s = p + q + 1e-37 keeps lg2 finite where both terms vanish; the shift is below one ulp of any s that matters
-            const uint64_t ia2 = pack2(ia, ia), ib2 = pack2(ib, ib), tiny2 = pack2(1e-37f, 1e-37f);
-#pragma unroll
-            for (int s = 0; s < kMaxStagesPerPair; ++s) {
-                if (s < ns) {
-                    float e[VPT][EPT];
-                    if (s < NT) {
-#pragma unroll
-                        for (int v = 0; v < VPT; ++v) tmem_ld<EPT>(taddr + (s * VPT + v) * EPT, e[v]);
-                        tmem_wait_ld();
-                    } else {
-#pragma unroll
-                        for (int v = 0; v < VPT; ++v) {
-#pragma unroll
-                            for (int j = 0; j < EPT; ++j) e[v][j] = ereg[(s - NT < 0 ? 0 : s - NT) * EPS + v * EPT + j];
-                        }
-                    }
-#pragma unroll
-                    for (int v = 0; v < VPT; ++v) {
-#pragma unroll
-                        for (int j = 0; j < EPV; j += 2) {
-                            const uint64_t ea2 = pack2(e[v][j], e[v][j + 1]), eb2 = pack2(e[v][EPV + j], e[v][EPV + j + 1]);
-                            if constexpr (DIV == FSD_DIV_JS) {
-                                const uint64_t s2 = fma2(eb2, ib2, fma2(ea2, ia2, tiny2));
-                                float s0, s1;
-                                unpack2(s2, s0, s1);
-                                x2 = fma2(s2, pack2(lg2(s0), lg2(s1)), x2);
-                            } else {
-                                // separately rounded products: a fused p - q would make TV(p, p) != 0
-                                const uint64_t d2 = fma2(mul2(eb2, ib2), pack2(-1.f, -1.f), mul2(ea2, ia2));
-                                float d0, d1;
-                                unpack2(d2, d0, d1);
-                                xt += fabsf(d0) + fabsf(d1);
-                            }
-                        }
-                    }
-                }
-            }
-            float x = sum2(x2) + xt;
-#pragma unroll
-            for (int m = 16; m > 0; m >>= 1) x += __shfl_xor_sync(0xffffffffu, x, m);
-            x_carry = x;
-        }
-
-        // ---- next pair ----
-        g += ns;
-        ++li;
-        item = sh.items[li & 7];
-    }
-
-    // ---- release tensor memory ----
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    if (tid == 0) {
-        // Every copy started into this virtual CTA's ring has landed before the CTA may leave: normally the
-        // first sweep consumed them all and these waits return at once; after a wait that ran out
-        // some may still be on their way (a copy, once started, always completes).
-        for (int slot = 0; slot < kRing; ++slot) {
-            const uint32_t n = sh.armed[slot];
-            if (n == 0) continue;
+        // Every copy started has landed before the block may leave: normally the rounds consumed them all;
+        // after a wait that ran out some may still be on their way (a copy, once started, always completes).
+        for (int k = in > P.ring ? in - P.ring : 0; k < in; ++k) {
 #pragma unroll 1
             for (uint32_t i = 0; i < kSpinLimit; ++i)
-                if (mbar_try_wait(&sh.full[slot], (n - 1) & 1)) break;
+                if (__all_sync(0xffffffffu, mbar_try_wait(&sh.full[k % P.ring], (k / P.ring) & 1))) break;
         }
     }
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*tmem_base_slot), "r"(kStreamHalves * kTmemCols) : "memory");
+
+    if constexpr (kSecondSweep) {
+        // ---- release tensor memory ----
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncthreads();
+        __syncwarp();
+        if (warp == kComputeWarps)
+            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(sh.tmem_base), "n"(kTmemCols) : "memory");
     }
 }
 

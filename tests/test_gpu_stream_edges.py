@@ -1,0 +1,87 @@
+"""The streaming kernel at the sizes where its partition can go wrong, against the oracle: rows of
+one entry to a few granules, either side of a step, of a block's slice and of the longest row it
+takes; rows and bases that are not 16-byte aligned; logits its quick form has to notice (a late
+spike, masked entries in some parts only); fewer pairs than a round and many rounds."""
+
+import numpy as np
+import pytest
+import torch
+
+import fsd_inputs as gi
+from tests import parity
+
+pytestmark = pytest.mark.gpu
+
+STEP = {"bf16": 256, "f32": 256}          # vocabulary entries of a step (32 lanes x 8)
+SLICE = {"bf16": 16384, "f32": 8192}      # of a block's largest slice
+LONGEST = {"bf16": 20 * 16384, "f32": 20 * 8192}
+
+
+def _chain(B, gamma, V, dtype, wid, **kw):
+    return gi.make_chain(B, gamma, V, dtype=dtype, recipe="zipf", sigma=(0.2, 1.5), sigma_mode="uniform",
+                         disjoint_frac=0.1, workload_id=wid, **kw)
+
+
+def _check(c, dev=None, **kw):
+    return parity.check_chain(c.target, c.draft, c.draft_tokens, c.u_accept, c.u_sample, c.dtype, dev=dev, **kw)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("edge", ["step", "slice", "two_slices", "longest"])
+@pytest.mark.parametrize("d", [-9, -8, -1, 0, 1, 8])
+def test_vocabulary_at_an_edge_of_the_partition(dtype, edge, d):
+    base = {"step": STEP, "slice": SLICE, "longest": LONGEST}.get(edge, {k: 2 * v for k, v in SLICE.items()})[dtype]
+    V = base + d
+    c = _chain(1 if edge == "longest" else 3, 2, V, dtype, 800)
+    for div in ("js", "kl", "tv") if edge != "longest" else ("js",):
+        r = _check(c, div=div, T=0.2)
+        assert not (r["gpu"].row_status & 2).any()
+
+
+@pytest.mark.parametrize("dtype,offset", [("bf16", 1), ("bf16", 3), ("bf16", 6), ("f32", 1), ("f32", 3)])
+@pytest.mark.parametrize("V", [5, 1001, 4096, 33003])
+def test_bases_and_rows_off_a_16_byte_boundary(dtype, offset, V):
+    c = _chain(3, 3, V, dtype, 801)
+
+    def shifted(a, off):
+        t = parity.to_device(a, dtype)
+        buf = torch.empty(t.numel() + off + 16, dtype=t.dtype, device="cuda")
+        v = buf[off:off + t.numel()].view(t.shape)
+        v.copy_(t)
+        return v
+
+    dev = dict(t=shifted(c.target, offset), d=shifted(c.draft, (3 * offset) % 8), tok=parity.to_device(c.draft_tokens, dtype),
+               ua=parity.to_device(c.u_accept, dtype), us=parity.to_device(c.u_sample, dtype))
+    for div in ("js", "kl", "tv"):
+        _check(c, dev=dev, div=div, T=0.1)
+    _check(c, dev=dev, mode="sd", T=0.0)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("V", [40000, 40003])
+def test_parts_the_quick_form_cannot_take(dtype, V):
+    """Spikes far above a part's first step, and entries of -inf in some parts: the warps concerned have
+    to notice and do the sweep over, in the first, a middle and the last round alike."""
+    B, gamma = 40, 5                                # several rounds per group
+    c = gi.make_chain(B, gamma, V, dtype=dtype, recipe="spike", sigma=(0.5, 1.0), workload_id=802)
+    f32 = dtype == "f32"
+    t = c.target if f32 else gi.bf16_bits_to_f32(c.target)
+    d = c.draft if f32 else gi.bf16_bits_to_f32(c.draft)
+    for b, v in ((0, 777), (13, 20011), (39, V - 1)):
+        t[b, :, v] += 60.0                          # 86 binades above the part's first step
+        d[b, :, (v + 4000) % V] += 45.0
+    t[5, 1, 9000:9300] = -np.inf
+    d[20, 2, ::97] = -np.inf
+    t[38, 4, : V // 2] = -np.inf
+    if not f32:
+        c.target[:] = gi.f32_to_bf16_bits(t)
+        c.draft[:] = gi.f32_to_bf16_bits(d)
+    for div in ("js", "kl", "tv"):
+        _check(c, div=div, T=0.25)
+
+
+@pytest.mark.parametrize("B,gamma,V", [(1, 1, 24), (2, 3, 8200), (200, 2, 520), (400, 3, 264), (64, 4, 16392)])
+def test_few_pairs_and_many_rounds(B, gamma, V):
+    c = _chain(B, gamma, V, "bf16", 803)
+    for div in ("js", "kl"):
+        _check(c, div=div, T=0.15)

@@ -325,6 +325,31 @@ int static_scratch(void** out) {
     return FSD_OK;
 }
 
+// A block on its own where a walk gives no thread more than one row: there the cluster's start and its
+// pushes cost more than they share out (300 x 6 on a B200: calibration 6.2 us in one block, 8.7 us in a
+// cluster; 4096 x 8: 34 and 11).
+bool tuning_in_one_block(int B) { return B <= kTuneThreads; }
+// A tuning kernel on `clusters` clusters; shared memory for as many of a block's rows as there are, up to what is staged.
+template <typename... KArgs, typename... Args>
+int launch_tuning(void (*kernel)(KArgs...), int threads, int cs, int clusters, int B, int G, void* stream, Args... args) {
+    // two tiles, or as much as the block's rows take (rounded out to 16 bytes at both ends)
+    const long long rows = ((B + 3ll) / 4 + cs - 1) / cs * 4, want = rows * G * 4 + 32;
+    const size_t bytes = static_cast<size_t>(want <= kTuneTileBytes - 16 ? want : 2 * kTuneTileBytes);
+    // (the calibration has 35 KB of its own; 48 KB in all need no attribute)
+    if (bytes > 12 * 1024 && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kTuneTileBytes) != cudaSuccess) return FSD_ERR_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(clusters) * cs, 1, 1);
+    cfg.blockDim = dim3(static_cast<unsigned>(threads), 1, 1);
+    cfg.dynamicSmemBytes = bytes;
+    cfg.stream = static_cast<cudaStream_t>(stream);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = cs; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cs > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...) == cudaSuccess ? FSD_OK : FSD_ERR_CUDA;
+}
+
 }  // namespace
 
 extern "C" {
@@ -509,9 +534,12 @@ int fsd_threshold_sweep(const float* divergence, int B, int positions, const flo
     if (B < 1 || positions < 1 || n_thresholds < 1) return FSD_ERR_SHAPE;
     if (static_cast<long long>(B) * positions > INT_MAX) return FSD_ERR_SHAPE;      // the kernels count in 32 bits
     if (compare != FSD_CMP_LT && compare != FSD_CMP_LE) return FSD_ERR_ENUM;
-    fsd_threshold_sweep_kernel<<<n_thresholds, 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        divergence, B, positions, thresholds, compare, mean_accept_len, accept_fraction);
-    return cudaGetLastError() == cudaSuccess ? FSD_OK : FSD_ERR_CUDA;
+    // a cluster per group of thresholds, as many as the GPU holds at once, and as few thresholds each as that gives
+    const bool one = tuning_in_one_block(B);
+    const int cs = one ? 1 : kTuneCluster, most = 148 / cs, rows = (B + cs - 1) / cs;
+    const int threads = rows >= kTuneThreads ? kTuneThreads : (rows + 31) / 32 * 32 < 64 ? 64 : (rows + 31) / 32 * 32;
+    return launch_tuning(one ? fsd_threshold_sweep_kernel<1> : fsd_threshold_sweep_kernel<kTuneCluster>, threads, cs, n_thresholds < most ? n_thresholds : most, B, positions, stream, divergence, B, positions, thresholds, n_thresholds,
+                         compare, mean_accept_len, accept_fraction);
 }
 
 int fsd_calibrate_threshold(const float* divergence, int B, int positions, float target_mean_accept_len, int compare,
@@ -520,9 +548,9 @@ int fsd_calibrate_threshold(const float* divergence, int B, int positions, float
     if (B < 1 || positions < 1 || !(target_mean_accept_len >= 0.f)) return FSD_ERR_SHAPE;   // NaN target included
     if (static_cast<long long>(B) * positions > INT_MAX) return FSD_ERR_SHAPE;      // the kernels count in 32 bits
     if (compare != FSD_CMP_LT && compare != FSD_CMP_LE) return FSD_ERR_ENUM;
-    fsd_calibrate_kernel<<<1, kTuneThreads, 0, static_cast<cudaStream_t>(stream)>>>(
-        divergence, B, positions, target_mean_accept_len, compare, threshold_out, achieved_out);
-    return cudaGetLastError() == cudaSuccess ? FSD_OK : FSD_ERR_CUDA;
+    const bool one = tuning_in_one_block(B);
+    return launch_tuning(one ? fsd_calibrate_kernel<1> : fsd_calibrate_kernel<kTuneCluster>, kTuneThreads, one ? 1 : kTuneCluster, 1, B, positions, stream, divergence, B, positions, target_mean_accept_len, compare,
+                         threshold_out, achieved_out);
 }
 
 int fsd_accept_labels(const float* divergence, int B, int positions, float threshold, int compare, uint8_t* labels,

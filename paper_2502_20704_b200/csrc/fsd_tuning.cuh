@@ -6,11 +6,22 @@
 //
 // With P[b, k] = max(D[b, 0..k]) (NaN once a NaN has been seen) the accepted length of row b is
 // the number of k with P[b, k] cmp T, so
-//   * a sweep needs one pass per candidate threshold, and
+//   * a sweep counts, for every candidate threshold, the prefix maxima that pass, and
 //   * the smallest T that reaches a wanted mean accepted length is an order statistic of the
 //     multiset {P[b, k]}: the ceil(target * B)-th smallest value v (T = v under <=, the next
-//     float above v under <).  It is found by a most-significant-byte-first radix selection on
-//     the float bit patterns (monotone for non-negative floats), four passes of 256 bins.
+//     float above v under <).  It is found by a most-significant-digit-first radix selection on
+//     the float bit patterns (monotone for non-negative floats): 12, 10 and 9 bits below the sign;
+//     when the first digit leaves few candidates they are ranked directly.  The first digit is wide because divergences sit in few binades: with 16 bins a binade the
+//     lanes of a warp seldom add to the same one.
+//
+// What bounds these kernels is latency: 4096 x 8 divergences are 128 KB.  Neither call has a
+// workspace, so the blocks that share a job are a cluster (8 blocks): one for the calibration, one
+// for every few thresholds of a sweep; few rows take single blocks.  A block's rows come to shared
+// memory by bulk copies and, where they all fit, stay there for every walk; a thread walks a row
+// in the widest loads its length allows, which also keeps lanes that walk neighbouring rows off one
+// another's banks.  What the blocks tell one another is pushed (st.async, bulk copies between the
+// blocks' shared memories) and counted in on the receiver's barrier: a cluster barrier orders all
+// memory first, and reading eight histograms back from the peers took longer than all the rest.
 #pragma once
 
 #include <cstdint>
@@ -20,7 +31,11 @@
 
 namespace fsd {
 
-constexpr int kTuneThreads = 1024;
+constexpr int kTuneThreads = 512;             // at most; a sweep over few rows takes fewer
+constexpr int kTuneCluster = 8;               // the portable size
+constexpr int kTuneBins = 4096;               // of the first digit; 1024 and 512 of the others
+constexpr int kTuneTileBytes = 72 * 1024;     // a tile of rows; two are in shared memory
+constexpr int kSweepAtOnce = 4;               // thresholds a thread counts for in one walk over its rows
 constexpr uint32_t kKeyInf = 0x7f800000u;     // keys above this are NaN (or negative): never accepted
 
 // Sortable key of a prefix maximum: divergences are >= 0, so the bit pattern orders them; -0 and
@@ -30,128 +45,424 @@ __device__ __forceinline__ uint32_t tune_key(float p) {
     return p <= 0.f ? 0u : __float_as_uint(p);
 }
 
-// ---- sweep: one CTA per candidate threshold -------------------------------------------------
-__global__ void __launch_bounds__(256) fsd_threshold_sweep_kernel(const float* __restrict__ D, int B, int G,
-                                                                  const float* __restrict__ thresholds, int cmp,
-                                                                  float* __restrict__ mean_len, float* __restrict__ frac) {
-    __shared__ unsigned long long part[8];
-    const float T = thresholds[blockIdx.x];
-    unsigned long long total = 0;
-    for (int b = threadIdx.x; b < B; b += blockDim.x) {
-        const float* row = D + static_cast<size_t>(b) * G;
-        int n = 0;
-        while (n < G && passes(row[n], T, cmp)) ++n;
-        total += static_cast<unsigned long long>(n);
-    }
-#pragma unroll
-    for (int m = 16; m > 0; m >>= 1) total += __shfl_xor_sync(0xffffffffu, total, m);
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = total;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long t = 0;
-        for (int w = 0; w < static_cast<int>(blockDim.x >> 5); ++w) t += part[w];
-        mean_len[blockIdx.x] = static_cast<float>(static_cast<double>(t) / static_cast<double>(B));
-        frac[blockIdx.x] = static_cast<float>(static_cast<double>(t) / (static_cast<double>(B) * static_cast<double>(G)));
-    }
+// ---- pushes between the blocks of a cluster -------------------------------------------------
+__device__ __forceinline__ uint32_t cluster_addr(const void* p, int rank) {       // of the same object in block `rank`
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void st_async(uint32_t addr, uint64_t v, uint32_t bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(addr), "l"(v), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void bulk_push(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(dst), "r"(smem_u32(src)), "r"(bytes), "r"(bar) : "memory");
+}
+// Bounded; what it waits for are copies already started or pushes of peers that run.
+__device__ __forceinline__ bool tune_wait(uint64_t* bar, uint32_t parity) {
+#pragma unroll 1
+    for (uint32_t i = 0; i < kSpinLimit; ++i)
+        if (mbar_try_wait(bar, parity)) return true;
+    return false;
 }
 
-// ---- calibration: one CTA, radix selection over the prefix maxima ----------------------------
-// Calls f(key, valid) for every prefix maximum of the rows this thread owns.  Every thread of the
-// CTA makes the same number of calls (rows past the end come with valid = false), so f may use
-// full-warp collectives.
-template <typename F>
-__device__ __forceinline__ void for_prefix_maxima(const float* __restrict__ D, int B, int G, F f) {
-    for (int b0 = 0; b0 < B; b0 += blockDim.x) {
-        const int b = b0 + threadIdx.x;
-        const bool valid = b < B;
-        const float* row = D + static_cast<size_t>(valid ? b : 0) * G;
-        float p = 0.f;
-        bool nan = false;
-        for (int k = 0; k < G; ++k) {
-            const float d = row[k];
-            nan = nan || d != d;
-            p = fmaxf(p, d);
-            f(nan ? 0xffffffffu : tune_key(p), valid);
+// ---- a block's rows [row0, row1) of the divergence matrix, tile by tile ---------------------
+// Two tiles are in shared memory at most; a block whose rows are no more than that copies them once.
+struct TuneRows {
+    const float* D;
+    int G, row0, rows, tile, tiles;       // rows a tile has (a multiple of four, so that tiles start 16 bytes apart like D), and tiles
+    int off;                              // words between a 16-byte boundary and D
+    bool staged;                          // (a single row longer than a tile is walked where it is)
+    float* buf;
+    uint64_t* bar;                        // [2]
+    int seq, issued;                      // tiles walked and asked for so far, over all walks
+};
+__device__ __forceinline__ void tune_issue(TuneRows& t) {         // one thread
+    const int i = t.issued % t.tiles, slot = t.issued & 1, n = min(t.tile, t.rows - i * t.tile);
+    const uintptr_t first = reinterpret_cast<uintptr_t>(t.D + static_cast<size_t>(t.row0 + i * t.tile) * t.G);
+    const uintptr_t a = first & ~uintptr_t(15), e = (first + static_cast<size_t>(n) * t.G * 4 + 15) & ~uintptr_t(15);
+    float* dst = t.buf + slot * (kTuneTileBytes / 4);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    mbar_arrive_expect_tx(&t.bar[slot], static_cast<uint32_t>(e - a));
+    bulk_g2s(dst, reinterpret_cast<const void*>(a), static_cast<uint32_t>(e - a), &t.bar[slot]);
+}
+// Rows of block `rank` of `cs`; starts the first copies.  `bar`: two barriers, initialised (count 1).
+__device__ __forceinline__ TuneRows tune_rows(const float* D, int B, int G, int rank, int cs, float* buf, uint64_t* bar) {
+    TuneRows t;
+    const int quads = (B + 3) / 4, base = quads / cs, rem = quads % cs;
+    t.D = D; t.G = G; t.buf = buf; t.bar = bar; t.seq = 0; t.issued = 0;
+    t.row0 = 4 * (rank * base + min(rank, rem));
+    t.rows = max(0, min(4 * (base + (rank < rem ? 1 : 0)), B - t.row0));
+    const long long quad_bytes = 16ll * G;
+    t.staged = quad_bytes + 16 <= kTuneTileBytes;
+    t.tile = t.staged ? 4 * static_cast<int>((kTuneTileBytes - 16) / quad_bytes) : t.rows;
+    t.tiles = t.staged ? (t.rows + t.tile - 1) / t.tile : (t.rows > 0 ? 1 : 0);
+    t.off = static_cast<int>((reinterpret_cast<uintptr_t>(D) & 15) / 4);
+    if (t.staged)
+        for (; t.issued < 2 && t.issued < t.tiles; ++t.issued)
+            if (threadIdx.x == 0) tune_issue(t);
+    return t;
+}
+// One thread's walk along one row: step(d) for every position in order, false to stop.
+template <int W, typename F>
+__device__ __forceinline__ void walk_row(const float* row, int G, F step) {
+    for (int k = 0; k < G; k += W) {
+        float d[W];
+        if constexpr (W == 4) { const float4 v = *reinterpret_cast<const float4*>(row + k); d[0] = v.x; d[1] = v.y; d[2] = v.z; d[3] = v.w; }
+        else if constexpr (W == 2) { const float2 v = *reinterpret_cast<const float2*>(row + k); d[0] = v.x; d[1] = v.y; }
+        else d[0] = row[k];
+#pragma unroll
+        for (int q = 0; q < W; ++q) step(d[q]);
+    }
+}
+// One walk over all of the block's rows: begin() / step(d) / end() per row.  All threads of the block take part.
+template <typename Begin, typename Step, typename End>
+__device__ __forceinline__ void tune_walk(TuneRows& t, Begin begin, Step step, End end) {
+    for (int i = 0; i < t.tiles; ++i) {
+        const int slot = t.seq & 1, n = min(t.tile, t.rows - i * t.tile);
+        const bool resident = t.tiles <= 2;
+        const float* base = t.D + static_cast<size_t>(t.row0 + i * t.tile) * t.G;
+        int width = 1;
+        if (t.staged) {
+            // a resident tile i is in slot i for good; others take turns
+            const int s = resident ? i : slot;
+            tune_wait(&t.bar[s], resident ? 0 : (t.seq >> 1) & 1);
+            base = t.buf + s * (kTuneTileBytes / 4) + t.off;
+            width = t.off == 0 && t.G % 4 == 0 ? 4 : t.off % 2 == 0 && t.G % 2 == 0 ? 2 : 1;
+        }
+        for (int r = threadIdx.x; r < n; r += blockDim.x) {
+            const float* row = base + static_cast<size_t>(r) * t.G;
+            begin();
+            if (width == 4) walk_row<4>(row, t.G, step);
+            else if (width == 2) walk_row<2>(row, t.G, step);
+            else walk_row<1>(row, t.G, step);
+            end();
+        }
+        ++t.seq;
+        if (t.staged && !resident) {
+            __syncthreads();                          // everybody is through with the slot
+            if (threadIdx.x == 0) tune_issue(t);      // (the walk after this one starts over: its first tiles are asked for too)
+            ++t.issued;
         }
     }
 }
+// No copy may still be on its way into a block that leaves.
+__device__ __forceinline__ void tune_drain(TuneRows& t) {
+    if (!t.staged) return;
+    if (t.tiles <= 2) {
+        for (int i = 0; i < t.tiles; ++i) tune_wait(&t.bar[i], 0);
+    } else {
+        for (int q = t.seq; q < t.issued; ++q) tune_wait(&t.bar[q & 1], (q >> 1) & 1);
+    }
+}
 
+// ---- sweep: a cluster (or a block) per group of candidate thresholds ---------------------------
+// Each block counts for its rows and pushes its counts to the cluster's first block.  On a B200, 64
+// thresholds: 4096 x 8 13.5 -> 4.6 us, 32768 x 20 245 -> 24 us (a block per threshold before, its
+// threads walking rows in global memory one dependent load at a time).
+template <int CS>
+__global__ void __launch_bounds__(kTuneThreads) fsd_threshold_sweep_kernel(const float* __restrict__ D, int B, int G,
+                                                                           const float* __restrict__ thresholds, int n_thresholds, int cmp,
+                                                                           float* __restrict__ mean_len, float* __restrict__ frac) {
+    extern __shared__ __align__(16) float tune_buf[];
+    __shared__ uint64_t bar[2], link[2];
+    __shared__ unsigned int part[kTuneThreads / 32][kSweepAtOnce];
+    __shared__ uint64_t got[2][kTuneCluster][kSweepAtOnce];      // (B * positions fits an int)
+    const int rank = CS == 1 ? 0 : static_cast<int>(cg::this_cluster().block_rank());
+    const int n_clusters = static_cast<int>(gridDim.x) / CS, cid = static_cast<int>(blockIdx.x) / CS;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) {
+        for (int k = 0; k < 2; ++k) { mbar_init(&bar[k], 1); mbar_init(&link[k], 1); }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    if constexpr (CS > 1) cg::this_cluster().barrier_arrive();   // "this block's barriers are ready": waited for before the first push
+    TuneRows rows = tune_rows(D, B, G, rank, CS, tune_buf, bar);
+    // thresholds cid, cid + n_clusters, ...: kSweepAtOnce of them in one walk
+    int turn = 0;
+    for (int t0 = cid; t0 < n_thresholds; t0 += n_clusters * kSweepAtOnce, ++turn) {
+        float T[kSweepAtOnce];
+        unsigned int n[kSweepAtOnce];
+#pragma unroll
+        for (int j = 0; j < kSweepAtOnce; ++j) {
+            const int t = t0 + j * n_clusters;
+            T[j] = t < n_thresholds ? thresholds[t] : __int_as_float(0x7fc00000);
+            n[j] = 0;
+        }
+        float p = 0.f;
+        const auto begin = [&] { p = -INFINITY; };
+        if (cmp == FSD_CMP_LE) {
+            tune_walk(rows, begin, [&](float d) {
+                p = fmax_nan(p, d);                   // NaN stays and never passes
+#pragma unroll
+                for (int j = 0; j < kSweepAtOnce; ++j) n[j] += p <= T[j];
+            }, [] {});
+        } else {
+            tune_walk(rows, begin, [&](float d) {
+                p = fmax_nan(p, d);
+#pragma unroll
+                for (int j = 0; j < kSweepAtOnce; ++j) n[j] += p < T[j];
+            }, [] {});
+        }
+#pragma unroll
+        for (int j = 0; j < kSweepAtOnce; ++j) {
+            const unsigned int w = __reduce_add_sync(0xffffffffu, n[j]);
+            if (lane == 0) part[warp][j] = w;
+        }
+        __syncthreads();
+        unsigned int sum = 0;
+        if (tid < kSweepAtOnce)
+            for (int w = 0; w < static_cast<int>(blockDim.x >> 5); ++w) sum += part[w][tid];
+        if constexpr (CS > 1) {
+            // (two buffers take turns; nobody is a turn ahead by more than one: see the barrier below)
+            if (turn == 0) cg::this_cluster().barrier_wait();
+            if (rank == 0 && tid == 0) mbar_arrive_expect_tx(&link[turn & 1], CS * kSweepAtOnce * 8);
+            if (tid < kSweepAtOnce) st_async(cluster_addr(&got[turn & 1][rank][tid], 0), sum, cluster_addr(&link[turn & 1], 0));
+            if (rank == 0 && tid < 32) {
+                tune_wait(&link[turn & 1], (turn >> 1) & 1);
+                if (tid < kSweepAtOnce) {
+                    sum = 0;
+                    for (int r = 0; r < CS; ++r) sum += static_cast<unsigned int>(got[turn & 1][r][tid]);
+                }
+            }
+            if (t0 + n_clusters * kSweepAtOnce < n_thresholds) cg::this_cluster().sync();   // more walks than one: nobody overtakes block 0
+        }
+        if (rank == 0 && tid < kSweepAtOnce && t0 + tid * n_clusters < n_thresholds) {
+            const int t = t0 + tid * n_clusters;
+            mean_len[t] = static_cast<float>(static_cast<double>(sum) / static_cast<double>(B));
+            frac[t] = static_cast<float>(static_cast<double>(sum) / (static_cast<double>(B) * static_cast<double>(G)));
+        }
+        __syncthreads();                              // `part` is free again
+    }
+    tune_drain(rows);
+}
+
+// ---- calibration: one cluster (or block), radix selection over the prefix maxima ----------------
+// Calls f(key, count) for every run of equal prefix maxima of this thread's rows.
+template <typename F>
+__device__ __forceinline__ void for_prefix_maxima(TuneRows& rows, F f) {
+    float p = 0.f;
+    uint32_t key = 0;
+    unsigned int run = 0;
+    tune_walk(rows, [&] { p = 0.f; key = 0; run = 0; },
+              [&](float d) {
+                  p = fmax_nan(p, d);
+                  const uint32_t kn = tune_key(p);
+                  if (kn != key && run > 0) { f(key, run); run = 0; }
+                  key = kn;
+                  ++run;
+              },
+              [&] { f(key, run); });
+}
+
+constexpr int kTuneList = kTuneBins / kTuneCluster;                        // candidates that are ranked directly
+struct CalibrateShared {
+    uint64_t bar[2];                                  // tiles
+    uint64_t link[3][3];                              // [digit][parts of the histogram | sums | the digit found]
+    uint64_t list_link;
+    unsigned int hist[kTuneBins];
+    unsigned int recv[kTuneCluster][kTuneBins / kTuneCluster];   // this block's part of the peers' histograms; later, in block 0,
+                                                      // everybody's candidates (sent when all have the first digit, so when all have read)
+    uint64_t sums[kTuneCluster];
+    uint64_t found[2];                                // digit | keys equal to it << 32, keys below it
+    uint32_t list[kTuneList];                         // this block's candidates
+    unsigned int warp_sum[kTuneThreads / 32];
+    unsigned int n_list, count;
+};
+
+// A row's prefix maxima never fall, so a thread adds once per distinct value (two or three a row of
+// eight).  Per digit: every block pushes the eighth of its histogram that block r is to add up to
+// block r, then its sum over that eighth to everybody, and the block whose eighth holds the wanted
+// rank pushes the digit to everybody.  If no more than kTuneList keys share the first digit, they are
+// pushed to block 0, which ranks them by counting.  4096 x 8: 57 -> 11 us, 32768 x 20: 821 -> 74 us (one
+// block and four 8-bit digits before), of which the walks' shared-memory atomics are the larger part.
+template <int CS>
 __global__ void __launch_bounds__(kTuneThreads) fsd_calibrate_kernel(const float* __restrict__ D, int B, int G, float target,
                                                                      int cmp, float* __restrict__ T_out,
                                                                      float* __restrict__ achieved_out) {
-    __shared__ unsigned int hist[256];         // B * positions fits an int
-    __shared__ unsigned long long s_total;
-    __shared__ unsigned long long s_rank;      // rank still to be found inside the selected bin (1-based)
-    __shared__ uint32_t s_prefix;              // the key's bytes selected so far
-    __shared__ int s_found;
+    extern __shared__ __align__(16) float tune_buf[];
+    __shared__ __align__(16) CalibrateShared sh;
+    const int rank = CS == 1 ? 0 : static_cast<int>(cg::this_cluster().block_rank());
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) {
+        for (int k = 0; k < 2; ++k) mbar_init(&sh.bar[k], 1);
+        for (int k = 0; k < 9; ++k) mbar_init(&sh.link[0][0] + k, 1);
+        mbar_init(&sh.list_link, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        sh.count = 0; sh.n_list = 0;
+    }
+    for (int i = tid; i < kTuneBins / 4; i += kTuneThreads) reinterpret_cast<uint4*>(sh.hist)[i] = make_uint4(0, 0, 0, 0);
+    for (int i = tid; i < kTuneList; i += kTuneThreads) sh.list[i] = 0xffffffffu;
+    __syncthreads();
+    if constexpr (CS > 1) cg::this_cluster().barrier_arrive();   // "this block's barriers are ready": waited for before the first push
+    TuneRows rows = tune_rows(D, B, G, rank, CS, tune_buf, sh.bar);
 
-    // positions that must be accepted: ceil(target * B), within [0, B * G]
+    // positions that must be accepted: ceil(target * B), within [0, B * G]  (the host refuses negative and NaN targets)
     const double want = ceil(static_cast<double>(target) * static_cast<double>(B));
     const double most = static_cast<double>(B) * static_cast<double>(G);
-    const unsigned long long need = want <= 0.0 ? 0ull : static_cast<unsigned long long>(want < most ? want : most);
-    // (the host refuses negative and NaN targets)
+    const unsigned int need = want <= 0.0 ? 0u : static_cast<unsigned int>(want < most ? want : most);
 
-    if (threadIdx.x == 0) { s_rank = need; s_prefix = 0; s_found = 1; }
-    __syncthreads();
-
+    uint32_t prefix = 0;
+    unsigned int left = need, below = 0, equal = 0;   // rank still to be found; keys below / equal to the prefix found
+    bool found = need > 0, ranked = false;
+    if constexpr (CS > 1) { if (need == 0) cg::this_cluster().barrier_wait(); }
     if (need > 0) {
-        for (int byte = 3; byte >= 0; --byte) {
-            for (int i = threadIdx.x; i < 256; i += blockDim.x) hist[i] = 0;
-            __syncthreads();
-            const uint32_t prefix = s_prefix;
-            const uint32_t high_mask = byte == 3 ? 0u : (0xffffffffu << (8 * (byte + 1)));
-            for_prefix_maxima(D, B, G, [&](uint32_t key, bool valid) {
-                // lanes that hit the same bin add once (keys cluster in a few bins: plain atomics would serialise)
-                const bool in = valid && key <= kKeyInf && (key & high_mask) == prefix;
-                const uint32_t bin = in ? ((key >> (8 * byte)) & 255u) : 256u;
-                const unsigned peers = __match_any_sync(0xffffffffu, bin);
-                if (in && (threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&hist[bin], static_cast<unsigned int>(__popc(peers)));
+#pragma unroll 1
+        for (int digit = 0; digit < 3; ++digit) {
+            const int shift = digit == 0 ? 19 : digit == 1 ? 9 : 0;
+            const uint32_t mask = digit == 0 ? 0u : digit == 1 ? 0xfff80000u : 0xfffffe00u;   // the digits before this one
+            const uint32_t width = digit == 0 ? 4095u : digit == 1 ? 1023u : 511u;
+            const int part = digit == 0 ? kTuneBins / CS : 1024 / CS;      // bins a block adds up
+            if (digit > 0) {
+                for (int i = tid; i < 1024 / 4; i += kTuneThreads) reinterpret_cast<uint4*>(sh.hist)[i] = make_uint4(0, 0, 0, 0);
+                __syncthreads();
+            }
+            for_prefix_maxima(rows, [&](uint32_t key, unsigned int count) {
+                if (key <= kKeyInf && (key & mask) == prefix) atomicAdd(&sh.hist[(key >> shift) & width], count);
             });
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                unsigned long long rank = s_rank, run = 0;
-                int bin = -1;
-                for (int i = 0; i < 256; ++i) {
-                    if (run + hist[i] >= rank) { bin = i; break; }
-                    run += hist[i];
+            const unsigned int (*mine)[kTuneBins / kTuneCluster] = sh.recv;
+            if constexpr (CS > 1) {
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                if (tid == 0) mbar_arrive_expect_tx(&sh.link[digit][0], static_cast<uint32_t>(part) * 4 * CS);
+                if (tid == 1) mbar_arrive_expect_tx(&sh.link[digit][1], 8 * CS);
+                if (tid == 2) mbar_arrive_expect_tx(&sh.link[digit][2], 16);
+                __syncthreads();
+                if (digit == 0) cg::this_cluster().barrier_wait();
+                if (tid < CS) bulk_push(cluster_addr(&sh.recv[rank][0], tid), sh.hist + tid * part, static_cast<uint32_t>(part) * 4, cluster_addr(&sh.link[digit][0], tid));
+                tune_wait(&sh.link[digit][0], 0);
+            } else {
+                __syncthreads();
+            }
+            // this block's part: its bins (8 a thread when a block has them all, else at most one) and their running sum
+            constexpr int kMost = CS > 1 ? 1 : kTuneBins / kTuneThreads;
+            unsigned int c[kMost], sum = 0;
+            const int per = CS > 1 ? 1 : part / kTuneThreads;
+#pragma unroll
+            for (int q = 0; q < kMost; ++q) {
+                c[q] = 0;
+                if (CS > 1) {
+                    if (tid < part) {
+#pragma unroll
+                        for (int r = 0; r < CS; ++r) c[q] += mine[r][tid];
+                    }
+                } else if (q < per) {
+                    c[q] = sh.hist[per * tid + q];
                 }
-                if (bin < 0) {
-                    s_found = 0;                        // fewer acceptable positions than needed
-                } else {
-                    s_rank = rank - run;
-                    s_prefix = prefix | (static_cast<uint32_t>(bin) << (8 * byte));
+                sum += c[q];
+            }
+            unsigned int incl = sum;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const unsigned int up = __shfl_up_sync(0xffffffffu, incl, d);
+                if (lane >= d) incl += up;
+            }
+            if (lane == 31) sh.warp_sum[warp] = incl;
+            __syncthreads();
+            unsigned int before = 0, all = 0;
+#pragma unroll
+            for (int w = 0; w < kTuneThreads / 32; ++w) { const unsigned int ws = sh.warp_sum[w]; if (w < warp) before += ws; all += ws; }
+            if constexpr (CS > 1) {
+                if (tid < CS) st_async(cluster_addr(&sh.sums[rank], tid), all, cluster_addr(&sh.link[digit][1], tid));
+                tune_wait(&sh.link[digit][1], 0);
+                all = 0;
+                for (int r = 0; r < CS; ++r) { const unsigned int v = static_cast<unsigned int>(sh.sums[r]); if (r < rank) before += v; all += v; }
+            }
+            if (all < left) { found = false; break; } // fewer acceptable positions than needed (the same for all)
+            unsigned int run = before + incl - sum;
+            if (left > run && left <= run + sum) {    // one thread of the cluster
+#pragma unroll
+                for (int q = 0; q < kMost; ++q) {
+                    if (left > run && left <= run + c[q]) {
+                        const uint64_t w0 = static_cast<uint32_t>((CS > 1 ? rank * part : 0) + per * tid + q) | static_cast<uint64_t>(c[q]) << 32, w1 = run;
+                        if constexpr (CS > 1) {
+                            for (int r = 0; r < CS; ++r) {
+                                st_async(cluster_addr(&sh.found[0], r), w0, cluster_addr(&sh.link[digit][2], r));
+                                st_async(cluster_addr(&sh.found[1], r), w1, cluster_addr(&sh.link[digit][2], r));
+                            }
+                        } else {
+                            sh.found[0] = w0; sh.found[1] = w1;
+                        }
+                        run = left;                   // (found: no other bin)
+                    }
+                    run += c[q];
                 }
             }
+            if constexpr (CS > 1) tune_wait(&sh.link[digit][2], 0); else __syncthreads();
+            const uint64_t w0 = sh.found[0];
+            prefix |= static_cast<uint32_t>(w0) << shift;
+            equal = static_cast<unsigned int>(w0 >> 32);
+            const unsigned int lower = static_cast<unsigned int>(sh.found[1]);
+            below += lower; left -= lower;
+            __syncthreads();                          // everybody has read: the histogram and the rest may be written again
+            if (digit == 0 && equal <= kTuneList) { ranked = true; break; }
+        }
+    }
+    if (ranked) {
+        // the keys that share the first digit, from all blocks to block 0
+        for_prefix_maxima(rows, [&](uint32_t key, unsigned int count) {
+            if ((key & 0xfff80000u) != prefix || key > kKeyInf) return;
+            const unsigned int at = atomicAdd(&sh.n_list, count);
+            for (unsigned int q = 0; q < count; ++q) sh.list[at + q] = key;       // (at most `equal` <= kTuneList in all)
+        });
+        if constexpr (CS > 1) {
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            if (rank == 0 && tid == 0) mbar_arrive_expect_tx(&sh.list_link, CS * kTuneList * 4);
             __syncthreads();
-            if (!s_found) break;
+            if (tid == 0) bulk_push(cluster_addr(&sh.recv[rank][0], 0), sh.list, kTuneList * 4, cluster_addr(&sh.list_link, 0));
+            if (rank == 0) {
+                tune_wait(&sh.list_link, 0);
+                if (tid == 0) sh.n_list = 0;
+                __syncthreads();
+                for (int i = tid; i < CS * kTuneList; i += kTuneThreads) {
+                    const uint32_t key = (&sh.recv[0][0])[i];
+                    if (key != 0xffffffffu) sh.list[atomicAdd(&sh.n_list, 1u)] = key;
+                }
+            }
+        }
+        __syncthreads();
+        if (rank == 0 && tid < static_cast<int>(equal)) {
+            const uint32_t key = sh.list[tid];
+            unsigned int less = 0, same = 0;
+            for (unsigned int q = 0; q < equal; ++q) { const uint32_t o = sh.list[q]; less += o < key; same += o == key; }
+            if (less < left && left <= less + same) { sh.found[0] = key | static_cast<uint64_t>(same) << 32; sh.found[1] = less; }   // (all that write, write this)
+        }
+        __syncthreads();
+        if (rank == 0) {
+            prefix = static_cast<uint32_t>(sh.found[0]);
+            equal = static_cast<unsigned int>(sh.found[0] >> 32);
+            below += static_cast<unsigned int>(sh.found[1]);
         }
     }
 
-    // the threshold, then the mean accepted length it gives (one more pass)
+    // the threshold, then the mean accepted length it gives: known from the counts, or (no selection, or +inf) one more walk
     float T;
     if (need == 0) {
         T = 0.f;
-    } else if (!s_found) {
+    } else if (!found) {
         T = INFINITY;
     } else {
-        const float v = __uint_as_float(s_prefix);
-        T = cmp == FSD_CMP_LE ? v : (v == INFINITY ? INFINITY : __uint_as_float(s_prefix + 1u));   // next float above v
+        const float v = __uint_as_float(prefix);
+        T = cmp == FSD_CMP_LE ? v : (v == INFINITY ? INFINITY : __uint_as_float(prefix + 1u));   // next float above v
     }
-    __syncthreads();
-    if (threadIdx.x == 0) s_total = 0;
-    __syncthreads();
-    unsigned long long mine = 0;
-    for_prefix_maxima(D, B, G, [&](uint32_t key, bool valid) {
-        if (valid && key <= kKeyInf && passes(__uint_as_float(key), T, cmp)) ++mine;
-    });
-#pragma unroll
-    for (int m = 16; m > 0; m >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, m);
-    if ((threadIdx.x & 31) == 0 && mine) atomicAdd(&s_total, mine);
-    __syncthreads();
-    if (threadIdx.x == 0) {
+    unsigned int total = below + equal;
+    // (a first digit of +inf's holds nothing else that counts, so that every block decides alike)
+    if (need == 0 || !found || (prefix & 0xfff80000u) == kKeyInf) {
+        unsigned int n = 0;
+        for_prefix_maxima(rows, [&](uint32_t key, unsigned int count) {
+            if (key <= kKeyInf && passes(__uint_as_float(key), T, cmp)) n += count;
+        });
+        n = __reduce_add_sync(0xffffffffu, n);
+        if (lane == 0 && n) atomicAdd(CS > 1 ? cg::this_cluster().map_shared_rank(&sh.count, 0) : &sh.count, n);
+        if constexpr (CS > 1) cg::this_cluster().sync(); else __syncthreads();
+        total = sh.count;                             // (block 0's is the one that is used)
+    } else if constexpr (CS > 1) {
+        cg::this_cluster().sync();                    // pushes from and to a block are through before it leaves
+    }
+    if (rank == 0 && tid == 0) {
         *T_out = T;
-        *achieved_out = static_cast<float>(static_cast<double>(s_total) / static_cast<double>(B));
+        *achieved_out = static_cast<float>(static_cast<double>(total) / static_cast<double>(B));
     }
+    tune_drain(rows);
 }
 
 // ---- labels: each position on its own ---------------------------------------------------------

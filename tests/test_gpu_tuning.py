@@ -111,3 +111,23 @@ def test_tuning_on_divergences_of_a_verify_call_reproduces_its_accept_lengths():
         m, _ = _gpu_sweep(D, [T], "lt")
         assert m[0] == F(g.accept_len.sum() / 12)
         assert np.array_equal(_gpu_labels(D, T, "lt"), (D < F(T)).astype(np.uint8))
+
+
+@pytest.mark.parametrize("B,G", [(1, 1), (7, 4607), (9, 4608), (8, 33), (512, 3), (513, 3), (70001, 9)])
+def test_rows_that_are_staged_in_one_tile_in_several_and_not_at_all(B, G):
+    """Either side of the staging limits: one row, rows longer than are staged, more rows than a block's
+    shared memory holds, more thresholds than are counted in one walk."""
+    rng = np.random.default_rng(33)
+    D = rng.gamma(0.7, 0.12, size=(B, G)).clip(0, 0.6931).astype(F)
+    D[rng.random((B, G)) < 0.001] = np.nan
+    Ts = np.linspace(0.0, 0.7, 150 if B < 100 else 5).astype(F)
+    for cmp in ("lt", "le"):
+        m, f = _gpu_sweep(D, Ts, cmp)
+        om, of = tun.threshold_sweep(D, Ts, cmp)
+        assert np.array_equal(m, om) and np.array_equal(f, of)
+        reach = float(tun.threshold_sweep(D, np.array([np.inf], dtype=F), cmp)[0][0])
+        for target in (0.3 * reach, 0.9 * reach):
+            T, got = _gpu_calibrate(D, target, cmp)
+            need = int(np.ceil(np.float64(F(target)) * B))
+            m, _ = tun.threshold_sweep(D, np.array([T, np.nextafter(F(T), F(-np.inf))], dtype=F), cmp)
+            assert m[0] == got and round(float(m[0]) * B) >= need > round(float(m[1]) * B)

@@ -68,11 +68,11 @@ int check_shape(int B, int G, int V) {
     return FSD_OK;
 }
 
+// CTAs per row of the finish kernel: one or two vectors of logits a thread, at most the portable cluster
+// size, and no more CTAs than one wave of two per SM (148 SMs) when the batch is large.
 int finish_cluster_size(int B, int V) {
-    // about 32 vocabulary entries per thread, at most the portable cluster size, and no more CTAs
-    // than one wave of two per SM (148 SMs) when the batch is large
     int cs = 1;
-    while (cs < kMaxClusterSize && static_cast<long long>(cs) * kFinishThreads * 32 < V &&
+    while (cs < kMaxClusterSize && static_cast<long long>(cs) * kFinishThreads * 8 < V &&
            static_cast<long long>(B) * cs * 2 <= 2 * 148)
         cs <<= 1;
     return cs;
@@ -238,8 +238,9 @@ int launch_all(const PairParams& pp, FinishParams fp, bool vec, int* flags, Grou
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    if (cudaLaunchKernelEx(&cfg, fsd_finish_kernel<DT>, fp) != cudaSuccess) return FSD_ERR_CUDA;
-    return FSD_OK;
+    const auto kernel = fp.mode != FSD_MODE_FSD ? fsd_finish_kernel<DT, kDrawResidual>
+                        : fp.sample == FSD_SAMPLE_GREEDY ? fsd_finish_kernel<DT, kDrawGreedy> : fsd_finish_kernel<DT, kDrawPt>;
+    return cudaLaunchKernelEx(&cfg, kernel, fp) == cudaSuccess ? FSD_OK : FSD_ERR_CUDA;
 }
 
 int verify_common(const void* target, const void* draft, const int32_t* tokens, const float* u_accept,

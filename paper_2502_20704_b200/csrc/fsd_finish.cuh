@@ -5,23 +5,33 @@
 //   3. Draws the replacement / bonus token from one target row (and, for the SD residual, one
 //      draft row) by an inverse CDF in vocabulary order.
 //
-// Drawing from P_T (the FSD rule, and every bonus token): each thread owns a contiguous chunk
-// of the vocabulary; the weights are single-precision exponentials (one MUFU ex2 each, relative
-// error at most a few 1e-7) summed in double precision, chunk sums are combined by a fixed-order
-// scan (thread -> warp -> CTA -> cluster), and the warp of the first thread whose inclusive sum
-// exceeds u * total re-walks that chunk with the same weights.  The cumulative sums therefore
-// differ from exact ones by less than 1e-6 of the total: the token is the exact one whenever
+// The kernel is serial by nature -- judge, choose the row, read it, total it, find the crossing -- and takes
+// 6 us on a small batch, most of them trips to L2 and instructions that run once.  So each kind of
+// draw is an instantiation of its own, the cluster's CTAs tell one another what they must by remote
+// stores that count themselves in (no cluster barrier in the path), and a row is read once.
+//
+// Drawing from P_T (the FSD rule, and every bonus token): each warp owns a contiguous run of the
+// vocabulary, each thread a reference exponent of its own, the largest logit it has met so far (moved by
+// exact powers of two); the weights are single-precision exponentials (one MUFU ex2 each, relative error
+// at most a few 1e-7) summed in double precision.  The sums, brought to one scale, are combined in a fixed
+// order (thread -> warp -> CTA -> cluster), and the CTA that owns the warp in whose run the total passes
+// u * total re-walks that run with the same weights, an iteration of it per warp.  The cumulative sums
+// therefore differ from exact ones by less than 1e-6 of the total: the token is the exact one whenever
 // u * total lies further than that from both ends of its interval, and a neighbour otherwise.
-// Drawing from the SD residual max(0, P_T - P_D) (Eq. 3) subtracts nearly equal numbers, so
-// there the exponentials are double precision (a 256-entry table times a degree-4 polynomial,
-// about ten fp64 operations) and the sums agree with a sequential double sum to rounding.
-// Usually one pass over the two rows suffices for it: which entries carry residual weight
-// depends on the ratio of the two normalisers only, the rejected pair's record gives that ratio
-// closely enough to class every entry that is not within a margin of the boundary, and the
-// chunk sums follow from the classed sums once the exact normalisers are known; entries inside
-// the margin are settled one by one afterwards, and a row with too many of them in one thread
-// takes a second pass.
+// Drawing from the SD residual max(0, P_T - P_D) (Eq. 3) subtracts nearly equal numbers, so there the
+// exponentials are double precision and the sums agree with a sequential double sum to rounding.
+// bf16 logits have few values: e^x comes from a table of all bf16 numbers between 2^-9 and 64 of either
+// sign (built while the streaming kernel drains), which leaves two shared-memory reads and four
+// double-precision instructions an entry.  fp32 logits take a 256-entry table times a degree-4
+// polynomial (about forty instructions).  Usually one pass over the two rows suffices: which
+// entries carry residual weight depends on the ratio of the two normalisers only, the rejected pair's
+// record gives that ratio closely enough to class every entry that is not within a margin of the
+// boundary, and the sums follow from the classed sums once the exact normalisers are known; entries
+// inside the margin are settled afterwards, and a row with too many of them in one thread takes a
+// second pass.
 #pragma once
+
+#include <climits>
 
 #include "fsd_device.cuh"
 #include "fsd_pair_generic.cuh"
@@ -56,31 +66,35 @@ struct FinishParams {
     int* debug_word;           // debug build: where failed range checks are recorded (may be null)
 };
 
-struct FinishExchange {        // what one CTA publishes to its cluster
-    double d[4];
-    int i[2];
-};
+constexpr int kExchangeDoubles = 5;      // most values a CTA tells its cluster at once
+// With more pairs than a CTA has warps, the cluster's CTAs share the judging (CTA r takes pairs r, r + cs, ...)
+// and tell one another the accept bits: up to 64 * kJudgeWords of them each.
+constexpr int kJudgeWords = kExchangeDoubles - 1;
 constexpr int kExpTable = 256;
+// e^x of the bf16 numbers with 2^-9 <= |x| < 64, both signs
+constexpr int kBf16Lowest = 118 << 7, kBf16Count = 15 << 7;
+// what a kernel draws: from P_T, its argmax, or (after a rejection) from the SD residual
+enum : int { kDrawPt = 0, kDrawGreedy = 1, kDrawResidual = 2 };
 
 struct FinishShared {
-    FinishExchange all[2][kMaxClusterSize];   // what the cluster's CTAs published, written by them (see cluster_exchange)
+    uint64_t link[2];              // barriers of the cluster's exchanges
+    double got[2][kMaxClusterSize][kExchangeDoubles];   // what the CTAs of the cluster sent (see cluster_exchange)
     double sc[kMaxClusterSize];
-    double gather_d[2][kMaxClusterSize];   // one value per CTA of the cluster, written by the peers (see cluster_gather)
-    int gather_i[2][kMaxClusterSize];
-    float kref[kMaxTreeNodes];          // per pair: integer reference at or just above the target row's log2-sum-exp (NaN: none)
-    double exp_table[kExpTable];   // 2^(j/256)
-    double exp_consts[8];          // the constants of exp2_table (see exp2_consts)
     double red_d[32 * 2];
     float red_f[32 * 2];
-    double warp_tot[32];
-    int amb;                   // residual draw: some entry could not be classed in the first pass
-    int cand;                  // lowest thread whose inclusive sum exceeds the target
+    double warp_tot[kFinishWarps];
+    double seg_tot[kFinishWarps];  // of the iterations find_crossing looks at
+    float warp_k[kFinishWarps];    // draw from P_T: the warps' largest references
+    unsigned long long bits[kJudgeWords];   // accept bits of the pairs this CTA judged for its cluster
+    int far;                   // draw from P_T: some thread's reference is out of a double's range; argmax: an invalid logit
+    int amb;                   // residual draw: 1 some thread needs the second pass, 2 some has close calls
+    int cand;                  // find_crossing: highest index with a positive weight
     int last_pos;              // highest index with a positive weight in this CTA
-    int token;
     int row_sel;               // target row the token is drawn from
     int n_acc;
     int bad;
     int best_key;              // depth * 2048 + (2047 - node) of the chosen tree node, or -1
+    int16_t tree_parent[kMaxTreeNodes];
     int16_t tree_jump[kMaxTreeNodes];
     int16_t tree_depth[kMaxTreeNodes];
     int8_t tree_ok[kMaxTreeNodes];
@@ -135,29 +149,28 @@ __device__ __forceinline__ double exp2_of_logit(float x, float xmin, double nk, 
     return exp2_table_fast(fma(static_cast<double>(fmaxf(x, xmin)), kLog2eD, nk), below, table, c);
 }
 
-// Every CTA of the cluster writes a FinishExchange into every CTA's shared memory (its own
-// included); after one cluster barrier sh.all[buf] holds everybody's, in rank order, in every CTA.
-// Like cluster_gather: `buf` alternates from one call to the next, and nobody reads a peer's
-// memory afterwards.  Every thread passes the same `mine`.
-__device__ __forceinline__ void cluster_exchange(cg::cluster_group& cluster, FinishShared& sh, int cs, int rank, int buf,
-                                                 const FinishExchange& mine) {
-    if (threadIdx.x < cs) cluster.map_shared_rank(&sh, threadIdx.x)->all[buf][rank] = mine;
-    cluster.sync();
-}
-
-// Light exchange: every CTA writes one double and one int into every CTA's shared memory (its
-// own included); after ONE cluster barrier sh.gather_d[buf] / gather_i[buf] hold the values of
-// all CTAs, in rank order, in every CTA, and nobody reads a peer's memory (so a CTA may leave
-// right afterwards).  `buf` alternates from one call to the next: a CTA that is already writing
-// the next exchange cannot disturb the values a slower peer is still reading.  The peers must be
-// known to have started (one cluster barrier earlier in the kernel).
-__device__ __forceinline__ void cluster_gather(cg::cluster_group& cluster, FinishShared& sh, int cs, int rank, int buf, double v, int iv) {
+// What the CTAs of a cluster tell one another: every CTA pushes a few doubles into every CTA's shared
+// memory (its own included) and waits for all of its own to arrive.  No cluster barrier, no fence: the
+// barrier.cluster form took twice as long.  Two barriers and buffers alternate, which is
+// enough: nobody can be two exchanges ahead of a CTA whose values it still lacks.  The peers must be
+// known to run (an arrive at kernel entry that is waited for before the first exchange); a CTA that
+// has had its last exchange may leave.  Called by all threads with the same values, and with a barrier
+// of the CTA between two calls; returns the buffer: got[rank][k].
+template <int N>
+__device__ __forceinline__ const double (*cluster_exchange(FinishShared& sh, int cs, int rank, int& turn, const double (&v)[N]))[kExchangeDoubles] {
+    static_assert(N <= kExchangeDoubles, "width of the exchange buffer");
+    const int buf = turn & 1;
+    if (threadIdx.x == 0) mbar_arrive_expect_tx(&sh.link[buf], static_cast<uint32_t>(cs) * N * 8);
     if (threadIdx.x < cs) {
-        FinishShared* rs = cluster.map_shared_rank(&sh, threadIdx.x);
-        rs->gather_d[buf][rank] = v;
-        rs->gather_i[buf][rank] = iv;
+        const uint32_t dst = cluster_addr(&sh.got[buf][rank][0], threadIdx.x), bar = cluster_addr(&sh.link[buf], threadIdx.x);
+#pragma unroll
+        for (int k = 0; k < N; ++k) st_async(dst + 8 * k, static_cast<uint64_t>(__double_as_longlong(v[k])), bar);
     }
-    cluster.sync();
+#pragma unroll 1
+    for (uint32_t i = 0; i < kSpinLimit; ++i)
+        if (mbar_try_wait(&sh.link[buf], (turn >> 1) & 1)) break;
+    ++turn;
+    return sh.got[buf];
 }
 
 // Divergence, accept bit and status of one pair from the streaming kernel's totals.
@@ -211,8 +224,9 @@ __device__ inline PairTotals fold_record(const PairRecord* rec, int div) {
     return t;
 }
 
+// (x, ax, bx: the candidate and its two logits, for the ratio test)
 __device__ inline void judge_record(const FinishParams& P, int item, const PairTotals& r, double lnZa, double lnZb,
-                                    const void* a_row, const void* b_row, int dt, float& D_out, int& bit_out, int& st_out) {
+                                    int x, float ax, float bx, float& D_out, int& bit_out, int& st_out) {
     if (r.state & kRecordBadTree) {
         D_out = __int_as_float(0x7fc00000); bit_out = 0; st_out = FSD_ROW_BADTREE;
         return;
@@ -225,10 +239,7 @@ __device__ inline void judge_record(const FinishParams& P, int item, const PairT
     if (P.mode != FSD_MODE_FSD) {
         bool ratio_ok = false;
         if (finite) {
-            const int x = P.tokens[item];
             if (x >= 0 && x < P.V) {
-                const float ax = dt == FSD_BF16 ? load_logit<FSD_BF16>(a_row, x) : load_logit<FSD_F32>(a_row, x);
-                const float bx = dt == FSD_BF16 ? load_logit<FSD_BF16>(b_row, x) : load_logit<FSD_F32>(b_row, x);
                 double pacc;                                                    // Eq. 1
                 if (bx == -INFINITY) {
                     pacc = (ax != -INFINITY) ? 1.0 : 0.0;
@@ -247,27 +258,158 @@ __device__ inline void judge_record(const FinishParams& P, int item, const PairT
     D_out = D; bit_out = bit; st_out = finite ? 0 : FSD_ROW_NONFINITE;
 }
 
-// Calls f(k, a_k, b_k) for k in [k0, k1) in order; 16-byte loads when `vec` (then k0 is a
-// multiple of the vector width and V a multiple of it).  b_k is 0 unless `with_b`.
+// ---- how a row is shared out for the draw -------------------------------------------------------
+// In units, a 16-byte vector of the row (rows off a 16-byte boundary: the aligned granules that cover it), or one
+// entry.  A warp of the cluster owns `iters` times 32 consecutive units, its lanes read neighbours: consecutive
+// threads on consecutive addresses.  (With a run of units per thread a warp's load touched 32 lines, which were
+// gone from L1 when the next one wanted the rest of them.)
+struct Draw {
+    const char* a_row;
+    const char* b_row;
+    int b, n, V, cs, rank;
+    bool shared_out;           // the cluster's CTAs have shared the judging: no pair's reference is at hand
+    bool vec;                  // both rows are whole vectors on 16-byte boundaries
+    double u;
+};
+struct Share { int units, iters, first; };            // units of the row, iterations of a warp, the warp's first unit
+__device__ __forceinline__ Share row_share(int units, int cs, int rank, int warp) {      // cs: a power of two
+    const int shift = 9 + 31 - __clz(cs);             // log2(cs * kFinishWarps * 32)
+    Share s;
+    s.units = units;
+    s.iters = static_cast<int>((static_cast<uint32_t>(units) + (1u << shift) - 1) >> shift);
+    const long long first = static_cast<long long>(rank * kFinishWarps + warp) * s.iters * 32;
+    s.first = first < units ? static_cast<int>(first) : units;
+    return s;
+}
+// The target row as granules: the granule that holds entry 0 starts `off` entries in front of it.
+template <int DT> struct Granules {
+    const void* base;
+    int off, count, V;
+    __device__ __forceinline__ Granules(const char* row, int v) : V(v) {
+        const int bytes = static_cast<int>(reinterpret_cast<uintptr_t>(row) & 15);
+        base = row - bytes;
+        off = bytes / Logit<DT>::kBytes;
+        count = (off + v + Logit<DT>::kPerVec - 1) / Logit<DT>::kPerVec;
+    }
+    __device__ __forceinline__ uint4 fetch(int g) const {                // -inf where there is no entry
+        constexpr uint32_t kNone = DT == FSD_BF16 ? 0xff80ff80u : 0xff800000u;
+        return g < count ? ldg_vec(base, g) : make_uint4(kNone, kNone, kNone, kNone);
+    }
+    __device__ __forceinline__ uint4 cut(uint4 v, int g) const {         // the first and last granule's entries that are not the row's
+        const int k0 = g * Logit<DT>::kPerVec - off;
+        return g < count && (k0 < 0 || k0 + Logit<DT>::kPerVec > V) ? masked_vector<DT>(v, k0, V, true) : v;
+    }
+};
+// Calls f(k, a_k, b_k) for this warp's entries, unit by unit: vectors where `vec`, else single entries.
 template <int DT, typename F>
-__device__ __forceinline__ void for_chunk(const void* a_row, const void* b_row, int k0, int k1, bool vec, bool with_b, F f) {
+__device__ __forceinline__ void for_units(const Draw& d, int warp, int lane, bool with_b, F f) {
     constexpr int EPV = Logit<DT>::kPerVec;
-    if (vec) {
-        for (int k = k0; k < k1; k += EPV) {
+    const Share s = row_share(d.vec ? d.V / EPV : d.V, d.cs, d.rank, warp);
+    for (int it = 0; it < s.iters; ++it) {
+        const int u = s.first + it * 32 + lane;
+        if (u >= s.units) break;
+        if (d.vec) {
             float xa[EPV], xb[EPV];
-            unpack_vec<DT>(ldg_vec(a_row, k / EPV), xa);
+            unpack_vec<DT>(ldg_vec(d.a_row, u), xa);
             if (with_b) {
-                unpack_vec<DT>(ldg_vec(b_row, k / EPV), xb);
+                unpack_vec<DT>(ldg_vec(d.b_row, u), xb);
             } else {
 #pragma unroll
                 for (int j = 0; j < EPV; ++j) xb[j] = 0.f;
             }
 #pragma unroll
-            for (int j = 0; j < EPV; ++j) f(k + j, xa[j], xb[j]);
+            for (int j = 0; j < EPV; ++j) f(u * EPV + j, xa[j], xb[j]);
+        } else {
+            f(u, load_logit<DT>(d.a_row, u), with_b ? load_logit<DT>(d.b_row, u) : 0.f);
         }
-    } else {
-        for (int k = k0; k < k1; ++k) f(k, load_logit<DT>(a_row, k), with_b ? load_logit<DT>(b_row, k) : 0.f);
     }
+}
+// One inclusive scan over a warp
+__device__ __forceinline__ double warp_scan(double v, int lane) {
+#pragma unroll
+    for (int q = 1; q < 32; q <<= 1) {
+        const double o = __shfl_up_sync(0xffffffffu, v, q);
+        if (lane >= q) v += o;
+    }
+    return v;
+}
+// Sixteen values, one a warp of the CTA, scanned by every warp for itself: lane w has warp w's.
+struct Prefix {
+    double v, upto, total;
+    __device__ __forceinline__ Prefix(double value, int lane) {
+        v = lane < kFinishWarps ? value : 0.0;
+        upto = warp_scan(v, lane);
+        total = __shfl_sync(0xffffffffu, upto, kFinishWarps - 1);
+    }
+    // the first whose running total (on top of `base`) passes t, or -1; and the total in front of it
+    __device__ __forceinline__ int passes(double base, double t, double& before) const {
+        const unsigned over = __ballot_sync(0xffffffffu, v > 0.0 && base + upto > t);
+        const int w = over != 0 ? __ffs(over) - 1 : -1;
+        before = base + __shfl_sync(0xffffffffu, upto - v, w < 0 ? 0 : w);
+        return w;
+    }
+    // the same, but the last with weight where rounding has lost the crossing
+    __device__ __forceinline__ int crossing(double t, double& before) const {
+        int w = passes(0.0, t, before);
+        if (w < 0) {
+            w = 31 - __clz(__ballot_sync(0xffffffffu, v > 0.0) | 1u);
+            before = __shfl_sync(0xffffffffu, upto - v, w);
+        }
+        return w;
+    }
+};
+// Finds the entry at which the running sum over a warp's share passes `target`: all warps of the CTA take an
+// iteration of that share each.  weights(unit, w[]) fills in the weights of a unit's EPU entries (0 where there is
+// none), first_entry(unit) is the index of its first.  The last entry with weight where rounding loses the crossing.
+template <int EPU, typename W, typename E>
+__device__ __forceinline__ void find_crossing(const FinishParams& P, FinishShared& sh, const Draw& d, const Share& share, double target, W weights, E first_entry) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    double base = 0.0;
+    int last = -1;                                    // highest index with weight this thread has seen
+#pragma unroll 1
+    for (int r0 = 0; r0 < share.iters; r0 += kFinishWarps) {
+        const int u = share.first + (r0 + warp) * 32 + lane;
+        double w[EPU], usum = 0.0;
+        int ulast = -1;
+#pragma unroll
+        for (int j = 0; j < EPU; ++j) w[j] = 0.0;
+        if (r0 + warp < share.iters && u < share.units) {
+            weights(u, w);
+#pragma unroll
+            for (int j = 0; j < EPU; ++j) { usum += w[j]; if (w[j] > 0.0) ulast = first_entry(u) + j; }
+        }
+        last = max(last, ulast);
+        const double upto = warp_scan(usum, lane);
+        if (lane == 31) sh.seg_tot[warp] = upto;
+        __syncthreads();
+        double before;
+        const Prefix seg(sh.seg_tot[lane & (kFinishWarps - 1)], lane);
+        const int found = seg.passes(base, target, before);
+        if (found >= 0) {                             // the same for all threads
+            if (warp != found) return;
+            const unsigned over = __ballot_sync(0xffffffffu, usum > 0.0 && before + upto > target), some = __ballot_sync(0xffffffffu, usum > 0.0);
+            const int src = over != 0 ? __ffs(over) - 1 : 31 - __clz(some);
+            if (lane == src) {
+                double run = before + upto - usum;
+                int tok = -1;
+#pragma unroll
+                for (int j = 0; j < EPU; ++j) {
+                    run += w[j];
+                    if (tok < 0 && w[j] > 0.0 && run > target) tok = first_entry(u) + j;
+                }
+                if (tok < 0) tok = ulast;             // lost to the order of the additions
+                FSD_CHECK(P.debug_word, tok >= 0 && tok < d.V, kChkToken);
+                P.next_token[d.b] = tok;
+            }
+            return;
+        }
+        base += seg.total;
+        __syncthreads();                              // seg_tot is free again
+    }
+    last = __reduce_max_sync(0xffffffffu, last);
+    if (lane == 0 && last >= 0) atomicMax(&sh.cand, last);
+    __syncthreads();
+    if (tid == 0) P.next_token[d.b] = sh.cand;
 }
 
 // Tree: the deepest node whose whole path passes (ties: lowest index), its depth and path.
@@ -276,20 +418,23 @@ __device__ __noinline__ void tree_select(const int32_t* par, int G, int max_dept
     const int tid = threadIdx.x, lane = tid & 31;
     // Depth of every node and "all nodes from the root down to it pass", by pointer jumping:
     // every node keeps (nodes counted, all pass, next ancestor) for the stretch of its path it
-    // has seen so far and doubles that stretch each round, so ceil(log2 N) rounds do for any
+    // has seen so far and doubles that stretch each round, so ceil(log2 depth) rounds do for any
     // tree shape (a serial walk takes N dependent steps for a chain-shaped tree of N nodes).
     const bool good = !(sh.bad & FSD_ROW_BADTREE);
     constexpr int kPer = (kMaxTreeNodes + kFinishThreads - 1) / kFinishThreads;
     if (tid == 0) sh.best_key = -1;
     if (good) {
         for (int j = tid; j < G; j += kFinishThreads) {
-            sh.tree_jump[j] = static_cast<int16_t>(par[j]);
+            const int16_t p = static_cast<int16_t>(par[j]);
+            sh.tree_parent[j] = p;
+            sh.tree_jump[j] = p;
             sh.tree_depth[j] = 1;
             sh.tree_ok[j] = sh.tree_bit[j];
         }
         __syncthreads();
         for (int span = 1; span < G; span <<= 1) {
             int nj[kPer], nd[kPer], no[kPer];
+            bool more = false;
 #pragma unroll
             for (int q = 0; q < kPer; ++q) {
                 const int j = tid + q * kFinishThreads;
@@ -298,9 +443,10 @@ __device__ __noinline__ void tree_select(const int32_t* par, int G, int max_dept
                     const int p = sh.tree_jump[j];
                     nj[q] = p; nd[q] = sh.tree_depth[j]; no[q] = sh.tree_ok[j];
                     if (p >= 0) { nj[q] = sh.tree_jump[p]; nd[q] += sh.tree_depth[p]; no[q] &= sh.tree_ok[p]; }
+                    more = more || nj[q] >= 0;
                 }
             }
-            __syncthreads();
+            const bool any = __syncthreads_or(more) != 0;
 #pragma unroll
             for (int q = 0; q < kPer; ++q) {
                 const int j = tid + q * kFinishThreads;
@@ -310,6 +456,7 @@ __device__ __noinline__ void tree_select(const int32_t* par, int G, int max_dept
                     sh.tree_ok[j] = static_cast<int8_t>(no[q]);
                 }
             }
+            if (!any) break;                          // every node has reached the root (what is read below, its reader wrote)
             __syncthreads();
         }
         // deepest passing node within max_depth, ties to the lowest index
@@ -325,25 +472,655 @@ __device__ __noinline__ void tree_select(const int32_t* par, int G, int max_dept
         if (lane == 0 && key >= 0) atomicMax(&sh.best_key, key);
     }
     __syncthreads();
-    if (tid == 0) {
-        const int key = sh.best_key;
-        const int best = key < 0 ? -1 : 2047 - (key & 2047), best_depth = key < 0 ? 0 : key >> 11;
-        sh.n_acc = best_depth;
-        sh.row_sel = best + 1;
-        if (pth != nullptr) {
-            for (int d = 0; d < max_depth; ++d) pth[d] = -1;
-            for (int j = best, d = best_depth - 1; j >= 0 && d >= 0; j = par[j], --d) pth[d] = j;
-        }
+    const int key = sh.best_key;
+    const int best = key < 0 ? -1 : 2047 - (key & 2047), best_depth = key < 0 ? 0 : key >> 11;
+    if (tid == 0) { sh.n_acc = best_depth; sh.row_sel = best + 1; }
+    if (pth != nullptr) {
+        for (int d = best_depth + tid; d < max_depth; d += kFinishThreads) pth[d] = -1;
+        if (tid == 0)
+            for (int j = best, d = best_depth - 1; j >= 0 && d >= 0; j = sh.tree_parent[j], --d) pth[d] = j;
     }
 }
 
+// ---- the draw from P_T ---------------------------------------------------------------------------
+__device__ __forceinline__ double pow2_any(int e) { return __hiloint2double((1023 + e) << 20, 0); }      // |e| < 1000
+
+// A weight (0 or a normal number up to 1) widened to double with integer instructions: the conversion instruction
+// shares the special-function pipe with ex2 and would double the pass' time there.  0 becomes 2^-127, which is
+// nothing beside the thread's largest weight, a half or more.
+__device__ __forceinline__ double widen(float w) {
+    const uint32_t u = __float_as_uint(w);
+    return __hiloint2double(static_cast<int>((u >> 3) + 0x38000000u), static_cast<int>(u << 29));
+}
+template <int DT> __device__ __forceinline__ float vector_max(const uint4& v) {          // NaN if one is
+    if constexpr (DT == FSD_BF16) {
+        const uint32_t m2 = bf16x2_max_nan(bf16x2_max_nan(v.x, v.y), bf16x2_max_nan(v.z, v.w));
+        return fmax_nan(bf16_lo(m2), bf16_hi(m2));
+    } else {
+        return fmax_nan(fmax_nan(__uint_as_float(v.x), __uint_as_float(v.y)), fmax_nan(__uint_as_float(v.z), __uint_as_float(v.w)));
+    }
+}
+
+// Inverse CDF over P_T.  Writes the row's accepted length, token and status; uniform over the cluster.
 template <int DT>
-__global__ void __launch_bounds__(kFinishThreads, 2) fsd_finish_kernel(FinishParams P) {
+__device__ __forceinline__ void draw_pt(const FinishParams& P, FinishShared& sh, const Draw& d, int& turn, int status) {
+    constexpr int EPV = Logit<DT>::kPerVec;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const Granules<DT> gr(d.a_row, d.V);
+    const Share mine = row_share(gr.count, d.cs, d.rank, warp);
+    FSD_CHECK(P.debug_word, mine.first >= 0 && mine.first <= gr.count && static_cast<long long>(mine.iters) * kFinishThreads * d.cs >= gr.count, kChkChunk);
+    // ---- one pass: this thread's weights 2^(logit * log2e - kr) in double, kr the largest logit's exponent so far;
+    //      four vectors are asked for before the first is used ----
+    constexpr int BV = 4;
+    double csum = 0.0;
+    float kr = -INFINITY;
+    for (int it = 0; it < mine.iters; it += BV) {
+        uint4 v[BV];
+#pragma unroll
+        for (int q = 0; q < BV; ++q) v[q] = gr.fetch(it + q < mine.iters ? mine.first + (it + q) * 32 + lane : INT_MAX);
+        float vm = -INFINITY;
+#pragma unroll
+        for (int q = 0; q < BV; ++q) {
+            if (it + q < mine.iters) v[q] = gr.cut(v[q], mine.first + (it + q) * 32 + lane);
+            vm = fmax_nan(vm, vector_max<DT>(v[q]));
+        }
+        if (!(vm * kLog2e <= kr)) {                   // (a NaN comes through here and stays in csum)
+            const float kn = ceilf(vm * kLog2e);
+            csum = kr == -INFINITY ? 0.0 : csum * pow2_int_d(static_cast<double>(kr) - kn);
+            kr = kn;
+        }
+        const float nk = kr == -INFINITY ? 0.f : -kr;
+        double part[BV];
+#pragma unroll
+        for (int q = 0; q < BV; ++q) {
+            part[q] = 0.0;
+            if (it + q < mine.iters) {
+                float x[EPV];
+                unpack_vec<DT>(v[q], x);
+#pragma unroll
+                for (int e = 0; e < EPV; ++e) part[q] += widen(ex2(fmaf(x[e], kLog2e, nk)));
+            }
+        }
+        csum += (part[0] + part[1]) + (part[2] + part[3]);
+        if (!(vm < INFINITY)) csum = vm - vm;         // (a NaN or +inf logit: `widen` takes finite weights)
+    }
+    const bool usable = kr > -INFINITY && kr < INFINITY;
+    const bool far = usable && fabsf(kr) > 900.f;
+    if (far) sh.far = 1;
+    const float wk = warp_redux_max_nan(usable ? kr : -INFINITY);
+    if (lane == 0) sh.warp_k[warp] = wk;
+
+    // ---- totals of warp, CTA and cluster, in a fixed order and on one scale: 2^0, or where a reference is out of a
+    //      double's reach the largest reference of the cluster ----
+    double K = 0.0, W, w_v, w_upto;
+    const double (*all)[kExchangeDoubles];
+#pragma unroll 1
+    for (bool scaled = false;; scaled = true) {
+        double val = kr == -INFINITY ? 0.0 : !usable ? csum * static_cast<double>(__int_as_float(0x7fc00000))
+                     : scaled ? csum * pow2_int_d(static_cast<double>(kr) - K) : far ? 0.0 : csum * pow2_any(static_cast<int>(kr));
+        val = warp_sum(val);
+        if (lane == 0) sh.warp_tot[warp] = val;
+        __syncthreads();
+        const Prefix pre(sh.warp_tot[lane & (kFinishWarps - 1)], lane);
+        w_v = pre.v; w_upto = pre.upto;
+        const double mine2[2] = {pre.total, scaled ? 0.0 : static_cast<double>(sh.far)};
+        all = cluster_exchange(sh, d.cs, d.rank, turn, mine2);
+        double any = 0.0;
+        W = 0.0;
+        for (int r = 0; r < d.cs; ++r) { W += all[r][0]; any += all[r][1]; }
+        if (any == 0.0) break;
+        float m = -INFINITY;
+        for (int w = 0; w < kFinishWarps; ++w) m = fmaxf(m, sh.warp_k[w]);
+        __syncthreads();
+        const double mk[1] = {m};
+        all = cluster_exchange(sh, d.cs, d.rank, turn, mk);
+        K = -INFINITY;
+        for (int r = 0; r < d.cs; ++r) K = fmax(K, all[r][0]);
+    }
+    if (!(isfinite(W) && W > 0.0)) {                  // a NaN or +inf logit, or no finite one: uniform over the cluster
+        if (d.rank == 0 && tid == 0) { P.accept_len[d.b] = d.n; P.next_token[d.b] = -1; P.row_status[d.b] = status | FSD_ROW_NONFINITE; }
+        return;
+    }
+    if (d.rank == 0 && tid == 0) { P.accept_len[d.b] = d.n; P.row_status[d.b] = status; }
+    const double t = d.u * W;
+    double run = 0.0, cpre = 0.0;
+    int owner = -1;
+    for (int r = 0; r < d.cs && owner < 0; ++r) {
+        cpre = run;
+        run += all[r][0];
+        if (run > t) owner = r;
+    }
+    if (owner < 0) {                                  // t >= W after rounding (uniform): the last token that has weight
+        int lastp = -1;
+        const float nk = kr == -INFINITY ? 0.f : -kr;
+        for (int it = 0; it < mine.iters; ++it) {
+            const int g = mine.first + it * 32 + lane;
+            if (g >= gr.count) break;
+            float x[EPV];
+            unpack_vec<DT>(gr.cut(gr.fetch(g), g), x);
+#pragma unroll
+            for (int e = 0; e < EPV; ++e) if (ex2(fmaf(x[e], kLog2e, nk)) > 0.f) lastp = g * EPV - gr.off + e;
+        }
+        lastp = __reduce_max_sync(0xffffffffu, lastp);
+        if (lane == 0 && lastp >= 0) atomicMax(&sh.last_pos, lastp);
+        __syncthreads();
+        const double mine1[1] = {static_cast<double>(sh.last_pos)};
+        all = cluster_exchange(sh, d.cs, d.rank, turn, mine1);
+        int best = -1;
+        for (int r = 0; r < d.cs; ++r) best = max(best, static_cast<int>(all[r][0]));
+        if (d.rank == 0 && tid == 0) P.next_token[d.b] = best;
+        return;
+    }
+    if (owner != d.rank) return;
+    // the warp in whose share the total passes the target, and the target on that warp's own scale
+    Prefix pre(0.0, lane);
+    pre.v = w_v; pre.upto = w_upto;
+    double before;
+    const int cw = pre.crossing(t - cpre, before);
+    const float ck = sh.warp_k[cw];
+    const double up = pow2_int_d(-fabs(static_cast<double>(ck) - K)), rest = t - cpre - before;
+    const double target = static_cast<double>(ck) > K ? rest * up : rest / up;
+    const float nk = -ck;
+    find_crossing<EPV>(P, sh, d, row_share(gr.count, d.cs, d.rank, cw), target,
+        [&](int g, double (&w)[EPV]) {
+            float x[EPV];
+            unpack_vec<DT>(gr.cut(gr.fetch(g), g), x);
+#pragma unroll
+            for (int e = 0; e < EPV; ++e) w[e] = static_cast<double>(ex2(fmaf(x[e], kLog2e, nk)));
+        },
+        [&](int g) { return g * EPV - gr.off; });
+}
+
+// argmax of P_T == argmax of the logits, ties to the lowest index.  One pass: the largest logit, its index, and
+// whether the row is a valid distribution (no NaN, no +inf, something finite).
+template <int DT>
+__device__ __forceinline__ void draw_argmax(const FinishParams& P, FinishShared& sh, const Draw& d, int& turn, int status) {
+    constexpr int EPV = Logit<DT>::kPerVec;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const Granules<DT> gr(d.a_row, d.V);
+    const Share mine = row_share(gr.count, d.cs, d.rank, warp);
+    float best = -INFINITY;
+    int idx = 0x7fffffff;
+    bool bad = false;
+#pragma unroll 4
+    for (int it = 0; it < mine.iters; ++it) {
+        const int g = mine.first + it * 32 + lane;
+        const uint4 v = gr.cut(gr.fetch(g), g);
+        const float vm = vector_max<DT>(v);
+        bad = bad || !(vm < INFINITY);
+        if (vm > best) {
+            best = vm;
+            float x[EPV];
+            unpack_vec<DT>(v, x);
+#pragma unroll
+            for (int j = EPV - 1; j >= 0; --j) if (x[j] == vm) idx = g * EPV - gr.off + j;
+        }
+    }
+    const float wb = warp_redux_max_nan(best);                            // (best is never NaN)
+    const int wi = __reduce_min_sync(0xffffffffu, best == wb ? idx : 0x7fffffff);
+    const bool wbad = __any_sync(0xffffffffu, bad);
+    if (lane == 0) { sh.red_f[warp] = wb; sh.red_d[warp] = wi; if (wbad) sh.far = 1; }
+    __syncthreads();
+    const float lb = lane < kFinishWarps ? sh.red_f[lane] : -INFINITY;
+    const int li = lane < kFinishWarps ? static_cast<int>(sh.red_d[lane]) : 0x7fffffff;
+    const float cb = warp_redux_max_nan(lb);
+    const int ci = __reduce_min_sync(0xffffffffu, lb == cb ? li : 0x7fffffff);
+    const double mine3[3] = {cb, static_cast<double>(ci), static_cast<double>(sh.far)};
+    const double (*all)[kExchangeDoubles] = cluster_exchange(sh, d.cs, d.rank, turn, mine3);
+    if (d.rank == 0 && threadIdx.x == 0) {
+        double gb = all[0][0], gi = all[0][1], gbad = all[0][2];
+        for (int r = 1; r < d.cs; ++r) {
+            if (all[r][0] > gb || (all[r][0] == gb && all[r][1] < gi)) { gb = all[r][0]; gi = all[r][1]; }
+            gbad += all[r][2];
+        }
+        const bool ok = gbad == 0.0 && gb > -INFINITY;
+        P.accept_len[d.b] = d.n;
+        P.next_token[d.b] = ok ? static_cast<int>(gi) : -1;
+        P.row_status[d.b] = status | (ok ? 0 : FSD_ROW_NONFINITE);
+    }
+}
+
+// ---- the draw from the SD residual -----------------------------------------------------------------
+constexpr int kPairRefs = 32;                         // (a pair beyond these has its record folded again)
+struct PairRef { double za, zb; float ka, kb; };      // normalisers relative to 2^ka, 2^kb; ka NaN: not usable
+struct ResidualShared {
+    double exp_table[kExpTable];                      // 2^(j/256)
+    double exp_consts[8];                             // the constants of exp2_table (see exp2_consts)
+    PairRef ref[kPairRefs];                           // of the pairs this CTA has judged
+    double4 wsum[kFinishWarps];                       // the warps' za, zb, sa, sb
+};
+template <int DT> struct ExpTable {};                // (fp32 logits have no table of their own)
+// e^x of the bf16 numbers from 2^-9 to 64, at [sign << 11 | magnitude's bits - kBf16Lowest].  Logits of a row lie
+// close together and mostly share a sign: neighbours fall on different banks.
+constexpr int kBf16Sign = 1 << 11;
+static_assert(kBf16Count <= kBf16Sign, "eleven bits index a sign's entries");
+template <> struct ExpTable<FSD_BF16> {
+    double e[2 * kBf16Sign];
+};
+// e^x of a bf16 number, to double precision, whatever it is
+__device__ __noinline__ double exp_bf16(float x, const ExpTable<FSD_BF16>& t) {
+    const uint32_t bits = __float_as_uint(x) >> 16, m = (bits & 0x7fffu) - kBf16Lowest;
+    if (m < static_cast<uint32_t>(kBf16Count)) return t.e[(bits >> 15) * kBf16Sign + m];
+    if (static_cast<int>(m) < 0) {                    // |x| < 2^-9: the series' next term is below 2^-51
+        const double y = x;
+        return fma(fma(fma(fma(y, 1.0 / 24, 1.0 / 6), y, 0.5), y, 1.0), y, 1.0);
+    }
+    if (x < -700.f) return 0.0;                       // (-inf among them)
+    return exp(static_cast<double>(x));
+}
+// All sixteen entries of two vectors within the table
+__device__ __forceinline__ bool in_table(const uint4& a, const uint4& b) {
+    constexpr uint32_t kMag = 0x7fff7fffu;
+    const uint32_t w[8] = {a.x & kMag, a.y & kMag, a.z & kMag, a.w & kMag, b.x & kMag, b.y & kMag, b.z & kMag, b.w & kMag};
+    uint32_t lo = w[0], hi = w[0];
+#pragma unroll
+    for (int i = 1; i < 8; ++i) { lo = __vminu2(lo, w[i]); hi = __vmaxu2(hi, w[i]); }
+    return (lo & 0xffffu) >= kBf16Lowest && (lo >> 16) >= kBf16Lowest && (hi & 0xffffu) < kBf16Lowest + kBf16Count && (hi >> 16) < kBf16Lowest + kBf16Count;
+}
+// e^x of both entries of a packed pair there; `table` is its shared-memory address
+__device__ __forceinline__ void table_exp2(uint32_t pair, uint32_t table, double& e0, double& e1) {
+    const uint32_t m = pair - kBf16Lowest * 0x10001u;                       // (no borrow between the halves)
+    const uint32_t idx = (m & 0x07ff07ffu) | (m >> 4 & 0x08000800u);        // the sign comes down to bit 11
+    asm("ld.shared.f64 %0, [%1];" : "=d"(e0) : "r"(table + (idx & 0xffffu) * 8));
+    asm("ld.shared.f64 %0, [%1];" : "=d"(e1) : "r"(table + (idx >> 13)));
+}
+// What a pass over a thread's entries leaves: normalisers; sums over the entries clearly above the ratio; sums over the
+// first kind of close call (entries whose logits differ by qd); the other close calls.  An entry is above where its
+// logits differ by more than ln rho: `hi` and `lo` are ln rho_est plus and minus the margin.
+struct Classed {
+    double za, zb, sa, sb, qa, qb;
+    float qd;                                         // NaN: none yet
+    int close, k0, k1;                                // number and indices of the other close calls
+    __device__ __forceinline__ void close_call(int k, float d, double pa, double pb) {
+        if (qd != qd) qd = d;
+        if (d == qd) { qa += pa; qb += pb; return; }
+        if (close == 0) k0 = k; else k1 = k;
+        ++close;
+    }
+    __device__ __forceinline__ void entry(int k, float xa, float xb, double pa, double pb, float hi, float lo) {
+        const float d = xa - xb;                      // (both -inf: NaN, no weight)
+        za += pa;
+        zb += pb;
+        if (d > hi) { sa += pa; sb += pb; }
+        else if (d >= lo) close_call(k, d, pa, pb);
+    }
+};
+// The pass over bf16 vectors, by the table.  A function of its own: the registers of everything around it would
+// otherwise be spilled inside its loop.  About twenty instructions an entry (two of them shared-memory reads, four
+// double-precision).
+__device__ __noinline__ void classed_pass_bf16(const void* a_row, const void* b_row, const Share share, float hi, float lo,
+                                               const ExpTable<FSD_BF16>& bt, Classed& out) {
+    const uint32_t table = smem_u32(bt.e);
+    const int u0 = share.first + (threadIdx.x & 31), u1 = min(share.first + share.iters * 32, share.units);
+    const float mid = 0.5f * (hi + lo), half = 0.51f * (hi - lo);     // (a rounded test that misses no close call)
+    Classed c = out;
+    uint4 na = make_uint4(0, 0, 0, 0), nb = na;       // the vectors after these, on their way
+    if (u0 < u1) { na = ldg_vec(a_row, u0); nb = ldg_vec(b_row, u0); }
+#pragma unroll 1
+    for (int u = u0; u < u1; u += 32) {
+        const uint4 va = na, vb = nb;
+        if (u + 32 < u1) { na = ldg_vec(a_row, u + 32); nb = ldg_vec(b_row, u + 32); }
+        const int k = u * 8;
+        if (!in_table(va, vb)) {                      // an entry of the vectors is small, large or -inf
+#pragma unroll 1
+            for (int e = 0; e < 8; ++e) {
+                const float xa = load_logit<FSD_BF16>(a_row, k + e), xb = load_logit<FSD_BF16>(b_row, k + e);
+                c.entry(k + e, xa, xb, exp_bf16(xa, bt), exp_bf16(xb, bt), hi, lo);
+            }
+            continue;
+        }
+        const uint32_t wa[4] = {va.x, va.y, va.z, va.w}, wb[4] = {vb.x, vb.y, vb.z, vb.w};
+        bool close = false;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            double pa[2], pb[2];
+            table_exp2(wa[q], table, pa[0], pa[1]);
+            table_exp2(wb[q], table, pb[0], pb[1]);
+            const float d[2] = {bf16_lo(wa[q]) - bf16_lo(wb[q]), bf16_hi(wa[q]) - bf16_hi(wb[q])};
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const double one = __hiloint2double(d[e] > hi ? 0x3ff00000 : 0, 0);
+                c.za += pa[e];
+                c.zb += pb[e];
+                c.sa = fma(pa[e], one, c.sa);
+                c.sb = fma(pb[e], one, c.sb);
+                close = close || fabsf(d[e] - mid) <= half;
+            }
+        }
+        if (close) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const float xa = (e & 1) ? bf16_hi(wa[e >> 1]) : bf16_lo(wa[e >> 1]), xb = (e & 1) ? bf16_hi(wb[e >> 1]) : bf16_lo(wb[e >> 1]);
+                const float d = xa - xb;
+                if (d >= lo && !(d > hi)) c.close_call(k + e, d, exp_bf16(xa, bt), exp_bf16(xb, bt));
+            }
+        }
+    }
+    out = c;
+}
+constexpr double kResidualMargin = 2e-5;              // the record's ratio is good to a few 1e-6 at worst
+
+template <int DT>
+__device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShared& sh, ResidualShared& rs, const ExpTable<DT>& bt,
+                                              const Draw& d, int& turn, int status, bool greedy) {
+    constexpr int EPV = Logit<DT>::kPerVec;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int b = d.b, n = d.n, cs = d.cs, rank = d.rank, G = P.G;
+    const char *a_row = d.a_row, *b_row = d.b_row;
+    const double* tab = rs.exp_table;
+    double* const sc = sh.sc;
+    // ---- references.  The rejected pair's record has references (log2 domain) for both rows, near their maxima and
+    //      common to the cluster; without a record one pass for the CTA-local maxima (exact) ----
+    double kra = 0.0, krb = 0.0;
+    double zea = 0.0, zeb = 0.0;
+    bool common = false;
+    if (P.records != nullptr) {
+        PairRef ref;
+        ref.za = 0.0; ref.zb = 0.0; ref.ka = __int_as_float(0x7fc00000); ref.kb = ref.ka;
+        if (n < kPairRefs && !d.shared_out) {
+            ref = rs.ref[n];
+        } else {
+            const PairTotals t = fold_record(P.records + (static_cast<size_t>(b) * G + n), P.div);
+            if (t.state & kRecordStats) { ref.za = t.Za; ref.zb = t.Zb; ref.ka = t.ka; ref.kb = t.kb; }
+        }
+        if (isfinite(ref.ka) && isfinite(ref.kb)) {
+            kra = ref.ka; krb = ref.kb; zea = ref.za; zeb = ref.zb;
+            if constexpr (DT == FSD_BF16) {
+                // plain e^x (no reference) as long as it neither overflows nor leaves the table for good: largest logits of
+                // about -64 to 64 (a record's reference can be 2^30 below its row's largest entry, no more)
+                common = fabsf(ref.ka) <= 92.f && fabsf(ref.kb) <= 92.f;
+                if (common) { zea *= pow2_any(static_cast<int>(ref.ka)); zeb *= pow2_any(static_cast<int>(ref.kb)); }
+            } else {
+                common = true;
+            }
+        }
+    }
+    float mx[2] = {-INFINITY, -INFINITY};
+    if (!common) {
+        for_units<DT>(d, warp, lane, true, [&](int, float xa, float xb) {
+            mx[0] = fmaxf(mx[0], xa);
+            mx[1] = fmaxf(mx[1], xb);
+        });
+        block_max<2>(mx, sh.red_f);
+    }
+    const double Ra = common ? 0.0 : mx[0], Rb = common ? 0.0 : mx[1];   // this CTA's references (logit domain)
+
+    // fp32 with common references: y = x * log2e - k; logits below xmin give 2^y < 2^-990 and count as 0
+    const Exp2Consts ec = exp2_consts(rs.exp_consts);
+    const double nka = -kra, nkb = -krb;
+    const float xmin_a = static_cast<float>((kra - 990.0) * kLn2D), xmin_b = static_cast<float>((krb - 990.0) * kLn2D);
+    auto exp_a = [&](float x) -> double { if constexpr (DT == FSD_BF16) return exp_bf16(x, bt); else return exp2_of_logit(x, xmin_a, nka, tab, ec); };
+    auto exp_b = [&](float x) -> double { if constexpr (DT == FSD_BF16) return exp_bf16(x, bt); else return exp2_of_logit(x, xmin_b, nkb, tab, ec); };
+
+    // ---- global normalisers of both rows (double) ----
+    double Ma, Mb, iZa = 0.0, iZb = 0.0;
+    bool residual = true;
+    // One pass instead of two, where it can be shown to give the same sums.  An entry has residual
+    // weight iff e_a / Z_a > e_b / Z_b, i.e. e_a > rho * e_b with rho = Z_a / Z_b, which is known
+    // only after the pass -- but the record gives rho to about 1e-6.  Entries are classed against
+    // rho_est * (1 +- margin): for those clearly above, e_a and e_b are summed separately, and their
+    // residual weight is then sum e_a / Z_a - sum e_b / Z_b with the exact normalisers.
+    // The few entries between the two bounds are settled with the exact normalisers afterwards: bf16 logits
+    // differ by multiples of a step, so where ln rho falls next to one (0 above all, two rows with the same
+    // normaliser) hundreds of entries do, but they all have the same difference, hence the same ratio and
+    // the same answer: the first such difference a thread meets has sums of its own.  Two entries of another
+    // difference are remembered; a thread with more of them, or an estimate that turns out further off than
+    // half the margin, sends the whole row through the second pass instead.
+    Classed c = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, __int_as_float(0x7fc00000), 0, -1, -1};
+    bool one_pass = false;
+    double Za = 0.0, Zb = 0.0, flags = 1.0;               // flags, cluster-wide: 0 no close calls, 2 some, 1 a second pass is needed
+    const double (*all)[kExchangeDoubles];
+    if (common) {
+        // the usual case (a rejected pair with a record): both rows, two independent exponentials an entry
+        const bool classify = !greedy && zea > 0.0 && zeb > 0.0 && isfinite(zea) && isfinite(zeb);
+        const double ln_rho = classify ? log(zea / zeb) + (DT == FSD_F32 ? (kra - krb) * kLn2D : 0.0) : 0.0;
+        const float hi = static_cast<float>(ln_rho + kResidualMargin), lo = static_cast<float>(ln_rho - kResidualMargin);
+        bool done = false;
+        if constexpr (DT == FSD_BF16) {
+            if (d.vec) { classed_pass_bf16(a_row, b_row, row_share(d.V / 8, cs, rank, warp), hi, lo, bt, c); done = true; }
+        }
+        if (!done) for_units<DT>(d, warp, lane, true, [&](int k, float xa, float xb) { c.entry(k, xa, xb, exp_a(xa), exp_b(xb), hi, lo); });
+        const int mine_amb = !classify || c.close > 2 ? 1 : (c.qd == c.qd || c.close > 0) ? 2 : 0;
+        if (mine_amb) atomicOr(&sh.amb, mine_amb);
+        const double4 ws = make_double4(warp_sum(c.za), warp_sum(c.zb), warp_sum(c.sa), warp_sum(c.sb));
+        if (lane == 0) rs.wsum[warp] = ws;
+        __syncthreads();
+        double4 t = make_double4(0.0, 0.0, 0.0, 0.0);
+        if (lane < kFinishWarps) t = rs.wsum[lane];
+        const int amb = sh.amb;
+        const double mine[5] = {warp_sum(t.x), warp_sum(t.y), warp_sum(t.z), warp_sum(t.w), static_cast<double>((amb & 1) ? 1 : amb)};
+        all = cluster_exchange(sh, cs, rank, turn, mine);
+        Ma = 0.0; Mb = 0.0; flags = 0.0;
+        for (int r = 0; r < cs; ++r) { Za += all[r][0]; Zb += all[r][1]; flags = all[r][4] == 1.0 || flags == 1.0 ? 1.0 : fmax(flags, all[r][4]); }
+    } else {
+        double z[2] = {0.0, 0.0};
+        for_units<DT>(d, warp, lane, true, [&](int, float xa, float xb) {
+            if (Ra > -INFINITY) z[0] += exp2_table((static_cast<double>(xa) - Ra) * kLog2eD, tab);
+            if (Rb > -INFINITY) z[1] += exp2_table((static_cast<double>(xb) - Rb) * kLog2eD, tab);
+        });
+        block_sum<2>(z, sh.red_d);
+        const double mine[4] = {Ra, Rb, z[0], z[1]};
+        all = cluster_exchange(sh, cs, rank, turn, mine);
+        Ma = -INFINITY; Mb = -INFINITY;
+        for (int r = 0; r < cs; ++r) { Ma = fmax(Ma, all[r][0]); Mb = fmax(Mb, all[r][1]); }
+        for (int r = 0; r < cs; ++r) {
+            if (all[r][0] > -INFINITY) Za += all[r][2] * exp2_table((all[r][0] - Ma) * kLog2eD, tab);
+            if (all[r][1] > -INFINITY) Zb += all[r][3] * exp2_table((all[r][1] - Mb) * kLog2eD, tab);
+        }
+    }
+    {
+        const bool a_ok = isfinite(Ma) && isfinite(Za) && Za > 0.0, b_ok = isfinite(Mb) && isfinite(Zb) && Zb > 0.0;
+        if (!a_ok) {                                      // uniform over the cluster
+            if (rank == 0 && tid == 0) { P.accept_len[b] = n; P.next_token[b] = -1; P.row_status[b] = status | FSD_ROW_NONFINITE; }
+            return;
+        }
+        if (!b_ok) { residual = false; status |= FSD_ROW_NONFINITE; }
+        else { iZa = 1.0 / Za; iZb = 1.0 / Zb; }
+        one_pass = b_ok && flags != 1.0 && fabs(zea * Zb - zeb * Za) <= 0.5 * kResidualMargin * zeb * Za;
+    }
+
+    // the residual weights of a unit of vectors (the usual case)
+    auto vector_weights = [&](int u, double (&w)[EPV]) {
+        if constexpr (DT == FSD_BF16) {
+            const uint4 va = ldg_vec(a_row, u), vb = ldg_vec(b_row, u);
+            if (in_table(va, vb)) {
+                const uint32_t wa[4] = {va.x, va.y, va.z, va.w}, wb[4] = {vb.x, vb.y, vb.z, vb.w}, table = smem_u32(bt.e);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    double a0, a1, b0, b1;
+                    table_exp2(wa[q], table, a0, a1);
+                    table_exp2(wb[q], table, b0, b1);
+                    w[2 * q] = fmax(a0 * iZa - b0 * iZb, 0.0);
+                    w[2 * q + 1] = fmax(a1 * iZa - b1 * iZb, 0.0);
+                }
+                return;
+            }
+        }
+#pragma unroll 1
+        for (int e = 0; e < EPV; ++e) {
+            const double v = fmax(exp_a(load_logit<DT>(a_row, u * EPV + e)) * iZa - exp_b(load_logit<DT>(b_row, u * EPV + e)) * iZb, 0.0);
+#pragma unroll
+            for (int q = 0; q < EPV; ++q) if (q == e) w[q] = v;
+        }
+    };
+    // No close call in the whole row: the classed sums, already exchanged, are all there is to know.
+    if (one_pass && flags == 0.0 && d.vec) {
+        double W = 0.0, cpre = 0.0, run = 0.0;
+        for (int r = 0; r < cs; ++r) W += fmax(all[r][2] * iZa - all[r][3] * iZb, 0.0);
+        const double t = d.u * W;
+        int owner = -1;
+        for (int r = 0; r < cs && owner < 0; ++r) {
+            cpre = run;
+            run += fmax(all[r][2] * iZa - all[r][3] * iZb, 0.0);
+            if (run > t) owner = r;
+        }
+        if (owner >= 0) {                                 // (no mass, or lost to rounding at the very end: the general way)
+            if (rank == 0 && tid == 0) { P.accept_len[b] = n; P.row_status[b] = status; }
+            if (owner != rank) return;
+            const double4 ws = rs.wsum[lane & (kFinishWarps - 1)];
+            double before;
+            const int cw = Prefix(fmax(ws.z * iZa - ws.w * iZb, 0.0), lane).crossing(t - cpre, before);
+            find_crossing<EPV>(P, sh, d, row_share(d.V / EPV, cs, rank, cw), t - cpre - before, vector_weights, [&](int u) { return u * EPV; });
+            return;
+        }
+    }
+
+    for (int attempt = 0; attempt < 2; ++attempt) {
+        // weight of one vocabulary entry: the SD residual, or (no residual mass) P_T on the pass' scale
+        auto weight = [&](float xa, float xb) -> double {
+            if (common) {
+                const double pa = exp_a(xa);
+                if (!residual) return pa;
+                const double r = pa * iZa - exp_b(xb) * iZb;
+                return r > 0.0 ? r : 0.0;
+            }
+            if (!residual) return Ra > -INFINITY ? exp2_table((static_cast<double>(xa) - Ra) * kLog2eD, tab) : 0.0;
+            const double r = exp2_table((static_cast<double>(xa) - Ma) * kLog2eD, tab) * iZa -
+                             exp2_table((static_cast<double>(xb) - Mb) * kLog2eD, tab) * iZb;
+            return r > 0.0 ? r : 0.0;
+        };
+        double csum = 0.0, wbest = 0.0;
+        int kbest = 0x7fffffff;
+        if (attempt == 0 && one_pass && residual) {
+            csum = c.sa * iZa - c.sb * iZb;
+            if (!(csum > 0.0)) csum = 0.0;
+            const double q = c.qa * iZa - c.qb * iZb;
+            if (q > 0.0) csum += q;
+            for (int j = 0; j < c.close; ++j) {           // the entries that were too close to call, now with the exact normalisers
+                const int k = j == 0 ? c.k0 : c.k1;
+                const double r = exp_a(load_logit<DT>(a_row, k)) * iZa - exp_b(load_logit<DT>(b_row, k)) * iZb;
+                if (r > 0.0) csum += r;
+            }
+        } else if (d.vec && common && residual) {
+            const Share share = row_share(d.V / EPV, cs, rank, warp);
+#pragma unroll 1
+            for (int u = share.first + lane; u < min(share.first + share.iters * 32, share.units); u += 32) {
+                double w[EPV];
+                vector_weights(u, w);
+#pragma unroll
+                for (int e = 0; e < EPV; ++e) {
+                    csum += w[e];
+                    if (greedy && w[e] > wbest) { wbest = w[e]; kbest = u * EPV + e; }
+                }
+            }
+        } else {
+            for_units<DT>(d, warp, lane, residual, [&](int k, float xa, float xb) {
+                const double w = weight(xa, xb);
+                csum += w;
+                if (greedy && w > wbest) { wbest = w; kbest = k; }
+            });
+        }
+        // totals of warp and CTA, in a fixed order
+        csum = warp_sum(csum);
+        if (lane == 0) sh.warp_tot[warp] = csum;
+        if (greedy) {                                     // arg-max of the warp, ties to the lowest index
+#pragma unroll
+            for (int m = 16; m > 0; m >>= 1) {
+                const double ob = shfl_xor_d(wbest, m);
+                const int oi = __shfl_xor_sync(0xffffffffu, kbest, m);
+                if (ob > wbest || (ob == wbest && oi < kbest)) { wbest = ob; kbest = oi; }
+            }
+            if (lane == 0) { sh.red_d[warp * 2] = wbest; sh.red_d[warp * 2 + 1] = kbest; }
+        }
+        __syncthreads();
+        const Prefix pre(sh.warp_tot[lane & (kFinishWarps - 1)], lane);
+        if (greedy) {
+            wbest = sh.red_d[0]; kbest = static_cast<int>(sh.red_d[1]);
+            for (int w = 1; w < kFinishWarps; ++w) {
+                const double ob = sh.red_d[w * 2];
+                const int oi = static_cast<int>(sh.red_d[w * 2 + 1]);
+                if (ob > wbest || (ob == wbest && oi < kbest)) { wbest = ob; kbest = oi; }
+            }
+        }
+        const double mine[4] = {pre.total, Ra, wbest, static_cast<double>(kbest)};
+        all = cluster_exchange(sh, cs, rank, turn, mine);
+
+        // cluster totals on a common reference
+        double M = -INFINITY;
+        for (int r = 0; r < cs; ++r) M = fmax(M, all[r][1]);
+        double W = 0.0;
+        __syncthreads();                                  // everybody is done with the last attempt's factors
+        if (tid < cs) sc[tid] = residual || common ? 1.0 : (all[tid][1] > -INFINITY ? exp2_table((all[tid][1] - M) * kLog2eD, tab) : 0.0);
+        __syncthreads();
+        for (int r = 0; r < cs; ++r) W += all[r][0] * sc[r];
+        if (residual && !(W > 0.0)) {                     // no residual mass: draw from P_T (uniform decision)
+            residual = false;
+            continue;
+        }
+        if (!residual && !(isfinite(M) && isfinite(W) && W > 0.0)) {     // uniform over the cluster
+            if (rank == 0 && tid == 0) { P.accept_len[b] = n; P.next_token[b] = -1; P.row_status[b] = status | FSD_ROW_NONFINITE; }
+            return;
+        }
+        if (rank == 0 && tid == 0) { P.accept_len[b] = n; P.row_status[b] = status; }
+
+        if (greedy) {                                     // arg-max over the cluster
+            double gb = all[0][2] * sc[0];
+            int gi = static_cast<int>(all[0][3]);
+            for (int r = 1; r < cs; ++r) {
+                const double rb = all[r][2] * sc[r];
+                if (rb > gb || (rb == gb && static_cast<int>(all[r][3]) < gi)) { gb = rb; gi = static_cast<int>(all[r][3]); }
+            }
+            if (rank == 0 && tid == 0) P.next_token[b] = gi;
+            return;
+        }
+
+        const double t = d.u * W;
+        double cpre = 0.0, run = 0.0;
+        int owner = -1;
+        for (int r = 0; r < cs && owner < 0; ++r) {
+            cpre = run;
+            run += all[r][0] * sc[r];
+            if (run > t) owner = r;
+        }
+        if (owner < 0) {                                  // t >= W after rounding (uniform): the last token that has weight
+            int lastp = -1;
+            for_units<DT>(d, warp, lane, residual, [&](int k, float xa, float xb) { if (weight(xa, xb) > 0.0) lastp = k; });
+            lastp = __reduce_max_sync(0xffffffffu, lastp);
+            if (lane == 0 && lastp >= 0) atomicMax(&sh.last_pos, lastp);
+            __syncthreads();
+            const double mine1[1] = {static_cast<double>(sh.last_pos)};
+            all = cluster_exchange(sh, cs, rank, turn, mine1);
+            int best = -1;
+            for (int r = 0; r < cs; ++r) best = max(best, static_cast<int>(all[r][0]));
+            if (rank == 0 && tid == 0) P.next_token[b] = best;
+            return;
+        }
+        if (owner != rank) return;
+        const double t_local = (t - cpre) / sc[owner];    // the target on this CTA's own scale
+        double before;
+        const int cw = pre.crossing(t_local, before);
+        const double target = t_local - before;
+        if (d.vec && common && residual) {
+            find_crossing<EPV>(P, sh, d, row_share(d.V / EPV, cs, rank, cw), target, vector_weights, [&](int u) { return u * EPV; });
+        } else if (d.vec) {
+            find_crossing<EPV>(P, sh, d, row_share(d.V / EPV, cs, rank, cw), target,
+                [&](int u, double (&w)[EPV]) {
+#pragma unroll 1
+                    for (int e = 0; e < EPV; ++e) {
+                        const double v = weight(load_logit<DT>(a_row, u * EPV + e), residual ? load_logit<DT>(b_row, u * EPV + e) : 0.f);
+#pragma unroll
+                        for (int q = 0; q < EPV; ++q) if (q == e) w[q] = v;
+                    }
+                },
+                [&](int u) { return u * EPV; });
+        } else {
+            find_crossing<1>(P, sh, d, row_share(d.V, cs, rank, cw), target,
+                [&](int u, double (&w)[1]) { w[0] = weight(load_logit<DT>(a_row, u), residual ? load_logit<DT>(b_row, u) : 0.f); },
+                [&](int u) { return u; });
+        }
+        return;
+    }
+}
+
+template <int DT, int KIND>
+__global__ void __launch_bounds__(kFinishThreads, 2) fsd_finish_kernel(const __grid_constant__ FinishParams P) {
     __shared__ FinishShared sh;
+    __shared__ ResidualShared rs;                        // (used by the residual's instantiation alone)
+    __shared__ ExpTable<DT> bt;
     cg::cluster_group cluster = cg::this_cluster();
     const int cs = static_cast<int>(cluster.num_blocks());
     const int rank = static_cast<int>(cluster.block_rank());
-    const int b = blockIdx.x / cs;
+    const int b = static_cast<int>(blockIdx.x) / cs;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int G = P.G, V = P.V;
     const size_t rb = static_cast<size_t>(V) * Logit<DT>::kBytes;
@@ -351,48 +1128,83 @@ __global__ void __launch_bounds__(kFinishThreads, 2) fsd_finish_kernel(FinishPar
     const char* d_base = static_cast<const char*>(P.draft) + static_cast<size_t>(b) * G * rb;
     const bool tree = P.parent != nullptr;
 
+    if (tid == 0) {
+        mbar_init(&sh.link[0], 1); mbar_init(&sh.link[1], 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");     // "this CTA has started": waited for below
-    if (tid == 0) { sh.cand = 0x7fffffff; sh.last_pos = -1; sh.n_acc = G; sh.bad = 0; sh.row_sel = 0; sh.token = -1; sh.amb = 0; }
+    if (tid == 0) { sh.cand = -1; sh.last_pos = -1; sh.n_acc = G; sh.bad = 0; sh.row_sel = 0; sh.amb = 0; sh.far = 0; }
+    if (tid < kJudgeWords) sh.bits[tid] = 0;
+    if constexpr (KIND == kDrawResidual) {
+        // the tables: nothing they need is the streaming kernel's, so they are built while it drains
+        if (tid < kExpTable) rs.exp_table[tid] = exp2(static_cast<double>(tid) * (1.0 / kExpTable));
+        if (tid == 0) {
+            rs.exp_consts[0] = 6755399441055744.0; rs.exp_consts[1] = 256.0;
+            rs.exp_consts[2] = 2.239395190875157e-12; rs.exp_consts[3] = 3.308302680541371e-09;
+            rs.exp_consts[4] = 3.665565596910106e-06; rs.exp_consts[5] = 2.7076061740622863e-03;
+        }
+        if constexpr (DT == FSD_BF16) {
+            __syncthreads();
+            for (int i = tid; i < kBf16Count; i += kFinishThreads) {
+                const double x = __uint_as_float(static_cast<uint32_t>(kBf16Lowest + i) << 16);
+                bt.e[i] = exp2_table(x * kLog2eD, rs.exp_table);
+                bt.e[kBf16Sign + i] = exp2_table(-x * kLog2eD, rs.exp_table);
+            }
+        }
+    }
     __syncthreads();
     // everything above touched no global memory; what follows reads what the pair kernel wrote
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");       // every CTA of the cluster runs: its shared memory may be written
+    int turn = 0;                                                              // exchanges so far
 
     // ---- 1. divergences, accept bits, status of this row's pairs ----
     // (asked for now, needed later: each is a trip to L2 or HBM of its own)
     const float u_draw = P.u_sample[b];
     int st = 0, first = G;
     if (tid == 0 && P.timeout_flag != nullptr && *reinterpret_cast<const volatile int*>(P.timeout_flag) != 0) st |= FSD_ROW_TIMEOUT;
+    const bool shared_out = P.records != nullptr && cs > 1 && G > kFinishWarps && G <= 64 * kJudgeWords * cs;
     if (P.records != nullptr) {
         // a pair per warp: its lanes fold the parts of the pair's record, the first of them judges it
-        for (int i = warp; i < G; i += blockDim.x >> 5) {
+        const int step = shared_out ? cs : 1, i0 = shared_out ? rank : 0;
+        for (int i = warp * step + i0; i < G; i += kFinishWarps * step) {
             const int item = b * G + i;
+            int x = -1;
+            float ax = 0.f, bx = 0.f;
+            if constexpr (KIND == kDrawResidual) {       // the candidate's logits, on their way while the record is folded
+                x = P.tokens[item];
+                if (x >= 0 && x < V) {
+                    ax = load_logit<DT>(t_base + static_cast<size_t>(i) * rb, x);
+                    bx = load_logit<DT>(d_base + static_cast<size_t>(i) * rb, x);
+                }
+            }
             const PairTotals tot = fold_record(P.records + item, P.div);
             // the two logarithms the judgement needs, by two lanes at once
             const double lz = log(lane == 1 ? tot.Zb : tot.Za);
             const double lnZa = lz, lnZb = __shfl_down_sync(0xffffffffu, lz, 1);
             if (lane == 0) {
-                int trow = i;
-                if (tree) {
-                    const int par = P.parent[item];
-                    trow = (par >= -1 && par < i) ? par + 1 : 0;
-                }
                 float D;
                 int bit, s;
-                judge_record(P, item, tot, lnZa, lnZb, t_base + static_cast<size_t>(trow) * rb, d_base + static_cast<size_t>(i) * rb, DT, D, bit, s);
-                if (rank == 0) P.divergence[item] = D;
-                st |= s;
-                if (i < kMaxTreeNodes) {
-                    const float za = static_cast<float>(tot.Za);
-                    const bool ok = s == 0 && isfinite(tot.ka) && za > 0.f && za < 3.0e38f;
-                    sh.kref[i] = ok ? ceilf(tot.ka + log2f(za)) : __int_as_float(0x7fc00000);
+                judge_record(P, item, tot, lnZa, lnZb, x, ax, bx, D, bit, s);
+                if (shared_out || rank == 0) P.divergence[item] = D;
+                if constexpr (KIND == kDrawResidual) {
+                    if (i < kPairRefs) {
+                        PairRef ref;
+                        ref.za = tot.Za; ref.zb = tot.Zb; ref.ka = (tot.state & kRecordStats) ? tot.ka : __int_as_float(0x7fc00000); ref.kb = tot.kb;
+                        rs.ref[i] = ref;
+                    }
                 }
-                if (tree) sh.tree_bit[i] = static_cast<int8_t>(bit);
-                else if (!bit && i < first) first = i;
+                st |= s;
+                if (tree) {
+                    if (!shared_out) sh.tree_bit[i] = static_cast<int8_t>(bit);
+                    else if (bit) atomicOr(&sh.bits[i / cs >> 6], 1ull << (i / cs & 63));
+                } else if (!bit && i < first) {
+                    first = i;
+                }
             }
         }
     } else {
-        for (int i = tid; i < G; i += blockDim.x) {
+        for (int i = tid; i < G; i += kFinishThreads) {
             const int item = b * G + i;
             const int bit = P.item_bits[item];
             st |= P.item_status[item];
@@ -407,531 +1219,60 @@ __global__ void __launch_bounds__(kFinishThreads, 2) fsd_finish_kernel(FinishPar
         if (!tree) atomicMin(&sh.n_acc, first);
     }
     __syncthreads();
+    if (shared_out) {
+        // (the bits travel as what a double's bits are; nothing computes with them)
+        double mine[kExchangeDoubles];
+        mine[0] = __longlong_as_double(static_cast<long long>(sh.bad) << 32 | sh.n_acc);
+#pragma unroll
+        for (int k = 0; k < kJudgeWords; ++k) mine[1 + k] = __longlong_as_double(static_cast<long long>(sh.bits[k]));
+        const double (*all)[kExchangeDoubles] = cluster_exchange(sh, cs, rank, turn, mine);
+        int bad = 0, prefix = G;
+        for (int r = 0; r < cs; ++r) {
+            const long long w = __double_as_longlong(all[r][0]);
+            bad |= static_cast<int>(w >> 32);
+            prefix = min(prefix, static_cast<int>(w & 0xffffffff));
+        }
+        if (tree)
+            for (int i = tid; i < G; i += kFinishThreads)
+                sh.tree_bit[i] = static_cast<int8_t>(__double_as_longlong(all[i % cs][1 + (i / cs >> 6)]) >> (i / cs & 63) & 1);
+        __syncthreads();
+        if (tid == 0) { sh.bad = bad; sh.n_acc = prefix; }
+        __syncthreads();
+    }
 
     // ---- 2. accepted prefix (chain) or deepest accepted path (tree) ----
-    if (!tree) {
-        if (tid == 0) sh.row_sel = sh.n_acc;
-    } else {
+    int n, row_sel;
+    if (tree) {
         tree_select(P.parent + static_cast<size_t>(b) * G, G, P.max_depth,
                     rank == 0 ? P.path + static_cast<size_t>(b) * P.max_depth : nullptr, sh);
         __syncthreads();
-        FSD_CHECK(P.debug_word, sh.row_sel >= 0 && sh.row_sel <= G && sh.n_acc >= 0 && sh.n_acc <= P.max_depth, kChkPath);
+        n = sh.n_acc; row_sel = sh.row_sel;
+        FSD_CHECK(P.debug_word, row_sel >= 0 && row_sel <= G && n >= 0 && n <= P.max_depth, kChkPath);
+    } else {
+        n = sh.n_acc; row_sel = n;
     }
-    __syncthreads();
-    const int n = sh.n_acc, row_sel = sh.row_sel;
     FSD_CHECK(P.debug_word, row_sel >= 0 && row_sel <= G && n >= 0 && n <= (tree ? P.max_depth : G), kChkRow);
-    int status = sh.bad;
+    const int status = sh.bad;
     if (status & FSD_ROW_BADTREE) {                      // uniform over the cluster
         if (rank == 0 && tid == 0) { P.accept_len[b] = 0; P.next_token[b] = -1; P.row_status[b] = status; }
         return;
     }
 
     // ---- 3. token draw ----
-    constexpr int EPV = Logit<DT>::kPerVec;
-    const bool vec = P.vec != 0;
-    const bool residual0 = (P.mode != FSD_MODE_FSD) && !tree && n < G;
-    const bool greedy = P.sample == FSD_SAMPLE_GREEDY;
-    const char* a_row = t_base + static_cast<size_t>(row_sel) * rb;
-    const char* b_row = d_base + static_cast<size_t>(residual0 ? n : 0) * rb;
-    const double* tab = sh.exp_table;
-
-    // contiguous chunk of the vocabulary owned by this thread
-    const int tt = cs * blockDim.x;
-    const int L = vec ? ((V / EPV + tt - 1) / tt) * EPV : (V + tt - 1) / tt;
-    const long long k0l = static_cast<long long>(rank * blockDim.x + tid) * L;
-    const int k0 = k0l < V ? static_cast<int>(k0l) : V;
-    const int k1 = (k0l + L) < V ? static_cast<int>(k0l + L) : V;
-    FSD_CHECK(P.debug_word, k0 >= 0 && k0 <= k1 && k1 <= V && (!vec || k0 % EPV == 0), kChkChunk);
-    FinishExchange mine;
-    const FinishExchange* all = sh.all[0];
-    double* const sc = sh.sc;
-
-    // ---- fast path: inverse CDF over P_T (the FSD rule, and every bonus token) ----
-    if (!residual0 && !greedy) {
-        // Reference exponent k (log2 domain, an integer) at or just above the row's log-sum-exp, so
-        // that every exponent is <= 0 and those of the entries that carry mass are small (their
-        // rounding error stays far below the 1e-6 the draw may be off by).  When the row was a
-        // pair's target row the pair's record gives the log-sum-exp; otherwise one pass for the
-        // row maximum.
-        float kref = 0.f;
-        bool have_ref = false;
-        if (P.records != nullptr && !tree && n < G && n < kMaxTreeNodes) {
-            kref = sh.kref[n];                            // left by the thread that judged the rejected pair
-            have_ref = kref == kref;
-        }
-        if (!have_ref) {
-            float m[1] = {-INFINITY};
-            for_chunk<DT>(a_row, b_row, k0, k1, vec, false, [&](int, float xa, float) { m[0] = fmaxf(m[0], xa); });
-            block_max<1>(m, sh.red_f);
-            cluster_gather(cluster, sh, cs, rank, 0, m[0], 0);
-            double M = -INFINITY;
-            for (int r = 0; r < cs; ++r) M = fmax(M, sh.gather_d[0][r]);
-            if (!isfinite(M)) {                           // no finite logit, or +inf: uniform over the cluster
-                if (rank == 0 && tid == 0) { P.accept_len[b] = n; P.next_token[b] = -1; P.row_status[b] = status | FSD_ROW_NONFINITE; }
-                return;
-            }
-            kref = ceilf(static_cast<float>(M) * kLog2e);
-        }
-        // weight of one entry: 2^(logit * log2e - k), the same float in every pass
-        const float nk = -kref;
-        auto weight = [&](float xa) -> float { return ex2(fmaf(xa, kLog2e, nk)); };
-        double csum = 0.0;
-        for_chunk<DT>(a_row, b_row, k0, k1, vec, false, [&](int, float xa, float) { csum += static_cast<double>(weight(xa)); });
-        // inclusive / exclusive scan of the chunk sums over the CTA, fixed order
-        double incl = csum;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const double up = __shfl_up_sync(0xffffffffu, incl, d);
-            if (lane >= d) incl += up;
-        }
-        double excl = __shfl_up_sync(0xffffffffu, incl, 1);
-        if (lane == 0) excl = 0.0;
-        if (lane == 31) sh.warp_tot[warp] = incl;
-        __syncthreads();
-        double wpre = 0.0, cta_tot = 0.0;
-        for (int w = 0; w < kFinishWarps; ++w) {
-            if (w == warp) wpre = cta_tot;
-            cta_tot += sh.warp_tot[w];
-        }
-        incl += wpre;
-        excl += wpre;
-        cluster_gather(cluster, sh, cs, rank, 1, cta_tot, 0);
-        double W = 0.0;
-        for (int r = 0; r < cs; ++r) W += sh.gather_d[1][r];
-        if (!(isfinite(W) && W > 0.0)) {                  // NaN logit (or nothing representable): uniform over the cluster
-            if (rank == 0 && tid == 0) { P.accept_len[b] = n; P.next_token[b] = -1; P.row_status[b] = status | FSD_ROW_NONFINITE; }
-            return;
-        }
-        if (rank == 0 && tid == 0) { P.accept_len[b] = n; P.row_status[b] = status; }
-        const double t = static_cast<double>(u_draw) * W;
-        double cpre = 0.0, run = 0.0;
-        int owner = -1;
-        for (int r = 0; r < cs && owner < 0; ++r) {
-            cpre = run;
-            run += sh.gather_d[1][r];
-            if (run > t) owner = r;
-        }
-        auto last_with_weight = [&]() -> int {           // highest index of this thread's chunk whose weight is positive
-            int lastp = -1;
-            for_chunk<DT>(a_row, b_row, k0, k1, vec, false, [&](int k, float xa, float) { if (weight(xa) > 0.f) lastp = k; });
-            return lastp;
-        };
-        if (owner < 0) {                                  // t >= W after rounding (uniform): the last token that has weight
-            const int lp = __reduce_max_sync(0xffffffffu, last_with_weight());
-            if (lane == 0 && lp >= 0) atomicMax(&sh.last_pos, lp);
-            __syncthreads();
-            cluster_gather(cluster, sh, cs, rank, 0, 0.0, sh.last_pos);
-            int best = -1;
-            for (int r = 0; r < cs; ++r) best = sh.gather_i[0][r] > best ? sh.gather_i[0][r] : best;
-            if (rank == 0 && tid == 0) P.next_token[b] = best;
-            return;
-        }
-        if (owner != rank) return;
-        const double t_local = t - cpre;
-        if (csum > 0.0 && incl > t_local) atomicMin(&sh.cand, tid);
-        __syncthreads();
-        const int c = sh.cand;
-        if (c == 0x7fffffff) {                            // crossing lost to rounding inside this CTA
-            const int lp = __reduce_max_sync(0xffffffffu, last_with_weight());
-            if (lane == 0 && lp >= 0) atomicMax(&sh.last_pos, lp);
-            __syncthreads();
-            if (tid == 0) P.next_token[b] = sh.last_pos;
-        } else if (warp == (c >> 5)) {
-            // The warp of the thread whose chunk holds the crossing walks that chunk together: lane j
-            // takes the chunk's j-th unit (a 16-byte vector, or one entry of an unaligned row) and sums
-            // its weights in index order; every lane then adds the units' sums in order until the
-            // running sum passes the target, and the lane of that unit finds the entry.
-            const int src = c & 31;
-            const int ck0 = __shfl_sync(0xffffffffu, k0, src), ck1 = __shfl_sync(0xffffffffu, k1, src);
-            double run = __shfl_sync(0xffffffffu, excl, src);
-            const int U = vec ? EPV : 1;
-            int tok = -1, lastp = -1;
-            for (int u0 = ck0; u0 < ck1 && tok < 0; u0 += 32 * U) {
-                const int uk = u0 + lane * U;
-                float w[EPV];
-#pragma unroll
-                for (int j = 0; j < EPV; ++j) w[j] = 0.f;
-                if (uk < ck1) {
-                    if (vec) {
-                        float xa[EPV];
-                        unpack_vec<DT>(ldg_vec(a_row, uk / EPV), xa);
-#pragma unroll
-                        for (int j = 0; j < EPV; ++j) w[j] = weight(xa[j]);
-                    } else {
-                        w[0] = weight(load_logit<DT>(a_row, uk));
-                    }
-                }
-                double usum = 0.0;
-                int ulast = -1;
-#pragma unroll
-                for (int j = 0; j < EPV; ++j) {
-                    usum += static_cast<double>(w[j]);
-                    if (w[j] > 0.f) ulast = uk + j;
-                }
-                int hit = -1;                            // unit in which the running sum passes the target
-                double before = 0.0;                     // the running sum in front of that unit
-                const int nunits = min(32, (ck1 - u0 + U - 1) / U);
-                for (int j = 0; j < nunits; ++j) {
-                    const double sj = __shfl_sync(0xffffffffu, usum, j);
-                    if (hit < 0) {
-                        if (sj > 0.0 && run + sj > t_local) { hit = j; before = run; }
-                        else run += sj;
-                    }
-                }
-                lastp = max(lastp, __reduce_max_sync(0xffffffffu, ulast));
-                if (hit >= 0) {
-                    int t_here = -1;
-                    if (lane == hit) {
-                        double r2 = before;
-#pragma unroll
-                        for (int j = 0; j < EPV; ++j) {
-                            r2 += static_cast<double>(w[j]);
-                            if (t_here < 0 && w[j] > 0.f && r2 > t_local) t_here = uk + j;
-                        }
-                        if (t_here < 0) t_here = ulast;   // lost to the order of the additions: the unit's last entry with weight
-                    }
-                    tok = __shfl_sync(0xffffffffu, t_here, hit);
-                }
-            }
-            if (tok < 0) tok = lastp;
-            FSD_CHECK(P.debug_word, tok >= -1 && tok < V, kChkToken);
-            if (lane == 0) P.next_token[b] = tok;
-        }
-        return;
-    }
-
-    // the paths below take their exponentials in double precision from a table
-    if (tid < kExpTable) sh.exp_table[tid] = exp2(static_cast<double>(tid) * (1.0 / kExpTable));
-    if (tid == 0) {
-        sh.exp_consts[0] = 6755399441055744.0; sh.exp_consts[1] = 256.0;
-        sh.exp_consts[2] = 2.239395190875157e-12; sh.exp_consts[3] = 3.308302680541371e-09;
-        sh.exp_consts[4] = 3.665565596910106e-06; sh.exp_consts[5] = 2.7076061740622863e-03;
-    }
-    __syncthreads();
-
-    // ---- references.  A residual draw follows a rejection, so the rejected pair's record has
-    //      references (log2 domain) for both rows, near their maxima and common to the cluster;
-    //      otherwise one pass for the CTA-local maxima (exact), and for the greedy FSD choice the
-    //      argmax of the logits ----
-    double kra = 0.0, krb = 0.0;
-    double zea = 0.0, zeb = 0.0;
-    bool common = false;
-    if (residual0 && P.records != nullptr) {
-        const PairRecord* r = P.records + (static_cast<size_t>(b) * G + n);
-        if (r->state & kRecordStats) {
-            float fa = -INFINITY, fb = -INFINITY;
-            bool nan = false;
-            for (uint32_t c = 0; c < r->ncta && c < kMaxGroupSize; ++c) {
-                const float a = r->part[c].ka, q = r->part[c].kb;
-                nan = nan || a != a || q != q;
-                fa = fmaxf(fa, a); fb = fmaxf(fb, q);
-            }
-            if (!nan && isfinite(fa) && isfinite(fb)) {
-                kra = fa; krb = fb; common = true;
-                // the record's (single-precision) normalisers on these references: an estimate of Z_a / Z_b
-                for (uint32_t c = 0; c < r->ncta && c < kMaxGroupSize; ++c) {
-                    const float a = r->part[c].ka, q = r->part[c].kb;
-                    if (a != -INFINITY) zea += static_cast<double>(r->part[c].za) * pow2_int_d(static_cast<double>(a) - fa);
-                    if (q != -INFINITY) zeb += static_cast<double>(r->part[c].zb) * pow2_int_d(static_cast<double>(q) - fb);
-                }
-            }
-        }
-    }
-    float mx[2] = {-INFINITY, -INFINITY};
-    int amax = 0x7fffffff;
-    float amax_v = -INFINITY;
-    if (!common) {
-        for_chunk<DT>(a_row, b_row, k0, k1, vec, residual0, [&](int k, float xa, float xb) {
-            if (xa > amax_v) { amax_v = xa; amax = k; }
-            mx[1] = fmaxf(mx[1], xb);
-        });
-        mx[0] = amax_v;
-        block_max<2>(mx, sh.red_f);
-    }
-    const double Ra = common ? 0.0 : mx[0], Rb = common ? 0.0 : mx[1];   // this CTA's references (logit domain)
-
-    if (greedy && !residual0) {
-        // argmax of P_T == argmax of the logits, ties to the lowest index
-        float best = amax_v;
-        int idx = amax;
-#pragma unroll
-        for (int m = 16; m > 0; m >>= 1) {
-            const float ob = __shfl_xor_sync(0xffffffffu, best, m);
-            const int oi = __shfl_xor_sync(0xffffffffu, idx, m);
-            if (ob > best || (ob == best && oi < idx)) { best = ob; idx = oi; }
-        }
-        if (lane == 0) { sh.red_d[warp * 2] = best; sh.red_d[warp * 2 + 1] = idx; }
-        __syncthreads();
-        best = static_cast<float>(sh.red_d[0]); idx = static_cast<int>(sh.red_d[1]);
-        for (int w = 1; w < kFinishWarps; ++w) {
-            const float ob = static_cast<float>(sh.red_d[w * 2]);
-            const int oi = static_cast<int>(sh.red_d[w * 2 + 1]);
-            if (ob > best || (ob == best && oi < idx)) { best = ob; idx = oi; }
-        }
-        // a NaN or +inf logit, or no finite logit, makes the row invalid: detect through the sum of the logits' signs
-        float bad_v = 0.f;
-        for_chunk<DT>(a_row, b_row, k0, k1, vec, false, [&](int, float xa, float) { if (xa != xa || xa == INFINITY) bad_v = 1.f; });
-        float bv[1] = {bad_v};
-        block_max<1>(bv, sh.red_f);
-        mine.d[0] = best; mine.d[1] = bv[0]; mine.d[2] = 0; mine.d[3] = 0; mine.i[0] = idx; mine.i[1] = 0;
-        cluster_exchange(cluster, sh, cs, rank, 0, mine);
-        double gb = all[0].d[0], gbad = all[0].d[1];
-        int gi = all[0].i[0];
-        for (int r = 1; r < cs; ++r) {
-            if (all[r].d[0] > gb || (all[r].d[0] == gb && all[r].i[0] < gi)) { gb = all[r].d[0]; gi = all[r].i[0]; }
-            gbad = fmax(gbad, all[r].d[1]);
-        }
-        const bool ok = gbad == 0.0 && gb > -INFINITY;
-        if (rank == 0 && tid == 0) {
-            P.accept_len[b] = n;
-            P.next_token[b] = ok ? gi : -1;
-            P.row_status[b] = status | (ok ? 0 : FSD_ROW_NONFINITE);
-        }
-        return;
-    }
-
-    // with common references (the usual case): y = x * log2e - k; logits below xmin give 2^y < 2^-990 and count as 0
-    const Exp2Consts ec = exp2_consts(sh.exp_consts);
-    const double nka = -kra, nkb = -krb;
-    const float xmin_a = static_cast<float>((kra - 990.0) * kLn2D), xmin_b = static_cast<float>((krb - 990.0) * kLn2D);
-
-    // ---- residual only: global normalisers of both rows (double) ----
-    double Ma = Ra, Mb = Rb, iZa = 0.0, iZb = 0.0;
-    bool residual = residual0;
-    // One pass instead of two, where it can be shown to give the same sums.  An entry has residual
-    // weight iff e_a / Z_a > e_b / Z_b, i.e. e_a > rho * e_b with rho = Z_a / Z_b, which is known
-    // only after the pass -- but the record gives rho to about 1e-6.  Entries are classed against
-    // rho_est * (1 +- 1e-4): for those clearly above, e_a and e_b are summed separately, and the
-    // chunk's residual weight is then sum e_a / Z_a - sum e_b / Z_b with the exact normalisers.
-    // The few entries between the two bounds (about one in 10^4) are remembered, two a thread, and
-    // settled with the exact normalisers afterwards; a thread with more of them, or an estimate
-    // that turns out further than 5e-5 off, sends the whole row through the second pass instead.
-    double sa = 0.0, sb = 0.0;
-    int lastp1 = -1, amb = 0, namb = 0, ak0 = -1, ak1 = -1;
-    bool one_pass = false;
-    if (residual0) {
-        double z[2] = {0.0, 0.0};
-        if (common && vec) {
-            // the usual case (a rejected pair with a record): both rows, two independent exponentials an entry
-            const bool classify = !greedy && zea > 0.0 && zeb > 0.0 && isfinite(zea) && isfinite(zeb);
-            const double rho_est = classify ? zea / zeb : 0.0;
-            const double rho_hi = rho_est * (1.0 + 1e-4), rho_lo = rho_est * (1.0 - 1e-4);
-            for (int k = k0; k < k1; k += EPV) {
-                float xa[EPV], xb[EPV];
-                unpack_vec<DT>(ldg_vec(a_row, k / EPV), xa);
-                unpack_vec<DT>(ldg_vec(b_row, k / EPV), xb);
-#pragma unroll
-                for (int e = 0; e < EPV; ++e) {
-                    const double pa = exp2_of_logit(xa[e], xmin_a, nka, tab, ec);
-                    const double pb = exp2_of_logit(xb[e], xmin_b, nkb, tab, ec);
-                    z[0] += pa;
-                    z[1] += pb;
-                    if (pa > rho_hi * pb) { sa += pa; sb += pb; lastp1 = k + e; }
-                    else if (!(pa < rho_lo * pb) && pa > 0.0) {            // (pa == 0: no weight whatever rho is)
-                        if (namb == 0) ak0 = k + e; else ak1 = k + e;
-                        ++namb;
-                    }
-                }
-            }
-            if (!classify || namb > 2) amb = 1;
-            if (amb) atomicOr(&sh.amb, 1);
-        } else
-        for_chunk<DT>(a_row, b_row, k0, k1, vec, true, [&](int, float xa, float xb) {
-            if (common) {
-                z[0] += exp2_of_logit(xa, xmin_a, nka, tab, ec);
-                z[1] += exp2_of_logit(xb, xmin_b, nkb, tab, ec);
-            } else {
-                if (Ra > -INFINITY) z[0] += exp2_table((static_cast<double>(xa) - Ra) * kLog2eD, tab);
-                if (Rb > -INFINITY) z[1] += exp2_table((static_cast<double>(xb) - Rb) * kLog2eD, tab);
-            }
-        });
-        block_sum<2>(z, sh.red_d);                        // (its barriers also order the flag above)
-        mine.d[0] = Ra; mine.d[1] = Rb; mine.d[2] = z[0]; mine.d[3] = z[1]; mine.i[0] = (common && vec) ? sh.amb : 1; mine.i[1] = 0;
-        cluster_exchange(cluster, sh, cs, rank, 0, mine);
-        Ma = -INFINITY; Mb = -INFINITY;
-        for (int r = 0; r < cs; ++r) { Ma = fmax(Ma, all[r].d[0]); Mb = fmax(Mb, all[r].d[1]); }
-        double Za = 0.0, Zb = 0.0;
-        for (int r = 0; r < cs; ++r) {
-            if (all[r].d[0] > -INFINITY) Za += all[r].d[2] * exp2_table((all[r].d[0] - Ma) * kLog2eD, tab);
-            if (all[r].d[1] > -INFINITY) Zb += all[r].d[3] * exp2_table((all[r].d[1] - Mb) * kLog2eD, tab);
-        }
-        const bool a_ok = isfinite(Ma) && isfinite(Za) && Za > 0.0, b_ok = isfinite(Mb) && isfinite(Zb) && Zb > 0.0;
-        if (!a_ok) {                                      // uniform over the cluster
-            if (rank == 0 && tid == 0) { P.accept_len[b] = n; P.next_token[b] = -1; P.row_status[b] = status | FSD_ROW_NONFINITE; }
-            return;
-        }
-        if (!b_ok) { residual = false; status |= FSD_ROW_NONFINITE; }
-        else { iZa = 1.0 / Za; iZb = 1.0 / Zb; }
-        int any_amb = 0;
-        for (int r = 0; r < cs; ++r) any_amb |= all[r].i[0];
-        one_pass = b_ok && any_amb == 0 && fabs(zea * Zb - zeb * Za) <= 5e-5 * zeb * Za;     // |rho_est - rho| <= 5e-5 rho
-    }
-
-    for (int attempt = 0; attempt < 2; ++attempt) {
-        // weight of one vocabulary entry: P_T relative to this CTA's maximum, or the SD residual
-        auto weight = [&](float xa, float xb) -> double {
-            if (common) {                                  // the same values as the tight loops
-                const double pa = exp2_of_logit(xa, xmin_a, nka, tab, ec);
-                if (!residual) return pa;
-                const double r = pa * iZa - exp2_of_logit(xb, xmin_b, nkb, tab, ec) * iZb;
-                return r > 0.0 ? r : 0.0;
-            }
-            if (!residual) return Ra > -INFINITY ? exp2_table((static_cast<double>(xa) - Ra) * kLog2eD, tab) : 0.0;
-            const double r = exp2_table((static_cast<double>(xa) - Ma) * kLog2eD, tab) * iZa -
-                             exp2_table((static_cast<double>(xb) - Mb) * kLog2eD, tab) * iZb;
-            return r > 0.0 ? r : 0.0;
-        };
-        double csum = 0.0, wbest = 0.0;
-        int lastp = -1, kbest = 0x7fffffff;
-        if (attempt == 0 && one_pass && residual) {
-            csum = sa * iZa - sb * iZb;
-            if (!(csum > 0.0)) csum = 0.0;
-            lastp = csum > 0.0 ? lastp1 : -1;
-            for (int j = 0; j < namb; ++j) {              // the entries that were too close to call, now with the exact normalisers
-                const int k = j == 0 ? ak0 : ak1;
-                const double r = exp2_of_logit(load_logit<DT>(a_row, k), xmin_a, nka, tab, ec) * iZa -
-                                 exp2_of_logit(load_logit<DT>(b_row, k), xmin_b, nkb, tab, ec) * iZb;
-                if (r > 0.0) { csum += r; lastp = k > lastp ? k : lastp; }
-            }
-        } else if (common && vec && residual && !greedy) {
-            for (int k = k0; k < k1; k += EPV) {
-                float xa[EPV], xb[EPV];
-                unpack_vec<DT>(ldg_vec(a_row, k / EPV), xa);
-                unpack_vec<DT>(ldg_vec(b_row, k / EPV), xb);
-#pragma unroll
-                for (int e = 0; e < EPV; ++e) {
-                    const double pa = exp2_of_logit(xa[e], xmin_a, nka, tab, ec);
-                    const double pb = exp2_of_logit(xb[e], xmin_b, nkb, tab, ec);
-                    const double r = pa * iZa - pb * iZb;
-                    if (r > 0.0) { csum += r; lastp = k + e; }
-                }
-            }
-        } else
-        for_chunk<DT>(a_row, b_row, k0, k1, vec, residual, [&](int k, float xa, float xb) {
-            const double w = weight(xa, xb);
-            csum += w;
-            if (w > 0.0) lastp = k;
-            if (greedy && w > wbest) { wbest = w; kbest = k; }
-        });
-        // inclusive / exclusive scan of the chunk sums over the CTA, fixed order
-        double incl = csum;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const double up = __shfl_up_sync(0xffffffffu, incl, d);
-            if (lane >= d) incl += up;
-        }
-        double excl = __shfl_up_sync(0xffffffffu, incl, 1);
-        if (lane == 0) excl = 0.0;
-        if (lane == 31) sh.warp_tot[warp] = incl;
-        if (greedy) {                                     // residual arg-max of the warp, ties to the lowest index
-#pragma unroll
-            for (int m = 16; m > 0; m >>= 1) {
-                const double ob = shfl_xor_d(wbest, m);
-                const int oi = __shfl_xor_sync(0xffffffffu, kbest, m);
-                if (ob > wbest || (ob == wbest && oi < kbest)) { wbest = ob; kbest = oi; }
-            }
-            if (lane == 0) { sh.red_d[warp * 2] = wbest; sh.red_d[warp * 2 + 1] = kbest; }
-        }
-        const int lp = __reduce_max_sync(0xffffffffu, lastp);
-        if (lane == 0 && lp >= 0) atomicMax(&sh.last_pos, lp);
-        __syncthreads();
-        double wpre = 0.0, cta_tot = 0.0;
-        for (int w = 0; w < kFinishWarps; ++w) {
-            if (w == warp) wpre = cta_tot;
-            cta_tot += sh.warp_tot[w];
-        }
-        incl += wpre;
-        excl += wpre;
-        if (greedy) {
-            wbest = sh.red_d[0]; kbest = static_cast<int>(sh.red_d[1]);
-            for (int w = 1; w < kFinishWarps; ++w) {
-                const double ob = sh.red_d[w * 2];
-                const int oi = static_cast<int>(sh.red_d[w * 2 + 1]);
-                if (ob > wbest || (ob == wbest && oi < kbest)) { wbest = ob; kbest = oi; }
-            }
-        }
-        mine.d[0] = cta_tot; mine.d[1] = Ra; mine.d[2] = wbest; mine.d[3] = 0; mine.i[0] = sh.last_pos; mine.i[1] = kbest;
-        cluster_exchange(cluster, sh, cs, rank, 1 - (attempt & 1), mine);
-        all = sh.all[1 - (attempt & 1)];
-
-        // cluster totals on a common reference
-        double M = -INFINITY;
-        for (int r = 0; r < cs; ++r) M = fmax(M, all[r].d[1]);
-        double W = 0.0;
-        __syncthreads();                                  // everybody is done with the last attempt's factors
-        if (tid < cs) sc[tid] = residual ? 1.0 : (all[tid].d[1] > -INFINITY ? exp2_table((all[tid].d[1] - M) * kLog2eD, tab) : 0.0);
-        __syncthreads();
-        for (int r = 0; r < cs; ++r) W += all[r].d[0] * sc[r];
-        if (residual && !(W > 0.0)) {                     // no residual mass: draw from P_T (uniform decision)
-            residual = false;
-            __syncthreads();
-            if (tid == 0) sh.last_pos = -1;
-            __syncthreads();
-            continue;
-        }
-        if (!residual && !(isfinite(M) && isfinite(W) && W > 0.0)) {     // uniform over the cluster
-            if (rank == 0 && tid == 0) { P.accept_len[b] = n; P.next_token[b] = -1; P.row_status[b] = status | FSD_ROW_NONFINITE; }
-            return;
-        }
-        if (rank == 0 && tid == 0) { P.accept_len[b] = n; P.row_status[b] = status; }
-
-        if (greedy) {                                     // residual arg-max over the cluster
-            double gb = all[0].d[2];
-            int gi = all[0].i[1];
-            for (int r = 1; r < cs; ++r)
-                if (all[r].d[2] > gb || (all[r].d[2] == gb && all[r].i[1] < gi)) { gb = all[r].d[2]; gi = all[r].i[1]; }
-            if (rank == 0 && tid == 0) P.next_token[b] = gi;
-            return;
-        }
-
-        const double t = static_cast<double>(u_draw) * W;
-        double cpre = 0.0, run = 0.0;
-        int owner = -1, last_any = -1;
-        for (int r = 0; r < cs; ++r) {
-            if (owner < 0) {
-                cpre = run;
-                run += all[r].d[0] * sc[r];
-                if (run > t) owner = r;
-            }
-            if (all[r].i[0] > last_any) last_any = all[r].i[0];
-        }
-        if (owner < 0) {                                  // t >= W after rounding: the last token that has weight
-            if (rank == 0 && tid == 0) P.next_token[b] = last_any;
-            return;
-        }
-        if (owner != rank) return;
-        const double t_local = (t - cpre) / sc[owner];    // the target on this CTA's own scale
-        if (csum > 0.0 && incl > t_local) atomicMin(&sh.cand, tid);
-        __syncthreads();
-        const int c = sh.cand;
-        if (c == 0x7fffffff) {                            // crossing lost to rounding inside this CTA
-            if (tid == 0) P.next_token[b] = sh.last_pos;
-        } else if (warp == (c >> 5)) {
-            // the warp of the thread whose chunk holds the crossing walks that chunk together
-            const int src = c & 31;
-            const int ck0 = __shfl_sync(0xffffffffu, k0, src), ck1 = __shfl_sync(0xffffffffu, k1, src);
-            double base = __shfl_sync(0xffffffffu, excl, src);
-            int tok = 0x7fffffff;
-            const int fallback = __shfl_sync(0xffffffffu, lastp, src);
-            for (int kb = ck0; kb < ck1; kb += 32) {
-                const int k = kb + lane;
-                double w = 0.0;
-                if (k < ck1) w = weight(load_logit<DT>(a_row, k), residual ? load_logit<DT>(b_row, k) : 0.f);
-                double run = w;
-#pragma unroll
-                for (int d = 1; d < 32; d <<= 1) {
-                    const double up = __shfl_up_sync(0xffffffffu, run, d);
-                    if (lane >= d) run += up;
-                }
-                run += base;
-                if (k < ck1 && run > t_local && k < tok) tok = k;
-                base = __shfl_sync(0xffffffffu, run, 31);
-            }
-            tok = __reduce_min_sync(0xffffffffu, tok);
-            FSD_CHECK(P.debug_word, (tok != 0x7fffffff ? tok : fallback) >= -1 && (tok != 0x7fffffff ? tok : fallback) < V, kChkToken);
-            if (lane == 0) P.next_token[b] = tok != 0x7fffffff ? tok : fallback;
-        }
-        return;
+    const bool residual = KIND == kDrawResidual && n < G;
+    Draw d;
+    d.a_row = t_base + static_cast<size_t>(row_sel) * rb;
+    d.b_row = d_base + static_cast<size_t>(residual ? n : 0) * rb;
+    d.b = b; d.n = n; d.V = V; d.cs = cs; d.rank = rank; d.shared_out = shared_out; d.vec = P.vec != 0; d.u = static_cast<double>(u_draw);
+    if constexpr (KIND == kDrawPt) {
+        draw_pt<DT>(P, sh, d, turn, status);
+    } else if constexpr (KIND == kDrawGreedy) {
+        draw_argmax<DT>(P, sh, d, turn, status);
+    } else {
+        const bool greedy = P.sample == FSD_SAMPLE_GREEDY;
+        if (residual) draw_residual<DT>(P, sh, rs, bt, d, turn, status, greedy);
+        else if (greedy) draw_argmax<DT>(P, sh, d, turn, status);
+        else draw_pt<DT>(P, sh, d, turn, status);
     }
 }
 }  // namespace fsd

@@ -167,6 +167,17 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, int* t
     return warp_wait_slow(bar, parity, timeout_flag);
 }
 
+// Pushes between the blocks of a cluster: the address of the same object in block `rank`, and a remote
+// store that counts its eight bytes in on a barrier of the receiver.
+__device__ __forceinline__ uint32_t cluster_addr(const void* p, int rank) {
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void st_async(uint32_t addr, uint64_t v, uint32_t bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(addr), "l"(v), "r"(bar) : "memory");
+}
+
 // tensor memory: 16 columns of this warp's 32 lanes, one value a lane and column
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&r)[16]) {
     asm volatile(
@@ -351,16 +362,17 @@ __device__ __forceinline__ uint4 shifted(const uint4& lo, const uint4& hi, uint3
     return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// The vector's entries outside [0, V) read as -1e30 (2^y = 0); k0 is the index of its first entry
+// The vector's entries outside [0, V) read as -1e30 (2^y = 0), or as -inf; k0 is the index of its first entry
 template <int DT>
-__device__ __noinline__ uint4 masked_vector(uint4 v, int k0, int V) {
+__device__ __noinline__ uint4 masked_vector(uint4 v, int k0, int V, bool minus_inf = false) {
     constexpr int EPV = Logit<DT>::kPerVec;
     uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    const uint32_t fill = minus_inf ? 0xff800000u : 0xf1490000u;
 #pragma unroll
     for (int j = 0; j < EPV; ++j) {
         if (k0 + j >= 0 && k0 + j < V) continue;
-        if constexpr (DT == FSD_BF16) w[j >> 1] = (j & 1) ? ((w[j >> 1] & 0x0000ffffu) | 0xf1490000u) : ((w[j >> 1] & 0xffff0000u) | 0x0000f149u);
-        else w[j] = 0xf149f2cau;
+        if constexpr (DT == FSD_BF16) w[j >> 1] = (j & 1) ? ((w[j >> 1] & 0x0000ffffu) | fill) : ((w[j >> 1] & 0xffff0000u) | fill >> 16);
+        else w[j] = minus_inf ? fill : 0xf149f2cau;
     }
     return make_uint4(w[0], w[1], w[2], w[3]);
 }

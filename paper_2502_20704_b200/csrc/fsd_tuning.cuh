@@ -27,7 +27,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
-#include "fsd_device.cuh"
+#include "fsd_pair_stream.cuh"
 
 namespace fsd {
 
@@ -45,15 +45,6 @@ __device__ __forceinline__ uint32_t tune_key(float p) {
     return p <= 0.f ? 0u : __float_as_uint(p);
 }
 
-// ---- pushes between the blocks of a cluster -------------------------------------------------
-__device__ __forceinline__ uint32_t cluster_addr(const void* p, int rank) {       // of the same object in block `rank`
-    uint32_t r;
-    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
-    return r;
-}
-__device__ __forceinline__ void st_async(uint32_t addr, uint64_t v, uint32_t bar) {
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(addr), "l"(v), "r"(bar) : "memory");
-}
 __device__ __forceinline__ void bulk_push(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
     asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(dst), "r"(smem_u32(src)), "r"(bytes), "r"(bar) : "memory");

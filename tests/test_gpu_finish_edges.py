@@ -1,0 +1,98 @@
+"""The finish kernel where its forms part ways, against the oracle: residual draws between rows whose
+normalisers are equal (every entry on which they agree is a close call), logits outside the table of
+exponentials (tiny, beyond 64, of one sign, -inf), references out of a double's range, rows off a
+16-byte boundary, and trees and chains whose judging the cluster's thread blocks share."""
+
+import numpy as np
+import pytest
+
+import fsd_inputs as gi
+from tests import parity
+
+pytestmark = pytest.mark.gpu
+
+
+def _store(c, t, d):
+    if c.dtype == "f32":
+        c.target[:], c.draft[:] = t, d
+    else:
+        c.target[:], c.draft[:] = gi.f32_to_bf16_bits(t), gi.f32_to_bf16_bits(d)
+
+
+def _wide(c):
+    f32 = c.dtype == "f32"
+    return (c.target.copy(), c.draft.copy()) if f32 else (gi.bf16_bits_to_f32(c.target).copy(), gi.bf16_bits_to_f32(c.draft).copy())
+
+
+def _check(c, **kw):
+    return parity.check_chain(c.target, c.draft, c.draft_tokens, c.u_accept, c.u_sample, c.dtype, **kw)
+
+
+@pytest.mark.parametrize("dtype,V", [("bf16", 24000), ("bf16", 24003), ("f32", 24000), ("bf16", 152064)])
+def test_residual_between_rows_with_the_same_normaliser(dtype, V):
+    """The draft row is the target row moved round by a third: equal normalisers, and thousands of entries
+    on which the two rows agree exactly.  Their weight is 0 to rounding, so the draw is of the others."""
+    c = gi.make_chain(5, 2, V, dtype=dtype, recipe="zipf", sigma=(0.5,), workload_id=900)
+    t, d = _wide(c)
+    if dtype == "f32":
+        t = gi.bf16_bits_to_f32(gi.f32_to_bf16_bits(t))             # few values, so that many agree
+    d[:] = np.roll(t[:, :2], V // 3, axis=2)
+    _store(c, t, d)
+    c.draft_tokens[:] = d.argmax(axis=2)                            # proposed where q is far above p: rejected
+    c.u_accept[:] = 0.999
+    r = _check(c, mode="sd")
+    assert (r["accept_len"] < 2).any()
+    _check(c, mode="sd", sample="greedy")
+    _check(c, mode="rfsd", T=0.0)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("V", [4096, 20008, 20011])
+@pytest.mark.parametrize("kind", ["tiny", "large", "below", "masked", "steep"])
+def test_logits_outside_the_table(dtype, V, kind):
+    c = gi.make_chain(6, 2, V, dtype=dtype, recipe="spike", sigma=(0.4, 1.2), sigma_mode="uniform", workload_id=901)
+    t, d = _wide(c)
+    rng = np.random.default_rng(5)
+    if kind == "tiny":
+        t *= 1e-4; d *= 1e-4                                        # all below 2^-9 but a few
+        t[:, :, ::5] = 0.0
+    elif kind == "large":
+        t += 70.0; d += 75.0                                        # beyond 64, still without a reference
+    elif kind == "below":
+        t -= 150.0; d -= 140.0                                      # needs a reference
+    elif kind == "masked":
+        t[:, :, rng.random(V) < 0.4] = -np.inf
+        d[:, :, rng.random(V) < 0.4] = -np.inf
+    else:
+        k = np.arange(V, dtype=np.float32) / V
+        t += 120.0 * k; d += 110.0 * (1.0 - k)
+    _store(c, t, d)
+    c.u_accept[:] = np.where(np.arange(12).reshape(6, 2) % 3 == 0, 0.9999, c.u_accept)
+    for sample in ("invcdf", "greedy"):
+        _check(c, mode="sd", sample=sample)
+        _check(c, mode="fsd", T=0.3, sample=sample)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("shift", [-3000.0, 650.0, 3000.0])
+def test_draw_from_the_target_with_references_out_of_range(dtype, shift):
+    c = gi.make_chain(4, 2, 9001, dtype=dtype, recipe="zipf", sigma=(0.5,), workload_id=902)
+    t, d = _wide(c)
+    # (bf16 steps of 8 or 16 up there: keep the values on them)
+    if dtype == "bf16":
+        t *= 16.0; d *= 16.0
+    _store(c, t + np.float32(shift), d + np.float32(shift))
+    c.u_sample[:] = np.array([0.0, 0.3, 0.77, np.nextafter(np.float32(1), np.float32(0))], np.float32)
+    _check(c, T=10.0)
+    _check(c, T=0.0)
+
+
+@pytest.mark.parametrize("N,B,V", [(17, 3, 4096), (60, 2, 9000), (257, 2, 520), (600, 1, 4100)])
+def test_judging_shared_by_the_cluster(N, B, V):
+    t = gi.make_tree(B, N, V, dtype="bf16", sigma=0.5, max_depth=7, max_children=4, workload_id=903)
+    for T in (0.02, 0.05, 1.0):
+        parity.check_tree(t, T=T)
+    parity.check_tree(t, T=0.04, sample="greedy")
+    c = gi.make_chain(B, min(N, 70), V, dtype="bf16", recipe="zipf", sigma=(0.05, 0.4), sigma_mode="uniform", workload_id=904)
+    _check(c, T=0.06)
+    _check(c, mode="sd")

@@ -68,11 +68,12 @@ int check_shape(int B, int G, int V) {
     return FSD_OK;
 }
 
-// CTAs per row of the finish kernel: one or two vectors of logits a thread, at most the portable cluster
-// size, and no more CTAs than one wave of two per SM (148 SMs) when the batch is large.
-int finish_cluster_size(int B, int V) {
+// CTAs per row of the finish kernel: one or two vectors of logits a thread and a warp for every pair to be
+// judged, at most the portable cluster size, and no more CTAs than one wave of two per SM (148 SMs) when the
+// batch is large.
+int finish_cluster_size(int B, int G, int V) {
     int cs = 1;
-    while (cs < kMaxClusterSize && static_cast<long long>(cs) * kFinishThreads * 8 < V &&
+    while (cs < kMaxClusterSize && (static_cast<long long>(cs) * kFinishThreads * 8 < V || cs * kFinishWarps < G) &&
            static_cast<long long>(B) * cs * 2 <= 2 * 148)
         cs <<= 1;
     return cs;
@@ -220,7 +221,7 @@ int launch_all(const PairParams& pp, FinishParams fp, bool vec, int* flags, Grou
     if (void* ev = g_stage_event.load()) {
         if (cudaEventRecord(static_cast<cudaEvent_t>(ev), s) != cudaSuccess) return FSD_ERR_CUDA;
     }
-    const int cs = finish_cluster_size(fp.B, fp.V);
+    const int cs = finish_cluster_size(fp.B, fp.G, fp.V);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(fp.B) * cs, 1, 1);
     cfg.blockDim = dim3(kFinishThreads, 1, 1);

@@ -32,8 +32,8 @@
  *   - Calls are asynchronous on `stream` (a cudaStream_t passed as void*; NULL is the
  *     default stream).  Outputs are valid once the stream has been synchronised.
  *   - The return value is a host-side status: FSD_OK (0) or a negative FSD_ERR_*.
- *     On error no kernel of the call has run (a launch the runtime refuses, FSD_ERR_CUDA, can
- *     leave a 256-byte memset of the workspace's flag block on the stream; everything that
+ *     On error no kernel of the call has run (unless the runtime refuses the second launch,
+ *     FSD_ERR_CUDA, after the first; everything that
  *     can fail before that is checked first).  Nothing aborts, throws or traps.
  *   - Conditions found on the device are reported per batch row in row_status.
  *   - -inf logits are legal (probability zero).  A row holding NaN, +inf or no finite
@@ -118,7 +118,7 @@ int fsd_workspace_bytes(int B, int positions, int V, const fsd_opts *opts, size_
  *   workspace     device scratch, 256-byte aligned, at least fsd_workspace_bytes() bytes;
  *                 contents need not be initialised and are not preserved
  * Calls that share a workspace must be ordered on the stream(s) that use it.
- * The call enqueues a memset and two kernels (the first a cooperative launch of at most one
+ * The call enqueues two kernels (the first a cooperative launch of at most one
  * thread block per SM) and nothing else, so it can be captured in a CUDA graph and replayed --
  * after one ordinary call with the same options on that device, which sets the kernels'
  * attributes (that cannot be done under capture). */
@@ -215,8 +215,8 @@ int fsd_set_stage_event(void *event);
 /* Test aid (no counterpart in the paper).  Every wait inside the streaming kernel is bounded; a
  * wait that runs out raises a flag in the workspace, the thread blocks that see it take no
  * further work, the call still returns, and every row's row_status carries FSD_ROW_TIMEOUT (its
- * other outputs are then not valid).  mode 1: verify calls raise that flag themselves (a 4-byte
- * memset between the two kernels), which exercises the reporting path alone.  mode 2: in the
+ * other outputs are then not valid).  mode 1: verify calls raise that flag themselves (an 8-byte
+ * copy between the two kernels), which exercises the reporting path alone.  mode 2: in the
  * streaming kernel one thread block keeps its first statistics message to itself and the limit
  * of the exchange wait is lowered to about a tenth of a second, so its partners' wait really
  * runs out and the kernel's own give-up path runs (every wait stays bounded; nothing faults).

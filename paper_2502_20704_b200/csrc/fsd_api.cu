@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <atomic>
 #include <mutex>
+#include <random>
 
 #include "fsd_verify.h"
 #include "fsd_device.cuh"
@@ -26,8 +27,8 @@ inline bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_
 struct Workspace {
     int32_t* item_bits;
     int32_t* item_status;
-    int* flags;                // [0] = a bounded device-side wait ran out
-    GroupMsg* exchange;        // the streaming kernel's statistics exchange (directly after the flags: one memset clears both)
+    int* flags;                // [0..1]: the nonce of a call of which a bounded device-side wait ran out; [2]: debug word
+    GroupMsg* exchange;        // the streaming kernel's statistics exchange
     PairRecord* records;       // per-pair totals of the streaming kernel
     size_t bytes;
 };
@@ -82,6 +83,17 @@ int finish_cluster_size(int B, int G, int V) {
 std::atomic<void*> g_stage_event{nullptr};   // see fsd_set_stage_event
 std::atomic<int> g_mark_timeout{0};          // see fsd_set_timeout_injection
 std::atomic<int> g_group_size{0};            // see fsd_set_group_size
+
+// A number no other call carries: what the streaming kernel's messages and its timeout flag are marked with, so
+// that whatever a workspace held before is not taken for this call's.  The counter's values are spread over 64 bits
+// by an invertible mixing (the finalizer of splitmix64), from a start that differs from process to process.
+uint64_t next_nonce() {
+    static std::atomic<uint64_t> counter{(static_cast<uint64_t>(std::random_device{}()) << 32) ^ std::random_device{}()};
+    uint64_t x = counter.fetch_add(0x9e3779b97f4a7c15ull);
+    x = (x ^ (x >> 30)) * 0xbf58476d1ce4e5b9ull;
+    x = (x ^ (x >> 27)) * 0x94d049bb133111ebull;
+    return x ^ (x >> 31);
+}
 
 // ---- streaming kernel launch -----------------------------------------------------------
 constexpr int kMaxDev = 64;
@@ -177,10 +189,16 @@ int launch_all(const PairParams& pp, FinishParams fp, bool vec, int* flags, Grou
     // an unaligned row covers at most as many 16-byte granules as one that starts at a granule's last element
     const size_t nvec_row = vec ? row_bytes / 16 : (row_bytes + 16 - Logit<DT>::kBytes + 15) / 16;
     const int C = nvec_row <= static_cast<size_t>(kMaxGroupSize) * StreamShape<DT>::kBlockVecs ? group_size<DT>(static_cast<int>(nvec_row), items, nsm) : 0;
+#ifdef FSD_DEBUG_CHECKS
+    if (cudaMemsetAsync(flags, 0, kAlign, s) != cudaSuccess) return FSD_ERR_CUDA;   // the debug word starts at zero
+#endif
+    fp.nonce = 0; fp.exchange = nullptr; fp.exchange_units = 0;
     if (C > 0) {
         StreamParams sp;
         sp.target = pp.target; sp.draft = pp.draft; sp.parent = pp.parent; sp.G = pp.G;
-        sp.nvec_row = static_cast<int>(nvec_row); sp.row_bytes = row_bytes; sp.n_items = items; sp.records = records; sp.timeout_flag = flags;
+        sp.nvec_row = static_cast<int>(nvec_row); sp.row_bytes = row_bytes; sp.n_items = items; sp.records = records;
+        const uint64_t nonce = next_nonce();
+        sp.nonce = nonce; sp.timeout_flag = reinterpret_cast<uint64_t*>(flags); sp.debug_word = flags + 2;
         sp.C = C; sp.exchange = exchange;
         const int slice = static_cast<int>((nvec_row + C - 1) / C);
         sp.slot_row_bytes = slot_row_bytes<DT>(slice); sp.slot_bytes = slot_bytes<DT>(slice, !vec);
@@ -199,18 +217,18 @@ int launch_all(const PairParams& pp, FinishParams fp, bool vec, int* flags, Grou
         // the first thing put on the stream
         int rc = stream_prepare<DT>(pp.div, !vec)(dev);
         if (rc != FSD_OK) return rc;
-        // the flag block and the exchange buffer start every call at zero: flags [0] timeout
-        if (cudaMemsetAsync(flags, 0, kAlign + kExchangeBytes, s) != cudaSuccess) return FSD_ERR_CUDA;
         rc = stream_launch<DT>(pp.div, !vec)(sp, nsm, s);
         if (rc != FSD_OK) return rc;
         // test aid: behave as if a bounded wait of the streaming kernel had run out
-        if (g_mark_timeout.load() == 1 && cudaMemsetAsync(flags, 1, sizeof(int), s) != cudaSuccess) return FSD_ERR_CUDA;
-        fp.timeout_flag = flags;
+        if (g_mark_timeout.load() == 1 && cudaMemcpyAsync(flags, &nonce, sizeof(nonce), cudaMemcpyHostToDevice, s) != cudaSuccess) return FSD_ERR_CUDA;
+        fp.nonce = nonce;
+        fp.timeout_flag = reinterpret_cast<const uint64_t*>(flags);
+        if (pp.div != FSD_DIV_KL) {                  // (KL exchanges nothing)
+            fp.exchange = reinterpret_cast<uint4*>(exchange);
+            fp.exchange_units = static_cast<int>(2 * sizeof(GroupMsg) / sizeof(uint4)) * (nsm < kMaxBlocks ? nsm : kMaxBlocks);
+        }
         fp.records = records;
     } else {
-#ifdef FSD_DEBUG_CHECKS
-        if (cudaMemsetAsync(flags, 0, kAlign, s) != cudaSuccess) return FSD_ERR_CUDA;   // the debug word starts at zero here too
-#endif
         if (vec) fsd_pair_generic_kernel<DT, true><<<items, 512, 0, s>>>(pp);
         else     fsd_pair_generic_kernel<DT, false><<<items, 512, 0, s>>>(pp);
         if (cudaGetLastError() != cudaSuccess) return FSD_ERR_CUDA;

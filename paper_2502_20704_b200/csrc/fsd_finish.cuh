@@ -57,7 +57,10 @@ struct FinishParams {
     const PairRecord* records; // per-pair totals of the streaming kernel, or null (generic kernel ran)
     int32_t* item_bits;        // [B, G] read when records == null
     int32_t* item_status;      // [B, G] read when records == null
-    const int* timeout_flag;   // nonzero: a bounded wait of the streaming kernel ran out (may be null)
+    uint64_t nonce;            // of the call (see StreamParams)
+    const uint64_t* timeout_flag;   // holds the nonce: a bounded wait of the streaming kernel ran out (may be null)
+    uint4* exchange;           // the streaming kernel's messages, cleared here: a replay of the call carries the same nonce
+    int exchange_units;
     float* divergence;         // [B, G] written here when records != null
     int32_t* accept_len;       // [B]
     int32_t* path;             // [B, max_depth] (tree) or null
@@ -1157,12 +1160,14 @@ __global__ void __launch_bounds__(kFinishThreads, 2) fsd_finish_kernel(const __g
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");       // every CTA of the cluster runs: its shared memory may be written
     int turn = 0;                                                              // exchanges so far
+    for (int i = static_cast<int>(blockIdx.x) * kFinishThreads + tid; i < P.exchange_units; i += static_cast<int>(gridDim.x) * kFinishThreads)
+        P.exchange[i] = make_uint4(0, 0, 0, 0);
 
     // ---- 1. divergences, accept bits, status of this row's pairs ----
     // (asked for now, needed later: each is a trip to L2 or HBM of its own)
     const float u_draw = P.u_sample[b];
     int st = 0, first = G;
-    if (tid == 0 && P.timeout_flag != nullptr && *reinterpret_cast<const volatile int*>(P.timeout_flag) != 0) st |= FSD_ROW_TIMEOUT;
+    if (tid == 0 && P.timeout_flag != nullptr && *reinterpret_cast<const volatile uint64_t*>(P.timeout_flag) == P.nonce) st |= FSD_ROW_TIMEOUT;
     const bool shared_out = P.records != nullptr && cs > 1 && G > kFinishWarps && G <= 64 * kJudgeWords * cs;
     if (P.records != nullptr) {
         // a pair per warp: its lanes fold the parts of the pair's record, the first of them judges it

@@ -86,10 +86,11 @@ static_assert(sizeof(PairRecord) == 736, "PairRecord layout");
 constexpr uint32_t kRecordStats = 1, kRecordBadTree = 2;
 
 // One block's statistics of a round as they cross global memory: 16-byte units, each stored whole
-// and ending in the round's tag, so that a reader knows a unit is this round's without any fence or
-// flag (a unit whose tag is older is fetched again).
+// and ending in 64 bits of call and round, so that a reader knows a unit is this round's without any fence
+// or flag (a unit of another round or call, or what the workspace held before, is fetched again).  That is why
+// nothing has to be cleared in front of a call, which took a memset of 1.5 us in a call of 16.
 struct alignas(16) GroupMsg {
-    uint4 u[2];                // {ka, kb, za, tag}, {zb, 0, 0, tag}
+    uint4 u[2];                // target row: {reference, Z, nonce's high half, nonce's low half + round}; draft row: the same
 };
 static_assert(sizeof(GroupMsg) == 32, "GroupMsg layout");
 
@@ -104,11 +105,13 @@ struct StreamParams {
     int slot_row_bytes, slot_bytes, ring;    // of the shared-memory ring (see slot_bytes())
     int n_items;               // B * G
     PairRecord* records;       // [B * G]
-    int* timeout_flag;         // set to 1 if a bounded wait ran out; zero at launch
+    uint64_t nonce;            // the call's own number: what its messages and its flag carry
+    uint64_t* timeout_flag;    // set to the nonce if a bounded wait ran out (anything else: not raised)
+    int* debug_word;           // debug build: where failed range checks are recorded
     int C;                     // blocks per group (<= kMaxGroupSize)
     uint32_t poll_limit;       // fetches of the group's messages before the exchange gives up (kSpinLimit normally)
     int silent_rank;           // test aid: this rank of group 0 keeps its first message to itself (-1: nobody)
-    GroupMsg* exchange;        // [groups][2][C], zero at launch
+    GroupMsg* exchange;        // [groups][2][C]; holds no unit of this call at launch (the finish kernel clears it behind a call)
 };
 
 // ---- PTX wrappers -----------------------------------------------------------------
@@ -142,10 +145,13 @@ __device__ __forceinline__ uint64_t global_ns() {
     asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
     return t;
 }
+__device__ __forceinline__ void raise_flag(uint64_t* flag, uint64_t nonce) {
+    atomicExch(reinterpret_cast<unsigned long long*>(flag), static_cast<unsigned long long>(nonce));
+}
 // Bounded wait of a whole warp for a phase of an mbarrier: kSpinLimit polls or kWaitNs, whatever is
 // first.  False (for every lane) and the flag raised if the phase never completes or somebody else's
 // wait has run out already.
-__device__ __noinline__ bool warp_wait_slow(uint64_t* bar, uint32_t parity, int* timeout_flag) {
+__device__ __noinline__ bool warp_wait_slow(uint64_t* bar, uint32_t parity, uint64_t* timeout_flag, uint64_t nonce) {
     uint64_t t0 = 0;
 #pragma unroll 1
     for (uint32_t i = 0; i < kSpinLimit / 64; ++i) {
@@ -157,14 +163,14 @@ __device__ __noinline__ bool warp_wait_slow(uint64_t* bar, uint32_t parity, int*
         // somebody has given up already: nothing this warp waits for is certain to come
         const uint64_t t = global_ns();
         if (t0 == 0) t0 = t;
-        if (__any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(timeout_flag) != 0 || t - t0 > kWaitNs)) break;
+        if (__any_sync(0xffffffffu, *reinterpret_cast<volatile uint64_t*>(timeout_flag) == nonce || t - t0 > kWaitNs)) break;
     }
-    if ((threadIdx.x & 31) == 0) atomicExch(timeout_flag, 1);
+    if ((threadIdx.x & 31) == 0) raise_flag(timeout_flag, nonce);
     return false;
 }
-__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, int* timeout_flag) {
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, const StreamParams& P) {
     if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
-    return warp_wait_slow(bar, parity, timeout_flag);
+    return warp_wait_slow(bar, parity, P.timeout_flag, P.nonce);
 }
 
 // Pushes between the blocks of a cluster: the address of the same object in block `rank`, and a remote
@@ -405,7 +411,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
     const int vbeg = rank * base + (rank < rem ? rank : rem), vcnt = base + (rank < rem ? 1 : 0);
     const WarpPart mine = warp_part(warp < kComputeWarps ? warp : lane & (kComputeWarps - 1), vcnt, SV);
     const int steps = mine.steps;
-    FSD_CHECK(P.timeout_flag + 2, steps <= S::kSteps && vbeg + vcnt <= P.nvec_row && mine.count >= 0 && mine.first + mine.count <= (steps == 0 ? INT_MAX : vcnt), kChkSlice);
+    FSD_CHECK(P.debug_word, steps <= S::kSteps && vbeg + vcnt <= P.nvec_row && mine.count >= 0 && mine.first + mine.count <= (steps == 0 ? INT_MAX : vcnt), kChkSlice);
 
     // ---- the helper warp starts the copies ----
     int in_slot = 0, in = 0, in_item = group_id, in_par = 0;      // the pair whose slices are asked for next: its number among the group's, its id, its parent node (trees)
@@ -413,13 +419,13 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
         if (in >= R) return;
         const int slot = in_slot;
         const int b = P.G == 1 ? in_item : static_cast<int>(__umulhi(static_cast<uint32_t>(in_item), P.g_magic) >> P.g_shift);
-        FSD_CHECK(P.timeout_flag + 2, in_item >= 0 && in_item < P.n_items && b == in_item / P.G, kChkItem);
+        FSD_CHECK(P.debug_word, in_item >= 0 && in_item < P.n_items && b == in_item / P.G, kChkItem);
         int arow = in_item + b;                                      // chain: b * (G + 1) + i
         if (P.parent != nullptr) {
             const int i = in_item - b * P.G;
             arow = b * (P.G + 1) + ((in_par >= -1 && in_par < i) ? in_par + 1 : 0);   // an invalid node still moves (ignored) data
         }
-        FSD_CHECK(P.timeout_flag + 2, vcnt >= 0 && vcnt <= S::kBlockVecs && arow >= 0, kChkStage);
+        FSD_CHECK(P.debug_word, vcnt >= 0 && vcnt <= S::kBlockVecs && arow >= 0, kChkStage);
         const char* arow_p = static_cast<const char*>(P.target) + static_cast<size_t>(arow) * P.row_bytes;
         const char* brow_p = static_cast<const char*>(P.draft) + static_cast<size_t>(in_item) * P.row_bytes;
         unsigned char* dst = smem + slot * P.slot_bytes;
@@ -585,7 +591,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
         uint32_t phase = 0;                          // of the next pair's slot
         bool careful = false;                        // this warp has met logits that the quick form of the first sweep cannot take
         if (R > 0) {
-            dead = !warp_wait(&sh.full[0], 0, P.timeout_flag);
+            dead = !warp_wait(&sh.full[0], 0, P);
             if (!dead) {
                 if constexpr (RAGGED) {
                     const uint32_t meta = sh.meta[0];
@@ -636,7 +642,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
                         if constexpr (kSecondSweep) {
                             if (old) tmem_wait_ld();
                             if (live) {
-                                FSD_CHECK(P.timeout_flag + 2, (s + 1) * kParkCols <= 64, kChkTmem);
+                                FSD_CHECK(P.debug_word, (s + 1) * kParkCols <= 64, kChkTmem);
                                 tmem_st16(tslot + s * kParkCols, e);
                             }
                             if (old) {
@@ -671,13 +677,13 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
             if (nslot == P.ring) { nslot = 0; nso = 0; phase ^= 1; }
             uint32_t meta = 0;
             if (n + 1 < R) {
-                if (!warp_wait(&sh.full[nslot], phase, P.timeout_flag)) { dead = true; break; }
+                if (!warp_wait(&sh.full[nslot], phase, P)) { dead = true; break; }
                 if constexpr (RAGGED) meta = sh.meta[nslot];
             }
             // ---- the totals of pair n - 2 ----
             float ia = 0.f, ib = 0.f;
             if (n >= 2) {
-                if (!warp_wait(&sh.totals[n & 1], ((n - 2) >> 1) & 1, P.timeout_flag)) { dead = true; break; }
+                if (!warp_wait(&sh.totals[n & 1], ((n - 2) >> 1) & 1, P)) { dead = true; break; }
                 if constexpr (kSecondSweep) {
                     const float4 t = sh.tot[n & 1];
                     ia = pow2_ref(ka2, t.x) * t.y;
@@ -755,14 +761,14 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
 #pragma unroll 1
         for (int n = 0; n < n_end; ++n, item += n_groups) {
             const int par = n & 1;
-            const uint32_t tag = static_cast<uint32_t>(n) + 1;       // what this round's messages carry (never 0, the buffer's initial state)
+            const uint32_t tag = static_cast<uint32_t>(P.nonce) + static_cast<uint32_t>(n), high = static_cast<uint32_t>(P.nonce >> 32);   // what this round's messages carry
             bool bad = false;
             if (n < R && rank == 0 && P.parent != nullptr) {
                 const int pr = __ldg(P.parent + item);
                 bad = pr < -1 || pr >= item % P.G;
             }
-            if (!warp_wait(&sh.posted[par], (n >> 1) & 1, P.timeout_flag)) break;
-            FSD_CHECK(P.timeout_flag + 2, n >= R || (item >= 0 && item < P.n_items && rank < kMaxGroupSize), kChkRecord);
+            if (!warp_wait(&sh.posted[par], (n >> 1) & 1, P)) break;
+            FSD_CHECK(P.debug_word, n >= R || (item >= 0 && item < P.n_items && rank < kMaxGroupSize), kChkRecord);
             // What the compute warps wait for comes first: Z and the references.  Lanes 0..15 take the
             // target row's of one warp each, lanes 16..31 the draft row's.
             __syncwarp();
@@ -781,7 +787,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
                 if constexpr (kSecondSweep) {
                     // lanes 0 and 16 each store one 16-byte unit of this block's message; every unit ends in the round's tag
                     if ((lane & 15) == 0 && !(n == 0 && group_id == 0 && rank == P.silent_rank))
-                        st_unit(&xg[par * C + rank].u[b_side], b_side ? Kb : Ka, z, 0.f, tag);
+                        st_unit(&xg[par * C + rank].u[b_side], b_side ? Kb : Ka, z, __uint_as_float(high), tag);
                     // (while it travels: the slot all warps are through with takes the pair after the next two)
                     __syncwarp();
                     issue_slices();
@@ -795,20 +801,20 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
                         bool ok = true;
                         if (r0 < C) {
                             const uint4 u = ld_unit(&xg[par * C + r0].u[b_side]);
-                            ok = u.w == tag;
+                            ok = u.w == tag && u.z == high;
                             tk0 = __uint_as_float(u.x); tz0 = __uint_as_float(u.y);
                         }
                         if (r0 + 16 < C) {
                             const uint4 u = ld_unit(&xg[par * C + r0 + 16].u[b_side]);
-                            ok = ok && u.w == tag;
+                            ok = ok && u.w == tag && u.z == high;
                             tk1 = __uint_as_float(u.x); tz1 = __uint_as_float(u.y);
                         }
                         if (__all_sync(0xffffffffu, ok)) { got = true; break; }
                         // has anybody's wait run out?  (then nothing this warp waits for is certain to come)
-                        if ((i & 255u) == 255u && __any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(P.timeout_flag) != 0)) break;
+                        if ((i & 255u) == 255u && __any_sync(0xffffffffu, *reinterpret_cast<volatile uint64_t*>(P.timeout_flag) == P.nonce)) break;
                     }
                     if (!got) {
-                        if (lane == 0) atomicExch(P.timeout_flag, 1);
+                        if (lane == 0) raise_flag(P.timeout_flag, P.nonce);
                         break;
                     }
                     const float tk = fmax_nan(tk0, tk1);

@@ -359,7 +359,7 @@ def main():
     ws = torch.empty(wsb, dtype=torch.uint8, device="cuda")
     stream = torch.cuda.current_stream()
     sptr = stream.cuda_stream
-    launches_per_step = 2                              # pair kernel + finish kernel (the flag memset is not a kernel of this library)
+    launches_per_step = 2                              # pair kernel + finish kernel
 
     def call(t, d):
         if tree:
@@ -486,12 +486,11 @@ def main():
         pair_bytes = c.elem_size * B * P * 2 * V
     achieved = pair_bytes / (pair_ms * 1e-3) / 1e9
     call_achieved = ideal / (ms_per_step * 1e-3) / 1e9
-    kname = "fsd_pair_stream_kernel" if -(-V * c.elem_size // 16) <= 40000 else "fsd_pair_generic_kernel"
+    kname = "fsd_pair_stream_kernel" if -(-V * c.elem_size // 16) <= (49152 if c.dtype == "bf16" else 73728) else "fsd_pair_generic_kernel"
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "traffic": PAIR_KERNEL_DRAM_BYTES if headline else None, "peak_kind": f"of {peak_kind}",
                 "frac_of_nominal_8000": achieved / NOMINAL_HBM_GBS,
-                "kernel": f"pair kernel ({kname}<{c.dtype}, {args.div.upper()}>; the interval includes the "
-                          "memset of flags and exchange buffer in front of it)",
+                "kernel": f"pair kernel ({kname}<{c.dtype}, {args.div.upper()}>)",
                 "algorithmic_bytes_per_launch": pair_bytes, "ms_per_launch": pair_ms,
                 "finish_kernel_ms": finish_ms,
                 "attribution_note": "pair + finish intervals are taken with an event recorded between the two "

@@ -1,17 +1,17 @@
 // Streaming per-(row, position) kernel: every logit is read from HBM once.
 //
-// A (row, position) pair is split along the vocabulary over a GROUP of C thread blocks (C <= 20,
+// A (row, position) pair is split along the vocabulary over a GROUP of C thread blocks (C <= 24,
 // chosen by the host from what fits on chip and the number of pairs), one block of sixteen compute
 // warps and one helper warp per SM.  The launch is cooperative (all blocks resident: the blocks of a
 // group wait for one another) and the groups are persistent: group g takes pairs g, g + groups, ...
 //
 // A block's slice of a pair's two rows arrives in a ring of shared-memory slots (bulk asynchronous
-// copies started by the helper warp; the ring is as deep as the slices allow, three slots at least).
+// copies started by the helper warp; the ring is as deep as the slices allow, two slots at least).
 // The compute warps are independent of one another: a warp owns a fixed run of the slice's 16-byte
 // vectors (at most four steps of eight entries a lane), and in round n it does, step by step,
 //   1. the first sweep of pair n: e = 2^(logit * log2e - k), the sums Z = sum e and S = sum e*y (or
 //      the KL sum), a bitwise "rows differ" flag.  The references k (integers in the log2 domain) come
-//      from the maxima of the part's first step, looked at a round earlier.  That is near enough for
+//      from the maxima of the part's first step, looked at when the round before is done.  That is near enough for
 //      any ordinary logits; a warp whose sums say it was not (a later logit 2^30 above it, a -inf in
 //      the entropy sums) does the sweep over with exact maxima and clamped logits;
 //   2. interleaved with it, the SECOND sweep of pair n - 2 over the e values parked two rounds
@@ -54,7 +54,7 @@ constexpr int kStepEntries = 8;                            // vocabulary entries
 constexpr int kTmemCols = 512;                             // all of the SM's columns: warp w owns 32 lanes x 128 columns
 constexpr int kParkCols = 2 * kStepEntries;                // e values a lane parks per step (both rows)
 constexpr int kMaxClusterSize = 8;                         // finish kernel (portable size)
-constexpr int kMaxGroupSize = 20;                          // most blocks in a group of the streaming kernel
+constexpr int kMaxGroupSize = 24;                          // most blocks in a group of the streaming kernel
 constexpr uint32_t kSpinLimit = 1u << 24;                  // polls before a wait gives up
 constexpr uint64_t kWaitNs = 4000000000ull;                // and its limit in time
 constexpr uint32_t kSleepNs = 40;                          // sleep between two polls of a barrier in shared memory
@@ -82,7 +82,7 @@ struct alignas(16) PairRecord {
     uint32_t state;            // kRecordStats | kRecordBadTree
     uint32_t pad[2];
 };
-static_assert(sizeof(PairRecord) == 736, "PairRecord layout");
+static_assert(sizeof(PairRecord) == 880, "PairRecord layout");
 constexpr uint32_t kRecordStats = 1, kRecordBadTree = 2;
 
 // One block's statistics of a round as they cross global memory: 16-byte units, each stored whole
@@ -302,21 +302,21 @@ __device__ __forceinline__ void st_shared16(uint32_t addr, const uint4& v) {
 // (its last vector straddles two), so there the parts lie a granule further apart.
 template <int DT> struct StreamShape {
     static constexpr int kVecPerStep = kStepEntries / Logit<DT>::kPerVec;   // 16-byte vectors a lane handles per step and row
-    static constexpr int kSteps = DT == FSD_BF16 ? 4 : 2;                   // most steps of a warp's part: 2 KB of each row
+    static constexpr int kSteps = DT == FSD_BF16 ? 4 : 3;                   // most steps of a warp's part: 2 or 3 KB of each row
     static constexpr int kWarpVecs = 32 * kVecPerStep * kSteps;
     static constexpr int kBlockVecs = kComputeWarps * kWarpVecs;
     static constexpr int kStepVecs = 32 * kVecPerStep;
 };
 static_assert(StreamShape<FSD_BF16>::kSteps <= kMaxSteps && StreamShape<FSD_F32>::kSteps <= kMaxSteps, "two parts fit a warp's tensor memory");
-constexpr int kRingBytes = 224 * 1024;                     // shared memory for the ring (two slots are in use, the rest in flight)
-constexpr int kMaxRing = 8, kMinRing = 3;
+constexpr int kRingBytes = 224 * 1024;                     // shared memory for the ring (one slot is in use, the rest in flight)
+constexpr int kMaxRing = 8, kMinRing = 2;
 // bytes from a slot's start to its draft part, and of a whole slot, for slices of up to `slice` vectors
 template <int DT> constexpr int slot_row_bytes(int slice) {
     return (slice + StreamShape<DT>::kStepVecs - 1) / StreamShape<DT>::kStepVecs * StreamShape<DT>::kStepVecs * 16;
 }
 template <int DT> constexpr int slot_bytes(int slice, bool ragged) { return 2 * slot_row_bytes<DT>(slice) + (ragged ? kComputeWarps * 16 : 0); }
 static_assert(kMinRing * slot_bytes<FSD_BF16>(StreamShape<FSD_BF16>::kBlockVecs, true) <= kRingBytes &&
-              kMinRing * slot_bytes<FSD_F32>(StreamShape<FSD_F32>::kBlockVecs, true) <= kRingBytes, "the largest slices have three slots");
+              kMinRing * slot_bytes<FSD_F32>(StreamShape<FSD_F32>::kBlockVecs, true) <= kRingBytes, "the largest slices have two slots");
 
 // A warp's part of the block's slice: whole steps, dealt out as evenly as they go.  The warps that share
 // a scheduler with the helper warp get a step more last.
@@ -588,29 +588,29 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
         float ka = -INFINITY, kb = -INFINITY;        // references of pair n
         int slot = 0;
         uint32_t so = 0;                             // its slot, and the slot's byte offset
-        uint32_t phase = 0;                          // of the next pair's slot
+        uint32_t phase = 0;                          // of its slot
         bool careful = false;                        // this warp has met logits that the quick form of the first sweep cannot take
-        if (R > 0) {
-            dead = !warp_wait(&sh.full[0], 0, P);
-            if (!dead) {
-                if constexpr (RAGGED) {
-                    const uint32_t meta = sh.meta[0];
-                    for (int v = 0; v < steps * VPS; ++v) align_vector(0, meta, v);
-                }
-                if (steps > 0) {
-#pragma unroll
-                    for (int v = 0; v < VPS; ++v) maxima(ld_shared16(my_a + v * 512), ld_shared16(my_b + v * 512));
-                }
-                references(ka, kb);
+        // A pair's part, in slot `s` at byte offset `o`: aligned (an unaligned row's), its first step looked at for the
+        // references.  Done for the next pair at the end of a round, so that two slots suffice.
+        auto look = [&](int s, uint32_t o, float& ra, float& rb) {
+            if constexpr (RAGGED) {
+                const uint32_t meta = sh.meta[s];
+#pragma unroll 1
+                for (int v = 0; v < steps * VPS; ++v) align_vector(o, meta, v);
+                __syncwarp();
             }
-        }
-        // Both sweeps of a round, step by step.  FULL: a pair in every stage (this one's first sweep, the second sweep of
-        // n - 2, a look at the first step of n + 1), so that a step is one run of straight-line code whose strands cover one
-        // another's latencies; otherwise (the first and last rounds, and careful ones) each strand is looked at.
-        auto sweeps = [&](auto full_tag, const int n, const bool first, const uint32_t nso, [[maybe_unused]] const uint32_t meta,
-                          const float ia, const float ib, Sums& t, uint64_t& x2) {
+            if (steps > 0) {
+#pragma unroll
+                for (int v = 0; v < VPS; ++v) maxima(ld_shared16(my_a + o + v * 512), ld_shared16(my_b + o + v * 512));
+            }
+            references(ra, rb);
+        };
+        // Both sweeps of a round, step by step.  FULL: a pair in both (this one's first sweep, the second sweep of n - 2), so
+        // that a step is one run of straight-line code whose two strands cover one another's latencies; otherwise (the first
+        // and last rounds, and careful ones) each strand is looked at.
+        auto sweeps = [&](auto full_tag, const int n, const bool first, const float ia, const float ib, Sums& t, uint64_t& x2) {
             constexpr bool FULL = decltype(full_tag)::value;
-            const bool live = FULL || first, next = FULL || n + 1 < R;
+            const bool live = FULL || first;
             [[maybe_unused]] const bool old = FULL || n >= 2;
             {
                 const float ca = ka == -INFINITY ? 0.f : -ka, cb = kb == -INFINITY ? 0.f : -kb;
@@ -624,17 +624,6 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
                 for (int s = 0; s < S::kSteps; ++s) {
                     if (s < steps) {
                         [[maybe_unused]] float eo[kParkCols], e[kParkCols];
-                        if (next) {
-                            if constexpr (RAGGED) {
-#pragma unroll
-                                for (int v = 0; v < VPS; ++v) align_vector(nso, meta, s * VPS + v);
-                                __syncwarp();
-                            }
-                            if (s == 0) {
-#pragma unroll
-                                for (int v = 0; v < VPS; ++v) maxima(ld_shared16(my_a + nso + (s * VPS + v) * 512), ld_shared16(my_b + nso + (s * VPS + v) * 512));
-                            }
-                        }
                         if constexpr (kSecondSweep) {
                             if (old) tmem_ld16(tslot + s * kParkCols, eo);
                         }
@@ -669,17 +658,13 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
             }
         };
 
+        if (R > 0) {
+            dead = !warp_wait(&sh.full[0], 0, P);
+            if (!dead) look(0, 0, ka, kb);
+        }
 #pragma unroll 1
         for (int n = 0; n < n_end && !dead; ++n) {
             const bool live = n < R;
-            int nslot = slot + 1;
-            uint32_t nso = so + P.slot_bytes;
-            if (nslot == P.ring) { nslot = 0; nso = 0; phase ^= 1; }
-            uint32_t meta = 0;
-            if (n + 1 < R) {
-                if (!warp_wait(&sh.full[nslot], phase, P)) { dead = true; break; }
-                if constexpr (RAGGED) meta = sh.meta[nslot];
-            }
             // ---- the totals of pair n - 2 ----
             float ia = 0.f, ib = 0.f;
             if (n >= 2) {
@@ -692,8 +677,8 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
             }
             Sums t = zero_sums();
             uint64_t x2 = 0;
-            if (n >= 2 && n + 1 < R && !careful) sweeps(std::true_type{}, n, true, nso, meta, ia, ib, t, x2);
-            else sweeps(std::false_type{}, n, live && !careful, nso, meta, ia, ib, t, x2);
+            if (n >= 2 && live && !careful) sweeps(std::true_type{}, n, true, ia, ib, t, x2);
+            else sweeps(std::false_type{}, n, live && !careful, ia, ib, t, x2);
             // Were the references near enough?  A lane's Z up to 4e10 (an entry may exceed 2^k by about 2^30, as the
             // exponents' rounding allows), no NaN (-inf * 0 in the entropy sums), and a reference at all.  If not, the
             // first sweep is done (over) with exact maxima and clamped logits, and this warp stays with that form.
@@ -703,12 +688,8 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
                 if constexpr (DIV == FSD_DIV_JS) near = near && fabsf(sum2(t.sa2)) + fabsf(sum2(t.sb2)) < 1.0e15f;
                 if (careful || __any_sync(0xffffffffu, !near)) {
                     careful = true;
-                    float na = ma, nb = mb;          // (the next pair's maxima are in flight)
-                    const uint32_t npa = pa, npb = pb;
-                    ma = -INFINITY; mb = -INFINITY; pa = kMinusInf2; pb = kMinusInf2;
                     for (int v = 0; v < steps * VPS; ++v) maxima(ld_shared16(my_a + so + v * 512), ld_shared16(my_b + so + v * 512));
                     references(ka, kb);
-                    ma = na; mb = nb; pa = npa; pb = npb;
                     const float ca = ka == -INFINITY ? 0.f : -ka, cb = kb == -INFINITY ? 0.f : -kb;
                     t = zero_sums();
                     __syncwarp();
@@ -737,20 +718,24 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
                     k += __shfl_xor_sync(0xffffffffu, k, m);
                     if constexpr (kSecondSweep) x += __shfl_xor_sync(0xffffffffu, x, m);
                 }
-                float kan, kbn;
-                references(kan, kbn);                // (of the next pair)
                 const bool differ = DIV == FSD_DIV_TV || __any_sync(0xffffffffu, t.diff != 0);
                 WarpPost& w = sh.post[n & 1][warp];
                 if ((lane & 7) == 0) w.z[lane >> 3] = k;
                 if (lane == 1) *reinterpret_cast<float4*>(&w.ka) = make_float4(ka, kb, x, __uint_as_float(differ ? 1u : 0u));
                 __syncwarp();                        // (every lane is through with the slot, too: it takes the pair after the next two)
                 if (lane == 0) mbar_arrive(&sh.posted[n & 1]);
-                ka2 = ka1; kb2 = kb1; ka1 = ka; kb1 = kb; ka = kan; kb = kbn;
             }
-            slot = nslot; so = nso;
+            ka2 = ka1; kb2 = kb1; ka1 = ka; kb1 = kb;
             if constexpr (kSecondSweep) {
                 __syncwarp();                        // tensor-memory instructions want the warp converged
                 tmem_wait_st();
+            }
+            // ---- the next pair: its slot, its references ----
+            if (++slot == P.ring) { slot = 0; so = 0; phase ^= 1; } else { so += P.slot_bytes; }
+            ka = -INFINITY; kb = -INFINITY;
+            if (n + 1 < R) {
+                if (!warp_wait(&sh.full[slot], phase, P)) { dead = true; break; }
+                look(slot, so, ka, kb);
             }
         }
     } else {

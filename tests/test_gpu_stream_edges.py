@@ -13,8 +13,8 @@ from tests import parity
 pytestmark = pytest.mark.gpu
 
 STEP = {"bf16": 256, "f32": 256}          # vocabulary entries of a step (32 lanes x 8)
-SLICE = {"bf16": 16384, "f32": 8192}      # of a block's largest slice
-LONGEST = {"bf16": 20 * 16384, "f32": 20 * 8192}
+SLICE = {"bf16": 16384, "f32": 12288}     # of a block's largest slice
+LONGEST = {"bf16": 24 * 16384, "f32": 24 * 12288}
 
 
 def _chain(B, gamma, V, dtype, wid, **kw):

@@ -150,10 +150,11 @@ int fsd_verify_tree(const void *target_logits, const void *draft_logits,
 
 /* Chain verification with HOST buffers (same computation as fsd_verify_chain).
  * Every h_* pointer is a HOST pointer (pinned memory makes the copies faster; pageable works).
- * The call copies the inputs into `staging` (device scratch, 256-byte aligned, at least
+ * The call copies the logits into `staging` (device scratch, 256-byte aligned, at least
  * fsd_host_staging_bytes() bytes, owned by the caller), runs fsd_verify_chain on them on
- * `stream`, copies the four outputs back and synchronises the stream before it returns, so the
- * host outputs are valid on return.  h_draft_tokens / h_u_accept may be NULL in FSD mode.
+ * `stream` and synchronises the stream before it returns, so the host outputs are valid on
+ * return.  The other arrays are copied too where they are pageable; pinned ones are read and
+ * written by the kernels where they are.  h_draft_tokens / h_u_accept may be NULL in FSD mode.
  * Errors as fsd_verify_chain; a failed copy gives FSD_ERR_CUDA. */
 int fsd_host_staging_bytes(int B, int gamma, int V, const fsd_opts *opts, size_t *bytes_out);
 int fsd_verify_chain_host(const void *h_target_logits, const void *h_draft_logits,

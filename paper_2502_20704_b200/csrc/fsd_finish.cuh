@@ -89,6 +89,7 @@ struct FinishShared {
     double seg_tot[kFinishWarps];  // of the iterations find_crossing looks at
     float warp_k[kFinishWarps];    // draw from P_T: the warps' largest references
     unsigned long long bits[kJudgeWords];   // accept bits of the pairs this CTA judged for its cluster
+    float u;                   // the row's uniform
     int far;                   // draw from P_T: some thread's reference is out of a double's range; argmax: an invalid logit
     int amb;                   // residual draw: 1 some thread needs the second pass, 2 some has close calls
     int cand;                  // find_crossing: highest index with a positive weight
@@ -1165,7 +1166,8 @@ __global__ void __launch_bounds__(kFinishThreads, 2) fsd_finish_kernel(const __g
 
     // ---- 1. divergences, accept bits, status of this row's pairs ----
     // (asked for now, needed later: each is a trip to L2 or HBM of its own)
-    const float u_draw = P.u_sample[b];
+    float u_mine = 0.f;                               // (one load: the array may be in host memory)
+    if (tid == 0) u_mine = P.u_sample[b];
     int st = 0, first = G;
     if (tid == 0 && P.timeout_flag != nullptr && *reinterpret_cast<const volatile uint64_t*>(P.timeout_flag) == P.nonce) st |= FSD_ROW_TIMEOUT;
     const bool shared_out = P.records != nullptr && cs > 1 && G > kFinishWarps && G <= 64 * kJudgeWords * cs;
@@ -1217,6 +1219,7 @@ __global__ void __launch_bounds__(kFinishThreads, 2) fsd_finish_kernel(const __g
             else if (!bit && i < first) first = i;
         }
     }
+    if (tid == 0) sh.u = u_mine;
     st = __reduce_or_sync(0xffffffffu, st);
     first = __reduce_min_sync(0xffffffffu, first);
     if (lane == 0) {
@@ -1268,7 +1271,7 @@ __global__ void __launch_bounds__(kFinishThreads, 2) fsd_finish_kernel(const __g
     Draw d;
     d.a_row = t_base + static_cast<size_t>(row_sel) * rb;
     d.b_row = d_base + static_cast<size_t>(residual ? n : 0) * rb;
-    d.b = b; d.n = n; d.V = V; d.cs = cs; d.rank = rank; d.shared_out = shared_out; d.vec = P.vec != 0; d.u = static_cast<double>(u_draw);
+    d.b = b; d.n = n; d.V = V; d.cs = cs; d.rank = rank; d.shared_out = shared_out; d.vec = P.vec != 0; d.u = static_cast<double>(sh.u);
     if constexpr (KIND == kDrawPt) {
         draw_pt<DT>(P, sh, d, turn, status);
     } else if constexpr (KIND == kDrawGreedy) {

@@ -118,8 +118,8 @@ int fsd_workspace_bytes(int B, int positions, int V, const fsd_opts *opts, size_
  *   workspace     device scratch, 256-byte aligned, at least fsd_workspace_bytes() bytes;
  *                 contents need not be initialised and are not preserved
  * Calls that share a workspace must be ordered on the stream(s) that use it.
- * The call enqueues two kernels (the first a cooperative launch of at most one
- * thread block per SM) and nothing else, so it can be captured in a CUDA graph and replayed --
+ * The call enqueues two kernels (the first of at most one thread block per SM, both with
+ * programmatic stream serialization) and nothing else, so it can be captured in a CUDA graph and replayed --
  * after one ordinary call with the same options on that device, which sets the kernels'
  * attributes (that cannot be done under capture). */
 int fsd_verify_chain(const void *target_logits, const void *draft_logits,
@@ -221,6 +221,9 @@ int fsd_set_stage_event(void *event);
  * streaming kernel one thread block keeps its first statistics message to itself and the limit
  * of the exchange wait is lowered to about a tenth of a second, so its partners' wait really
  * runs out and the kernel's own give-up path runs (every wait stays bounded; nothing faults).
+ * mode 3, in a build with -DFSD_DEBUG_CHECKS only: the block keeps its message to itself and the
+ * others do without, as they do when a block of a group is not running: they sum its slice
+ * themselves after about a millisecond, and the call's results are ordinary ones.
  * mode 0: off (the default).  Process-wide, read when a call is made.  Returns FSD_OK, or
  * FSD_ERR_ENUM for another mode. */
 int fsd_set_timeout_injection(int mode);

@@ -98,7 +98,7 @@ uint64_t next_nonce() {
 // ---- streaming kernel launch -----------------------------------------------------------
 constexpr int kMaxDev = 64;
 
-// One block per SM, all resident (cooperative launch).  Puts nothing on a stream.
+// One block per SM.  Puts nothing on a stream.
 template <int DT, int DIV, bool RAGGED>
 int prepare_stream(int dev) {
     static bool ready[kMaxDev] = {};
@@ -109,7 +109,7 @@ int prepare_stream(int dev) {
     if (!ready[dev]) {
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kStreamSmemBytes)) != cudaSuccess)
             return FSD_ERR_CUDA;
-        int per = 0;                                 // one block must fit an SM, or the cooperative launch is refused
+        int per = 0;                                 // one block must fit an SM
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, kStreamThreads, kStreamSmemBytes) != cudaSuccess || per < 1)
             return FSD_ERR_CUDA;
         ready[dev] = true;
@@ -130,8 +130,9 @@ int launch_stream(const StreamParams& gp, int nsm, cudaStream_t s) {
     cfg.dynamicSmemBytes = kStreamSmemBytes;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;     // the groups' blocks wait for one another: all must be resident
-    attr[0].val.cooperative = 1;
+    // Set up while the kernel in front drains; the kernel waits for its end itself.  (A cooperative launch ignores this.)
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if (cudaLaunchKernelEx(&cfg, fsd_pair_stream_kernel<DT, DIV, RAGGED>, gp) != cudaSuccess) return FSD_ERR_CUDA;
@@ -209,9 +210,12 @@ int launch_all(const PairParams& pp, FinishParams fp, bool vec, int* flags, Grou
         sp.g_magic = l == 0 ? 0u : static_cast<uint32_t>(((1ull << (31 + l)) + pp.G - 1) / pp.G);
         sp.g_shift = l == 0 ? 0u : static_cast<uint32_t>(l - 1);
         // test aid: one block keeps its first message to itself, so that its group's exchange
-        // runs out (after a shorter limit: about a tenth of a second) and the kernel's own give-up path runs
-        const bool silent = g_mark_timeout.load() == 2;
+        // runs out (after a shorter limit: about a tenth of a second) and the kernel's own give-up path runs;
+        // mode 3: so that the others sum its slice themselves
+        const int injection = g_mark_timeout.load();
+        const bool silent = injection >= 2;
         sp.poll_limit = silent ? (1u << 17) : kSpinLimit;
+        sp.help_after = injection == 2 ? 0xffffffffu : 1024;     // about a millisecond of fetches
         sp.silent_rank = silent ? C - 1 : -1;
         // everything that can fail without a launch (attributes, the occupancy query) comes before
         // the first thing put on the stream
@@ -557,7 +561,12 @@ int fsd_debug_checks(int B, int positions, size_t* word_offset) {
 }
 
 int fsd_set_timeout_injection(int mode) {
-    if (mode < 0 || mode > 2) return FSD_ERR_ENUM;
+#ifdef FSD_DEBUG_CHECKS
+    constexpr int kModes = 3;
+#else
+    constexpr int kModes = 2;
+#endif
+    if (mode < 0 || mode > kModes) return FSD_ERR_ENUM;
     g_mark_timeout.store(mode);
     return FSD_OK;
 }

@@ -2,8 +2,12 @@
 //
 // A (row, position) pair is split along the vocabulary over a GROUP of C thread blocks (C <= 24,
 // chosen by the host from what fits on chip and the number of pairs), one block of sixteen compute
-// warps and one helper warp per SM.  The launch is cooperative (all blocks resident: the blocks of a
-// group wait for one another) and the groups are persistent: group g takes pairs g, g + groups, ...
+// warps and one helper warp per SM.  The groups are persistent: group g takes pairs g, g + groups, ...
+//
+// The blocks of a group wait for one another's sums, and usually all of them run.  The launch does not promise it: a
+// cooperative launch would, but it starts only when the kernel in front has ended and that end has been polled for (a
+// period of 2.05 us; calls in a row took multiples of it), while a launch with programmatic stream serialization is set
+// up before.  So a block that has waited for about a millisecond sums the missing slices itself and goes on.
 //
 // A block's slice of a pair's two rows arrives in a ring of shared-memory slots (bulk asynchronous
 // copies started by the helper warp; the ring is as deep as the slices allow, two slots at least).
@@ -110,6 +114,7 @@ struct StreamParams {
     int* debug_word;           // debug build: where failed range checks are recorded
     int C;                     // blocks per group (<= kMaxGroupSize)
     uint32_t poll_limit;       // fetches of the group's messages before the exchange gives up (kSpinLimit normally)
+    uint32_t help_after;       // fetches after which a block computes what it waits for by itself (0xffffffff: never)
     int silent_rank;           // test aid: this rank of group 0 keeps its first message to itself (-1: nobody)
     GroupMsg* exchange;        // [groups][2][C]; holds no unit of this call at launch (the finish kernel clears it behind a call)
 };
@@ -383,6 +388,24 @@ __device__ __noinline__ uint4 masked_vector(uint4 v, int k0, int V, bool minus_i
     return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
+// Reference and Z of entries [k0, k1) of a row in global memory, by one warp: what a block's message says of its slice
+template <int DT>
+__device__ __noinline__ float2 slice_sum(const void* row, int k0, int k1) {
+    const int lane = threadIdx.x & 31;
+    float m = -INFINITY, z = 0.f;
+#pragma unroll 8
+    for (int k = k0 + lane; k < k1; k += 32) m = fmax_nan(m, load_logit<DT>(row, k));
+    __syncwarp();
+    m = warp_redux_max_nan(m);
+    const float K = m <= -9.9e29f ? -INFINITY : ceilf(m * kLog2e), c = K == -INFINITY ? 0.f : -K;
+#pragma unroll 8
+    for (int k = k0 + lane; k < k1; k += 32) z += ex2(fmaf(load_logit<DT>(row, k), kLog2e, c));
+    __syncwarp();
+#pragma unroll
+    for (int i = 16; i > 0; i >>= 1) z += __shfl_xor_sync(0xffffffffu, z, i);
+    return make_float2(K, z);
+}
+
 template <int DT, int DIV, bool RAGGED>
 __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(const __grid_constant__ StreamParams P) {
     using S = StreamShape<DT>;
@@ -466,13 +489,16 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         }
         __syncwarp();
+        // This warp alone touches global memory.  What is in front of the kernel in its stream has to be done first: it may
+        // have been launched before (programmatic stream serialization).
+        asm volatile("griddepcontrol.wait;" ::: "memory");
         if (P.parent != nullptr && R > 0) in_par = __ldg(P.parent + in_item);
         for (int q = 0; q < P.ring; ++q) issue_slices();
-        if constexpr (kSecondSweep) {
+    } else {
+        if (kSecondSweep && warp == 0) {
             asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh.tmem_base)), "n"(kTmemCols) : "memory");
             asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
         }
-    } else {
         // lanes without a vector in the slice's last step read "-inf" there: no copy ever writes behind the slice
         // (an unaligned draft row's vectors there are masked)
         const int end = (vcnt + SV - 1) / SV * SV;
@@ -743,6 +769,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
         // where this group exchanges its statistics: [parity][rank] messages
         GroupMsg* const xg = P.exchange + static_cast<size_t>(group_id < n_groups ? group_id : 0) * 2 * C;
         int item = group_id;
+        uint32_t help_after = P.help_after;
 #pragma unroll 1
         for (int n = 0; n < n_end; ++n, item += n_groups) {
             const int par = n & 1;
@@ -783,18 +810,45 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
                     bool got = false;
 #pragma unroll 1
                     for (uint32_t i = 0; i < P.poll_limit; ++i) {
-                        bool ok = true;
+                        bool ok0 = true, ok1 = true;
                         if (r0 < C) {
                             const uint4 u = ld_unit(&xg[par * C + r0].u[b_side]);
-                            ok = u.w == tag && u.z == high;
+                            ok0 = u.w == tag && u.z == high;
                             tk0 = __uint_as_float(u.x); tz0 = __uint_as_float(u.y);
                         }
                         if (r0 + 16 < C) {
                             const uint4 u = ld_unit(&xg[par * C + r0 + 16].u[b_side]);
-                            ok = ok && u.w == tag && u.z == high;
+                            ok1 = u.w == tag && u.z == high;
                             tk1 = __uint_as_float(u.x); tz1 = __uint_as_float(u.y);
                         }
-                        if (__all_sync(0xffffffffu, ok)) { got = true; break; }
+                        if (__all_sync(0xffffffffu, ok0 && ok1)) { got = true; break; }
+                        // A block of the group that has sent nothing for this long may not be running at all: nothing makes the
+                        // blocks of this launch resident together, another stream's kernels may hold SMs.  Its slices are summed
+                        // here then, so no block ever needs another one in order to finish.  (From then on the others' rounds
+                        // and this block's are apart, and it does not wait as long again.)
+                        if (i >= help_after) {
+                            const uint32_t miss0 = __ballot_sync(0xffffffffu, !ok0), miss1 = __ballot_sync(0xffffffffu, !ok1);
+                            const int b = item / P.G, V = static_cast<int>(P.row_bytes / Logit<DT>::kBytes);
+                            int arow = item + b;
+                            if (P.parent != nullptr) {
+                                const int pr = __ldg(P.parent + item), k = item - b * P.G;
+                                arow = b * (P.G + 1) + (pr >= -1 && pr < k ? pr + 1 : 0);
+                            }
+                            const char* arow_p = static_cast<const char*>(P.target) + static_cast<size_t>(arow) * P.row_bytes;
+                            const char* brow_p = static_cast<const char*>(P.draft) + static_cast<size_t>(item) * P.row_bytes;
+                            const int oa = RAGGED ? static_cast<int>(reinterpret_cast<uintptr_t>(arow_p) & 15) / Logit<DT>::kBytes : 0;
+#pragma unroll 1
+                            for (int r = 0; r < C; ++r) {
+                                if (((r < 16 ? miss0 : miss1) >> (r & 15) & 0x10001u) == 0) continue;
+                                const int k0 = (r * base + min(r, rem)) * EPV - oa, k1 = min(k0 + (base + (r < rem ? 1 : 0)) * EPV, V);
+                                const float2 ta = slice_sum<DT>(arow_p, max(k0, 0), k1), tb = slice_sum<DT>(brow_p, max(k0, 0), k1);
+                                if (r0 == r) { tk0 = b_side ? tb.x : ta.x; tz0 = b_side ? tb.y : ta.y; }
+                                if (r0 + 16 == r) { tk1 = b_side ? tb.x : ta.x; tz1 = b_side ? tb.y : ta.y; }
+                            }
+                            help_after = 32;
+                            got = true;
+                            break;
+                        }
                         // has anybody's wait run out?  (then nothing this warp waits for is certain to come)
                         if ((i & 255u) == 255u && __any_sync(0xffffffffu, *reinterpret_cast<volatile uint64_t*>(P.timeout_flag) == P.nonce)) break;
                     }
@@ -861,7 +915,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
         __syncwarp();
-        if (warp == kComputeWarps)
+        if (warp == 0)
             asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(sh.tmem_base), "n"(kTmemCols) : "memory");
     }
 }

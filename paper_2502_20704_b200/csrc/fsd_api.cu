@@ -373,11 +373,13 @@ int launch_tuning(void (*kernel)(KArgs...), int threads, int cs, int clusters, i
     cfg.blockDim = dim3(static_cast<unsigned>(threads), 1, 1);
     cfg.dynamicSmemBytes = bytes;
     cfg.stream = static_cast<cudaStream_t>(stream);
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = cs; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cs; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = cs > 1 ? 1 : 0;
+    cfg.numAttrs = cs > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...) == cudaSuccess ? FSD_OK : FSD_ERR_CUDA;
 }
 
@@ -610,8 +612,16 @@ int fsd_accept_labels(const float* divergence, int B, int positions, float thres
     if (compare != FSD_CMP_LT && compare != FSD_CMP_LE) return FSD_ERR_ENUM;
     const size_t n = static_cast<size_t>(B) * positions;
     const unsigned blocks = static_cast<unsigned>(n / 256 + 1 < 1184 ? n / 256 + 1 : 1184);
-    fsd_accept_labels_kernel<<<blocks, 256, 0, static_cast<cudaStream_t>(stream)>>>(divergence, n, threshold, compare, labels);
-    return cudaGetLastError() == cudaSuccess ? FSD_OK : FSD_ERR_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks, 1, 1);
+    cfg.blockDim = dim3(256, 1, 1);
+    cfg.stream = static_cast<cudaStream_t>(stream);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, fsd_accept_labels_kernel, divergence, n, threshold, compare, labels) == cudaSuccess ? FSD_OK : FSD_ERR_CUDA;
 }
 
 }  // extern "C"

@@ -57,6 +57,14 @@ __device__ __forceinline__ bool tune_wait(uint64_t* bar, uint32_t parity) {
     return false;
 }
 
+// These kernels are a few microseconds each and follow one another: all are launched with programmatic stream
+// serialization.  What is in front of a kernel in its stream has ended (or it is waited for here, before global memory
+// is touched); what comes behind it may be set up meanwhile.
+__device__ __forceinline__ void launch_in_turn() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // ---- a block's rows [row0, row1) of the divergence matrix, tile by tile ---------------------
 // Two tiles are in shared memory at most; a block whose rows are no more than that copies them once.
 struct TuneRows {
@@ -168,6 +176,7 @@ __global__ void __launch_bounds__(kTuneThreads) fsd_threshold_sweep_kernel(const
     }
     __syncthreads();
     if constexpr (CS > 1) cg::this_cluster().barrier_arrive();   // "this block's barriers are ready": waited for before the first push
+    launch_in_turn();
     TuneRows rows = tune_rows(D, B, G, rank, CS, tune_buf, bar);
     // thresholds cid, cid + n_clusters, ...: kSweepAtOnce of them in one walk
     int turn = 0;
@@ -286,6 +295,7 @@ __global__ void __launch_bounds__(kTuneThreads) fsd_calibrate_kernel(const float
     for (int i = tid; i < kTuneList; i += kTuneThreads) sh.list[i] = 0xffffffffu;
     __syncthreads();
     if constexpr (CS > 1) cg::this_cluster().barrier_arrive();   // "this block's barriers are ready": waited for before the first push
+    launch_in_turn();
     TuneRows rows = tune_rows(D, B, G, rank, CS, tune_buf, sh.bar);
 
     // positions that must be accepted: ceil(target * B), within [0, B * G]  (the host refuses negative and NaN targets)
@@ -458,6 +468,7 @@ __global__ void __launch_bounds__(kTuneThreads) fsd_calibrate_kernel(const float
 
 // ---- labels: each position on its own ---------------------------------------------------------
 __global__ void fsd_accept_labels_kernel(const float* __restrict__ D, size_t n, float T, int cmp, uint8_t* __restrict__ labels) {
+    launch_in_turn();
     const size_t stride = static_cast<size_t>(gridDim.x) * blockDim.x;
     for (size_t i = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += stride)
         labels[i] = passes(D[i], T, cmp) ? 1 : 0;

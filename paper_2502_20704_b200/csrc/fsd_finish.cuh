@@ -1056,6 +1056,7 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
             return;
         }
         if (rank == 0 && tid == 0) { P.accept_len[b] = n; P.row_status[b] = status; }
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
         if (greedy) {                                     // arg-max over the cluster
             double gb = all[0][2] * sc[0];
@@ -1157,6 +1158,9 @@ __global__ void __launch_bounds__(kFinishThreads, 2) fsd_finish_kernel(const __g
         }
     }
     __syncthreads();
+    // What comes behind this kernel may be set up while it runs.  (A residual draw allows that when its pass is through:
+    // earlier, the next call's blocks are spread over the SMs as its rows end, 64 x 8 x 152064 136.5 -> 140 us.)
+    if constexpr (KIND != kDrawResidual) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // everything above touched no global memory; what follows reads what the pair kernel wrote
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");       // every CTA of the cluster runs: its shared memory may be written
@@ -1278,6 +1282,7 @@ __global__ void __launch_bounds__(kFinishThreads, 2) fsd_finish_kernel(const __g
         draw_argmax<DT>(P, sh, d, turn, status);
     } else {
         const bool greedy = P.sample == FSD_SAMPLE_GREEDY;
+        if (!residual) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
         if (residual) draw_residual<DT>(P, sh, rs, bt, d, turn, status, greedy);
         else if (greedy) draw_argmax<DT>(P, sh, d, turn, status);
         else draw_pt<DT>(P, sh, d, turn, status);

@@ -727,27 +727,29 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
                     }
                 }
             }
-            // ---- fold over the lanes: four sums by halving (six shuffles), the second-sweep sum by a butterfly ----
+            // ---- fold over the lanes: sums by halving, the second-sweep sum joins where the four have become one ----
             {
                 const float v0 = sum2(t.za2), v1 = sum2(t.zb2), v2 = DIV == FSD_DIV_KL ? t.kk : sum2(t.sa2), v3 = sum2(t.sb2);
                 const bool hi = (lane & 16) != 0, up = (lane & 8) != 0;
                 float k0 = (hi ? v2 : v0) + __shfl_xor_sync(0xffffffffu, hi ? v0 : v2, 16);
                 float k1 = (hi ? v3 : v1) + __shfl_xor_sync(0xffffffffu, hi ? v1 : v3, 16);
                 float k = (up ? k1 : k0) + __shfl_xor_sync(0xffffffffu, up ? k0 : k1, 8);
-                float x = sum2(x2);
                 if constexpr (kSecondSweep) {
+                    float x = sum2(x2);
                     x += __shfl_xor_sync(0xffffffffu, x, 16);
                     x += __shfl_xor_sync(0xffffffffu, x, 8);
-                }
+                    const bool odd = (lane & 4) != 0;                    // from here on, these lanes carry x
+                    k = (odd ? x : k) + __shfl_xor_sync(0xffffffffu, odd ? k : x, 4);
+                    k += __shfl_xor_sync(0xffffffffu, k, 2);
+                    k += __shfl_xor_sync(0xffffffffu, k, 1);
+                } else {
 #pragma unroll
-                for (int m = 4; m > 0; m >>= 1) {
-                    k += __shfl_xor_sync(0xffffffffu, k, m);
-                    if constexpr (kSecondSweep) x += __shfl_xor_sync(0xffffffffu, x, m);
+                    for (int m = 4; m > 0; m >>= 1) k += __shfl_xor_sync(0xffffffffu, k, m);
                 }
                 const bool differ = DIV == FSD_DIV_TV || __any_sync(0xffffffffu, t.diff != 0);
                 WarpPost& w = sh.post[n & 1][warp];
                 if ((lane & 7) == 0) w.z[lane >> 3] = k;
-                if (lane == 1) *reinterpret_cast<float4*>(&w.ka) = make_float4(ka, kb, x, __uint_as_float(differ ? 1u : 0u));
+                if (lane == 4) *reinterpret_cast<float4*>(&w.ka) = make_float4(ka, kb, k, __uint_as_float(differ ? 1u : 0u));
                 __syncwarp();                        // (every lane is through with the slot, too: it takes the pair after the next two)
                 if (lane == 0) mbar_arrive(&sh.posted[n & 1]);
             }

@@ -69,13 +69,13 @@ struct FinishParams {
     int* debug_word;           // debug build: where failed range checks are recorded (may be null)
 };
 
-constexpr int kExchangeDoubles = 5;      // most values a CTA tells its cluster at once
+constexpr int kExchangeDoubles = 7;      // most values a CTA tells its cluster at once
 // With more pairs than a CTA has warps, the cluster's CTAs share the judging (CTA r takes pairs r, r + cs, ...)
 // and tell one another the accept bits: up to 64 * kJudgeWords of them each.
-constexpr int kJudgeWords = kExchangeDoubles - 1;
+constexpr int kJudgeWords = 4;
 constexpr int kExpTable = 256;
-// e^x of the bf16 numbers with 2^-9 <= |x| < 64, both signs
-constexpr int kBf16Lowest = 118 << 7, kBf16Count = 15 << 7;
+// e^x of the bf16 numbers with 2^-13 <= |x| < 64, both signs
+constexpr int kBf16Lowest = 114 << 7, kBf16Count = 19 << 7;
 // what a kernel draws: from P_T, its argmax, or (after a rejection) from the SD residual
 enum : int { kDrawPt = 0, kDrawGreedy = 1, kDrawResidual = 2 };
 
@@ -91,19 +91,25 @@ struct FinishShared {
     unsigned long long bits[kJudgeWords];   // accept bits of the pairs this CTA judged for its cluster
     float u;                   // the row's uniform
     int far;                   // draw from P_T: some thread's reference is out of a double's range; argmax: an invalid logit
-    int amb;                   // residual draw: 1 some thread needs the second pass, 2 some has close calls
+    int amb;                   // residual draw: some thread needs the second pass
+    int n_close;               // how many threads have close calls; two where one has some of two kinds
+    int next;                  // part of the table to be built next
     int cand;                  // find_crossing: highest index with a positive weight
     int last_pos;              // highest index with a positive weight in this CTA
     int row_sel;               // target row the token is drawn from
     int n_acc;
     int bad;
     int best_key;              // depth * 2048 + (2047 - node) of the chosen tree node, or -1
-    int16_t tree_parent[kMaxTreeNodes];
-    int16_t tree_jump[kMaxTreeNodes];
-    int16_t tree_depth[kMaxTreeNodes];
-    int8_t tree_ok[kMaxTreeNodes];
-    int8_t tree_bit[kMaxTreeNodes];
 };
+
+struct TreeShared {
+    int16_t parent[kMaxTreeNodes];
+    int16_t jump[kMaxTreeNodes];
+    int16_t depth[kMaxTreeNodes];
+    int8_t ok[kMaxTreeNodes];
+    int8_t bit[kMaxTreeNodes];
+};
+struct NoTree {};                  // (a residual draw is never a tree's)
 
 // 2^y in double precision (relative error about 2e-16) for -1000 < y < 1000; 0 below, NaN for NaN.
 // y = (k + r) / 256 with integer k and |r| <= 1/2: 2^y = 2^(k >> 8) * table[k & 255] * 2^(r/256),
@@ -228,9 +234,9 @@ __device__ inline PairTotals fold_record(const PairRecord* rec, int div) {
     return t;
 }
 
-// (x, ax, bx: the candidate and its two logits, for the ratio test)
-__device__ inline void judge_record(const FinishParams& P, int item, const PairTotals& r, double lnZa, double lnZb,
-                                    int x, float ax, float bx, float& D_out, int& bit_out, int& st_out) {
+// (x, ax, bx, ua: the candidate, its two logits and its uniform, for the ratio test)
+__device__ inline void judge_record(const FinishParams& P, const PairTotals& r, double lnZa, double lnZb,
+                                    int x, float ax, float bx, float ua, float& D_out, int& bit_out, int& st_out) {
     if (r.state & kRecordBadTree) {
         D_out = __int_as_float(0x7fc00000); bit_out = 0; st_out = FSD_ROW_BADTREE;
         return;
@@ -254,7 +260,7 @@ __device__ inline void judge_record(const FinishParams& P, int item, const PairT
                     pacc = exp(la - lb);
                     pacc = pacc < 1.0 ? pacc : 1.0;
                 }
-                ratio_ok = static_cast<double>(P.u_accept[item]) < pacc;        // Eq. 2
+                ratio_ok = static_cast<double>(ua) < pacc;        // Eq. 2
             }
         }
         bit = P.mode == FSD_MODE_SD ? ratio_ok : (div_ok || ratio_ok);          // Eq. 6
@@ -418,7 +424,7 @@ __device__ __forceinline__ void find_crossing(const FinishParams& P, FinishShare
 
 // Tree: the deepest node whose whole path passes (ties: lowest index), its depth and path.
 // Called by all threads of the CTA; leaves sh.n_acc / sh.row_sel and writes the path if `pth` is given.
-__device__ __noinline__ void tree_select(const int32_t* par, int G, int max_depth, int32_t* pth, FinishShared& sh) {
+__device__ __noinline__ void tree_select(const int32_t* par, int G, int max_depth, int32_t* pth, FinishShared& sh, TreeShared& tr) {
     const int tid = threadIdx.x, lane = tid & 31;
     // Depth of every node and "all nodes from the root down to it pass", by pointer jumping:
     // every node keeps (nodes counted, all pass, next ancestor) for the stretch of its path it
@@ -430,10 +436,10 @@ __device__ __noinline__ void tree_select(const int32_t* par, int G, int max_dept
     if (good) {
         for (int j = tid; j < G; j += kFinishThreads) {
             const int16_t p = static_cast<int16_t>(par[j]);
-            sh.tree_parent[j] = p;
-            sh.tree_jump[j] = p;
-            sh.tree_depth[j] = 1;
-            sh.tree_ok[j] = sh.tree_bit[j];
+            tr.parent[j] = p;
+            tr.jump[j] = p;
+            tr.depth[j] = 1;
+            tr.ok[j] = tr.bit[j];
         }
         __syncthreads();
         for (int span = 1; span < G; span <<= 1) {
@@ -444,9 +450,9 @@ __device__ __noinline__ void tree_select(const int32_t* par, int G, int max_dept
                 const int j = tid + q * kFinishThreads;
                 nj[q] = -1; nd[q] = 0; no[q] = 0;
                 if (j < G) {
-                    const int p = sh.tree_jump[j];
-                    nj[q] = p; nd[q] = sh.tree_depth[j]; no[q] = sh.tree_ok[j];
-                    if (p >= 0) { nj[q] = sh.tree_jump[p]; nd[q] += sh.tree_depth[p]; no[q] &= sh.tree_ok[p]; }
+                    const int p = tr.jump[j];
+                    nj[q] = p; nd[q] = tr.depth[j]; no[q] = tr.ok[j];
+                    if (p >= 0) { nj[q] = tr.jump[p]; nd[q] += tr.depth[p]; no[q] &= tr.ok[p]; }
                     more = more || nj[q] >= 0;
                 }
             }
@@ -455,9 +461,9 @@ __device__ __noinline__ void tree_select(const int32_t* par, int G, int max_dept
             for (int q = 0; q < kPer; ++q) {
                 const int j = tid + q * kFinishThreads;
                 if (j < G) {
-                    sh.tree_jump[j] = static_cast<int16_t>(nj[q]);
-                    sh.tree_depth[j] = static_cast<int16_t>(nd[q]);
-                    sh.tree_ok[j] = static_cast<int8_t>(no[q]);
+                    tr.jump[j] = static_cast<int16_t>(nj[q]);
+                    tr.depth[j] = static_cast<int16_t>(nd[q]);
+                    tr.ok[j] = static_cast<int8_t>(no[q]);
                 }
             }
             if (!any) break;                          // every node has reached the root (what is read below, its reader wrote)
@@ -466,8 +472,8 @@ __device__ __noinline__ void tree_select(const int32_t* par, int G, int max_dept
         // deepest passing node within max_depth, ties to the lowest index
         int key = -1;
         for (int j = tid; j < G; j += kFinishThreads) {
-            const int d = sh.tree_depth[j];
-            if (sh.tree_ok[j] && d <= max_depth) {
+            const int d = tr.depth[j];
+            if (tr.ok[j] && d <= max_depth) {
                 const int k = d * 2048 + (2047 - j);
                 key = k > key ? k : key;
             }
@@ -482,7 +488,7 @@ __device__ __noinline__ void tree_select(const int32_t* par, int G, int max_dept
     if (pth != nullptr) {
         for (int d = best_depth + tid; d < max_depth; d += kFinishThreads) pth[d] = -1;
         if (tid == 0)
-            for (int j = best, d = best_depth - 1; j >= 0 && d >= 0; j = sh.tree_parent[j], --d) pth[d] = j;
+            for (int j = best, d = best_depth - 1; j >= 0 && d >= 0; j = tr.parent[j], --d) pth[d] = j;
     }
 }
 
@@ -686,26 +692,26 @@ __device__ __forceinline__ void draw_argmax(const FinishParams& P, FinishShared&
 
 // ---- the draw from the SD residual -----------------------------------------------------------------
 constexpr int kPairRefs = 32;                         // (a pair beyond these has its record folded again)
-struct PairRef { double za, zb; float ka, kb; };      // normalisers relative to 2^ka, 2^kb; ka NaN: not usable
+struct PairRef { double za, zb, ln_rho; float ka, kb; };      // normalisers relative to 2^ka, 2^kb, log of their ratio; ka NaN: not usable
 struct ResidualShared {
     double exp_table[kExpTable];                      // 2^(j/256)
     double exp_consts[8];                             // the constants of exp2_table (see exp2_consts)
     PairRef ref[kPairRefs];                           // of the pairs this CTA has judged
-    double4 wsum[kFinishWarps];                       // the warps' za, zb, sa, sb
+    double wsum[kFinishWarps][4];                     // the warps' za, zb, sa, sb
+    double cq[2];                                     // the close calls' e_a, e_b where one thread of the CTA has some, of one kind
+    int cq_warp;
 };
 template <int DT> struct ExpTable {};                // (fp32 logits have no table of their own)
-// e^x of the bf16 numbers from 2^-9 to 64, at [sign << 11 | magnitude's bits - kBf16Lowest].  Logits of a row lie
-// close together and mostly share a sign: neighbours fall on different banks.
-constexpr int kBf16Sign = 1 << 11;
-static_assert(kBf16Count <= kBf16Sign, "eleven bits index a sign's entries");
+// e^x of the bf16 numbers from 2^-13 to 64, at [sign * kBf16Count + magnitude's bits - kBf16Lowest].  (From 2^-9 on, every
+// fourth warp of the pass met a smaller logit in a step, and its lane's sixteen entries one by one took as long as all others.)
 template <> struct ExpTable<FSD_BF16> {
-    double e[2 * kBf16Sign];
+    double e[2 * kBf16Count];
 };
 // e^x of a bf16 number, to double precision, whatever it is
 __device__ __noinline__ double exp_bf16(float x, const ExpTable<FSD_BF16>& t) {
     const uint32_t bits = __float_as_uint(x) >> 16, m = (bits & 0x7fffu) - kBf16Lowest;
-    if (m < static_cast<uint32_t>(kBf16Count)) return t.e[(bits >> 15) * kBf16Sign + m];
-    if (static_cast<int>(m) < 0) {                    // |x| < 2^-9: the series' next term is below 2^-51
+    if (m < static_cast<uint32_t>(kBf16Count)) return t.e[(bits >> 15) * kBf16Count + m];
+    if (static_cast<int>(m) < 0) {                    // |x| < 2^-13: the series' next term is below 2^-71
         const double y = x;
         return fma(fma(fma(fma(y, 1.0 / 24, 1.0 / 6), y, 0.5), y, 1.0), y, 1.0);
     }
@@ -724,9 +730,9 @@ __device__ __forceinline__ bool in_table(const uint4& a, const uint4& b) {
 // e^x of both entries of a packed pair there; `table` is its shared-memory address
 __device__ __forceinline__ void table_exp2(uint32_t pair, uint32_t table, double& e0, double& e1) {
     const uint32_t m = pair - kBf16Lowest * 0x10001u;                       // (no borrow between the halves)
-    const uint32_t idx = (m & 0x07ff07ffu) | (m >> 4 & 0x08000800u);        // the sign comes down to bit 11
+    const uint32_t idx = (m & 0x0fff0fffu) + (m >> 15 & 0x00010001u) * kBf16Count;
     asm("ld.shared.f64 %0, [%1];" : "=d"(e0) : "r"(table + (idx & 0xffffu) * 8));
-    asm("ld.shared.f64 %0, [%1];" : "=d"(e1) : "r"(table + (idx >> 13)));
+    asm("ld.shared.f64 %0, [%1];" : "=d"(e1) : "r"(table + (idx >> 16) * 8));
 }
 // What a pass over a thread's entries leaves: normalisers; sums over the entries clearly above the ratio; sums over the
 // first kind of close call (entries whose logits differ by qd); the other close calls.  An entry is above where its
@@ -802,6 +808,16 @@ __device__ __noinline__ void classed_pass_bf16(const void* a_row, const void* b_
     }
     out = c;
 }
+// Four values summed over the warp: lanes 8 q to 8 q + 7 return the q-th sum.
+__device__ __forceinline__ double fold_four(double v0, double v1, double v2, double v3, int lane) {
+    const bool hi = (lane & 16) != 0, up = (lane & 8) != 0;
+    const double k0 = (hi ? v2 : v0) + shfl_xor_d(hi ? v0 : v2, 16);
+    const double k1 = (hi ? v3 : v1) + shfl_xor_d(hi ? v1 : v3, 16);
+    double k = (up ? k1 : k0) + shfl_xor_d(up ? k0 : k1, 8);
+#pragma unroll
+    for (int m = 4; m > 0; m >>= 1) k += shfl_xor_d(k, m);
+    return k;
+}
 constexpr double kResidualMargin = 2e-5;              // the record's ratio is good to a few 1e-6 at worst
 
 template <int DT>
@@ -816,19 +832,20 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
     // ---- references.  The rejected pair's record has references (log2 domain) for both rows, near their maxima and
     //      common to the cluster; without a record one pass for the CTA-local maxima (exact) ----
     double kra = 0.0, krb = 0.0;
-    double zea = 0.0, zeb = 0.0;
+    double zea = 0.0, zeb = 0.0, ln_rho = 0.0;
     bool common = false;
     if (P.records != nullptr) {
         PairRef ref;
-        ref.za = 0.0; ref.zb = 0.0; ref.ka = __int_as_float(0x7fc00000); ref.kb = ref.ka;
+        ref.za = 0.0; ref.zb = 0.0; ref.ln_rho = 0.0; ref.ka = __int_as_float(0x7fc00000); ref.kb = ref.ka;
         if (n < kPairRefs && !d.shared_out) {
             ref = rs.ref[n];
         } else {
             const PairTotals t = fold_record(P.records + (static_cast<size_t>(b) * G + n), P.div);
-            if (t.state & kRecordStats) { ref.za = t.Za; ref.zb = t.Zb; ref.ka = t.ka; ref.kb = t.kb; }
+            if (t.state & kRecordStats) { ref.za = t.Za; ref.zb = t.Zb; ref.ln_rho = log(t.Za) - log(t.Zb); ref.ka = t.ka; ref.kb = t.kb; }
         }
         if (isfinite(ref.ka) && isfinite(ref.kb)) {
             kra = ref.ka; krb = ref.kb; zea = ref.za; zeb = ref.zb;
+            ln_rho = ref.ln_rho + (kra - krb) * kLn2D;
             if constexpr (DT == FSD_BF16) {
                 // plain e^x (no reference) as long as it neither overflows nor leaves the table for good: largest logits of
                 // about -64 to 64 (a record's reference can be 2^30 below its row's largest entry, no more)
@@ -872,27 +889,40 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
     // half the margin, sends the whole row through the second pass instead.
     Classed c = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, __int_as_float(0x7fc00000), 0, -1, -1};
     bool one_pass = false;
-    double Za = 0.0, Zb = 0.0, flags = 1.0;               // flags, cluster-wide: 0 no close calls, 2 some, 1 a second pass is needed
+    double Za = 0.0, Zb = 0.0, flags = 1.0;               // flags, cluster-wide: 0 no CTA has close calls of two threads or kinds, 2 some has, 1 a second pass is needed
     const double (*all)[kExchangeDoubles];
     if (common) {
         // the usual case (a rejected pair with a record): both rows, two independent exponentials an entry
         const bool classify = !greedy && zea > 0.0 && zeb > 0.0 && isfinite(zea) && isfinite(zeb);
-        const double ln_rho = classify ? log(zea / zeb) + (DT == FSD_F32 ? (kra - krb) * kLn2D : 0.0) : 0.0;
         const float hi = static_cast<float>(ln_rho + kResidualMargin), lo = static_cast<float>(ln_rho - kResidualMargin);
         bool done = false;
         if constexpr (DT == FSD_BF16) {
             if (d.vec) { classed_pass_bf16(a_row, b_row, row_share(d.V / 8, cs, rank, warp), hi, lo, bt, c); done = true; }
         }
         if (!done) for_units<DT>(d, warp, lane, true, [&](int k, float xa, float xb) { c.entry(k, xa, xb, exp_a(xa), exp_b(xb), hi, lo); });
-        const int mine_amb = !classify || c.close > 2 ? 1 : (c.qd == c.qd || c.close > 0) ? 2 : 0;
-        if (mine_amb) atomicOr(&sh.amb, mine_amb);
-        const double4 ws = make_double4(warp_sum(c.za), warp_sum(c.zb), warp_sum(c.sa), warp_sum(c.sb));
-        if (lane == 0) rs.wsum[warp] = ws;
+        if (!classify || c.close > 2) {
+            atomicOr(&sh.amb, 1);
+        } else if (c.qd == c.qd) {
+            if (atomicAdd(&sh.n_close, c.close > 0 ? 2 : 1) == 0) { rs.cq[0] = c.qa; rs.cq[1] = c.qb; rs.cq_warp = warp; }
+        }
+        {
+            const double k = fold_four(c.za, c.zb, c.sa, c.sb, lane);
+            if ((lane & 7) == 0) rs.wsum[warp][lane >> 3] = k;
+        }
         __syncthreads();
-        double4 t = make_double4(0.0, 0.0, 0.0, 0.0);
-        if (lane < kFinishWarps) t = rs.wsum[lane];
-        const int amb = sh.amb;
-        const double mine[5] = {warp_sum(t.x), warp_sum(t.y), warp_sum(t.z), warp_sum(t.w), static_cast<double>((amb & 1) ? 1 : amb)};
+        double mine[7] = {};                              // (the first warp sends)
+        if (warp == 0) {
+            static_assert(kFinishWarps == 16, "two warps' sums a lane");
+            double k = rs.wsum[lane & 7][lane >> 3] + rs.wsum[8 + (lane & 7)][lane >> 3];
+#pragma unroll
+            for (int m = 4; m > 0; m >>= 1) k += shfl_xor_d(k, m);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) mine[q] = __shfl_sync(0xffffffffu, k, 8 * q);
+            const bool one = sh.n_close == 1;
+            mine[4] = sh.amb ? 1.0 : sh.n_close > 1 ? 2.0 : 0.0;
+            mine[5] = one ? rs.cq[0] : 0.0;
+            mine[6] = one ? rs.cq[1] : 0.0;
+        }
         all = cluster_exchange(sh, cs, rank, turn, mine);
         Ma = 0.0; Mb = 0.0; flags = 0.0;
         for (int r = 0; r < cs; ++r) { Za += all[r][0]; Zb += all[r][1]; flags = all[r][4] == 1.0 || flags == 1.0 ? 1.0 : fmax(flags, all[r][4]); }
@@ -947,23 +977,27 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
             for (int q = 0; q < EPV; ++q) if (q == e) w[q] = v;
         }
     };
-    // No close call in the whole row: the classed sums, already exchanged, are all there is to know.
+    // No close call in the whole row, or those of one thread a CTA (the usual case): the classed sums, already exchanged,
+    // are all there is to know.
+    const auto residual_of = [&](double sa, double sb, double qa, double qb) { return fmax(sa * iZa - sb * iZb, 0.0) + fmax(qa * iZa - qb * iZb, 0.0); };
     if (one_pass && flags == 0.0 && d.vec) {
         double W = 0.0, cpre = 0.0, run = 0.0;
-        for (int r = 0; r < cs; ++r) W += fmax(all[r][2] * iZa - all[r][3] * iZb, 0.0);
+        for (int r = 0; r < cs; ++r) W += residual_of(all[r][2], all[r][3], all[r][5], all[r][6]);
         const double t = d.u * W;
         int owner = -1;
         for (int r = 0; r < cs && owner < 0; ++r) {
             cpre = run;
-            run += fmax(all[r][2] * iZa - all[r][3] * iZb, 0.0);
+            run += residual_of(all[r][2], all[r][3], all[r][5], all[r][6]);
             if (run > t) owner = r;
         }
         if (owner >= 0) {                                 // (no mass, or lost to rounding at the very end: the general way)
             if (rank == 0 && tid == 0) { P.accept_len[b] = n; P.row_status[b] = status; }
             if (owner != rank) return;
-            const double4 ws = rs.wsum[lane & (kFinishWarps - 1)];
+            asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+            const int w = lane & (kFinishWarps - 1);
+            const bool one = sh.n_close == 1 && rs.cq_warp == w;
             double before;
-            const int cw = Prefix(fmax(ws.z * iZa - ws.w * iZb, 0.0), lane).crossing(t - cpre, before);
+            const int cw = Prefix(residual_of(rs.wsum[w][2], rs.wsum[w][3], one ? rs.cq[0] : 0.0, one ? rs.cq[1] : 0.0), lane).crossing(t - cpre, before);
             find_crossing<EPV>(P, sh, d, row_share(d.V / EPV, cs, rank, cw), t - cpre - before, vector_weights, [&](int u) { return u * EPV; });
             return;
         }
@@ -1122,6 +1156,7 @@ __global__ void __launch_bounds__(kFinishThreads, 2) fsd_finish_kernel(const __g
     __shared__ FinishShared sh;
     __shared__ ResidualShared rs;                        // (used by the residual's instantiation alone)
     __shared__ ExpTable<DT> bt;
+    __shared__ std::conditional_t<KIND == kDrawResidual, NoTree, TreeShared> tr;
     cg::cluster_group cluster = cg::this_cluster();
     const int cs = static_cast<int>(cluster.num_blocks());
     const int rank = static_cast<int>(cluster.block_rank());
@@ -1131,30 +1166,21 @@ __global__ void __launch_bounds__(kFinishThreads, 2) fsd_finish_kernel(const __g
     const size_t rb = static_cast<size_t>(V) * Logit<DT>::kBytes;
     const char* t_base = static_cast<const char*>(P.target) + static_cast<size_t>(b) * (G + 1) * rb;
     const char* d_base = static_cast<const char*>(P.draft) + static_cast<size_t>(b) * G * rb;
-    const bool tree = P.parent != nullptr;
+    const bool tree = KIND != kDrawResidual && P.parent != nullptr;
 
     if (tid == 0) {
         mbar_init(&sh.link[0], 1); mbar_init(&sh.link[1], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");     // "this CTA has started": waited for below
-    if (tid == 0) { sh.cand = -1; sh.last_pos = -1; sh.n_acc = G; sh.bad = 0; sh.row_sel = 0; sh.amb = 0; sh.far = 0; }
+    if (tid == 0) { sh.cand = -1; sh.last_pos = -1; sh.n_acc = G; sh.bad = 0; sh.row_sel = 0; sh.amb = 0; sh.n_close = 0; sh.next = 0; sh.far = 0; }
     if (tid < kJudgeWords) sh.bits[tid] = 0;
     if constexpr (KIND == kDrawResidual) {
-        // the tables: nothing they need is the streaming kernel's, so they are built while it drains
         if (tid < kExpTable) rs.exp_table[tid] = exp2(static_cast<double>(tid) * (1.0 / kExpTable));
         if (tid == 0) {
             rs.exp_consts[0] = 6755399441055744.0; rs.exp_consts[1] = 256.0;
             rs.exp_consts[2] = 2.239395190875157e-12; rs.exp_consts[3] = 3.308302680541371e-09;
             rs.exp_consts[4] = 3.665565596910106e-06; rs.exp_consts[5] = 2.7076061740622863e-03;
-        }
-        if constexpr (DT == FSD_BF16) {
-            __syncthreads();
-            for (int i = tid; i < kBf16Count; i += kFinishThreads) {
-                const double x = __uint_as_float(static_cast<uint32_t>(kBf16Lowest + i) << 16);
-                bt.e[i] = exp2_table(x * kLog2eD, rs.exp_table);
-                bt.e[kBf16Sign + i] = exp2_table(-x * kLog2eD, rs.exp_table);
-            }
         }
     }
     __syncthreads();
@@ -1189,6 +1215,8 @@ __global__ void __launch_bounds__(kFinishThreads, 2) fsd_finish_kernel(const __g
                     bx = load_logit<DT>(d_base + static_cast<size_t>(i) * rb, x);
                 }
             }
+            float ua = 0.f;
+            if constexpr (KIND == kDrawResidual) ua = P.u_accept[item];
             const PairTotals tot = fold_record(P.records + item, P.div);
             // the two logarithms the judgement needs, by two lanes at once
             const double lz = log(lane == 1 ? tot.Zb : tot.Za);
@@ -1196,19 +1224,21 @@ __global__ void __launch_bounds__(kFinishThreads, 2) fsd_finish_kernel(const __g
             if (lane == 0) {
                 float D;
                 int bit, s;
-                judge_record(P, item, tot, lnZa, lnZb, x, ax, bx, D, bit, s);
+                judge_record(P, tot, lnZa, lnZb, x, ax, bx, ua, D, bit, s);
                 if (shared_out || rank == 0) P.divergence[item] = D;
                 if constexpr (KIND == kDrawResidual) {
                     if (i < kPairRefs) {
                         PairRef ref;
-                        ref.za = tot.Za; ref.zb = tot.Zb; ref.ka = (tot.state & kRecordStats) ? tot.ka : __int_as_float(0x7fc00000); ref.kb = tot.kb;
+                        ref.za = tot.Za; ref.zb = tot.Zb; ref.ln_rho = lnZa - lnZb; ref.ka = (tot.state & kRecordStats) ? tot.ka : __int_as_float(0x7fc00000); ref.kb = tot.kb;
                         rs.ref[i] = ref;
                     }
                 }
                 st |= s;
                 if (tree) {
-                    if (!shared_out) sh.tree_bit[i] = static_cast<int8_t>(bit);
-                    else if (bit) atomicOr(&sh.bits[i / cs >> 6], 1ull << (i / cs & 63));
+                    if constexpr (KIND != kDrawResidual) {
+                        if (!shared_out) tr.bit[i] = static_cast<int8_t>(bit);
+                        else if (bit) atomicOr(&sh.bits[i / cs >> 6], 1ull << (i / cs & 63));
+                    }
                 } else if (!bit && i < first) {
                     first = i;
                 }
@@ -1219,8 +1249,22 @@ __global__ void __launch_bounds__(kFinishThreads, 2) fsd_finish_kernel(const __g
             const int item = b * G + i;
             const int bit = P.item_bits[item];
             st |= P.item_status[item];
-            if (tree) sh.tree_bit[i] = static_cast<int8_t>(bit);
-            else if (!bit && i < first) first = i;
+            if constexpr (KIND != kDrawResidual) { if (tree) tr.bit[i] = static_cast<int8_t>(bit); }
+            if (!tree && !bit && i < first) first = i;
+        }
+    }
+    if constexpr (KIND == kDrawResidual && DT == FSD_BF16) {
+        // The table, by whichever warps have no pair to judge (left), a warp's worth at a time: judging is trips to L2 and
+        // chains of double-precision latencies, the table 1.2 us of instruction issue.
+        for (;;) {
+            int part = 0;
+            if (lane == 0) part = atomicAdd(&sh.next, 1);
+            part = __shfl_sync(0xffffffffu, part, 0);
+            if (part >= kBf16Count / 32) break;
+            const int i = part * 32 + lane;
+            const double x = __uint_as_float(static_cast<uint32_t>(kBf16Lowest + i) << 16);
+            bt.e[i] = exp2_table(x * kLog2eD, rs.exp_table);
+            bt.e[kBf16Count + i] = exp2_table(-x * kLog2eD, rs.exp_table);
         }
     }
     if (tid == 0) sh.u = u_mine;
@@ -1233,7 +1277,7 @@ __global__ void __launch_bounds__(kFinishThreads, 2) fsd_finish_kernel(const __g
     __syncthreads();
     if (shared_out) {
         // (the bits travel as what a double's bits are; nothing computes with them)
-        double mine[kExchangeDoubles];
+        double mine[1 + kJudgeWords];
         mine[0] = __longlong_as_double(static_cast<long long>(sh.bad) << 32 | sh.n_acc);
 #pragma unroll
         for (int k = 0; k < kJudgeWords; ++k) mine[1 + k] = __longlong_as_double(static_cast<long long>(sh.bits[k]));
@@ -1244,24 +1288,24 @@ __global__ void __launch_bounds__(kFinishThreads, 2) fsd_finish_kernel(const __g
             bad |= static_cast<int>(w >> 32);
             prefix = min(prefix, static_cast<int>(w & 0xffffffff));
         }
-        if (tree)
-            for (int i = tid; i < G; i += kFinishThreads)
-                sh.tree_bit[i] = static_cast<int8_t>(__double_as_longlong(all[i % cs][1 + (i / cs >> 6)]) >> (i / cs & 63) & 1);
+        if constexpr (KIND != kDrawResidual)
+            for (int i = tree ? tid : G; i < G; i += kFinishThreads)
+                tr.bit[i] = static_cast<int8_t>(__double_as_longlong(all[i % cs][1 + (i / cs >> 6)]) >> (i / cs & 63) & 1);
         __syncthreads();
         if (tid == 0) { sh.bad = bad; sh.n_acc = prefix; }
         __syncthreads();
     }
 
     // ---- 2. accepted prefix (chain) or deepest accepted path (tree) ----
-    int n, row_sel;
-    if (tree) {
-        tree_select(P.parent + static_cast<size_t>(b) * G, G, P.max_depth,
-                    rank == 0 ? P.path + static_cast<size_t>(b) * P.max_depth : nullptr, sh);
-        __syncthreads();
-        n = sh.n_acc; row_sel = sh.row_sel;
-        FSD_CHECK(P.debug_word, row_sel >= 0 && row_sel <= G && n >= 0 && n <= P.max_depth, kChkPath);
-    } else {
-        n = sh.n_acc; row_sel = n;
+    int n = sh.n_acc, row_sel = n;
+    if constexpr (KIND != kDrawResidual) {
+        if (tree) {
+            tree_select(P.parent + static_cast<size_t>(b) * G, G, P.max_depth,
+                        rank == 0 ? P.path + static_cast<size_t>(b) * P.max_depth : nullptr, sh, tr);
+            __syncthreads();
+            n = sh.n_acc; row_sel = sh.row_sel;
+            FSD_CHECK(P.debug_word, row_sel >= 0 && row_sel <= G && n >= 0 && n <= P.max_depth, kChkPath);
+        }
     }
     FSD_CHECK(P.debug_word, row_sel >= 0 && row_sel <= G && n >= 0 && n <= (tree ? P.max_depth : G), kChkRow);
     const int status = sh.bad;

@@ -818,7 +818,12 @@ __device__ __forceinline__ double fold_four(double v0, double v1, double v2, dou
     for (int m = 4; m > 0; m >>= 1) k += shfl_xor_d(k, m);
     return k;
 }
-constexpr double kResidualMargin = 2e-5;              // the record's ratio is good to a few 1e-6 at worst
+// How far from ln rho_est an entry's difference has to be to be classed in the pass.  The record's ratio is good to about
+// 2e-7 (measured), and the difference and the bounds, numbers of about ln rho, are rounded to single precision (6e-8 of
+// them each): half the margin covers the one (checked afterwards), half the other.  With 2e-5 throughout, four rows in ten
+// of 32000 fp32 entries, and nearly all of 152064, had close calls (16 x 6 x 64000 fp32 36.5 us, now 35.1).
+__device__ __forceinline__ float residual_margin(double ln_rho) { return fabs(ln_rho) < 8.0 ? 2e-6f : 2e-5f; }
+constexpr double kMostLnRho = 80.0;
 
 template <int DT>
 __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShared& sh, ResidualShared& rs, const ExpTable<DT>& bt,
@@ -889,12 +894,14 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
     // half the margin, sends the whole row through the second pass instead.
     Classed c = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, __int_as_float(0x7fc00000), 0, -1, -1};
     bool one_pass = false;
+    float margin = 0.f;
     double Za = 0.0, Zb = 0.0, flags = 1.0;               // flags, cluster-wide: 0 no CTA has close calls of two threads or kinds, 2 some has, 1 a second pass is needed
     const double (*all)[kExchangeDoubles];
     if (common) {
         // the usual case (a rejected pair with a record): both rows, two independent exponentials an entry
-        const bool classify = !greedy && zea > 0.0 && zeb > 0.0 && isfinite(zea) && isfinite(zeb);
-        const float hi = static_cast<float>(ln_rho + kResidualMargin), lo = static_cast<float>(ln_rho - kResidualMargin);
+        const bool classify = !greedy && zea > 0.0 && zeb > 0.0 && isfinite(zea) && isfinite(zeb) && fabs(ln_rho) < kMostLnRho;
+        margin = residual_margin(ln_rho);
+        const float hi = static_cast<float>(ln_rho + margin), lo = static_cast<float>(ln_rho - margin);
         bool done = false;
         if constexpr (DT == FSD_BF16) {
             if (d.vec) { classed_pass_bf16(a_row, b_row, row_share(d.V / 8, cs, rank, warp), hi, lo, bt, c); done = true; }
@@ -950,7 +957,7 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
         }
         if (!b_ok) { residual = false; status |= FSD_ROW_NONFINITE; }
         else { iZa = 1.0 / Za; iZb = 1.0 / Zb; }
-        one_pass = b_ok && flags != 1.0 && fabs(zea * Zb - zeb * Za) <= 0.5 * kResidualMargin * zeb * Za;
+        one_pass = b_ok && flags != 1.0 && fabs(zea * Zb - zeb * Za) <= 0.5 * margin * zeb * Za;
     }
 
     // the residual weights of a unit of vectors (the usual case)

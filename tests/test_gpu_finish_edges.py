@@ -1,5 +1,5 @@
 """The finish kernel where its forms part ways, against the oracle: residual draws between rows whose
-normalisers are equal (every entry on which they agree is a close call), logits outside the table of
+normalisers are equal (every entry on which they agree is a close call) or far apart, logits outside the table of
 exponentials (tiny, beyond 64, of one sign, -inf), references out of a double's range, rows off a
 16-byte boundary, and trees and chains whose judging the cluster's thread blocks share."""
 
@@ -43,6 +43,26 @@ def test_residual_between_rows_with_the_same_normaliser(dtype, V):
     r = _check(c, mode="sd")
     assert (r["accept_len"] < 2).any()
     _check(c, mode="sd", sample="greedy")
+    _check(c, mode="rfsd", T=0.0)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("offset", [0.0, -0.001, 7.75, -8.25, 60.0, -79.5, 81.0])
+def test_residual_between_rows_whose_normalisers_are_far_apart(dtype, offset):
+    """The log of the normalisers' ratio decides how close to it an entry may be classed at once; a few
+    entries lie right at it, whichever side, and one of them alone in its block's share."""
+    c = gi.make_chain(6, 2, 32000, dtype=dtype, recipe="zipf", sigma=(0.4, 1.2), sigma_mode="uniform", workload_id=902)
+    t, d = _wide(c)
+    d += offset
+    lse = lambda x: np.log(np.exp(x - x.max(axis=2, keepdims=True).astype(np.float64)).sum(axis=2)) + x.max(axis=2)
+    rho = (lse(t[:, :2]) - lse(d)).astype(np.float32)               # an entry at t - rho in the draft is as likely in both rows
+    for k in (17, 9000, 9001, 25000):
+        d[:, :, k] = t[:, :2, k] - rho
+    _store(c, t, d)
+    c.draft_tokens[:] = (d - t[:, :2]).argmax(axis=2)               # proposed where q is far above p: rejected
+    c.u_accept[:] = 0.999
+    r = _check(c, mode="sd")
+    assert (r["accept_len"] < 2).any()
     _check(c, mode="rfsd", T=0.0)
 
 

@@ -42,7 +42,7 @@ import fsd_inputs as gi  # noqa: E402
 NOMINAL_HBM_GBS = 8000.0
 # DRAM bytes (read + written) of one pair-kernel launch on the headline workload, from the ncu
 # capture summarised under profiles/; None whenever that kernel has changed since the capture.
-PAIR_KERNEL_DRAM_BYTES = None
+PAIR_KERNEL_DRAM_BYTES = 316_160_000
 FALLBACK_HBM_GBS = 6650.0
 L2_BYTES = 126 * 1024 * 1024
 D_BAND = 1e-5          # |D_oracle - T| below this: the fp32 and fp64 decisions may differ

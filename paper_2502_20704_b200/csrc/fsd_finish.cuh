@@ -184,7 +184,7 @@ __device__ __forceinline__ const double (*cluster_exchange(FinishShared& sh, int
 }
 
 // Divergence, accept bit and status of one pair from the streaming kernel's totals.
-// A pair's totals from the parts its record holds (one per virtual CTA of the streaming group), in
+// A pair's totals from the parts its record holds (one per block of the streaming group), in
 // double: Z = sum 2^y, S = sum 2^y * y, K = sum 2^ya (ya - yb), all relative to the largest
 // part reference (the parts' references are integers, so the factors are exact powers of two).
 struct PairTotals {

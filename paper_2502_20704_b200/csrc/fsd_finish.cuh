@@ -762,7 +762,6 @@ __device__ __noinline__ void classed_pass_bf16(const void* a_row, const void* b_
                                                const ExpTable<FSD_BF16>& bt, Classed& out) {
     const uint32_t table = smem_u32(bt.e);
     const int u0 = share.first + (threadIdx.x & 31), u1 = min(share.first + share.iters * 32, share.units);
-    const float mid = 0.5f * (hi + lo), half = 0.51f * (hi - lo);     // (a rounded test that misses no close call)
     Classed c = out;
     uint4 na = make_uint4(0, 0, 0, 0), nb = na;       // the vectors after these, on their way
     if (u0 < u1) { na = ldg_vec(a_row, u0); nb = ldg_vec(b_row, u0); }
@@ -794,7 +793,7 @@ __device__ __noinline__ void classed_pass_bf16(const void* a_row, const void* b_
                 c.zb += pb[e];
                 c.sa = fma(pa[e], one, c.sa);
                 c.sb = fma(pb[e], one, c.sb);
-                close = close || fabsf(d[e] - mid) <= half;
+                close = close || (d[e] >= lo && !(d[e] > hi));         // (as in Classed::entry: between the bounds, both included)
             }
         }
         if (close) {

@@ -66,6 +66,42 @@ def test_residual_between_rows_whose_normalisers_are_far_apart(dtype, offset):
     _check(c, mode="rfsd", T=0.0)
 
 
+def test_residual_entries_that_lie_on_the_bound_of_a_close_call():
+    """Nearly all of both rows differs by exactly 45, and ln(Z_a / Z_b) is 45 - 2.1e-5, so that the upper bound of the
+    close calls (the log plus 2e-5, rounded to single precision) is 45 itself: those entries are not above it, and
+    they carry half of the residual.  The other half is one entry's at the row's end, which a draw that loses
+    the first half takes every time."""
+    B, V = 16, 8200
+    c = gi.make_chain(B, 1, V, dtype="bf16", recipe="spike", sigma=(0.5,), workload_id=905)
+    t, d = _wide(c)
+    rng = np.random.default_rng(7)
+    x = -24.0 + rng.integers(0, 64, size=8000) / 8.0                # bf16 steps of 1/8 here and at x + 45
+    zx, off = np.exp(x).sum(), 2.1e-5                               # hi == 45 for 45 - ln rho from 2.01e-5 to 2.19e-5
+    y = np.round(8.0 * np.log(zx * off / (np.e - 1.0))) / 8.0       # one entry, 46 apart: about as much residual again
+    rest, extra = zx * off + np.exp(y) * (np.e - 1.0), []           # what only the draft has, from bf16 numbers
+    while len(extra) < 100:
+        v = gi.bf16_bits_to_f32(gi.f32_to_bf16_bits(np.array([np.log(rest)], np.float32)))[0]
+        v = v if np.exp(np.float64(v)) < rest else np.float32(v - 0.125)
+        extra.append(v)
+        rest -= np.exp(np.float64(v))
+        if rest < 1e-8 * zx:
+            break
+    t[:], d[:] = -np.inf, -np.inf
+    d[:, 0, :8000], t[:, 0, :8000] = x, x + 45.0
+    d[:, 0, 8191], t[:, 0, 8191] = y, y + 46.0
+    d[:, 0, 8000:8000 + len(extra)] = extra
+    t[:, 1] = 0.0
+    _store(c, t, d)
+    ln_rho = np.log(np.exp(t[0, 0].astype(np.float64)).sum()) - np.log(np.exp(d[0, 0].astype(np.float64)).sum())
+    assert 2.02e-5 < 45.0 - ln_rho < 2.18e-5
+    c.draft_tokens[:] = 8000                                        # nothing of the target's: rejected
+    c.u_sample[:] = (np.arange(B) + 0.5) / B
+    r = _check(c, mode="sd")
+    assert (r["accept_len"] == 0).all()
+    tok = r["gpu"].next_token
+    assert (tok < 8000).any() and (tok == 8191).any()
+
+
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 @pytest.mark.parametrize("V", [4096, 20008, 20011])
 @pytest.mark.parametrize("kind", ["tiny", "large", "below", "masked", "steep"])

@@ -216,8 +216,9 @@ int fsd_set_stage_event(void *event);
 /* Test aid (no counterpart in the paper).  Every wait inside the streaming kernel is bounded; a
  * wait that runs out raises a flag in the workspace, the thread blocks that see it take no
  * further work, the call still returns, and every row's row_status carries FSD_ROW_TIMEOUT (its
- * other outputs are then not valid).  mode 1: verify calls raise that flag themselves (an 8-byte
- * copy between the two kernels), which exercises the reporting path alone.  mode 2: in the
+ * other outputs are then not valid).  The flag is that call's own, and of a call in a graph that
+ * replay's.  mode 1: the streaming kernel's first block raises that flag as it ends, which
+ * exercises the reporting path alone.  mode 2: in the
  * streaming kernel one thread block keeps its first statistics message to itself and the limit
  * of the exchange wait is lowered to about a tenth of a second, so its partners' wait really
  * runs out and the kernel's own give-up path runs (every wait stays bounded; nothing faults).

@@ -27,7 +27,7 @@ inline bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_
 struct Workspace {
     int32_t* item_bits;
     int32_t* item_status;
-    int* flags;                // [0..1]: the nonce of a call of which a bounded device-side wait ran out; [2]: debug word
+    CallFlags* flags;
     GroupMsg* exchange;        // the streaming kernel's statistics exchange
     PairRecord* records;       // per-pair totals of the streaming kernel
     size_t bytes;
@@ -41,7 +41,7 @@ Workspace carve(void* base, int B, int G) {
     p += align_up(items * sizeof(int32_t));
     w.item_status = reinterpret_cast<int32_t*>(p);
     p += align_up(items * sizeof(int32_t));
-    w.flags = reinterpret_cast<int*>(p);
+    w.flags = reinterpret_cast<CallFlags*>(p);
     p += kAlign;
     w.exchange = reinterpret_cast<GroupMsg*>(p);
     p += kExchangeBytes;
@@ -84,9 +84,8 @@ std::atomic<void*> g_stage_event{nullptr};   // see fsd_set_stage_event
 std::atomic<int> g_mark_timeout{0};          // see fsd_set_timeout_injection
 std::atomic<int> g_group_size{0};            // see fsd_set_group_size
 
-// A number no other call carries: what the streaming kernel's messages and its timeout flag are marked with, so
-// that whatever a workspace held before is not taken for this call's.  The counter's values are spread over 64 bits
-// by an invertible mixing (the finalizer of splitmix64), from a start that differs from process to process.
+// A number no other launch is given, of which a call's number is made (see CallFlags).  The counter's values are spread
+// over 64 bits by an invertible mixing (the finalizer of splitmix64), from a start that differs from process to process.
 uint64_t next_nonce() {
     static std::atomic<uint64_t> counter{(static_cast<uint64_t>(std::random_device{}()) << 32) ^ std::random_device{}()};
     uint64_t x = counter.fetch_add(0x9e3779b97f4a7c15ull);
@@ -180,7 +179,7 @@ int group_size(int nvec_row, int items, int nsm) {
 }
 
 template <int DT>
-int launch_all(const PairParams& pp, FinishParams fp, bool vec, int* flags, GroupMsg* exchange, PairRecord* records, cudaStream_t s) {
+int launch_all(PairParams pp, FinishParams fp, bool vec, CallFlags* flags, GroupMsg* exchange, PairRecord* records, cudaStream_t s) {
     const int items = pp.B * pp.G;
     int dev = 0, nsm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -191,15 +190,15 @@ int launch_all(const PairParams& pp, FinishParams fp, bool vec, int* flags, Grou
     const size_t nvec_row = vec ? row_bytes / 16 : (row_bytes + 16 - Logit<DT>::kBytes + 15) / 16;
     const int C = nvec_row <= static_cast<size_t>(kMaxGroupSize) * StreamShape<DT>::kBlockVecs ? group_size<DT>(static_cast<int>(nvec_row), items, nsm) : 0;
 #ifdef FSD_DEBUG_CHECKS
-    if (cudaMemsetAsync(flags, 0, kAlign, s) != cudaSuccess) return FSD_ERR_CUDA;   // the debug word starts at zero
+    if (cudaMemsetAsync(&flags->debug, 0, sizeof(int), s) != cudaSuccess) return FSD_ERR_CUDA;   // the debug word starts at zero
 #endif
-    fp.nonce = 0; fp.exchange = nullptr; fp.exchange_units = 0;
+    pp.nonce = next_nonce(); pp.flags = flags;
+    fp.flags = flags;
     if (C > 0) {
         StreamParams sp;
         sp.target = pp.target; sp.draft = pp.draft; sp.parent = pp.parent; sp.G = pp.G;
         sp.nvec_row = static_cast<int>(nvec_row); sp.row_bytes = row_bytes; sp.n_items = items; sp.records = records;
-        const uint64_t nonce = next_nonce();
-        sp.nonce = nonce; sp.timeout_flag = reinterpret_cast<uint64_t*>(flags); sp.debug_word = flags + 2;
+        sp.nonce = pp.nonce; sp.flags = flags;
         sp.C = C; sp.exchange = exchange;
         const int slice = static_cast<int>((nvec_row + C - 1) / C);
         sp.slot_row_bytes = slot_row_bytes<DT>(slice); sp.slot_bytes = slot_bytes<DT>(slice, !vec);
@@ -217,26 +216,18 @@ int launch_all(const PairParams& pp, FinishParams fp, bool vec, int* flags, Grou
         sp.poll_limit = silent ? (1u << 17) : kSpinLimit;
         sp.help_after = injection == 2 ? 0xffffffffu : 1024;     // about a millisecond of fetches
         sp.silent_rank = silent ? C - 1 : -1;
+        sp.raise = injection == 1;                    // behave as if a bounded wait had run out
         // everything that can fail without a launch (attributes, the occupancy query) comes before
         // the first thing put on the stream
         int rc = stream_prepare<DT>(pp.div, !vec)(dev);
         if (rc != FSD_OK) return rc;
         rc = stream_launch<DT>(pp.div, !vec)(sp, nsm, s);
         if (rc != FSD_OK) return rc;
-        // test aid: behave as if a bounded wait of the streaming kernel had run out
-        if (g_mark_timeout.load() == 1 && cudaMemcpyAsync(flags, &nonce, sizeof(nonce), cudaMemcpyHostToDevice, s) != cudaSuccess) return FSD_ERR_CUDA;
-        fp.nonce = nonce;
-        fp.timeout_flag = reinterpret_cast<const uint64_t*>(flags);
-        if (pp.div != FSD_DIV_KL) {                  // (KL exchanges nothing)
-            fp.exchange = reinterpret_cast<uint4*>(exchange);
-            fp.exchange_units = static_cast<int>(2 * sizeof(GroupMsg) / sizeof(uint4)) * (nsm < kMaxBlocks ? nsm : kMaxBlocks);
-        }
         fp.records = records;
     } else {
         if (vec) fsd_pair_generic_kernel<DT, true><<<items, 512, 0, s>>>(pp);
         else     fsd_pair_generic_kernel<DT, false><<<items, 512, 0, s>>>(pp);
         if (cudaGetLastError() != cudaSuccess) return FSD_ERR_CUDA;
-        fp.timeout_flag = nullptr;
         fp.records = nullptr;
     }
 
@@ -285,7 +276,6 @@ int verify_common(const void* target, const void* draft, const int32_t* tokens, 
     pp.B = B; pp.G = G; pp.V = V;
     pp.div = o->divergence; pp.mode = o->mode; pp.cmp = o->compare; pp.T = o->threshold;
     pp.divergence = divergence; pp.item_bits = ws.item_bits; pp.item_status = ws.item_status;
-    pp.debug_word = ws.flags + 2;
 
     FinishParams fp;
     fp.target = target; fp.draft = draft; fp.parent = parent; fp.u_sample = u_sample;
@@ -293,9 +283,8 @@ int verify_common(const void* target, const void* draft, const int32_t* tokens, 
     fp.tokens = tokens; fp.u_accept = u_accept;
     fp.div = o->divergence; fp.mode = o->mode; fp.cmp = o->compare; fp.sample = o->sample; fp.max_depth = max_depth;
     fp.T = o->threshold; fp.records = nullptr; fp.divergence = divergence;
-    fp.item_bits = ws.item_bits; fp.item_status = ws.item_status; fp.timeout_flag = nullptr;
+    fp.item_bits = ws.item_bits; fp.item_status = ws.item_status;
     fp.accept_len = accept_len; fp.path = path; fp.next_token = next_token; fp.row_status = row_status;
-    fp.debug_word = ws.flags + 2;
 
     const bool vec = (static_cast<size_t>(V) * es) % 16 == 0 && aligned(target, 16) && aligned(draft, 16);
     fp.vec = vec ? 1 : 0;
@@ -553,7 +542,7 @@ int fsd_set_stage_event(void* event) {
 int fsd_debug_checks(int B, int positions, size_t* word_offset) {
     if (word_offset != nullptr && B >= 1 && positions >= 1) {
         const Workspace w = carve(nullptr, B, positions);
-        *word_offset = static_cast<size_t>(reinterpret_cast<char*>(w.flags + 2) - static_cast<char*>(nullptr));
+        *word_offset = static_cast<size_t>(reinterpret_cast<char*>(&w.flags->debug) - static_cast<char*>(nullptr));
     }
 #ifdef FSD_DEBUG_CHECKS
     return 1;

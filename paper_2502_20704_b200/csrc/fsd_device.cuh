@@ -11,9 +11,9 @@
 // Index and range checks of the debug build (-DFSD_DEBUG_CHECKS, see build.py): a failed check
 // sets a bit in the workspace's debug word and the access goes ahead as in the release build --
 // the checks are there to show that it never happens, on inputs of every shape the tests run.
-// `word` is the third int of the workspace's flag block; null disables the check.
+// `word` points to the debug word of the workspace's block of flags.
 #ifdef FSD_DEBUG_CHECKS
-#define FSD_CHECK(word, cond, code) do { if ((word) != nullptr && !(cond)) atomicOr((word), (code)); } while (0)
+#define FSD_CHECK(word, cond, code) do { if (!(cond)) atomicOr((word), (code)); } while (0)
 #else
 #define FSD_CHECK(word, cond, code) do { } while (0)
 #endif
@@ -25,6 +25,26 @@ namespace cg = cooperative_groups;
 // bits of the debug word
 constexpr int kChkItem = 1, kChkSlice = 2, kChkStage = 4, kChkTmem = 8, kChkRecord = 16, kChkRow = 32, kChkChunk = 64,
               kChkToken = 128, kChkPath = 256;
+
+// The workspace's block of flags.  A verify call is known by a number of its own: what its messages between thread
+// blocks and its timeout flag carry, so that nothing the workspace held before is taken for this call's and
+// nothing has to be cleared in front of a call.  The number is the nonce the host gives the launch plus a multiple of
+// the epoch, a count of the calls on this workspace (from whatever it held), which the finish kernel moves
+// on: the replays of a captured call all carry one nonce.
+struct CallFlags {
+    uint64_t raised;           // the number of a call of which a bounded device-side wait ran out
+    int debug;                 // debug build: what range checks have failed
+    int pad;
+    uint64_t epoch;
+    uint64_t number;           // of the latest call, left by its pair kernel for its finish kernel
+};
+static_assert(sizeof(CallFlags) <= 256, "the block of flags in a workspace");
+__device__ __forceinline__ uint64_t call_number(const CallFlags* flags, uint64_t nonce) {
+    return nonce + *reinterpret_cast<const volatile uint64_t*>(&flags->epoch) * 0x9e3779b97f4a7c15ull;    // (odd, both halves move each time)
+}
+__device__ __forceinline__ bool timed_out(const CallFlags* flags, uint64_t number) {
+    return *reinterpret_cast<const volatile uint64_t*>(&flags->raised) == number;
+}
 
 constexpr float  kLog2e  = 1.4426950408889634f;
 constexpr double kLog2eD = 1.4426950408889634074;

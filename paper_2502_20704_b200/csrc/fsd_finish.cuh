@@ -57,16 +57,12 @@ struct FinishParams {
     const PairRecord* records; // per-pair totals of the streaming kernel, or null (generic kernel ran)
     int32_t* item_bits;        // [B, G] read when records == null
     int32_t* item_status;      // [B, G] read when records == null
-    uint64_t nonce;            // of the call (see StreamParams)
-    const uint64_t* timeout_flag;   // holds the nonce: a bounded wait of the streaming kernel ran out (may be null)
-    uint4* exchange;           // the streaming kernel's messages, cleared here: a replay of the call carries the same nonce
-    int exchange_units;
+    CallFlags* flags;
     float* divergence;         // [B, G] written here when records != null
     int32_t* accept_len;       // [B]
     int32_t* path;             // [B, max_depth] (tree) or null
     int32_t* next_token;       // [B]
     int32_t* row_status;       // [B]
-    int* debug_word;           // debug build: where failed range checks are recorded (may be null)
 };
 
 constexpr int kExchangeDoubles = 7;      // most values a CTA tells its cluster at once
@@ -408,7 +404,7 @@ __device__ __forceinline__ void find_crossing(const FinishParams& P, FinishShare
                     if (tok < 0 && w[j] > 0.0 && run > target) tok = first_entry(u) + j;
                 }
                 if (tok < 0) tok = ulast;             // lost to the order of the additions
-                FSD_CHECK(P.debug_word, tok >= 0 && tok < d.V, kChkToken);
+                FSD_CHECK(&P.flags->debug, tok >= 0 && tok < d.V, kChkToken);
                 P.next_token[d.b] = tok;
             }
             return;
@@ -518,7 +514,7 @@ __device__ __forceinline__ void draw_pt(const FinishParams& P, FinishShared& sh,
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const Granules<DT> gr(d.a_row, d.V);
     const Share mine = row_share(gr.count, d.cs, d.rank, warp);
-    FSD_CHECK(P.debug_word, mine.first >= 0 && mine.first <= gr.count && static_cast<long long>(mine.iters) * kFinishThreads * d.cs >= gr.count, kChkChunk);
+    FSD_CHECK(&P.flags->debug, mine.first >= 0 && mine.first <= gr.count && static_cast<long long>(mine.iters) * kFinishThreads * d.cs >= gr.count, kChkChunk);
     // ---- one pass: this thread's weights 2^(logit * log2e - kr) in double, kr the largest logit's exponent so far;
     //      four vectors are asked for before the first is used ----
     constexpr int BV = 4;
@@ -1197,15 +1193,14 @@ __global__ void __launch_bounds__(kFinishThreads, 2) fsd_finish_kernel(const __g
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");       // every CTA of the cluster runs: its shared memory may be written
     int turn = 0;                                                              // exchanges so far
-    for (int i = static_cast<int>(blockIdx.x) * kFinishThreads + tid; i < P.exchange_units; i += static_cast<int>(gridDim.x) * kFinishThreads)
-        P.exchange[i] = make_uint4(0, 0, 0, 0);
+    if (blockIdx.x == 0 && tid == 0) atomicAdd(reinterpret_cast<unsigned long long*>(&P.flags->epoch), 1ull);     // (nothing here reads it)
 
     // ---- 1. divergences, accept bits, status of this row's pairs ----
     // (asked for now, needed later: each is a trip to L2 or HBM of its own)
     float u_mine = 0.f;                               // (one load: the array may be in host memory)
     if (tid == 0) u_mine = P.u_sample[b];
     int st = 0, first = G;
-    if (tid == 0 && P.timeout_flag != nullptr && *reinterpret_cast<const volatile uint64_t*>(P.timeout_flag) == P.nonce) st |= FSD_ROW_TIMEOUT;
+    if (tid == 0 && timed_out(P.flags, *reinterpret_cast<const volatile uint64_t*>(&P.flags->number))) st |= FSD_ROW_TIMEOUT;
     const bool shared_out = P.records != nullptr && cs > 1 && G > kFinishWarps && G <= 64 * kJudgeWords * cs;
     if (P.records != nullptr) {
         // a pair per warp: its lanes fold the parts of the pair's record, the first of them judges it
@@ -1310,10 +1305,10 @@ __global__ void __launch_bounds__(kFinishThreads, 2) fsd_finish_kernel(const __g
                         rank == 0 ? P.path + static_cast<size_t>(b) * P.max_depth : nullptr, sh, tr);
             __syncthreads();
             n = sh.n_acc; row_sel = sh.row_sel;
-            FSD_CHECK(P.debug_word, row_sel >= 0 && row_sel <= G && n >= 0 && n <= P.max_depth, kChkPath);
+            FSD_CHECK(&P.flags->debug, row_sel >= 0 && row_sel <= G && n >= 0 && n <= P.max_depth, kChkPath);
         }
     }
-    FSD_CHECK(P.debug_word, row_sel >= 0 && row_sel <= G && n >= 0 && n <= (tree ? P.max_depth : G), kChkRow);
+    FSD_CHECK(&P.flags->debug, row_sel >= 0 && row_sel <= G && n >= 0 && n <= (tree ? P.max_depth : G), kChkRow);
     const int status = sh.bad;
     if (status & FSD_ROW_BADTREE) {                      // uniform over the cluster
         if (rank == 0 && tid == 0) { P.accept_len[b] = 0; P.next_token[b] = -1; P.row_status[b] = status; }

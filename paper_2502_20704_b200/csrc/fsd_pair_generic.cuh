@@ -22,7 +22,8 @@ struct PairParams {
     float* divergence;         // [B, G]
     int32_t* item_bits;        // [B, G] accept bit per pair
     int32_t* item_status;      // [B, G] FSD_ROW_* flags per pair
-    int* debug_word;           // debug build: where failed range checks are recorded (may be null)
+    uint64_t nonce;            // what the call's number is made of (see CallFlags)
+    CallFlags* flags;
 };
 
 // Final scalar work for one pair, done by one thread in double precision.
@@ -191,8 +192,9 @@ __global__ void __launch_bounds__(512) fsd_pair_generic_kernel(PairParams P) {
     __shared__ float red_f[32 * 2];
 
     const int item = blockIdx.x;
+    if (item == 0 && threadIdx.x == 0) P.flags->number = call_number(P.flags, P.nonce);
     const int b = item / P.G, i = item - b * P.G;
-    FSD_CHECK(P.debug_word, b < P.B, kChkItem);
+    FSD_CHECK(&P.flags->debug, b < P.B, kChkItem);
     int trow = i;
     if (P.parent != nullptr) {
         const int par = P.parent[item];

@@ -90,11 +90,11 @@ static_assert(sizeof(PairRecord) == 880, "PairRecord layout");
 constexpr uint32_t kRecordStats = 1, kRecordBadTree = 2;
 
 // One block's statistics of a round as they cross global memory: 16-byte units, each stored whole
-// and ending in 64 bits of call and round, so that a reader knows a unit is this round's without any fence
+// and ending in 64 bits of call and round (see CallFlags), so that a reader knows a unit is this round's without any fence
 // or flag (a unit of another round or call, or what the workspace held before, is fetched again).  That is why
 // nothing has to be cleared in front of a call, which took a memset of 1.5 us in a call of 16.
 struct alignas(16) GroupMsg {
-    uint4 u[2];                // target row: {reference, Z, nonce's high half, nonce's low half + round}; draft row: the same
+    uint4 u[2];                // target row: {reference, Z, call number's high half, its low half + round}; draft row: the same
 };
 static_assert(sizeof(GroupMsg) == 32, "GroupMsg layout");
 
@@ -109,14 +109,14 @@ struct StreamParams {
     int slot_row_bytes, slot_bytes, ring;    // of the shared-memory ring (see slot_bytes())
     int n_items;               // B * G
     PairRecord* records;       // [B * G]
-    uint64_t nonce;            // the call's own number: what its messages and its flag carry
-    uint64_t* timeout_flag;    // set to the nonce if a bounded wait ran out (anything else: not raised)
-    int* debug_word;           // debug build: where failed range checks are recorded
+    uint64_t nonce;            // what the call's number is made of (see CallFlags)
+    CallFlags* flags;
     int C;                     // blocks per group (<= kMaxGroupSize)
     uint32_t poll_limit;       // fetches of the group's messages before the exchange gives up (kSpinLimit normally)
     uint32_t help_after;       // fetches after which a block computes what it waits for by itself (0xffffffff: never)
     int silent_rank;           // test aid: this rank of group 0 keeps its first message to itself (-1: nobody)
-    GroupMsg* exchange;        // [groups][2][C]; holds no unit of this call at launch (the finish kernel clears it behind a call)
+    int raise;                 // test aid: the first block raises the timeout flag as it ends
+    GroupMsg* exchange;        // [groups][2][C]
 };
 
 // ---- PTX wrappers -----------------------------------------------------------------
@@ -150,14 +150,15 @@ __device__ __forceinline__ uint64_t global_ns() {
     asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
     return t;
 }
-__device__ __forceinline__ void raise_flag(uint64_t* flag, uint64_t nonce) {
-    atomicExch(reinterpret_cast<unsigned long long*>(flag), static_cast<unsigned long long>(nonce));
+__device__ __forceinline__ void raise_flag(CallFlags* flags, uint64_t number) {
+    atomicExch(reinterpret_cast<unsigned long long*>(&flags->raised), static_cast<unsigned long long>(number));
 }
 // Bounded wait of a whole warp for a phase of an mbarrier: kSpinLimit polls or kWaitNs, whatever is
 // first.  False (for every lane) and the flag raised if the phase never completes or somebody else's
 // wait has run out already.
-__device__ __noinline__ bool warp_wait_slow(uint64_t* bar, uint32_t parity, uint64_t* timeout_flag, uint64_t nonce) {
+__device__ __noinline__ bool warp_wait_slow(uint64_t* bar, uint32_t parity, CallFlags* flags, uint64_t nonce) {
     uint64_t t0 = 0;
+    const uint64_t number = call_number(flags, nonce);
 #pragma unroll 1
     for (uint32_t i = 0; i < kSpinLimit / 64; ++i) {
 #pragma unroll 1
@@ -168,14 +169,14 @@ __device__ __noinline__ bool warp_wait_slow(uint64_t* bar, uint32_t parity, uint
         // somebody has given up already: nothing this warp waits for is certain to come
         const uint64_t t = global_ns();
         if (t0 == 0) t0 = t;
-        if (__any_sync(0xffffffffu, *reinterpret_cast<volatile uint64_t*>(timeout_flag) == nonce || t - t0 > kWaitNs)) break;
+        if (__any_sync(0xffffffffu, timed_out(flags, number) || t - t0 > kWaitNs)) break;
     }
-    if ((threadIdx.x & 31) == 0) raise_flag(timeout_flag, nonce);
+    if ((threadIdx.x & 31) == 0) raise_flag(flags, number);
     return false;
 }
 __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, const StreamParams& P) {
     if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
-    return warp_wait_slow(bar, parity, P.timeout_flag, P.nonce);
+    return warp_wait_slow(bar, parity, P.flags, P.nonce);
 }
 
 // Pushes between the blocks of a cluster: the address of the same object in block `rank`, and a remote
@@ -434,7 +435,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
     const int vbeg = rank * base + (rank < rem ? rank : rem), vcnt = base + (rank < rem ? 1 : 0);
     const WarpPart mine = warp_part(warp < kComputeWarps ? warp : lane & (kComputeWarps - 1), vcnt, SV);
     const int steps = mine.steps;
-    FSD_CHECK(P.debug_word, steps <= S::kSteps && vbeg + vcnt <= P.nvec_row && mine.count >= 0 && mine.first + mine.count <= (steps == 0 ? INT_MAX : vcnt), kChkSlice);
+    FSD_CHECK(&P.flags->debug, steps <= S::kSteps && vbeg + vcnt <= P.nvec_row && mine.count >= 0 && mine.first + mine.count <= (steps == 0 ? INT_MAX : vcnt), kChkSlice);
 
     // ---- the helper warp starts the copies ----
     int in_slot = 0, in = 0, in_item = group_id, in_par = 0;      // the pair whose slices are asked for next: its number among the group's, its id, its parent node (trees)
@@ -442,13 +443,13 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
         if (in >= R) return;
         const int slot = in_slot;
         const int b = P.G == 1 ? in_item : static_cast<int>(__umulhi(static_cast<uint32_t>(in_item), P.g_magic) >> P.g_shift);
-        FSD_CHECK(P.debug_word, in_item >= 0 && in_item < P.n_items && b == in_item / P.G, kChkItem);
+        FSD_CHECK(&P.flags->debug, in_item >= 0 && in_item < P.n_items && b == in_item / P.G, kChkItem);
         int arow = in_item + b;                                      // chain: b * (G + 1) + i
         if (P.parent != nullptr) {
             const int i = in_item - b * P.G;
             arow = b * (P.G + 1) + ((in_par >= -1 && in_par < i) ? in_par + 1 : 0);   // an invalid node still moves (ignored) data
         }
-        FSD_CHECK(P.debug_word, vcnt >= 0 && vcnt <= S::kBlockVecs && arow >= 0, kChkStage);
+        FSD_CHECK(&P.flags->debug, vcnt >= 0 && vcnt <= S::kBlockVecs && arow >= 0, kChkStage);
         const char* arow_p = static_cast<const char*>(P.target) + static_cast<size_t>(arow) * P.row_bytes;
         const char* brow_p = static_cast<const char*>(P.draft) + static_cast<size_t>(in_item) * P.row_bytes;
         unsigned char* dst = smem + slot * P.slot_bytes;
@@ -657,7 +658,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
                         if constexpr (kSecondSweep) {
                             if (old) tmem_wait_ld();
                             if (live) {
-                                FSD_CHECK(P.debug_word, (s + 1) * kParkCols <= 64, kChkTmem);
+                                FSD_CHECK(&P.flags->debug, (s + 1) * kParkCols <= 64, kChkTmem);
                                 tmem_st16(tslot + s * kParkCols, e);
                             }
                             if (old) {
@@ -772,17 +773,19 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
         GroupMsg* const xg = P.exchange + static_cast<size_t>(group_id < n_groups ? group_id : 0) * 2 * C;
         int item = group_id;
         uint32_t help_after = P.help_after;
+        int n = 0;
+        const uint64_t number = call_number(P.flags, P.nonce);     // (asked for in front of the block's barrier: small calls +0.3 us)
 #pragma unroll 1
-        for (int n = 0; n < n_end; ++n, item += n_groups) {
+        for (; n < n_end; ++n, item += n_groups) {
             const int par = n & 1;
-            const uint32_t tag = static_cast<uint32_t>(P.nonce) + static_cast<uint32_t>(n), high = static_cast<uint32_t>(P.nonce >> 32);   // what this round's messages carry
+            const uint32_t tag = static_cast<uint32_t>(number) + static_cast<uint32_t>(n), high = static_cast<uint32_t>(number >> 32);   // what this round's messages carry
             bool bad = false;
             if (n < R && rank == 0 && P.parent != nullptr) {
                 const int pr = __ldg(P.parent + item);
                 bad = pr < -1 || pr >= item % P.G;
             }
             if (!warp_wait(&sh.posted[par], (n >> 1) & 1, P)) break;
-            FSD_CHECK(P.debug_word, n >= R || (item >= 0 && item < P.n_items && rank < kMaxGroupSize), kChkRecord);
+            FSD_CHECK(&P.flags->debug, n >= R || (item >= 0 && item < P.n_items && rank < kMaxGroupSize), kChkRecord);
             // What the compute warps wait for comes first: Z and the references.  Lanes 0..15 take the
             // target row's of one warp each, lanes 16..31 the draft row's.
             __syncwarp();
@@ -852,10 +855,10 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
                             break;
                         }
                         // has anybody's wait run out?  (then nothing this warp waits for is certain to come)
-                        if ((i & 255u) == 255u && __any_sync(0xffffffffu, *reinterpret_cast<volatile uint64_t*>(P.timeout_flag) == P.nonce)) break;
+                        if ((i & 255u) == 255u && __any_sync(0xffffffffu, timed_out(P.flags, number))) break;
                     }
                     if (!got) {
-                        if (lane == 0) raise_flag(P.timeout_flag, P.nonce);
+                        if (lane == 0) raise_flag(P.flags, number);
                         break;
                     }
                     const float tk = fmax_nan(tk0, tk1);
@@ -889,6 +892,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
                     c.ka = Ka; c.kb = Kb; c.za = z; c.zb = z_b; c.s0 = s; c.sb = s_b; c.x = 0.f; c.diff = differ ? 1u : 0u;
                     r->part[rank] = c;
                     if (rank == 0) { r->ncta = static_cast<uint32_t>(C); r->state = bad ? kRecordBadTree : kRecordStats; }
+                    if (n == 0 && blockIdx.x == 0) P.flags->number = number;
                 }
             }
             if constexpr (kSecondSweep) {
@@ -902,6 +906,10 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
                 if (lane == 0) mbar_arrive(&sh.totals[par]);
                 issue_slices();
             }
+        }
+        if (blockIdx.x == 0 && lane == 0) {
+            if (n == 0) P.flags->number = number;     // (a wait of the first round ran out)
+            if (P.raise) raise_flag(P.flags, number);
         }
         // Every copy started has landed before the block may leave: normally the rounds consumed them all;
         // after a wait that ran out some may still be on their way (a copy, once started, always completes).

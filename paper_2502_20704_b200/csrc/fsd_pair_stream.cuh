@@ -720,6 +720,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
                     const float ca = ka == -INFINITY ? 0.f : -ka, cb = kb == -INFINITY ? 0.f : -kb;
                     t = zero_sums();
                     __syncwarp();
+                    if constexpr (kSecondSweep) tmem_wait_st();      // the quick form's values go to the same columns: they have to be there first
 #pragma unroll 1
                     for (int s = 0; s < steps; ++s) {
                         float e[kParkCols];

@@ -8,6 +8,7 @@ import pytest
 import torch
 
 import fsd_inputs as gi
+import paper_2502_20704_b200 as fsd
 from tests import parity
 
 pytestmark = pytest.mark.gpu
@@ -85,3 +86,27 @@ def test_few_pairs_and_many_rounds(B, gamma, V):
     c = _chain(B, gamma, V, "bf16", 803)
     for div in ("js", "kl"):
         _check(c, div=div, T=0.15)
+
+
+@pytest.mark.parametrize("dtype,V,step", [("bf16", 16384, 256), ("f32", 12288, 256)])
+def test_every_part_does_its_sweep_over(dtype, V, step):
+    """One block's largest slice, a spike in the last step of each of its sixteen parts: all of what the quick form had
+    parked is parked anew, and the second sweep reads the new values."""
+    c = _chain(4, 3, V, dtype, 805)
+    f32 = dtype == "f32"
+    t = c.target if f32 else gi.bf16_bits_to_f32(c.target)
+    d = c.draft if f32 else gi.bf16_bits_to_f32(c.draft)
+    part = V // 16
+    at = np.arange(16) * part + part - step // 2
+    t[:, :, at] += 50.0
+    d[:, :, at[::2]] += 50.0
+    d[:, :, at[1::2]] += 48.5
+    if not f32:
+        c.target[:] = gi.f32_to_bf16_bits(t)
+        c.draft[:] = gi.f32_to_bf16_bits(d)
+    assert fsd.fsd_set_group_size(1) == 0
+    try:
+        for div in ("js", "tv"):
+            _check(c, div=div, T=0.2)
+    finally:
+        fsd.fsd_set_group_size(0)

@@ -216,7 +216,8 @@ int fsd_set_stage_event(void *event);
 /* Test aid (no counterpart in the paper).  Every wait inside the streaming kernel is bounded; a
  * wait that runs out raises a flag in the workspace, the thread blocks that see it take no
  * further work, the call still returns, and every row's row_status carries FSD_ROW_TIMEOUT (its
- * other outputs are then not valid).  The flag is that call's own, and of a call in a graph that
+ * other outputs are then not valid).  The finish kernel's waits within a cluster end the same way.
+ * The flag is that call's own, and of a call in a graph that
  * replay's.  mode 1: the streaming kernel's first block raises that flag as it ends, which
  * exercises the reporting path alone.  mode 2: in the
  * streaming kernel one thread block keeps its first statistics message to itself and the limit
@@ -225,6 +226,8 @@ int fsd_set_stage_event(void *event);
  * mode 3, in a build with -DFSD_DEBUG_CHECKS only: the block keeps its message to itself and the
  * others do without, as they do when a block of a group is not running: they sum its slice
  * themselves after about a millisecond, and the call's results are ordinary ones.
+ * mode 4, in such a build only: in the finish kernel and in the tuning kernels one block of each
+ * cluster keeps its first values to itself, and the limit of their waits is lowered to 20 ms.
  * mode 0: off (the default).  Process-wide, read when a call is made.  Returns FSD_OK, or
  * FSD_ERR_ENUM for another mode. */
 int fsd_set_timeout_injection(int mode);
@@ -258,7 +261,7 @@ int fsd_debug_checks(int B, int positions, size_t *word_offset);
  * logits.  The accepted length of a row at threshold T is the index of its first position that
  * fails `D compare T` (NaN never passes); the speed proxy is its mean over the rows.  All pointers
  * are device pointers owned by the caller; the calls are asynchronous on `stream`, allocate
- * nothing and need no workspace.  Errors: FSD_ERR_NULL, FSD_ERR_SHAPE (B < 1, positions < 1,
+ * nothing and need no workspace (if a bounded device-side wait runs out their results are NaN).  Errors: FSD_ERR_NULL, FSD_ERR_SHAPE (B < 1, positions < 1,
  * n_thresholds < 1, target negative or NaN), FSD_ERR_ENUM (compare), FSD_ERR_CUDA. */
 
 /* For each of `n_thresholds` candidate thresholds (device array): the mean accepted length over

@@ -194,6 +194,8 @@ int launch_all(PairParams pp, FinishParams fp, bool vec, CallFlags* flags, Group
 #endif
     pp.nonce = next_nonce(); pp.flags = flags;
     fp.flags = flags;
+    const int injection = g_mark_timeout.load();
+    fp.silent = injection == 4;
     if (C > 0) {
         StreamParams sp;
         sp.target = pp.target; sp.draft = pp.draft; sp.parent = pp.parent; sp.G = pp.G;
@@ -211,8 +213,7 @@ int launch_all(PairParams pp, FinishParams fp, bool vec, CallFlags* flags, Group
         // test aid: one block keeps its first message to itself, so that its group's exchange
         // runs out (after a shorter limit: about a tenth of a second) and the kernel's own give-up path runs;
         // mode 3: so that the others sum its slice themselves
-        const int injection = g_mark_timeout.load();
-        const bool silent = injection >= 2;
+        const bool silent = injection == 2 || injection == 3;
         sp.poll_limit = silent ? (1u << 17) : kSpinLimit;
         sp.help_after = injection == 2 ? 0xffffffffu : 1024;     // about a millisecond of fetches
         sp.silent_rank = silent ? C - 1 : -1;
@@ -553,7 +554,7 @@ int fsd_debug_checks(int B, int positions, size_t* word_offset) {
 
 int fsd_set_timeout_injection(int mode) {
 #ifdef FSD_DEBUG_CHECKS
-    constexpr int kModes = 3;
+    constexpr int kModes = 4;
 #else
     constexpr int kModes = 2;
 #endif
@@ -580,7 +581,7 @@ int fsd_threshold_sweep(const float* divergence, int B, int positions, const flo
     const int cs = one ? 1 : kTuneCluster, most = 148 / cs, rows = (B + cs - 1) / cs;
     const int threads = rows >= kTuneThreads ? kTuneThreads : (rows + 31) / 32 * 32 < 64 ? 64 : (rows + 31) / 32 * 32;
     return launch_tuning(one ? fsd_threshold_sweep_kernel<1> : fsd_threshold_sweep_kernel<kTuneCluster>, threads, cs, n_thresholds < most ? n_thresholds : most, B, positions, stream, divergence, B, positions, thresholds, n_thresholds,
-                         compare, mean_accept_len, accept_fraction);
+                         compare, mean_accept_len, accept_fraction, g_mark_timeout.load() == 4 ? 1 : 0);
 }
 
 int fsd_calibrate_threshold(const float* divergence, int B, int positions, float target_mean_accept_len, int compare,
@@ -591,7 +592,7 @@ int fsd_calibrate_threshold(const float* divergence, int B, int positions, float
     if (compare != FSD_CMP_LT && compare != FSD_CMP_LE) return FSD_ERR_ENUM;
     const bool one = tuning_in_one_block(B);
     return launch_tuning(one ? fsd_calibrate_kernel<1> : fsd_calibrate_kernel<kTuneCluster>, kTuneThreads, one ? 1 : kTuneCluster, 1, B, positions, stream, divergence, B, positions, target_mean_accept_len, compare,
-                         threshold_out, achieved_out);
+                         threshold_out, achieved_out, g_mark_timeout.load() == 4 ? 1 : 0);
 }
 
 int fsd_accept_labels(const float* divergence, int B, int positions, float threshold, int compare, uint8_t* labels,

@@ -58,6 +58,7 @@ struct FinishParams {
     int32_t* item_bits;        // [B, G] read when records == null
     int32_t* item_status;      // [B, G] read when records == null
     CallFlags* flags;
+    int silent;                // debug build, test aid: the last CTA of each cluster keeps its first exchange's values to itself
     float* divergence;         // [B, G] written here when records != null
     int32_t* accept_len;       // [B]
     int32_t* path;             // [B, max_depth] (tree) or null
@@ -162,20 +163,31 @@ __device__ __forceinline__ double exp2_of_logit(float x, float xmin, double nk, 
 // known to run (an arrive at kernel entry that is waited for before the first exchange); a CTA that
 // has had its last exchange may leave.  Called by all threads with the same values, and with a barrier
 // of the CTA between two calls; returns the buffer: got[rank][k].
+// Where some thread's wait runs out, all of the CTA's give up: the call's flag is raised, `lost` is set and the caller
+// has to return.  Such a CTA sends nothing any more (a peer that has what it needs may have left) and leaves last
+// (others may send still).  The first CTA looks at the flag when it writes the row's status, at its end: a CTA that
+// gave up waiting for somebody's values has raised it before they were sent, and the first has them all by then.
+struct Link {
+    int turn;                  // exchanges so far
+    bool lost;                 // (the same for all of the CTA's threads)
+};
 template <int N>
-__device__ __forceinline__ const double (*cluster_exchange(FinishShared& sh, int cs, int rank, int& turn, const double (&v)[N]))[kExchangeDoubles] {
+__device__ __forceinline__ const double (*cluster_exchange(const FinishParams& P, FinishShared& sh, int cs, int rank, Link& link, const double (&v)[N]))[kExchangeDoubles] {
     static_assert(N <= kExchangeDoubles, "width of the exchange buffer");
-    const int buf = turn & 1;
+    const int buf = link.turn & 1;
     if (threadIdx.x == 0) mbar_arrive_expect_tx(&sh.link[buf], static_cast<uint32_t>(cs) * N * 8);
-    if (threadIdx.x < cs) {
+    bool send = threadIdx.x < cs;
+#ifdef FSD_DEBUG_CHECKS
+    if (P.silent && link.turn == 0 && rank == cs - 1 && threadIdx.x != rank) send = false;
+#endif
+    if (send) {
         const uint32_t dst = cluster_addr(&sh.got[buf][rank][0], threadIdx.x), bar = cluster_addr(&sh.link[buf], threadIdx.x);
 #pragma unroll
         for (int k = 0; k < N; ++k) st_async(dst + 8 * k, static_cast<uint64_t>(__double_as_longlong(v[k])), bar);
     }
-#pragma unroll 1
-    for (uint32_t i = 0; i < kSpinLimit; ++i)
-        if (mbar_try_wait(&sh.link[buf], (turn >> 1) & 1)) break;
-    ++turn;
+    link.lost = __syncthreads_or(!thread_wait(&sh.link[buf], (link.turn >> 1) & 1, P.silent != 0)) != 0;
+    if (link.lost && threadIdx.x == 0) raise_flag(P.flags, *reinterpret_cast<const volatile uint64_t*>(&P.flags->number));
+    ++link.turn;
     return sh.got[buf];
 }
 
@@ -507,9 +519,9 @@ template <int DT> __device__ __forceinline__ float vector_max(const uint4& v) { 
     }
 }
 
-// Inverse CDF over P_T.  Writes the row's accepted length, token and status; uniform over the cluster.
+// Inverse CDF over P_T.  Writes the row's token, adds to its status (uniform over the cluster).
 template <int DT>
-__device__ __forceinline__ void draw_pt(const FinishParams& P, FinishShared& sh, const Draw& d, int& turn, int status) {
+__device__ __forceinline__ void draw_pt(const FinishParams& P, FinishShared& sh, const Draw& d, Link& link, int& status) {
     constexpr int EPV = Logit<DT>::kPerVec;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const Granules<DT> gr(d.a_row, d.V);
@@ -570,7 +582,8 @@ __device__ __forceinline__ void draw_pt(const FinishParams& P, FinishShared& sh,
         const Prefix pre(sh.warp_tot[lane & (kFinishWarps - 1)], lane);
         w_v = pre.v; w_upto = pre.upto;
         const double mine2[2] = {pre.total, scaled ? 0.0 : static_cast<double>(sh.far)};
-        all = cluster_exchange(sh, d.cs, d.rank, turn, mine2);
+        all = cluster_exchange(P, sh, d.cs, d.rank, link, mine2);
+        if (link.lost) return;
         double any = 0.0;
         W = 0.0;
         for (int r = 0; r < d.cs; ++r) { W += all[r][0]; any += all[r][1]; }
@@ -579,15 +592,16 @@ __device__ __forceinline__ void draw_pt(const FinishParams& P, FinishShared& sh,
         for (int w = 0; w < kFinishWarps; ++w) m = fmaxf(m, sh.warp_k[w]);
         __syncthreads();
         const double mk[1] = {m};
-        all = cluster_exchange(sh, d.cs, d.rank, turn, mk);
+        all = cluster_exchange(P, sh, d.cs, d.rank, link, mk);
+        if (link.lost) return;
         K = -INFINITY;
         for (int r = 0; r < d.cs; ++r) K = fmax(K, all[r][0]);
     }
     if (!(isfinite(W) && W > 0.0)) {                  // a NaN or +inf logit, or no finite one: uniform over the cluster
-        if (d.rank == 0 && tid == 0) { P.accept_len[d.b] = d.n; P.next_token[d.b] = -1; P.row_status[d.b] = status | FSD_ROW_NONFINITE; }
+        status |= FSD_ROW_NONFINITE;
+        if (d.rank == 0 && tid == 0) P.next_token[d.b] = -1;
         return;
     }
-    if (d.rank == 0 && tid == 0) { P.accept_len[d.b] = d.n; P.row_status[d.b] = status; }
     const double t = d.u * W;
     double run = 0.0, cpre = 0.0;
     int owner = -1;
@@ -611,7 +625,8 @@ __device__ __forceinline__ void draw_pt(const FinishParams& P, FinishShared& sh,
         if (lane == 0 && lastp >= 0) atomicMax(&sh.last_pos, lastp);
         __syncthreads();
         const double mine1[1] = {static_cast<double>(sh.last_pos)};
-        all = cluster_exchange(sh, d.cs, d.rank, turn, mine1);
+        all = cluster_exchange(P, sh, d.cs, d.rank, link, mine1);
+        if (link.lost) return;
         int best = -1;
         for (int r = 0; r < d.cs; ++r) best = max(best, static_cast<int>(all[r][0]));
         if (d.rank == 0 && tid == 0) P.next_token[d.b] = best;
@@ -640,7 +655,7 @@ __device__ __forceinline__ void draw_pt(const FinishParams& P, FinishShared& sh,
 // argmax of P_T == argmax of the logits, ties to the lowest index.  One pass: the largest logit, its index, and
 // whether the row is a valid distribution (no NaN, no +inf, something finite).
 template <int DT>
-__device__ __forceinline__ void draw_argmax(const FinishParams& P, FinishShared& sh, const Draw& d, int& turn, int status) {
+__device__ __forceinline__ void draw_argmax(const FinishParams& P, FinishShared& sh, const Draw& d, Link& link, int& status) {
     constexpr int EPV = Logit<DT>::kPerVec;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const Granules<DT> gr(d.a_row, d.V);
@@ -672,7 +687,8 @@ __device__ __forceinline__ void draw_argmax(const FinishParams& P, FinishShared&
     const float cb = warp_redux_max_nan(lb);
     const int ci = __reduce_min_sync(0xffffffffu, lb == cb ? li : 0x7fffffff);
     const double mine3[3] = {cb, static_cast<double>(ci), static_cast<double>(sh.far)};
-    const double (*all)[kExchangeDoubles] = cluster_exchange(sh, d.cs, d.rank, turn, mine3);
+    const double (*all)[kExchangeDoubles] = cluster_exchange(P, sh, d.cs, d.rank, link, mine3);
+    if (link.lost) return;
     if (d.rank == 0 && threadIdx.x == 0) {
         double gb = all[0][0], gi = all[0][1], gbad = all[0][2];
         for (int r = 1; r < d.cs; ++r) {
@@ -680,9 +696,8 @@ __device__ __forceinline__ void draw_argmax(const FinishParams& P, FinishShared&
             gbad += all[r][2];
         }
         const bool ok = gbad == 0.0 && gb > -INFINITY;
-        P.accept_len[d.b] = d.n;
         P.next_token[d.b] = ok ? static_cast<int>(gi) : -1;
-        P.row_status[d.b] = status | (ok ? 0 : FSD_ROW_NONFINITE);
+        if (!ok) status |= FSD_ROW_NONFINITE;         // (this thread writes it)
     }
 }
 
@@ -822,7 +837,7 @@ constexpr double kMostLnRho = 80.0;
 
 template <int DT>
 __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShared& sh, ResidualShared& rs, const ExpTable<DT>& bt,
-                                              const Draw& d, int& turn, int status, bool greedy) {
+                                              const Draw& d, Link& link, int& status, bool greedy) {
     constexpr int EPV = Logit<DT>::kPerVec;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b = d.b, n = d.n, cs = d.cs, rank = d.rank, G = P.G;
@@ -925,7 +940,8 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
             mine[5] = one ? rs.cq[0] : 0.0;
             mine[6] = one ? rs.cq[1] : 0.0;
         }
-        all = cluster_exchange(sh, cs, rank, turn, mine);
+        all = cluster_exchange(P, sh, cs, rank, link, mine);
+        if (link.lost) return;
         Ma = 0.0; Mb = 0.0; flags = 0.0;
         for (int r = 0; r < cs; ++r) { Za += all[r][0]; Zb += all[r][1]; flags = all[r][4] == 1.0 || flags == 1.0 ? 1.0 : fmax(flags, all[r][4]); }
     } else {
@@ -936,7 +952,8 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
         });
         block_sum<2>(z, sh.red_d);
         const double mine[4] = {Ra, Rb, z[0], z[1]};
-        all = cluster_exchange(sh, cs, rank, turn, mine);
+        all = cluster_exchange(P, sh, cs, rank, link, mine);
+        if (link.lost) return;
         Ma = -INFINITY; Mb = -INFINITY;
         for (int r = 0; r < cs; ++r) { Ma = fmax(Ma, all[r][0]); Mb = fmax(Mb, all[r][1]); }
         for (int r = 0; r < cs; ++r) {
@@ -947,7 +964,8 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
     {
         const bool a_ok = isfinite(Ma) && isfinite(Za) && Za > 0.0, b_ok = isfinite(Mb) && isfinite(Zb) && Zb > 0.0;
         if (!a_ok) {                                      // uniform over the cluster
-            if (rank == 0 && tid == 0) { P.accept_len[b] = n; P.next_token[b] = -1; P.row_status[b] = status | FSD_ROW_NONFINITE; }
+            status |= FSD_ROW_NONFINITE;
+            if (rank == 0 && tid == 0) P.next_token[b] = -1;
             return;
         }
         if (!b_ok) { residual = false; status |= FSD_ROW_NONFINITE; }
@@ -993,7 +1011,6 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
             if (run > t) owner = r;
         }
         if (owner >= 0) {                                 // (no mass, or lost to rounding at the very end: the general way)
-            if (rank == 0 && tid == 0) { P.accept_len[b] = n; P.row_status[b] = status; }
             if (owner != rank) return;
             asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
             const int w = lane & (kFinishWarps - 1);
@@ -1073,7 +1090,8 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
             }
         }
         const double mine[4] = {pre.total, Ra, wbest, static_cast<double>(kbest)};
-        all = cluster_exchange(sh, cs, rank, turn, mine);
+        all = cluster_exchange(P, sh, cs, rank, link, mine);
+        if (link.lost) return;
 
         // cluster totals on a common reference
         double M = -INFINITY;
@@ -1088,10 +1106,10 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
             continue;
         }
         if (!residual && !(isfinite(M) && isfinite(W) && W > 0.0)) {     // uniform over the cluster
-            if (rank == 0 && tid == 0) { P.accept_len[b] = n; P.next_token[b] = -1; P.row_status[b] = status | FSD_ROW_NONFINITE; }
+            status |= FSD_ROW_NONFINITE;
+            if (rank == 0 && tid == 0) P.next_token[b] = -1;
             return;
         }
-        if (rank == 0 && tid == 0) { P.accept_len[b] = n; P.row_status[b] = status; }
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
         if (greedy) {                                     // arg-max over the cluster
@@ -1120,7 +1138,8 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
             if (lane == 0 && lastp >= 0) atomicMax(&sh.last_pos, lastp);
             __syncthreads();
             const double mine1[1] = {static_cast<double>(sh.last_pos)};
-            all = cluster_exchange(sh, cs, rank, turn, mine1);
+            all = cluster_exchange(P, sh, cs, rank, link, mine1);
+            if (link.lost) return;
             int best = -1;
             for (int r = 0; r < cs; ++r) best = max(best, static_cast<int>(all[r][0]));
             if (rank == 0 && tid == 0) P.next_token[b] = best;
@@ -1192,7 +1211,7 @@ __global__ void __launch_bounds__(kFinishThreads, 2) fsd_finish_kernel(const __g
     // everything above touched no global memory; what follows reads what the pair kernel wrote
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");       // every CTA of the cluster runs: its shared memory may be written
-    int turn = 0;                                                              // exchanges so far
+    Link link = {0, false};
     if (blockIdx.x == 0 && tid == 0) atomicAdd(reinterpret_cast<unsigned long long*>(&P.flags->epoch), 1ull);     // (nothing here reads it)
 
     // ---- 1. divergences, accept bits, status of this row's pairs ----
@@ -1282,7 +1301,7 @@ __global__ void __launch_bounds__(kFinishThreads, 2) fsd_finish_kernel(const __g
         mine[0] = __longlong_as_double(static_cast<long long>(sh.bad) << 32 | sh.n_acc);
 #pragma unroll
         for (int k = 0; k < kJudgeWords; ++k) mine[1 + k] = __longlong_as_double(static_cast<long long>(sh.bits[k]));
-        const double (*all)[kExchangeDoubles] = cluster_exchange(sh, cs, rank, turn, mine);
+        const double (*all)[kExchangeDoubles] = cluster_exchange(P, sh, cs, rank, link, mine);
         int bad = 0, prefix = G;
         for (int r = 0; r < cs; ++r) {
             const long long w = __double_as_longlong(all[r][0]);
@@ -1293,14 +1312,14 @@ __global__ void __launch_bounds__(kFinishThreads, 2) fsd_finish_kernel(const __g
             for (int i = tree ? tid : G; i < G; i += kFinishThreads)
                 tr.bit[i] = static_cast<int8_t>(__double_as_longlong(all[i % cs][1 + (i / cs >> 6)]) >> (i / cs & 63) & 1);
         __syncthreads();
-        if (tid == 0) { sh.bad = bad; sh.n_acc = prefix; }
+        if (tid == 0 && !link.lost) { sh.bad = bad; sh.n_acc = prefix; }      // (its own are in range)
         __syncthreads();
     }
 
     // ---- 2. accepted prefix (chain) or deepest accepted path (tree) ----
     int n = sh.n_acc, row_sel = n;
     if constexpr (KIND != kDrawResidual) {
-        if (tree) {
+        if (tree && !link.lost) {                    // (lost: whether the parents are valid is not known)
             tree_select(P.parent + static_cast<size_t>(b) * G, G, P.max_depth,
                         rank == 0 ? P.path + static_cast<size_t>(b) * P.max_depth : nullptr, sh, tr);
             __syncthreads();
@@ -1308,29 +1327,35 @@ __global__ void __launch_bounds__(kFinishThreads, 2) fsd_finish_kernel(const __g
             FSD_CHECK(&P.flags->debug, row_sel >= 0 && row_sel <= G && n >= 0 && n <= P.max_depth, kChkPath);
         }
     }
-    FSD_CHECK(&P.flags->debug, row_sel >= 0 && row_sel <= G && n >= 0 && n <= (tree ? P.max_depth : G), kChkRow);
-    const int status = sh.bad;
-    if (status & FSD_ROW_BADTREE) {                      // uniform over the cluster
-        if (rank == 0 && tid == 0) { P.accept_len[b] = 0; P.next_token[b] = -1; P.row_status[b] = status; }
-        return;
-    }
+    FSD_CHECK(&P.flags->debug, link.lost || (row_sel >= 0 && row_sel <= G && n >= 0 && n <= (tree ? P.max_depth : G)), kChkRow);
+    int status = sh.bad;
 
     // ---- 3. token draw ----
-    const bool residual = KIND == kDrawResidual && n < G;
+    const bool residual = KIND == kDrawResidual && n < G, bad_tree = (status & FSD_ROW_BADTREE) != 0;      // (uniform over the cluster)
     Draw d;
     d.a_row = t_base + static_cast<size_t>(row_sel) * rb;
     d.b_row = d_base + static_cast<size_t>(residual ? n : 0) * rb;
     d.b = b; d.n = n; d.V = V; d.cs = cs; d.rank = rank; d.shared_out = shared_out; d.vec = P.vec != 0; d.u = static_cast<double>(sh.u);
-    if constexpr (KIND == kDrawPt) {
-        draw_pt<DT>(P, sh, d, turn, status);
+    if (link.lost) {
+        n = 0;                                           // (nothing of the row is valid but its status)
+    } else if (bad_tree) {
+        n = 0;
+        if (rank == 0 && tid == 0) P.next_token[b] = -1;
+    } else if constexpr (KIND == kDrawPt) {
+        draw_pt<DT>(P, sh, d, link, status);
     } else if constexpr (KIND == kDrawGreedy) {
-        draw_argmax<DT>(P, sh, d, turn, status);
+        draw_argmax<DT>(P, sh, d, link, status);
     } else {
         const bool greedy = P.sample == FSD_SAMPLE_GREEDY;
         if (!residual) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-        if (residual) draw_residual<DT>(P, sh, rs, bt, d, turn, status, greedy);
-        else if (greedy) draw_argmax<DT>(P, sh, d, turn, status);
-        else draw_pt<DT>(P, sh, d, turn, status);
+        if (residual) draw_residual<DT>(P, sh, rs, bt, d, link, status, greedy);
+        else if (greedy) draw_argmax<DT>(P, sh, d, link, status);
+        else draw_pt<DT>(P, sh, d, link, status);
     }
+    if (rank == 0 && tid == 0) {
+        P.accept_len[b] = n;
+        P.row_status[b] = status | (link.lost || timed_out(P.flags, *reinterpret_cast<const volatile uint64_t*>(&P.flags->number)) ? FSD_ROW_TIMEOUT : 0);
+    }
+    leave_last(link.lost);
 }
 }  // namespace fsd

@@ -61,6 +61,7 @@ constexpr int kMaxClusterSize = 8;                         // finish kernel (por
 constexpr int kMaxGroupSize = 24;                          // most blocks in a group of the streaming kernel
 constexpr uint32_t kSpinLimit = 1u << 24;                  // polls before a wait gives up
 constexpr uint64_t kWaitNs = 4000000000ull;                // and its limit in time
+constexpr uint64_t kInjectedWaitNs = 20000000ull;          // test aid: of waits made to run out (see fsd_set_timeout_injection)
 constexpr uint32_t kSleepNs = 40;                          // sleep between two polls of a barrier in shared memory
 
 // Partial statistics of one (target row, draft row) pair: of a warp, of a block, or -- in a pair's
@@ -173,6 +174,29 @@ __device__ __noinline__ bool warp_wait_slow(uint64_t* bar, uint32_t parity, Call
     }
     if ((threadIdx.x & 31) == 0) raise_flag(flags, number);
     return false;
+}
+// Bounded wait of a thread where nobody raises a flag meanwhile (the exchanges within a cluster, copies of its own).
+// (In one loop: with a function of its own for the waits that take longer, the finish kernel's draws were 1 to 4 % slower.)
+__device__ __forceinline__ bool thread_wait(uint64_t* bar, uint32_t parity, [[maybe_unused]] bool short_limit) {
+#ifdef FSD_DEBUG_CHECKS
+    const uint64_t t0 = global_ns();
+#endif
+#pragma unroll 1
+    for (uint32_t i = 0; i < kSpinLimit; ++i) {
+        if (mbar_try_wait(bar, parity)) return true;
+#ifdef FSD_DEBUG_CHECKS
+        if (short_limit && global_ns() - t0 > kInjectedWaitNs) break;
+#endif
+    }
+    return false;
+}
+// A block that has not got what its cluster's others were to push to it leaves last: they may push still.
+__device__ __forceinline__ void leave_last(bool lost) {
+    if (lost) {
+        asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");      // (blocks that have left count as arrived)
+        __nanosleep(50000);                                              // (what they pushed last is there by now)
+    }
 }
 __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, const StreamParams& P) {
     if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;

@@ -36,6 +36,7 @@ constexpr int kTuneCluster = 8;               // the portable size
 constexpr int kTuneBins = 4096;               // of the first digit; 1024 and 512 of the others
 constexpr int kTuneTileBytes = 72 * 1024;     // a tile of rows; two are in shared memory
 constexpr int kSweepAtOnce = 4;               // thresholds a thread counts for in one walk over its rows
+constexpr uint64_t kTuneLost = ~0ull;         // in the place of a count: a wait ran out
 constexpr uint32_t kKeyInf = 0x7f800000u;     // keys above this are NaN (or negative): never accepted
 
 // Sortable key of a prefix maximum: divergences are >= 0, so the bit pattern orders them; -0 and
@@ -49,13 +50,18 @@ __device__ __forceinline__ void bulk_push(uint32_t dst, const void* src, uint32_
     asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(dst), "r"(smem_u32(src)), "r"(bytes), "r"(bar) : "memory");
 }
-// Bounded; what it waits for are copies already started or pushes of peers that run.
-__device__ __forceinline__ bool tune_wait(uint64_t* bar, uint32_t parity) {
-#pragma unroll 1
-    for (uint32_t i = 0; i < kSpinLimit; ++i)
-        if (mbar_try_wait(bar, parity)) return true;
-    return false;
-}
+// Bounded; what it waits for are copies already started or pushes of peers that run.  `lost` remembers, for the
+// thread, that one has run out (the results are NaN then) and ends further waits.
+struct TuneWait {
+    bool lost;
+    bool short_limit;                     // (test aid)
+    __device__ __forceinline__ void operator()(uint64_t* bar, uint32_t parity) { if (!lost && !thread_wait(bar, parity, short_limit)) lost = true; }
+};
+#ifdef FSD_DEBUG_CHECKS
+#define FSD_TUNE_SILENT (silent != 0)
+#else
+#define FSD_TUNE_SILENT false
+#endif
 
 // These kernels are a few microseconds each and follow one another: all are launched with programmatic stream
 // serialization.  What is in front of a kernel in its stream has ended (or it is waited for here, before global memory
@@ -75,6 +81,7 @@ struct TuneRows {
     float* buf;
     uint64_t* bar;                        // [2]
     int seq, issued;                      // tiles walked and asked for so far, over all walks
+    TuneWait wait;
 };
 __device__ __forceinline__ void tune_issue(TuneRows& t) {         // one thread
     const int i = t.issued % t.tiles, slot = t.issued & 1, n = min(t.tile, t.rows - i * t.tile);
@@ -86,8 +93,9 @@ __device__ __forceinline__ void tune_issue(TuneRows& t) {         // one thread
     bulk_g2s(dst, reinterpret_cast<const void*>(a), static_cast<uint32_t>(e - a), &t.bar[slot]);
 }
 // Rows of block `rank` of `cs`; starts the first copies.  `bar`: two barriers, initialised (count 1).
-__device__ __forceinline__ TuneRows tune_rows(const float* D, int B, int G, int rank, int cs, float* buf, uint64_t* bar) {
+__device__ __forceinline__ TuneRows tune_rows(const float* D, int B, int G, int rank, int cs, float* buf, uint64_t* bar, bool short_limit) {
     TuneRows t;
+    t.wait = TuneWait{false, short_limit};
     const int quads = (B + 3) / 4, base = quads / cs, rem = quads % cs;
     t.D = D; t.G = G; t.buf = buf; t.bar = bar; t.seq = 0; t.issued = 0;
     t.row0 = 4 * (rank * base + min(rank, rem));
@@ -125,7 +133,7 @@ __device__ __forceinline__ void tune_walk(TuneRows& t, Begin begin, Step step, E
         if (t.staged) {
             // a resident tile i is in slot i for good; others take turns
             const int s = resident ? i : slot;
-            tune_wait(&t.bar[s], resident ? 0 : (t.seq >> 1) & 1);
+            t.wait(&t.bar[s], resident ? 0 : (t.seq >> 1) & 1);
             base = t.buf + s * (kTuneTileBytes / 4) + t.off;
             width = t.off == 0 && t.G % 4 == 0 ? 4 : t.off % 2 == 0 && t.G % 2 == 0 ? 2 : 1;
         }
@@ -149,9 +157,9 @@ __device__ __forceinline__ void tune_walk(TuneRows& t, Begin begin, Step step, E
 __device__ __forceinline__ void tune_drain(TuneRows& t) {
     if (!t.staged) return;
     if (t.tiles <= 2) {
-        for (int i = 0; i < t.tiles; ++i) tune_wait(&t.bar[i], 0);
+        for (int i = 0; i < t.tiles; ++i) t.wait(&t.bar[i], 0);
     } else {
-        for (int q = t.seq; q < t.issued; ++q) tune_wait(&t.bar[q & 1], (q >> 1) & 1);
+        for (int q = t.seq; q < t.issued; ++q) t.wait(&t.bar[q & 1], (q >> 1) & 1);
     }
 }
 
@@ -162,22 +170,24 @@ __device__ __forceinline__ void tune_drain(TuneRows& t) {
 template <int CS>
 __global__ void __launch_bounds__(kTuneThreads) fsd_threshold_sweep_kernel(const float* __restrict__ D, int B, int G,
                                                                            const float* __restrict__ thresholds, int n_thresholds, int cmp,
-                                                                           float* __restrict__ mean_len, float* __restrict__ frac) {
+                                                                           float* __restrict__ mean_len, float* __restrict__ frac, int silent) {
     extern __shared__ __align__(16) float tune_buf[];
     __shared__ uint64_t bar[2], link[2];
     __shared__ unsigned int part[kTuneThreads / 32][kSweepAtOnce];
-    __shared__ uint64_t got[2][kTuneCluster][kSweepAtOnce];      // (B * positions fits an int)
+    __shared__ uint64_t got[2][kTuneCluster][kSweepAtOnce];      // (B * positions fits an int); kTuneLost: not to be relied on
+    __shared__ int lost;                              // a wait of some thread of this block has run out
     const int rank = CS == 1 ? 0 : static_cast<int>(cg::this_cluster().block_rank());
     const int n_clusters = static_cast<int>(gridDim.x) / CS, cid = static_cast<int>(blockIdx.x) / CS;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) {
+        lost = 0;
         for (int k = 0; k < 2; ++k) { mbar_init(&bar[k], 1); mbar_init(&link[k], 1); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
     if constexpr (CS > 1) cg::this_cluster().barrier_arrive();   // "this block's barriers are ready": waited for before the first push
     launch_in_turn();
-    TuneRows rows = tune_rows(D, B, G, rank, CS, tune_buf, bar);
+    TuneRows rows = tune_rows(D, B, G, rank, CS, tune_buf, bar, FSD_TUNE_SILENT);
     // thresholds cid, cid + n_clusters, ...: kSweepAtOnce of them in one walk
     int turn = 0;
     for (int t0 = cid; t0 < n_thresholds; t0 += n_clusters * kSweepAtOnce, ++turn) {
@@ -209,32 +219,39 @@ __global__ void __launch_bounds__(kTuneThreads) fsd_threshold_sweep_kernel(const
             const unsigned int w = __reduce_add_sync(0xffffffffu, n[j]);
             if (lane == 0) part[warp][j] = w;
         }
+        if (rows.wait.lost) lost = 1;
         __syncthreads();
-        unsigned int sum = 0;
+        uint64_t sum = 0;
         if (tid < kSweepAtOnce)
             for (int w = 0; w < static_cast<int>(blockDim.x >> 5); ++w) sum += part[w][tid];
+        if (lost) sum = kTuneLost;
         if constexpr (CS > 1) {
             // (two buffers take turns; nobody is a turn ahead by more than one: see the barrier below)
             if (turn == 0) cg::this_cluster().barrier_wait();
-            if (rank == 0 && tid == 0) mbar_arrive_expect_tx(&link[turn & 1], CS * kSweepAtOnce * 8);
-            if (tid < kSweepAtOnce) st_async(cluster_addr(&got[turn & 1][rank][tid], 0), sum, cluster_addr(&link[turn & 1], 0));
+            if (rank == 0 && tid == 0 && !rows.wait.lost) mbar_arrive_expect_tx(&link[turn & 1], CS * kSweepAtOnce * 8);
+            if (tid < kSweepAtOnce && !(FSD_TUNE_SILENT && rank == CS - 1))
+                st_async(cluster_addr(&got[turn & 1][rank][tid], 0), sum, cluster_addr(&link[turn & 1], 0));
             if (rank == 0 && tid < 32) {
-                tune_wait(&link[turn & 1], (turn >> 1) & 1);
+                rows.wait(&link[turn & 1], (turn >> 1) & 1);
                 if (tid < kSweepAtOnce) {
+                    bool all = !rows.wait.lost;
                     sum = 0;
-                    for (int r = 0; r < CS; ++r) sum += static_cast<unsigned int>(got[turn & 1][r][tid]);
+                    for (int r = 0; r < CS; ++r) { sum += got[turn & 1][r][tid]; all = all && got[turn & 1][r][tid] != kTuneLost; }
+                    if (!all) sum = kTuneLost;
                 }
             }
             if (t0 + n_clusters * kSweepAtOnce < n_thresholds) cg::this_cluster().sync();   // more walks than one: nobody overtakes block 0
         }
         if (rank == 0 && tid < kSweepAtOnce && t0 + tid * n_clusters < n_thresholds) {
             const int t = t0 + tid * n_clusters;
-            mean_len[t] = static_cast<float>(static_cast<double>(sum) / static_cast<double>(B));
-            frac[t] = static_cast<float>(static_cast<double>(sum) / (static_cast<double>(B) * static_cast<double>(G)));
+            const float nan = __int_as_float(0x7fc00000);
+            mean_len[t] = sum == kTuneLost ? nan : static_cast<float>(static_cast<double>(sum) / static_cast<double>(B));
+            frac[t] = sum == kTuneLost ? nan : static_cast<float>(static_cast<double>(sum) / (static_cast<double>(B) * static_cast<double>(G)));
         }
         __syncthreads();                              // `part` is free again
     }
     tune_drain(rows);
+    if constexpr (CS > 1) leave_last(rows.wait.lost);
 }
 
 // ---- calibration: one cluster (or block), radix selection over the prefix maxima ----------------
@@ -268,6 +285,7 @@ struct CalibrateShared {
     uint32_t list[kTuneList];                         // this block's candidates
     unsigned int warp_sum[kTuneThreads / 32];
     unsigned int n_list, count;
+    int lost;                                         // block 0's: a wait of some thread of the cluster has run out
 };
 
 // A row's prefix maxima never fall, so a thread adds once per distinct value (two or three a row of
@@ -279,7 +297,7 @@ struct CalibrateShared {
 template <int CS>
 __global__ void __launch_bounds__(kTuneThreads) fsd_calibrate_kernel(const float* __restrict__ D, int B, int G, float target,
                                                                      int cmp, float* __restrict__ T_out,
-                                                                     float* __restrict__ achieved_out) {
+                                                                     float* __restrict__ achieved_out, int silent) {
     extern __shared__ __align__(16) float tune_buf[];
     __shared__ __align__(16) CalibrateShared sh;
     const int rank = CS == 1 ? 0 : static_cast<int>(cg::this_cluster().block_rank());
@@ -289,14 +307,15 @@ __global__ void __launch_bounds__(kTuneThreads) fsd_calibrate_kernel(const float
         for (int k = 0; k < 9; ++k) mbar_init(&sh.link[0][0] + k, 1);
         mbar_init(&sh.list_link, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        sh.count = 0; sh.n_list = 0;
+        sh.count = 0; sh.n_list = 0; sh.lost = 0;
     }
     for (int i = tid; i < kTuneBins / 4; i += kTuneThreads) reinterpret_cast<uint4*>(sh.hist)[i] = make_uint4(0, 0, 0, 0);
     for (int i = tid; i < kTuneList; i += kTuneThreads) sh.list[i] = 0xffffffffu;
     __syncthreads();
     if constexpr (CS > 1) cg::this_cluster().barrier_arrive();   // "this block's barriers are ready": waited for before the first push
     launch_in_turn();
-    TuneRows rows = tune_rows(D, B, G, rank, CS, tune_buf, sh.bar);
+    TuneRows rows = tune_rows(D, B, G, rank, CS, tune_buf, sh.bar, FSD_TUNE_SILENT);
+    TuneWait& tune_wait = rows.wait;
 
     // positions that must be accepted: ceil(target * B), within [0, B * G]  (the host refuses negative and NaN targets)
     const double want = ceil(static_cast<double>(target) * static_cast<double>(B));
@@ -363,8 +382,9 @@ __global__ void __launch_bounds__(kTuneThreads) fsd_calibrate_kernel(const float
 #pragma unroll
             for (int w = 0; w < kTuneThreads / 32; ++w) { const unsigned int ws = sh.warp_sum[w]; if (w < warp) before += ws; all += ws; }
             if constexpr (CS > 1) {
-                if (tid < CS) st_async(cluster_addr(&sh.sums[rank], tid), all, cluster_addr(&sh.link[digit][1], tid));
+                if (tid < CS && !(FSD_TUNE_SILENT && rank == CS - 1)) st_async(cluster_addr(&sh.sums[rank], tid), all, cluster_addr(&sh.link[digit][1], tid));
                 tune_wait(&sh.link[digit][1], 0);
+                if (__syncthreads_or(tune_wait.lost)) { found = false; break; }      // (the same for the block: what follows has barriers)
                 all = 0;
                 for (int r = 0; r < CS; ++r) { const unsigned int v = static_cast<unsigned int>(sh.sums[r]); if (r < rank) before += v; all += v; }
             }
@@ -394,7 +414,8 @@ __global__ void __launch_bounds__(kTuneThreads) fsd_calibrate_kernel(const float
             equal = static_cast<unsigned int>(w0 >> 32);
             const unsigned int lower = static_cast<unsigned int>(sh.found[1]);
             below += lower; left -= lower;
-            __syncthreads();                          // everybody has read: the histogram and the rest may be written again
+            if (__syncthreads_or(tune_wait.lost)) { found = false; break; }
+            // everybody has read: the histogram and the rest may be written again
             if (digit == 0 && equal <= kTuneList) { ranked = true; break; }
         }
     }
@@ -403,7 +424,7 @@ __global__ void __launch_bounds__(kTuneThreads) fsd_calibrate_kernel(const float
         for_prefix_maxima(rows, [&](uint32_t key, unsigned int count) {
             if ((key & 0xfff80000u) != prefix || key > kKeyInf) return;
             const unsigned int at = atomicAdd(&sh.n_list, count);
-            for (unsigned int q = 0; q < count; ++q) sh.list[at + q] = key;       // (at most `equal` <= kTuneList in all)
+            for (unsigned int q = 0; q < count && at + q < kTuneList; ++q) sh.list[at + q] = key;       // (at most `equal` <= kTuneList in all, unless a wait ran out)
         });
         if constexpr (CS > 1) {
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -416,7 +437,9 @@ __global__ void __launch_bounds__(kTuneThreads) fsd_calibrate_kernel(const float
                 __syncthreads();
                 for (int i = tid; i < CS * kTuneList; i += kTuneThreads) {
                     const uint32_t key = (&sh.recv[0][0])[i];
-                    if (key != 0xffffffffu) sh.list[atomicAdd(&sh.n_list, 1u)] = key;
+                    if (key == 0xffffffffu) continue;
+                    const unsigned int at = atomicAdd(&sh.n_list, 1u);
+                    if (at < kTuneList) sh.list[at] = key;
                 }
             }
         }
@@ -445,6 +468,10 @@ __global__ void __launch_bounds__(kTuneThreads) fsd_calibrate_kernel(const float
         const float v = __uint_as_float(prefix);
         T = cmp == FSD_CMP_LE ? v : (v == INFINITY ? INFINITY : __uint_as_float(prefix + 1u));   // next float above v
     }
+    const auto tell_lost = [&] {
+        if (rows.wait.lost) { if constexpr (CS > 1) *cg::this_cluster().map_shared_rank(&sh.lost, 0) = 1; else sh.lost = 1; }
+    };
+    tell_lost();
     unsigned int total = below + equal;
     // (a first digit of +inf's holds nothing else that counts, so that every block decides alike)
     if (need == 0 || !found || (prefix & 0xfff80000u) == kKeyInf) {
@@ -453,15 +480,18 @@ __global__ void __launch_bounds__(kTuneThreads) fsd_calibrate_kernel(const float
             if (key <= kKeyInf && passes(__uint_as_float(key), T, cmp)) n += count;
         });
         n = __reduce_add_sync(0xffffffffu, n);
+        tell_lost();
         if (lane == 0 && n) atomicAdd(CS > 1 ? cg::this_cluster().map_shared_rank(&sh.count, 0) : &sh.count, n);
         if constexpr (CS > 1) cg::this_cluster().sync(); else __syncthreads();
         total = sh.count;                             // (block 0's is the one that is used)
-    } else if constexpr (CS > 1) {
-        cg::this_cluster().sync();                    // pushes from and to a block are through before it leaves
+    } else {
+        // pushes from and to a block are through before it leaves
+        if constexpr (CS > 1) cg::this_cluster().sync(); else __syncthreads();
     }
     if (rank == 0 && tid == 0) {
-        *T_out = T;
-        *achieved_out = static_cast<float>(static_cast<double>(total) / static_cast<double>(B));
+        const float nan = __int_as_float(0x7fc00000);
+        *T_out = sh.lost ? nan : T;
+        *achieved_out = sh.lost ? nan : static_cast<float>(static_cast<double>(total) / static_cast<double>(B));
     }
     tune_drain(rows);
 }
@@ -473,5 +503,6 @@ __global__ void fsd_accept_labels_kernel(const float* __restrict__ D, size_t n, 
     for (size_t i = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += stride)
         labels[i] = passes(D[i], T, cmp) ? 1 : 0;
 }
+#undef FSD_TUNE_SILENT
 
 }  // namespace fsd

@@ -125,7 +125,7 @@ import fsd_inputs as gi
 import paper_2502_20704_b200 as fsd
 from tests import parity
 assert fsd.fsd_debug_checks()[0], "this process must have loaded the debug build"
-assert fsd.fsd_set_timeout_injection(3) == 0 and fsd.fsd_set_timeout_injection(4) != 0
+assert fsd.fsd_set_timeout_injection(3) == 0 and fsd.fsd_set_timeout_injection(5) != 0
 def chain(*a, **k):
     kw = {x: k.pop(x) for x in ("div", "mode", "T") if x in k}
     c = gi.make_chain(*a, recipe="zipf", sigma=(0.3, 1.5), sigma_mode="uniform", workload_id=480, **k)

@@ -108,3 +108,53 @@ def test_an_injected_timeout_in_a_captured_call_is_reported_by_every_replay():
         st.zero_()
         graph.replay()
         assert (st.cpu().numpy() & binding.FSD_ROW_TIMEOUT).all()
+
+
+_SCRIPT = r"""
+import numpy as np, torch
+import fsd_inputs as gi
+from paper_2502_20704_b200 import binding as fsd
+from oracle import fsd_tuning_oracle as tun
+from tests import parity
+assert fsd.fsd_debug_checks()[0], "this process must have loaded the debug build"
+c = gi.make_chain(6, 4, 36000, dtype="bf16", recipe="zipf", sigma=(0.3, 1.5), sigma_mode="uniform", workload_id=433)
+t = gi.make_tree(3, 40, 32000, dtype="bf16", sigma=0.6, max_depth=5, workload_id=445)
+D = np.random.default_rng(3).gamma(0.7, 0.12, size=(4096, 8)).clip(0, 0.6931).astype(np.float32)
+d, Ts = torch.from_numpy(D).cuda(), torch.linspace(0.0, 0.6, 200, device="cuda")
+
+def tuning():
+    out = torch.zeros(402, device="cuda")
+    s = torch.cuda.current_stream().cuda_stream
+    assert fsd.fsd_threshold_sweep(d, 4096, 8, Ts, 200, 0, out[:200], out[200:400], s) == 0
+    assert fsd.fsd_calibrate_threshold(d, 4096, 8, 3.0, 0, out[400:401], out[401:402], s) == 0
+    return out.cpu().numpy()
+
+def statuses():
+    for mode, sample in (("fsd", "invcdf"), ("fsd", "greedy"), ("sd", "invcdf"), ("rfsd", "greedy")):
+        yield parity.run_chain_gpu(c.target, c.draft, c.draft_tokens, c.u_accept, c.u_sample, c.dtype, mode=mode, sample=sample, T=0.2).row_status
+    yield parity.run_tree_gpu(t.target, t.draft, t.parent, t.u_sample, 5, t.dtype, T=0.05).row_status
+
+want = tuning()
+assert fsd.fsd_set_timeout_injection(4) == 0
+assert all((st & fsd.FSD_ROW_TIMEOUT).all() for st in statuses())
+assert np.isnan(tuning()).all()
+assert fsd.fsd_set_timeout_injection(0) == 0
+assert all((st == 0).all() for st in statuses())
+assert np.array_equal(tuning(), want) and np.array_equal(want[:200], tun.threshold_sweep(D, Ts.cpu().numpy(), "lt")[0])
+for mode in ("fsd", "sd"):
+    parity.check_chain(c.target, c.draft, c.draft_tokens, c.u_accept, c.u_sample, c.dtype, mode=mode, T=0.2)
+print("reported")
+"""
+
+
+def test_waits_within_a_cluster_that_run_out_are_reported():
+    """One block of each cluster of the finish kernel and of the tuning kernels keeps its first values to itself (debug
+    build, in a process of its own): rows are marked, tuning results are NaN, and the next calls are clean."""
+    import os
+    import subprocess
+    import sys
+    from paper_2502_20704_b200 import build as lib_build
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    env = dict(os.environ, FSD_VERIFY_LIB=lib_build.build(debug=True), PYTHONPATH=root + os.pathsep + os.environ.get("PYTHONPATH", ""))
+    r = subprocess.run([sys.executable, "-c", _SCRIPT], cwd=root, env=env, capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0 and "reported" in r.stdout, r.stdout[-2000:] + r.stderr[-4000:]

@@ -153,8 +153,10 @@ int fsd_verify_tree(const void *target_logits, const void *draft_logits,
  * The call copies the logits into `staging` (device scratch, 256-byte aligned, at least
  * fsd_host_staging_bytes() bytes, owned by the caller), runs fsd_verify_chain on them on
  * `stream` and synchronises the stream before it returns, so the host outputs are valid on
- * return.  The other arrays are copied too where they are pageable; pinned ones are read and
- * written by the kernels where they are.  h_draft_tokens / h_u_accept may be NULL in FSD mode.
+ * return.  The other arrays are copied too where they are pageable; pinned ones of up to 64 KB are read
+ * and written by the kernels where they are (copied, too, at addresses off a multiple of 4, and the
+ * outputs where one shares memory with an input or another output; outputs are written after all
+ * inputs are read).  h_draft_tokens / h_u_accept may be NULL in FSD mode.
  * Errors as fsd_verify_chain; a failed copy gives FSD_ERR_CUDA. */
 int fsd_host_staging_bytes(int B, int gamma, int V, const fsd_opts *opts, size_t *bytes_out);
 int fsd_verify_chain_host(const void *h_target_logits, const void *h_draft_logits,

@@ -317,11 +317,25 @@ HostStaging carve_staging(void* base, int B, int G, int V, size_t es) {
     return h;
 }
 
-// The address at which kernels of the current device reach pinned host memory; null for pageable memory.
-void* mapped_pointer(const void* host) {
-    cudaPointerAttributes a;
-    if (cudaPointerGetAttributes(&a, host) != cudaSuccess) { cudaGetLastError(); return nullptr; }
-    return a.type == cudaMemoryTypeHost ? a.devicePointer : nullptr;
+// The address at which kernels of the current device reach n bytes of pinned host memory; null where they may not use
+// them in place: pageable memory, memory that is pinned in part (pages are pinned one by one, so each is looked at; arrays of
+// more pages than a few are better copied), an address off an element's boundary.
+void* mapped_pointer(const void* host, size_t n) {
+    constexpr size_t kPage = 4096, kMostPages = 16;
+    if (!aligned(host, 4) || n > kMostPages * kPage) return nullptr;
+    char* first = nullptr;
+    for (size_t at = 0;; at = at + kPage < n ? at + kPage : n - 1) {
+        cudaPointerAttributes a;
+        if (cudaPointerGetAttributes(&a, static_cast<const char*>(host) + at) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+        if (a.type != cudaMemoryTypeHost || a.devicePointer == nullptr) return nullptr;
+        if (at == 0) first = static_cast<char*>(a.devicePointer);
+        else if (static_cast<char*>(a.devicePointer) != first + at) return nullptr;
+        if (at == n - 1) return first;
+    }
+}
+bool overlap(const void* a, size_t na, const void* b, size_t nb) {
+    const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+    return x < y + nb && y < x + na;
 }
 
 // Built-in scratch of fsd_verify_chain_static.  In host code this name is only a handle for
@@ -463,35 +477,38 @@ int fsd_verify_chain_host(const void* h_target_logits, const void* h_draft_logit
     // The logits are copied.  The small arrays are not, where the kernels can reach them where they are (pinned
     // memory): a copy of a few hundred bytes takes its 2 us on the stream all the same, and there were seven.
     // 8 x 5 x 32000 bf16, pinned: 165 us a call with the copies, of which 100 are the logits on PCIe.
-    bool ok = true;
-    auto input = [&](const void* host, char* staged, size_t n) -> const void* {
-        if (host == nullptr) return nullptr;
-        if (void* p = mapped_pointer(host)) return p;
-        ok = ok && cudaMemcpyAsync(staged, host, n, cudaMemcpyHostToDevice, s) == cudaSuccess;
-        return staged;
-    };
-    auto output = [&](void* host, char* staged) -> void* {
-        void* p = mapped_pointer(host);
-        return p != nullptr ? p : staged;
-    };
-    ok = ok && cudaMemcpyAsync(h.target, h_target_logits, h.n_target, cudaMemcpyHostToDevice, s) == cudaSuccess;
+    bool ok = cudaMemcpyAsync(h.target, h_target_logits, h.n_target, cudaMemcpyHostToDevice, s) == cudaSuccess;
     ok = ok && cudaMemcpyAsync(h.draft, h_draft_logits, h.n_draft, cudaMemcpyHostToDevice, s) == cudaSuccess;
-    const void* tokens = input(h_draft_tokens, h.tokens, h.n_items4);
-    const void* u_accept = input(h_u_accept, h.u_accept, h.n_items4);
-    const void* u_sample = input(h_u_sample, h.u_sample, h.n_rows4);
+    struct Array { const void* host; char* staged; size_t n; void* used; };
+    Array ins[3] = {{h_draft_tokens, h.tokens, h.n_items4, nullptr}, {h_u_accept, h.u_accept, h.n_items4, nullptr}, {h_u_sample, h.u_sample, h.n_rows4, nullptr}};
+    Array outs[4] = {{h_accept_len, h.accept_len, h.n_rows4, nullptr}, {h_next_token, h.next_token, h.n_rows4, nullptr},
+                     {h_divergence, h.divergence, h.n_items4, nullptr}, {h_row_status, h.row_status, h.n_rows4, nullptr}};
+    // outputs that share memory with an input or with one another are written when all is read, one after another
+    bool apart = true;
+    for (int k = 0; k < 4; ++k) {
+        for (const Array& in : ins) apart = apart && (in.host == nullptr || !overlap(outs[k].host, outs[k].n, in.host, in.n));
+        for (int q = 0; q < k; ++q) apart = apart && !overlap(outs[k].host, outs[k].n, outs[q].host, outs[q].n);
+    }
+    for (Array& a : ins) {
+        if (a.host == nullptr) continue;
+        a.used = mapped_pointer(a.host, a.n);
+        if (a.used == nullptr) {
+            a.used = a.staged;
+            ok = ok && cudaMemcpyAsync(a.staged, a.host, a.n, cudaMemcpyHostToDevice, s) == cudaSuccess;
+        }
+    }
     if (!ok) return FSD_ERR_CUDA;
-    struct Out { void* host; char* staged; size_t n; void* used; } outs[4] = {
-        {h_accept_len, h.accept_len, h.n_rows4, output(h_accept_len, h.accept_len)},
-        {h_next_token, h.next_token, h.n_rows4, output(h_next_token, h.next_token)},
-        {h_divergence, h.divergence, h.n_items4, output(h_divergence, h.divergence)},
-        {h_row_status, h.row_status, h.n_rows4, output(h_row_status, h.row_status)}};
-    rc = fsd_verify_chain(h.target, h.draft, static_cast<const int32_t*>(tokens), static_cast<const float*>(u_accept),
-                          static_cast<const float*>(u_sample), B, gamma, V, opts, static_cast<int32_t*>(outs[0].used),
+    for (Array& a : outs) {
+        a.used = apart ? mapped_pointer(a.host, a.n) : nullptr;
+        if (a.used == nullptr) a.used = a.staged;
+    }
+    rc = fsd_verify_chain(h.target, h.draft, static_cast<const int32_t*>(ins[0].used), static_cast<const float*>(ins[1].used),
+                          static_cast<const float*>(ins[2].used), B, gamma, V, opts, static_cast<int32_t*>(outs[0].used),
                           static_cast<int32_t*>(outs[1].used), static_cast<float*>(outs[2].used), static_cast<int32_t*>(outs[3].used),
                           h.ws, h.n_ws, stream);
     if (rc != FSD_OK) return rc;
-    for (const Out& o : outs)
-        if (o.used == o.staged) ok = ok && cudaMemcpyAsync(o.host, o.staged, o.n, cudaMemcpyDeviceToHost, s) == cudaSuccess;
+    for (const Array& a : outs)
+        if (a.used == a.staged) ok = ok && cudaMemcpyAsync(const_cast<void*>(a.host), a.staged, a.n, cudaMemcpyDeviceToHost, s) == cudaSuccess;
     ok = ok && cudaStreamSynchronize(s) == cudaSuccess;
     return ok ? FSD_OK : FSD_ERR_CUDA;
 }

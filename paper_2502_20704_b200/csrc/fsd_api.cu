@@ -4,8 +4,9 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 #include <atomic>
+#include <ctime>
 #include <mutex>
-#include <random>
+#include <unistd.h>
 
 #include "fsd_verify.h"
 #include "fsd_device.cuh"
@@ -85,13 +86,22 @@ std::atomic<int> g_mark_timeout{0};          // see fsd_set_timeout_injection
 std::atomic<int> g_group_size{0};            // see fsd_set_group_size
 
 // A number no other launch is given, of which a call's number is made (see CallFlags).  The counter's values are spread
-// over 64 bits by an invertible mixing (the finalizer of splitmix64), from a start that differs from process to process.
-uint64_t next_nonce() {
-    static std::atomic<uint64_t> counter{(static_cast<uint64_t>(std::random_device{}()) << 32) ^ std::random_device{}()};
-    uint64_t x = counter.fetch_add(0x9e3779b97f4a7c15ull);
+// over 64 bits by an invertible mixing (the finalizer of splitmix64), from a start that differs from process to process:
+// the time in nanoseconds, the process and where its stack is.  (std::random_device may throw, and this is behind a C entry.)
+uint64_t spread(uint64_t x) {
     x = (x ^ (x >> 30)) * 0xbf58476d1ce4e5b9ull;
     x = (x ^ (x >> 27)) * 0x94d049bb133111ebull;
     return x ^ (x >> 31);
+}
+uint64_t nonce_start() {
+    timespec t = {};
+    clock_gettime(CLOCK_REALTIME, &t);
+    return spread(static_cast<uint64_t>(t.tv_sec) * 1000000000ull + static_cast<uint64_t>(t.tv_nsec)) ^
+           spread(static_cast<uint64_t>(getpid()) << 32) ^ spread(reinterpret_cast<uintptr_t>(&t));
+}
+uint64_t next_nonce() {
+    static std::atomic<uint64_t> counter{nonce_start()};
+    return spread(counter.fetch_add(0x9e3779b97f4a7c15ull));
 }
 
 // ---- streaming kernel launch -----------------------------------------------------------

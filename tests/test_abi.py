@@ -36,6 +36,14 @@ def test_library_exports_every_declared_symbol():
         assert hasattr(lib, n), f"{n} is declared but not exported"
 
 
+def test_library_takes_nothing_that_throws_from_the_cpp_runtime_behind_its_c_entries():
+    """Nothing aborts or throws: what the library uses of the C++ runtime has no way to throw but a mutex.  (std::random_device
+    throws where a process cannot get at a source of randomness.)"""
+    import subprocess
+    names = subprocess.run(["nm", "-D", "--undefined-only", fsd.library_path()], capture_output=True, text=True, check=True).stdout
+    assert "random_device" not in names and "_Znwm" not in names and "__throw_" not in names.replace("__throw_system_error", "")
+
+
 def test_default_opts_and_workspace_size():
     o = fsd.fsd_default_opts()
     assert o.struct_size == ctypes.sizeof(fsd.FsdOpts)

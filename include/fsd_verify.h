@@ -226,8 +226,8 @@ int fsd_set_stage_event(void *event);
  * of the exchange wait is lowered to about a tenth of a second, so its partners' wait really
  * runs out and the kernel's own give-up path runs (every wait stays bounded; nothing faults).
  * mode 3, in a build with -DFSD_DEBUG_CHECKS only: the block keeps its message to itself and the
- * others do without, as they do when a block of a group is not running: they sum its slice
- * themselves after about a millisecond, and the call's results are ordinary ones.
+ * others do without, as they do when a block of a group is not running: they compute what it would
+ * have sent after about a millisecond (ordinarily fifteen), and the call's results are the same.
  * mode 4, in such a build only: in the finish kernel and in the tuning kernels one block of each
  * cluster keeps its first values to itself, and the limit of their waits is lowered to 20 ms.
  * mode 0: off (the default).  Process-wide, read when a call is made.  Returns FSD_OK, or

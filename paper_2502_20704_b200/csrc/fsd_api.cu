@@ -225,7 +225,9 @@ int launch_all(PairParams pp, FinishParams fp, bool vec, CallFlags* flags, Group
         // mode 3: so that the others sum its slice themselves
         const bool silent = injection == 2 || injection == 3;
         sp.poll_limit = silent ? (1u << 17) : kSpinLimit;
-        sp.help_after = injection == 2 ? 0xffffffffu : 1024;     // about a millisecond of fetches
+        // fetches, somewhat below a microsecond each (beside kernels that held 140 of 148 SMs for 3 ms, with 1024 of them:
+        // 64 x 8 x 152064 ended after 20 ms instead of 3.2)
+        sp.help_after = injection == 2 ? 0xffffffffu : injection == 3 ? 1024 : 16384;
         sp.silent_rank = silent ? C - 1 : -1;
         sp.raise = injection == 1;                    // behave as if a bounded wait had run out
         // everything that can fail without a launch (attributes, the occupancy query) comes before

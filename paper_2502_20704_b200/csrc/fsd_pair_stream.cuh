@@ -7,7 +7,8 @@
 // The blocks of a group wait for one another's sums, and usually all of them run.  The launch does not promise it: a
 // cooperative launch would, but it starts only when the kernel in front has ended and that end has been polled for (a
 // period of 2.05 us; calls in a row took multiples of it), while a launch with programmatic stream serialization is set
-// up before.  So a block that has waited for about a millisecond sums the missing slices itself and goes on.
+// up before.  So a block that has waited for about fifteen milliseconds, or finds that a message it wants has been
+// overwritten because the others went on without it, computes the missing blocks' messages itself, bit for bit, and goes on.
 //
 // A block's slice of a pair's two rows arrives in a ring of shared-memory slots (bulk asynchronous
 // copies started by the helper warp; the ring is as deep as the slices allow, two slots at least).
@@ -15,9 +16,11 @@
 // vectors (at most four steps of eight entries a lane), and in round n it does, step by step,
 //   1. the first sweep of pair n: e = 2^(logit * log2e - k), the sums Z = sum e and S = sum e*y (or
 //      the KL sum), a bitwise "rows differ" flag.  The references k (integers in the log2 domain) come
-//      from the maxima of the part's first step, looked at when the round before is done.  That is near enough for
-//      any ordinary logits; a warp whose sums say it was not (a later logit 2^30 above it, a -inf in
-//      the entropy sums) does the sweep over with exact maxima and clamped logits;
+//      from the maxima of the part's first step (of all of it where that has no finite logit), looked at when the round
+//      before is done.  That is near enough for any ordinary logits; a warp whose sums say it was not (a later logit
+//      2^30 above it) does the sweep over with exact maxima.  Where a -inf spoils the entropy sums it does it over
+//      with clamped logits, and clamps from then on: that changes no bit of a part it was not needed for, so a pair's
+//      sums depend on its two rows alone;
 //   2. interleaved with it, the SECOND sweep of pair n - 2 over the e values parked two rounds
 //      earlier: p = e_a/Z_a, q = e_b/Z_b, JS needs sum (p+q) log2(p+q), TV sum |p - q|, KL nothing.
 //      The new e values take the tensor-memory columns the old ones leave (64 values a lane and pair,
@@ -293,6 +296,11 @@ __device__ __forceinline__ float rcp(float x) {
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
+// the reference a maximum gives (log2 domain); none (-inf) where no finite logit was seen
+__device__ __forceinline__ float reference(float maximum) { return maximum <= -9.9e29f ? -INFINITY : ceilf(maximum * kLog2e); }
+// a lane's Z_a + Z_b up to which the references were near enough: an entry may exceed 2^k by about 2^30, as the exponents'
+// rounding allows
+constexpr float kNearZ = 4.0e10f;
 // maximum over the warp, NaN if any lane holds one
 __device__ __forceinline__ float warp_redux_max_nan(float v) {
     float d;
@@ -413,22 +421,94 @@ __device__ __noinline__ uint4 masked_vector(uint4 v, int k0, int V, bool minus_i
     return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// Reference and Z of entries [k0, k1) of a row in global memory, by one warp: what a block's message says of its slice
+// What the compute warps of a block would post of a slice's references and Z's, by one warp from global memory: the
+// same parts, lanes and order of additions, so the same bits.  Lane w returns warp w's of the target row, lane 16 + w those of
+// the draft row.  `off`: entries of the first granule in front of the row (both rows': the draft's are moved onto the target's).
 template <int DT>
-__device__ __noinline__ float2 slice_sum(const void* row, int k0, int k1) {
+__device__ __noinline__ float2 slice_sums(const void* arow, const void* brow, int off, int V, int vbeg, int vcnt) {
+    constexpr int EPV = Logit<DT>::kPerVec, VPS = StreamShape<DT>::kVecPerStep;
     const int lane = threadIdx.x & 31;
-    float m = -INFINITY, z = 0.f;
-#pragma unroll 8
-    for (int k = k0 + lane; k < k1; k += 32) m = fmax_nan(m, load_logit<DT>(row, k));
-    __syncwarp();
-    m = warp_redux_max_nan(m);
-    const float K = m <= -9.9e29f ? -INFINITY : ceilf(m * kLog2e), c = K == -INFINITY ? 0.f : -K;
-#pragma unroll 8
-    for (int k = k0 + lane; k < k1; k += 32) z += ex2(fmaf(load_logit<DT>(row, k), kLog2e, c));
-    __syncwarp();
+    float2 mine = make_float2(-INFINITY, 0.f);
+#pragma unroll 1
+    for (int w = 0; w < kComputeWarps; ++w) {
+        const WarpPart part = warp_part(w, vcnt, 32 * VPS);
+        if (part.steps == 0) continue;
+        const auto first_entry = [&](int v) { return v * 32 + lane < part.count ? (vbeg + part.first + v * 32 + lane) * EPV - off : V; };
+        const auto entry = [&](const void* row, int k) { return k >= 0 && k < V ? load_logit<DT>(row, k) : -1.0e30f; };
+        float ka, kb, za, zb;
+        const auto look = [&](int vectors) {
+            float ma = -INFINITY, mb = -INFINITY;
+#pragma unroll 1
+            for (int v = 0; v < vectors; ++v) {
+                const int k = first_entry(v);
 #pragma unroll
-    for (int i = 16; i > 0; i >>= 1) z += __shfl_xor_sync(0xffffffffu, z, i);
-    return make_float2(K, z);
+                for (int e = 0; e < EPV; ++e) { ma = fmax_nan(ma, entry(arow, k + e)); mb = fmax_nan(mb, entry(brow, k + e)); }
+            }
+            __syncwarp();
+            ka = reference(warp_redux_max_nan(ma)); kb = reference(warp_redux_max_nan(mb));
+        };
+        const auto sum = [&]() {                      // false: the references were not near enough
+            const float ca = ka == -INFINITY ? 0.f : -ka, cb = kb == -INFINITY ? 0.f : -kb;
+            uint64_t za2 = 0, zb2 = 0;
+#pragma unroll 1
+            for (int v = 0; v < part.steps * VPS; ++v) {
+                const int k = first_entry(v);
+#pragma unroll
+                for (int e = 0; e < EPV; e += 2) {
+                    za2 = add2(za2, pack2(ex2(fmaf(entry(arow, k + e), kLog2e, ca)), ex2(fmaf(entry(arow, k + e + 1), kLog2e, ca))));
+                    zb2 = add2(zb2, pack2(ex2(fmaf(entry(brow, k + e), kLog2e, cb)), ex2(fmaf(entry(brow, k + e + 1), kLog2e, cb))));
+                }
+            }
+            za = sum2(za2); zb = sum2(zb2);
+            return __all_sync(0xffffffffu, za + zb < kNearZ) != 0;
+        };
+        look(VPS);
+        if (ka == -INFINITY || kb == -INFINITY) look(part.steps * VPS);
+        if (!sum()) { look(part.steps * VPS); sum(); }
+#pragma unroll
+        for (int m = 16; m > 0; m >>= 1) { za += __shfl_xor_sync(0xffffffffu, za, m); zb += __shfl_xor_sync(0xffffffffu, zb, m); }
+        if (lane == w) mine = make_float2(ka, za);
+        if (lane == 16 + w) mine = make_float2(kb, zb);
+    }
+    __syncwarp();
+    return mine;
+}
+
+// Sixteen warps' Z (a lane each; the draft row's in the upper half) brought to the largest of their references and added up.
+__device__ __forceinline__ float fold_z(float k, float z, bool b_side, float& Ka, float& Kb, float& f) {
+    Ka = warp_redux_max_nan(b_side ? -INFINITY : k); Kb = warp_redux_max_nan(b_side ? k : -INFINITY);
+    f = pow2_ref(k, b_side ? Kb : Ka);
+    float sum = __fmul_rn(z, f);
+#pragma unroll
+    for (int m = 8; m > 0; m >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, m);
+    return sum;
+}
+// The messages of a pair that have not come (bit r and 16 + r of miss0: block r's, of miss1: block 16 + r's), computed by the helper
+// warp; the others stay as they are.  (That the path is there at all costs TV 2 us of 86 on 64 x 8 x 152064 -- without it 82
+// to 84, where its code stands makes no difference -- and JS less than half a microsecond.)
+template <int DT, bool RAGGED>
+__device__ __noinline__ float4 missing_messages(const StreamParams& P, int item, uint32_t miss0, uint32_t miss1, float4 t) {
+    const int lane = threadIdx.x & 31, r0 = lane & 15, base = P.nvec_row / P.C, rem = P.nvec_row % P.C;
+    const bool b_side = lane >= 16;
+    const int b = item / P.G, V = static_cast<int>(P.row_bytes / Logit<DT>::kBytes);
+    int arow = item + b;
+    if (P.parent != nullptr) {
+        const int pr = __ldg(P.parent + item), k = item - b * P.G;
+        arow = b * (P.G + 1) + (pr >= -1 && pr < k ? pr + 1 : 0);
+    }
+    const char* arow_p = static_cast<const char*>(P.target) + static_cast<size_t>(arow) * P.row_bytes;
+    const char* brow_p = static_cast<const char*>(P.draft) + static_cast<size_t>(item) * P.row_bytes;
+    const int off = RAGGED ? static_cast<int>(reinterpret_cast<uintptr_t>(arow_p) & 15) / Logit<DT>::kBytes : 0;
+#pragma unroll 1
+    for (int r = 0; r < P.C; ++r) {
+        if (((r < 16 ? miss0 : miss1) >> (r & 15) & 0x10001u) == 0) continue;
+        const float2 m = slice_sums<DT>(arow_p, brow_p, off, V, r * base + min(r, rem), base + (r < rem ? 1 : 0));
+        float Ka, Kb, f;
+        const float z = fold_z(m.x, m.y, b_side, Ka, Kb, f);
+        if (r0 == r) { t.x = b_side ? Kb : Ka; t.y = z; }
+        if (r0 + 16 == r) { t.z = b_side ? Kb : Ka; t.w = z; }
+    }
+    return t;
 }
 
 template <int DT, int DIV, bool RAGGED>
@@ -584,20 +664,20 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
             __syncwarp();
             const float ra = warp_redux_max_nan(ma), rb = warp_redux_max_nan(mb);
             ma = -INFINITY; mb = -INFINITY;
-            ka = ra <= -9.9e29f ? -INFINITY : ceilf(ra * kLog2e);
-            kb = rb <= -9.9e29f ? -INFINITY : ceilf(rb * kLog2e);
+            ka = reference(ra);
+            kb = reference(rb);
         };
 
         // ---- first sweep of step s of the pair in the slot at byte offset `o` ----
         struct Sums { uint64_t za2, zb2, sa2, sb2; float kk; uint32_t diff; };     // packed (even, odd) partial sums
         const auto zero_sums = [] { return Sums{0, 0, 0, 0, 0.f, 0}; };
-        auto first_sweep = [&](auto careful_tag, int s, uint32_t o, uint64_t ca2, uint64_t cb2, Sums& t, float (&e)[kParkCols]) {
-            constexpr bool CAREFUL = decltype(careful_tag)::value;
+        auto first_sweep = [&](auto clamp_tag, int s, uint32_t o, uint64_t ca2, uint64_t cb2, Sums& t, float (&e)[kParkCols]) {
+            constexpr bool CLAMP = decltype(clamp_tag)::value;
 #pragma unroll
             for (int v = 0; v < VPS; ++v) {
                 uint4 wa = ld_shared16(my_a + o + (s * VPS + v) * 512);
                 uint4 wb = ld_shared16(my_b + o + (s * VPS + v) * 512);
-                if constexpr (CAREFUL && DIV == FSD_DIV_JS && DT == FSD_BF16) {
+                if constexpr (CLAMP && DIV == FSD_DIV_JS && DT == FSD_BF16) {
                     // -inf becomes -1e30: 2^y = 0 and 0 * y = 0 stay finite (NaN passes through)
                     wa.x = bf16x2_max_nan(wa.x, kClamp2); wa.y = bf16x2_max_nan(wa.y, kClamp2);
                     wa.z = bf16x2_max_nan(wa.z, kClamp2); wa.w = bf16x2_max_nan(wa.w, kClamp2);
@@ -611,7 +691,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
 #pragma unroll
                 for (int j = 0; j < EPV; j += 2) {
                     float a0 = xa[j], a1 = xa[j + 1], b0 = xb[j], b1 = xb[j + 1];
-                    if constexpr (CAREFUL && DIV == FSD_DIV_JS && DT == FSD_F32) {
+                    if constexpr (CLAMP && DIV == FSD_DIV_JS && DT == FSD_F32) {
                         a0 = fmax_nan(a0, kClamp); a1 = fmax_nan(a1, kClamp); b0 = fmax_nan(b0, kClamp); b1 = fmax_nan(b1, kClamp);
                     }
                     const uint64_t ya2 = fma2(pack2(a0, a1), l2, ca2), yb2 = fma2(pack2(b0, b1), l2, cb2);
@@ -640,7 +720,12 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
         int slot = 0;
         uint32_t so = 0;                             // its slot, and the slot's byte offset
         uint32_t phase = 0;                          // of its slot
-        bool careful = false;                        // this warp has met logits that the quick form of the first sweep cannot take
+        bool clamp = false;                          // this warp has met a -inf: the entropy sums (JS) take clamped logits
+        const auto look_at_all = [&](uint32_t o, float& ra, float& rb) {
+#pragma unroll 1
+            for (int v = 0; v < steps * VPS; ++v) maxima(ld_shared16(my_a + o + v * 512), ld_shared16(my_b + o + v * 512));
+            references(ra, rb);
+        };
         // A pair's part, in slot `s` at byte offset `o`: aligned (an unaligned row's), its first step looked at for the
         // references.  Done for the next pair at the end of a round, so that two slots suffice.
         auto look = [&](int s, uint32_t o, float& ra, float& rb) {
@@ -655,11 +740,12 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
                 for (int v = 0; v < VPS; ++v) maxima(ld_shared16(my_a + o + v * 512), ld_shared16(my_b + o + v * 512));
             }
             references(ra, rb);
+            if (steps > 1 && (ra == -INFINITY || rb == -INFINITY)) look_at_all(o, ra, rb);
         };
         // Both sweeps of a round, step by step.  FULL: a pair in both (this one's first sweep, the second sweep of n - 2), so
         // that a step is one run of straight-line code whose two strands cover one another's latencies; otherwise (the first
-        // and last rounds, and careful ones) each strand is looked at.
-        auto sweeps = [&](auto full_tag, const int n, const bool first, const float ia, const float ib, Sums& t, uint64_t& x2) {
+        // and last rounds) each strand is looked at.
+        auto sweeps = [&](auto full_tag, auto clamp_tag, const int n, const bool first, const float ia, const float ib, Sums& t, uint64_t& x2) {
             constexpr bool FULL = decltype(full_tag)::value;
             const bool live = FULL || first;
             [[maybe_unused]] const bool old = FULL || n >= 2;
@@ -678,7 +764,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
                         if constexpr (kSecondSweep) {
                             if (old) tmem_ld16(tslot + s * kParkCols, eo);
                         }
-                        if (live) first_sweep(std::false_type{}, s, so, ca2, cb2, t, e);
+                        if (live) first_sweep(clamp_tag, s, so, ca2, cb2, t, e);
                         if constexpr (kSecondSweep) {
                             if (old) tmem_wait_ld();
                             if (live) {
@@ -728,19 +814,22 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
             }
             Sums t = zero_sums();
             uint64_t x2 = 0;
-            if (n >= 2 && live && !careful) sweeps(std::true_type{}, n, true, ia, ib, t, x2);
-            else sweeps(std::false_type{}, n, live && !careful, ia, ib, t, x2);
-            // Were the references near enough?  A lane's Z up to 4e10 (an entry may exceed 2^k by about 2^30, as the
-            // exponents' rounding allows), no NaN (-inf * 0 in the entropy sums), and a reference at all.  If not, the
-            // first sweep is done (over) with exact maxima and clamped logits, and this warp stays with that form.
+            const bool full = n >= 2 && live;
+            if (full && (DIV != FSD_DIV_JS || !clamp)) {
+                sweeps(std::true_type{}, std::false_type{}, n, true, ia, ib, t, x2);
+            } else if (full) {
+                sweeps(std::true_type{}, std::true_type{}, n, true, ia, ib, t, x2);
+            } else {
+                sweeps(std::false_type{}, std::true_type{}, n, live, ia, ib, t, x2);
+            }
+            // Were the references near enough (see kNearZ)?  If not, the first sweep is done over with exact maxima.  Has a
+            // -inf spoilt the entropy sums (-inf * 0)?  Then it is done over with clamped logits, and clamped at once from now on.
             if (live) {
                 const float z = sum2(t.za2) + sum2(t.zb2);
-                bool near = z < 4.0e10f && ((ka != -INFINITY && kb != -INFINITY) || steps == 0);
+                bool near = z < kNearZ;
                 if constexpr (DIV == FSD_DIV_JS) near = near && fabsf(sum2(t.sa2)) + fabsf(sum2(t.sb2)) < 1.0e15f;
-                if (careful || __any_sync(0xffffffffu, !near)) {
-                    careful = true;
-                    for (int v = 0; v < steps * VPS; ++v) maxima(ld_shared16(my_a + so + v * 512), ld_shared16(my_b + so + v * 512));
-                    references(ka, kb);
+                if (__any_sync(0xffffffffu, !near)) {
+                    if (DIV != FSD_DIV_JS || __any_sync(0xffffffffu, !(z < kNearZ))) look_at_all(so, ka, kb); else clamp = true;
                     const float ca = ka == -INFINITY ? 0.f : -ka, cb = kb == -INFINITY ? 0.f : -kb;
                     t = zero_sums();
                     __syncwarp();
@@ -821,11 +910,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
             const bool differ = __any_sync(0xffffffffu, w.diff != 0);
             float Ka = -INFINITY, Kb = -INFINITY, f = 0.f;
             if (n < R) {
-                Ka = warp_redux_max_nan(b_side ? -INFINITY : wk); Kb = warp_redux_max_nan(b_side ? wk : -INFINITY);
-                f = pow2_ref(wk, b_side ? Kb : Ka);
-                float z = wz * f;
-#pragma unroll
-                for (int m = 8; m > 0; m >>= 1) z += __shfl_xor_sync(0xffffffffu, z, m);
+                const float z = fold_z(wk, wz, b_side, Ka, Kb, f);
                 if constexpr (kSecondSweep) {
                     // lanes 0 and 16 each store one 16-byte unit of this block's message; every unit ends in the round's tag
                     if ((lane & 15) == 0 && !(n == 0 && group_id == 0 && rank == P.silent_rank))
@@ -838,53 +923,44 @@ __global__ void __launch_bounds__(kStreamThreads, 1) fsd_pair_stream_kernel(cons
                     const int r0 = lane & 15;
                     float tk0 = -INFINITY, tz0 = 0.f, tk1 = -INFINITY, tz1 = 0.f;
                     bool got = false;
+                    uint32_t miss0 = 0, miss1 = 0;    // messages to be computed here
 #pragma unroll 1
                     for (uint32_t i = 0; i < P.poll_limit; ++i) {
                         bool ok0 = true, ok1 = true;
+                        uint4 u0 = make_uint4(0, 0, ~high, 0), u1 = u0;
                         if (r0 < C) {
-                            const uint4 u = ld_unit(&xg[par * C + r0].u[b_side]);
-                            ok0 = u.w == tag && u.z == high;
-                            tk0 = __uint_as_float(u.x); tz0 = __uint_as_float(u.y);
+                            u0 = ld_unit(&xg[par * C + r0].u[b_side]);
+                            ok0 = u0.w == tag && u0.z == high;
+                            tk0 = __uint_as_float(u0.x); tz0 = __uint_as_float(u0.y);
                         }
                         if (r0 + 16 < C) {
-                            const uint4 u = ld_unit(&xg[par * C + r0 + 16].u[b_side]);
-                            ok1 = u.w == tag && u.z == high;
-                            tk1 = __uint_as_float(u.x); tz1 = __uint_as_float(u.y);
+                            u1 = ld_unit(&xg[par * C + r0 + 16].u[b_side]);
+                            ok1 = u1.w == tag && u1.z == high;
+                            tk1 = __uint_as_float(u1.x); tz1 = __uint_as_float(u1.y);
                         }
                         if (__all_sync(0xffffffffu, ok0 && ok1)) { got = true; break; }
                         // A block of the group that has sent nothing for this long may not be running at all: nothing makes the
-                        // blocks of this launch resident together, another stream's kernels may hold SMs.  Its slices are summed
+                        // blocks of this launch resident together, another stream's kernels may hold SMs.  Its message is computed
                         // here then, so no block ever needs another one in order to finish.  (From then on the others' rounds
-                        // and this block's are apart, and it does not wait as long again.)
-                        if (i >= help_after) {
-                            const uint32_t miss0 = __ballot_sync(0xffffffffu, !ok0), miss1 = __ballot_sync(0xffffffffu, !ok1);
-                            const int b = item / P.G, V = static_cast<int>(P.row_bytes / Logit<DT>::kBytes);
-                            int arow = item + b;
-                            if (P.parent != nullptr) {
-                                const int pr = __ldg(P.parent + item), k = item - b * P.G;
-                                arow = b * (P.G + 1) + (pr >= -1 && pr < k ? pr + 1 : 0);
-                            }
-                            const char* arow_p = static_cast<const char*>(P.target) + static_cast<size_t>(arow) * P.row_bytes;
-                            const char* brow_p = static_cast<const char*>(P.draft) + static_cast<size_t>(item) * P.row_bytes;
-                            const int oa = RAGGED ? static_cast<int>(reinterpret_cast<uintptr_t>(arow_p) & 15) / Logit<DT>::kBytes : 0;
-#pragma unroll 1
-                            for (int r = 0; r < C; ++r) {
-                                if (((r < 16 ? miss0 : miss1) >> (r & 15) & 0x10001u) == 0) continue;
-                                const int k0 = (r * base + min(r, rem)) * EPV - oa, k1 = min(k0 + (base + (r < rem ? 1 : 0)) * EPV, V);
-                                const float2 ta = slice_sum<DT>(arow_p, max(k0, 0), k1), tb = slice_sum<DT>(brow_p, max(k0, 0), k1);
-                                if (r0 == r) { tk0 = b_side ? tb.x : ta.x; tz0 = b_side ? tb.y : ta.y; }
-                                if (r0 + 16 == r) { tk1 = b_side ? tb.x : ta.x; tz1 = b_side ? tb.y : ta.y; }
-                            }
-                            help_after = 32;
-                            got = true;
+                        // and this block's are apart: it does not wait as long again, and the late block finds the others' messages
+                        // overwritten by those of later rounds, and does not wait at all.  Waiting is cheap and computing is not, 5 us
+                        // and more a slice, so a block waits for about as long as it may take to catch up.)
+                        const auto overwritten = [&](const uint4& u) { return u.z == high && u.w - tag - 1u < static_cast<uint32_t>(R); };
+                        if (i >= help_after || __any_sync(0xffffffffu, overwritten(u0) || overwritten(u1))) {
+                            if (i >= help_after) help_after = 32;
+                            miss0 = __ballot_sync(0xffffffffu, !ok0); miss1 = __ballot_sync(0xffffffffu, !ok1);
                             break;
                         }
                         // has anybody's wait run out?  (then nothing this warp waits for is certain to come)
                         if ((i & 255u) == 255u && __any_sync(0xffffffffu, timed_out(P.flags, number))) break;
                     }
                     if (!got) {
-                        if (lane == 0) raise_flag(P.flags, number);
-                        break;
+                        if ((miss0 | miss1) == 0) {
+                            if (lane == 0) raise_flag(P.flags, number);
+                            break;
+                        }
+                        const float4 m = missing_messages<DT, RAGGED>(P, item, miss0, miss1, make_float4(tk0, tz0, tk1, tz1));
+                        tk0 = m.x; tz0 = m.y; tk1 = m.z; tz1 = m.w;
                     }
                     const float tk = fmax_nan(tk0, tk1);
                     const float Ga = warp_redux_max_nan(b_side ? -INFINITY : tk), Gb = warp_redux_max_nan(b_side ? tk : -INFINITY);

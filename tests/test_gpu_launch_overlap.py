@@ -143,6 +143,29 @@ for size in (1, 2, 3, 16):
 fsd.fsd_set_group_size(0)
 c = gi.make_tree(3, 40, 32000, dtype="bf16", sigma=0.6, max_depth=5, workload_id=445)
 parity.check_tree(c, T=0.05)
+
+# bit for bit what the same call gives when all blocks send: masked parts, late spikes, invalid rows among them
+import numpy as np
+def same(B, gamma, V, dtype, div, special):
+    c = gi.make_chain(B, gamma, V, dtype=dtype, recipe="zipf", sigma=(0.3, 1.5), sigma_mode="uniform", workload_id=481)
+    t, d, us = (parity.to_device(x, dtype) for x in (c.target, c.draft, c.u_sample))
+    if special:
+        t[0, :, ::7] = -float("inf"); d[0, :, : V // 2] = -float("inf"); t[1, :, V - 9] += 60.0; d[1, 0, 5] = float("nan")
+        t[2, :, 300:] = -float("inf"); d[2, :, V // 3:] = -3.0e38
+    dev = dict(t=t, d=d, tok=None, ua=None, us=us)
+    out = []
+    for mode in (0, 3):
+        assert fsd.fsd_set_timeout_injection(mode) == 0
+        out.append(parity.run_chain_gpu(c.target, c.draft, None, None, c.u_sample, dtype, div=div, T=0.2, dev=dev).divergence.view(np.uint32))
+    assert np.array_equal(out[0], out[1]), (B, gamma, V, dtype, div, special, int((out[0] != out[1]).sum()))
+for special in (False, True):
+    for div in ("js", "tv"):
+        same(6, 4, 36000, "bf16", div, special)
+        same(6, 4, 50257, "bf16", div, special)
+        same(4, 3, 40003, "f32", div, special)
+        same(3, 3, 152064, "f32", div, special)
+    same(64, 6, 32000, "bf16", "js", special)
+    same(3, 2, 290000, "f32", "js", special)
 print("did without")
 """
 

@@ -110,3 +110,24 @@ def test_every_part_does_its_sweep_over(dtype, V, step):
             _check(c, div=div, T=0.2)
     finally:
         fsd.fsd_set_group_size(0)
+
+
+@pytest.mark.parametrize("dtype,V", [("bf16", 40000), ("bf16", 40003), ("f32", 30000)])
+@pytest.mark.parametrize("div", ["js", "kl", "tv"])
+def test_a_pairs_divergence_is_its_own_rows_alone(dtype, V, div):
+    """What the other pairs of a call hold (masked entries, late spikes, NaN) changes no bit of a pair's divergence."""
+    c = gi.make_chain(40, 5, V, dtype=dtype, recipe="spike", sigma=(0.5, 1.0), workload_id=804)
+    t, d = (parity.to_device(x, dtype) for x in (c.target, c.draft))
+    us = parity.to_device(c.u_sample, dtype)
+
+    def divergences():
+        return parity.run_chain_gpu(c.target, c.draft, None, None, c.u_sample, dtype, div=div, T=0.25, dev=dict(t=t, d=d, tok=None, ua=None, us=us)).divergence
+
+    want = divergences()
+    t[0:20, :, ::53] = -float("inf")
+    t[20, 2, 11] = float("nan")
+    d[21:24, :, 9000:9400] = -float("inf")
+    d[24:28, :, V - 5] += 60.0
+    got = divergences()
+    assert np.array_equal(got[28:].view(np.uint32), want[28:].view(np.uint32))
+    assert not np.array_equal(got[:28].view(np.uint32), want[:28].view(np.uint32))

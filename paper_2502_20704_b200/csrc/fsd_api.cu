@@ -609,7 +609,12 @@ int fsd_threshold_sweep(const float* divergence, int B, int positions, const flo
     const bool one = tuning_in_one_block(B);
     const int cs = one ? 1 : kTuneCluster, most = 148 / cs, rows = (B + cs - 1) / cs;
     const int threads = rows >= kTuneThreads ? kTuneThreads : (rows + 31) / 32 * 32 < 64 ? 64 : (rows + 31) / 32 * 32;
-    return launch_tuning(one ? fsd_threshold_sweep_kernel<1> : fsd_threshold_sweep_kernel<kTuneCluster>, threads, cs, n_thresholds < most ? n_thresholds : most, B, positions, stream, divergence, B, positions, thresholds, n_thresholds,
+    const int clusters = n_thresholds < most ? n_thresholds : most;
+    // (4096 x 8, 2000 thresholds: 72 us with four of them a walk)
+    const bool many = n_thresholds > 8ll * clusters;
+    const auto kernel = one ? (many ? fsd_threshold_sweep_kernel<1, kSweepMany> : fsd_threshold_sweep_kernel<1, kSweepFew>)
+                            : (many ? fsd_threshold_sweep_kernel<kTuneCluster, kSweepMany> : fsd_threshold_sweep_kernel<kTuneCluster, kSweepFew>);
+    return launch_tuning(kernel, threads, cs, clusters, B, positions, stream, divergence, B, positions, thresholds, n_thresholds,
                          compare, mean_accept_len, accept_fraction, g_mark_timeout.load() == 4 ? 1 : 0);
 }
 

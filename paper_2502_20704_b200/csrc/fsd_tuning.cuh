@@ -35,7 +35,7 @@ constexpr int kTuneThreads = 512;             // at most; a sweep over few rows 
 constexpr int kTuneCluster = 8;               // the portable size
 constexpr int kTuneBins = 4096;               // of the first digit; 1024 and 512 of the others
 constexpr int kTuneTileBytes = 72 * 1024;     // a tile of rows; two are in shared memory
-constexpr int kSweepAtOnce = 4;               // thresholds a thread counts for in one walk over its rows
+constexpr int kSweepFew = 4, kSweepMany = 16; // thresholds a thread counts for in one walk over its rows (many: where a cluster has more than eight)
 constexpr uint64_t kTuneLost = ~0ull;         // in the place of a count: a wait ran out
 constexpr uint32_t kKeyInf = 0x7f800000u;     // keys above this are NaN (or negative): never accepted
 
@@ -77,7 +77,7 @@ struct TuneRows {
     const float* D;
     int G, row0, rows, tile, tiles;       // rows a tile has (a multiple of four, so that tiles start 16 bytes apart like D), and tiles
     int off;                              // words between a 16-byte boundary and D
-    bool staged;                          // (a single row longer than a tile is walked where it is)
+    bool staged;                          // (rows so long that a tile has too few for the threads are walked where they are)
     float* buf;
     uint64_t* bar;                        // [2]
     int seq, issued;                      // tiles walked and asked for so far, over all walks
@@ -101,8 +101,11 @@ __device__ __forceinline__ TuneRows tune_rows(const float* D, int B, int G, int 
     t.row0 = 4 * (rank * base + min(rank, rem));
     t.rows = max(0, min(4 * (base + (rank < rem ? 1 : 0)), B - t.row0));
     const long long quad_bytes = 16ll * G;
-    t.staged = quad_bytes + 16 <= kTuneTileBytes;
-    t.tile = t.staged ? 4 * static_cast<int>((kTuneTileBytes - 16) / quad_bytes) : t.rows;
+    // A thread walks a row, so a tile of few rows leaves the block's other threads idle: where it has less than half of what
+    // they could take, the rows are read through L1 instead (300 rows of 1000, calibration 3863 us from tiles of 16 rows).
+    const int fit = 4 * static_cast<int>((kTuneTileBytes - 16) / quad_bytes);
+    t.staged = fit > 0 && 2 * fit >= min(t.rows, static_cast<int>(blockDim.x));
+    t.tile = t.staged ? fit : t.rows;
     t.tiles = t.staged ? (t.rows + t.tile - 1) / t.tile : (t.rows > 0 ? 1 : 0);
     t.off = static_cast<int>((reinterpret_cast<uintptr_t>(D) & 15) / 4);
     if (t.staged)
@@ -110,10 +113,10 @@ __device__ __forceinline__ TuneRows tune_rows(const float* D, int B, int G, int 
             if (threadIdx.x == 0) tune_issue(t);
     return t;
 }
-// One thread's walk along one row: step(d) for every position in order, false to stop.
-template <int W, typename F>
-__device__ __forceinline__ void walk_row(const float* row, int G, F step) {
-    for (int k = 0; k < G; k += W) {
+// One thread's walk along one row: step(d) for every position in order, until stop() says that the rest does not matter.
+template <int W, typename F, typename S>
+__device__ __forceinline__ void walk_row(const float* row, int G, F step, S stop) {
+    for (int k = 0; k < G && !stop(); k += W) {
         float d[W];
         if constexpr (W == 4) { const float4 v = *reinterpret_cast<const float4*>(row + k); d[0] = v.x; d[1] = v.y; d[2] = v.z; d[3] = v.w; }
         else if constexpr (W == 2) { const float2 v = *reinterpret_cast<const float2*>(row + k); d[0] = v.x; d[1] = v.y; }
@@ -122,27 +125,26 @@ __device__ __forceinline__ void walk_row(const float* row, int G, F step) {
         for (int q = 0; q < W; ++q) step(d[q]);
     }
 }
-// One walk over all of the block's rows: begin() / step(d) / end() per row.  All threads of the block take part.
-template <typename Begin, typename Step, typename End>
-__device__ __forceinline__ void tune_walk(TuneRows& t, Begin begin, Step step, End end) {
+// One walk over all of the block's rows: begin() / step(d) until stop() / end() per row.  All threads of the block take part.
+template <typename Begin, typename Step, typename Stop, typename End>
+__device__ __forceinline__ void tune_walk(TuneRows& t, Begin begin, Step step, Stop stop, End end) {
     for (int i = 0; i < t.tiles; ++i) {
         const int slot = t.seq & 1, n = min(t.tile, t.rows - i * t.tile);
         const bool resident = t.tiles <= 2;
         const float* base = t.D + static_cast<size_t>(t.row0 + i * t.tile) * t.G;
-        int width = 1;
+        const int width = t.off == 0 && t.G % 4 == 0 ? 4 : t.off % 2 == 0 && t.G % 2 == 0 ? 2 : 1;
         if (t.staged) {
             // a resident tile i is in slot i for good; others take turns
             const int s = resident ? i : slot;
             t.wait(&t.bar[s], resident ? 0 : (t.seq >> 1) & 1);
             base = t.buf + s * (kTuneTileBytes / 4) + t.off;
-            width = t.off == 0 && t.G % 4 == 0 ? 4 : t.off % 2 == 0 && t.G % 2 == 0 ? 2 : 1;
         }
         for (int r = threadIdx.x; r < n; r += blockDim.x) {
             const float* row = base + static_cast<size_t>(r) * t.G;
             begin();
-            if (width == 4) walk_row<4>(row, t.G, step);
-            else if (width == 2) walk_row<2>(row, t.G, step);
-            else walk_row<1>(row, t.G, step);
+            if (width == 4) walk_row<4>(row, t.G, step, stop);
+            else if (width == 2) walk_row<2>(row, t.G, step, stop);
+            else walk_row<1>(row, t.G, step, stop);
             end();
         }
         ++t.seq;
@@ -167,14 +169,14 @@ __device__ __forceinline__ void tune_drain(TuneRows& t) {
 // Each block counts for its rows and pushes its counts to the cluster's first block.  On a B200, 64
 // thresholds: 4096 x 8 13.5 -> 4.6 us, 32768 x 20 245 -> 24 us (a block per threshold before, its
 // threads walking rows in global memory one dependent load at a time).
-template <int CS>
+template <int CS, int AT>
 __global__ void __launch_bounds__(kTuneThreads) fsd_threshold_sweep_kernel(const float* __restrict__ D, int B, int G,
                                                                            const float* __restrict__ thresholds, int n_thresholds, int cmp,
                                                                            float* __restrict__ mean_len, float* __restrict__ frac, int silent) {
     extern __shared__ __align__(16) float tune_buf[];
     __shared__ uint64_t bar[2], link[2];
-    __shared__ unsigned int part[kTuneThreads / 32][kSweepAtOnce];
-    __shared__ uint64_t got[2][kTuneCluster][kSweepAtOnce];      // (B * positions fits an int); kTuneLost: not to be relied on
+    __shared__ unsigned int part[kTuneThreads / 32][AT];
+    __shared__ uint64_t got[2][kTuneCluster][AT];      // (B * positions fits an int); kTuneLost: not to be relied on
     __shared__ int lost;                              // a wait of some thread of this block has run out
     const int rank = CS == 1 ? 0 : static_cast<int>(cg::this_cluster().block_rank());
     const int n_clusters = static_cast<int>(gridDim.x) / CS, cid = static_cast<int>(blockIdx.x) / CS;
@@ -188,61 +190,64 @@ __global__ void __launch_bounds__(kTuneThreads) fsd_threshold_sweep_kernel(const
     if constexpr (CS > 1) cg::this_cluster().barrier_arrive();   // "this block's barriers are ready": waited for before the first push
     launch_in_turn();
     TuneRows rows = tune_rows(D, B, G, rank, CS, tune_buf, bar, FSD_TUNE_SILENT);
-    // thresholds cid, cid + n_clusters, ...: kSweepAtOnce of them in one walk
+    // thresholds cid, cid + n_clusters, ...: AT of them in one walk
     int turn = 0;
-    for (int t0 = cid; t0 < n_thresholds; t0 += n_clusters * kSweepAtOnce, ++turn) {
-        float T[kSweepAtOnce];
-        unsigned int n[kSweepAtOnce];
+    for (int t0 = cid; t0 < n_thresholds; t0 += n_clusters * AT, ++turn) {
+        float T[AT];
+        unsigned int n[AT];
 #pragma unroll
-        for (int j = 0; j < kSweepAtOnce; ++j) {
+        for (int j = 0; j < AT; ++j) {
             const int t = t0 + j * n_clusters;
             T[j] = t < n_thresholds ? thresholds[t] : __int_as_float(0x7fc00000);
             n[j] = 0;
         }
-        float p = 0.f;
+        float p = 0.f, most = T[0];
+#pragma unroll
+        for (int j = 1; j < AT; ++j) most = fmaxf(most, T[j]);       // (a NaN threshold is no threshold)
         const auto begin = [&] { p = -INFINITY; };
+        const auto stop = [&] { return !(p <= most); };              // nothing passes from here on (a row's rest was never read)
         if (cmp == FSD_CMP_LE) {
             tune_walk(rows, begin, [&](float d) {
                 p = fmax_nan(p, d);                   // NaN stays and never passes
 #pragma unroll
-                for (int j = 0; j < kSweepAtOnce; ++j) n[j] += p <= T[j];
-            }, [] {});
+                for (int j = 0; j < AT; ++j) n[j] += p <= T[j];
+            }, stop, [] {});
         } else {
             tune_walk(rows, begin, [&](float d) {
                 p = fmax_nan(p, d);
 #pragma unroll
-                for (int j = 0; j < kSweepAtOnce; ++j) n[j] += p < T[j];
-            }, [] {});
+                for (int j = 0; j < AT; ++j) n[j] += p < T[j];
+            }, stop, [] {});
         }
 #pragma unroll
-        for (int j = 0; j < kSweepAtOnce; ++j) {
+        for (int j = 0; j < AT; ++j) {
             const unsigned int w = __reduce_add_sync(0xffffffffu, n[j]);
             if (lane == 0) part[warp][j] = w;
         }
         if (rows.wait.lost) lost = 1;
         __syncthreads();
         uint64_t sum = 0;
-        if (tid < kSweepAtOnce)
+        if (tid < AT)
             for (int w = 0; w < static_cast<int>(blockDim.x >> 5); ++w) sum += part[w][tid];
         if (lost) sum = kTuneLost;
         if constexpr (CS > 1) {
             // (two buffers take turns; nobody is a turn ahead by more than one: see the barrier below)
             if (turn == 0) cg::this_cluster().barrier_wait();
-            if (rank == 0 && tid == 0 && !rows.wait.lost) mbar_arrive_expect_tx(&link[turn & 1], CS * kSweepAtOnce * 8);
-            if (tid < kSweepAtOnce && !(FSD_TUNE_SILENT && rank == CS - 1))
+            if (rank == 0 && tid == 0 && !rows.wait.lost) mbar_arrive_expect_tx(&link[turn & 1], CS * AT * 8);
+            if (tid < AT && !(FSD_TUNE_SILENT && rank == CS - 1))
                 st_async(cluster_addr(&got[turn & 1][rank][tid], 0), sum, cluster_addr(&link[turn & 1], 0));
             if (rank == 0 && tid < 32) {
                 rows.wait(&link[turn & 1], (turn >> 1) & 1);
-                if (tid < kSweepAtOnce) {
+                if (tid < AT) {
                     bool all = !rows.wait.lost;
                     sum = 0;
                     for (int r = 0; r < CS; ++r) { sum += got[turn & 1][r][tid]; all = all && got[turn & 1][r][tid] != kTuneLost; }
                     if (!all) sum = kTuneLost;
                 }
             }
-            if (t0 + n_clusters * kSweepAtOnce < n_thresholds) cg::this_cluster().sync();   // more walks than one: nobody overtakes block 0
+            if (t0 + n_clusters * AT < n_thresholds) cg::this_cluster().sync();   // more walks than one: nobody overtakes block 0
         }
-        if (rank == 0 && tid < kSweepAtOnce && t0 + tid * n_clusters < n_thresholds) {
+        if (rank == 0 && tid < AT && t0 + tid * n_clusters < n_thresholds) {
             const int t = t0 + tid * n_clusters;
             const float nan = __int_as_float(0x7fc00000);
             mean_len[t] = sum == kTuneLost ? nan : static_cast<float>(static_cast<double>(sum) / static_cast<double>(B));
@@ -269,7 +274,7 @@ __device__ __forceinline__ void for_prefix_maxima(TuneRows& rows, F f) {
                   key = kn;
                   ++run;
               },
-              [&] { f(key, run); });
+              [] { return false; }, [&] { f(key, run); });
 }
 
 constexpr int kTuneList = kTuneBins / kTuneCluster;                        // candidates that are ranked directly

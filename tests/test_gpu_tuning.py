@@ -131,3 +131,26 @@ def test_rows_that_are_staged_in_one_tile_in_several_and_not_at_all(B, G):
             need = int(np.ceil(np.float64(F(target)) * B))
             m, _ = tun.threshold_sweep(D, np.array([T, np.nextafter(F(T), F(-np.inf))], dtype=F), cmp)
             assert m[0] == got and round(float(m[0]) * B) >= need > round(float(m[1]) * B)
+
+
+@pytest.mark.parametrize("B,G,K", [(300, 200, 16), (300, 1000, 9), (40, 2301, 33), (513, 702, 5), (2100, 300, 7), (1, 20000, 5),
+                                   (4096, 8, 1000), (513, 3, 145), (513, 3, 144), (100, 33, 3000), (64, 6, 1185)])
+def test_long_rows_and_many_thresholds(B, G, K):
+    """Rows of which a tile has too few for the threads, either side of that rule; rows left at their first failure, at NaN
+    and at a threshold itself; more thresholds than eight a cluster."""
+    rng = np.random.default_rng(34)
+    D = rng.gamma(0.7, 0.12, size=(B, G)).clip(0, 0.6931).astype(F)
+    D[rng.random((B, G)) < 0.001] = np.nan
+    D[: B // 2] *= F(0.01)                                              # rows that pass nearly everything
+    Ts = rng.permutation(np.concatenate([np.linspace(0.0, 0.7, K - 2), [np.inf, D[0, 0]]]).astype(F))
+    for cmp in ("lt", "le"):
+        m, f = _gpu_sweep(D, Ts, cmp)
+        at = np.arange(K) if B * G * K < 3e7 else rng.choice(K, 12, replace=False)
+        om, of = tun.threshold_sweep(D, Ts[at], cmp)
+        assert np.array_equal(m[at], om) and np.array_equal(f[at], of)
+        reach = float(tun.threshold_sweep(D, np.array([np.inf], dtype=F), cmp)[0][0])
+        for target in (0.3 * reach, 0.9 * reach):
+            T, got = _gpu_calibrate(D, target, cmp)
+            need = int(np.ceil(np.float64(F(target)) * B))
+            m, _ = tun.threshold_sweep(D, np.array([T, np.nextafter(F(T), F(-np.inf))], dtype=F), cmp)
+            assert m[0] == got and round(float(np.float64(m[0]) * B)) >= need > round(float(np.float64(m[1]) * B))

@@ -766,11 +766,20 @@ struct Classed {
         else if (d >= lo) close_call(k, d, pa, pb);
     }
 };
-// The pass over bf16 vectors, by the table.  A function of its own: the registers of everything around it would
-// otherwise be spilled inside its loop.  About twenty instructions an entry (two of them shared-memory reads, four
-// double-precision).
-__device__ __noinline__ void classed_pass_bf16(const void* a_row, const void* b_row, const Share share, float hi, float lo,
-                                               const ExpTable<FSD_BF16>& bt, Classed& out) {
+// e^x on a pass' scale by the 256-entry table and the polynomial, whatever x is but NaN (0 below xmin); with k = 0, bit for bit
+// what the table of bf16 exponentials holds
+struct RowExp {
+    double nk;
+    float xmin;
+    __device__ __forceinline__ RowExp(double k) : nk(-k), xmin(static_cast<float>((k - 990.0) * kLn2D)) {}
+    __device__ __forceinline__ double operator()(float x, const double* table, const Exp2Consts& c) const { return exp2_of_logit(x, xmin, nk, table, c); }
+};
+// The pass over bf16 vectors.  A function of its own: the registers of everything around it would
+// otherwise be spilled inside its loop.  By the table about twenty instructions an entry (two of them shared-memory reads,
+// four double-precision); a lane with an entry outside it (a masked one, above all) computes its sixteen
+// instead, and so do all where the logits lie so far off 0 that they need a reference (`tabled` false).
+__device__ __noinline__ void classed_pass_bf16(const void* a_row, const void* b_row, const Share share, float hi, float lo, const bool tabled,
+                                               const RowExp ea, const RowExp eb, const ResidualShared& rs, const ExpTable<FSD_BF16>& bt, Classed& out) {
     const uint32_t table = smem_u32(bt.e);
     const int u0 = share.first + (threadIdx.x & 31), u1 = min(share.first + share.iters * 32, share.units);
     Classed c = out;
@@ -781,38 +790,40 @@ __device__ __noinline__ void classed_pass_bf16(const void* a_row, const void* b_
         const uint4 va = na, vb = nb;
         if (u + 32 < u1) { na = ldg_vec(a_row, u + 32); nb = ldg_vec(b_row, u + 32); }
         const int k = u * 8;
-        if (!in_table(va, vb)) {                      // an entry of the vectors is small, large or -inf
-#pragma unroll 1
-            for (int e = 0; e < 8; ++e) {
-                const float xa = load_logit<FSD_BF16>(a_row, k + e), xb = load_logit<FSD_BF16>(b_row, k + e);
-                c.entry(k + e, xa, xb, exp_bf16(xa, bt), exp_bf16(xb, bt), hi, lo);
-            }
-            continue;
-        }
         const uint32_t wa[4] = {va.x, va.y, va.z, va.w}, wb[4] = {vb.x, vb.y, vb.z, vb.w};
         bool close = false;
+        const auto add = [&](float xa, float xb, double pa, double pb) {
+            const float d = xa - xb;                  // (both -inf: NaN, no weight)
+            const double one = __hiloint2double(d > hi ? 0x3ff00000 : 0, 0);
+            c.za += pa;
+            c.zb += pb;
+            c.sa = fma(pa, one, c.sa);
+            c.sb = fma(pb, one, c.sb);
+            close = close || (d >= lo && !(d > hi));  // (as in Classed::entry: between the bounds, both included)
+        };
+        if (tabled && in_table(va, vb)) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            double pa[2], pb[2];
-            table_exp2(wa[q], table, pa[0], pa[1]);
-            table_exp2(wb[q], table, pb[0], pb[1]);
-            const float d[2] = {bf16_lo(wa[q]) - bf16_lo(wb[q]), bf16_hi(wa[q]) - bf16_hi(wb[q])};
+            for (int q = 0; q < 4; ++q) {
+                double pa[2], pb[2];
+                table_exp2(wa[q], table, pa[0], pa[1]);
+                table_exp2(wb[q], table, pb[0], pb[1]);
+                add(bf16_lo(wa[q]), bf16_lo(wb[q]), pa[0], pb[0]);
+                add(bf16_hi(wa[q]), bf16_hi(wb[q]), pa[1], pb[1]);
+            }
+        } else {
+            const Exp2Consts ec = exp2_consts(rs.exp_consts);
 #pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const double one = __hiloint2double(d[e] > hi ? 0x3ff00000 : 0, 0);
-                c.za += pa[e];
-                c.zb += pb[e];
-                c.sa = fma(pa[e], one, c.sa);
-                c.sb = fma(pb[e], one, c.sb);
-                close = close || (d[e] >= lo && !(d[e] > hi));         // (as in Classed::entry: between the bounds, both included)
+            for (int q = 0; q < 4; ++q) {
+                add(bf16_lo(wa[q]), bf16_lo(wb[q]), ea(bf16_lo(wa[q]), rs.exp_table, ec), eb(bf16_lo(wb[q]), rs.exp_table, ec));
+                add(bf16_hi(wa[q]), bf16_hi(wb[q]), ea(bf16_hi(wa[q]), rs.exp_table, ec), eb(bf16_hi(wb[q]), rs.exp_table, ec));
             }
         }
         if (close) {
-#pragma unroll
+#pragma unroll 1
             for (int e = 0; e < 8; ++e) {
-                const float xa = (e & 1) ? bf16_hi(wa[e >> 1]) : bf16_lo(wa[e >> 1]), xb = (e & 1) ? bf16_hi(wb[e >> 1]) : bf16_lo(wb[e >> 1]);
-                const float d = xa - xb;
-                if (d >= lo && !(d > hi)) c.close_call(k + e, d, exp_bf16(xa, bt), exp_bf16(xb, bt));
+                const float xa = load_logit<FSD_BF16>(a_row, k + e), xb = load_logit<FSD_BF16>(b_row, k + e), d = xa - xb;
+                const Exp2Consts ec = exp2_consts(rs.exp_consts);
+                if (d >= lo && !(d > hi)) c.close_call(k + e, d, ea(xa, rs.exp_table, ec), eb(xb, rs.exp_table, ec));
             }
         }
     }
@@ -848,7 +859,7 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
     //      common to the cluster; without a record one pass for the CTA-local maxima (exact) ----
     double kra = 0.0, krb = 0.0;
     double zea = 0.0, zeb = 0.0, ln_rho = 0.0;
-    bool common = false;
+    bool common = false, tabled = false;
     if (P.records != nullptr) {
         PairRef ref;
         ref.za = 0.0; ref.zb = 0.0; ref.ln_rho = 0.0; ref.ka = __int_as_float(0x7fc00000); ref.kb = ref.ka;
@@ -861,14 +872,11 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
         if (isfinite(ref.ka) && isfinite(ref.kb)) {
             kra = ref.ka; krb = ref.kb; zea = ref.za; zeb = ref.zb;
             ln_rho = ref.ln_rho + (kra - krb) * kLn2D;
-            if constexpr (DT == FSD_BF16) {
-                // plain e^x (no reference) as long as it neither overflows nor leaves the table for good: largest logits of
-                // about -64 to 64 (a record's reference can be 2^30 below its row's largest entry, no more)
-                common = fabsf(ref.ka) <= 92.f && fabsf(ref.kb) <= 92.f;
-                if (common) { zea *= pow2_any(static_cast<int>(ref.ka)); zeb *= pow2_any(static_cast<int>(ref.kb)); }
-            } else {
-                common = true;
-            }
+            common = true;
+            // bf16: plain e^x (no reference), by the table, as long as it neither overflows nor leaves the table for good: largest
+            // logits of about -64 to 64 (a record's reference can be 2^30 below its row's largest entry, no more)
+            tabled = DT == FSD_BF16 && fabsf(ref.ka) <= 92.f && fabsf(ref.kb) <= 92.f;
+            if (tabled) { zea *= pow2_any(static_cast<int>(ref.ka)); zeb *= pow2_any(static_cast<int>(ref.kb)); kra = 0.0; krb = 0.0; }
         }
     }
     float mx[2] = {-INFINITY, -INFINITY};
@@ -881,12 +889,11 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
     }
     const double Ra = common ? 0.0 : mx[0], Rb = common ? 0.0 : mx[1];   // this CTA's references (logit domain)
 
-    // fp32 with common references: y = x * log2e - k; logits below xmin give 2^y < 2^-990 and count as 0
+    // common references: y = x * log2e - k; logits below xmin give 2^y < 2^-990 and count as 0
     const Exp2Consts ec = exp2_consts(rs.exp_consts);
-    const double nka = -kra, nkb = -krb;
-    const float xmin_a = static_cast<float>((kra - 990.0) * kLn2D), xmin_b = static_cast<float>((krb - 990.0) * kLn2D);
-    auto exp_a = [&](float x) -> double { if constexpr (DT == FSD_BF16) return exp_bf16(x, bt); else return exp2_of_logit(x, xmin_a, nka, tab, ec); };
-    auto exp_b = [&](float x) -> double { if constexpr (DT == FSD_BF16) return exp_bf16(x, bt); else return exp2_of_logit(x, xmin_b, nkb, tab, ec); };
+    const RowExp ea(kra), eb(krb);
+    auto exp_a = [&](float x) -> double { if constexpr (DT == FSD_BF16) { if (tabled) return exp_bf16(x, bt); } return ea(x, tab, ec); };
+    auto exp_b = [&](float x) -> double { if constexpr (DT == FSD_BF16) { if (tabled) return exp_bf16(x, bt); } return eb(x, tab, ec); };
 
     // ---- global normalisers of both rows (double) ----
     double Ma, Mb, iZa = 0.0, iZb = 0.0;
@@ -914,7 +921,7 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
         const float hi = static_cast<float>(ln_rho + margin), lo = static_cast<float>(ln_rho - margin);
         bool done = false;
         if constexpr (DT == FSD_BF16) {
-            if (d.vec) { classed_pass_bf16(a_row, b_row, row_share(d.V / 8, cs, rank, warp), hi, lo, bt, c); done = true; }
+            if (d.vec) { classed_pass_bf16(a_row, b_row, row_share(d.V / 8, cs, rank, warp), hi, lo, tabled, ea, eb, rs, bt, c); done = true; }
         }
         if (!done) for_units<DT>(d, warp, lane, true, [&](int k, float xa, float xb) { c.entry(k, xa, xb, exp_a(xa), exp_b(xb), hi, lo); });
         if (!classify || c.close > 2) {
@@ -977,7 +984,7 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
     auto vector_weights = [&](int u, double (&w)[EPV]) {
         if constexpr (DT == FSD_BF16) {
             const uint4 va = ldg_vec(a_row, u), vb = ldg_vec(b_row, u);
-            if (in_table(va, vb)) {
+            if (tabled && in_table(va, vb)) {
                 const uint32_t wa[4] = {va.x, va.y, va.z, va.w}, wb[4] = {vb.x, vb.y, vb.z, vb.w}, table = smem_u32(bt.e);
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {

@@ -152,3 +152,24 @@ def test_judging_shared_by_the_cluster(N, B, V):
     c = gi.make_chain(B, min(N, 70), V, dtype="bf16", recipe="zipf", sigma=(0.05, 0.4), sigma_mode="uniform", workload_id=904)
     _check(c, T=0.06)
     _check(c, mode="sd")
+
+
+@pytest.mark.parametrize("offsets", [(-100.0, -100.0), (0.0, 100.0), (-300.0, -20.0)])
+@pytest.mark.parametrize("V", [24000, 24003])
+def test_residual_of_bf16_rows_off_the_table_with_close_calls_and_masked_entries(offsets, V):
+    """Rows too far from 0 for the table of exponentials (one of them or both), entries on which they agree but for
+    the offset, and entries that one row or both mask."""
+    c = gi.make_chain(5, 2, V, dtype="bf16", recipe="spike", sigma=(0.5,), workload_id=906)
+    t, d = _wide(c)
+    t = np.round(t * 2.0)                                           # bf16 numbers with the offsets on them, too
+    d[:] = np.roll(t[:, :2], V // 3, axis=2) + offsets[1]
+    t += offsets[0]
+    t[:, :, 100:140] = -np.inf
+    d[:, :, 120:200] = -np.inf
+    _store(c, t, d)
+    c.draft_tokens[:] = d.argmax(axis=2)                            # proposed where q is far above p: rejected
+    c.u_accept[:] = 0.999
+    r = _check(c, mode="sd")
+    assert (r["accept_len"] < 2).any()
+    _check(c, mode="sd", sample="greedy")
+    _check(c, mode="rfsd", T=0.0)

@@ -235,7 +235,7 @@ int fsd_set_stage_event(void *event);
 int fsd_set_timeout_injection(int mode);
 
 /* Test and tuning aid (no counterpart in the paper).  The streaming kernel splits every
- * (row, position) pair along the vocabulary over a group of 1..16 thread blocks; the library
+ * (row, position) pair along the vocabulary over a group of 1..24 thread blocks; the library
  * picks the group size from the row length and the number of pairs.  A nonzero `group_size`
  * replaces that choice in later verify calls wherever it is possible (at least the smallest
  * size whose slice fits on chip, at most 16; otherwise the library's own choice stands); 0

@@ -35,14 +35,14 @@
 // kernel takes 92 us there (3.4 TB/s; the form in which all warps of a block waited for the group's
 // totals between the two sweeps of a pair took 127 us): 40 rounds of 2.0 us, of which the sweeps are
 // two thirds, the wait for data and totals a sixth, the fold a seventh, plus 3.5 us until the first
-// slices have landed.  KL has no second sweep and no exchange and runs at 4.7 TB/s.  Of what was
+// slices have landed.  KL has no second sweep and no exchange and runs at 5 TB/s.  Of what was
 // tried on it: ex2 on the FMA pipe for a part of the entries (+8 %, the extra instructions cost more
 // than the special-function pipe gains), five and more pairs in flight in smaller parts (more rounds,
 // the fold weighs more), reading the references from a full pass over the part (+1 %).
 //
 // Rows that are not whole 16-byte vectors (or start off a 16-byte boundary) are streamed as the
 // aligned 16-byte granules that cover them; the draft row's granules are shifted onto the target
-// row's in registers and the entries in front of and behind the rows are read as -inf.  A granule
+// row's in shared memory, in place, and the entries in front of and behind the rows become -1e30.  A granule
 // that holds at least one byte of a row never crosses into another page.
 #pragma once
 
@@ -245,11 +245,6 @@ __device__ __forceinline__ float fmax_nan(float a, float b) {
     asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
     return d;
 }
-__device__ __forceinline__ float warp_max_nan(float v) {
-#pragma unroll
-    for (int m = 16; m > 0; m >>= 1) v = fmax_nan(v, __shfl_xor_sync(0xffffffffu, v, m));
-    return v;
-}
 // ---- packed pairs of floats (one instruction works on two values) --------------------------
 __device__ __forceinline__ uint64_t pack2(float lo, float hi) {
     uint64_t r;
@@ -278,12 +273,6 @@ __device__ __forceinline__ float sum2(uint64_t v) {
     float lo, hi;
     unpack2(v, lo, hi);
     return lo + hi;
-}
-
-// 2^d for an integer-valued d <= 0 (exact); 0 below the normal range and for d = -inf; NaN for NaN
-__device__ __forceinline__ float pow2_int(float d) {
-    if (d != d) return d;
-    return d < -126.f ? 0.f : __int_as_float((static_cast<int>(d) + 127) << 23);
 }
 
 // 2^(k - K) for integer-valued k <= K, exact; 0 below the normal range, for k = -inf ("no reference"), and where

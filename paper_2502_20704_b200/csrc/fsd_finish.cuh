@@ -20,7 +20,7 @@
 // u * total lies further than that from both ends of its interval, and a neighbour otherwise.
 // Drawing from the SD residual max(0, P_T - P_D) (Eq. 3) subtracts nearly equal numbers, so there the
 // exponentials are double precision and the sums agree with a sequential double sum to rounding.
-// bf16 logits have few values: e^x comes from a table of all bf16 numbers between 2^-9 and 64 of either
+// bf16 logits have few values: e^x comes from a table of all bf16 numbers between 2^-13 and 64 of either
 // sign (built while the streaming kernel drains), which leaves two shared-memory reads and four
 // double-precision instructions an entry.  fp32 logits take a 256-entry table times a degree-4
 // polynomial (about forty instructions).  Usually one pass over the two rows suffices: which
@@ -774,12 +774,11 @@ struct RowExp {
     __device__ __forceinline__ RowExp(double k) : nk(-k), xmin(static_cast<float>((k - 990.0) * kLn2D)) {}
     __device__ __forceinline__ double operator()(float x, const double* table, const Exp2Consts& c) const { return exp2_of_logit(x, xmin, nk, table, c); }
 };
-// The pass over bf16 vectors.  A function of its own: the registers of everything around it would
-// otherwise be spilled inside its loop.  By the table about twenty instructions an entry (two of them shared-memory reads,
-// four double-precision); a lane with an entry outside it (a masked one, above all) computes its sixteen
-// instead, and so do all where the logits lie so far off 0 that they need a reference (`tabled` false).
-__device__ __noinline__ void classed_pass_bf16(const void* a_row, const void* b_row, const Share share, float hi, float lo, const bool tabled,
-                                               const RowExp ea, const RowExp eb, const ResidualShared& rs, const ExpTable<FSD_BF16>& bt, Classed& out) {
+// The pass over bf16 vectors, by the table.  A function of its own: the registers of everything around it would
+// otherwise be spilled inside its loop.  About twenty instructions an entry (two of them shared-memory reads, four
+// double-precision).
+__device__ __noinline__ void classed_pass_bf16(const void* a_row, const void* b_row, const Share share, float hi, float lo,
+                                               const ExpTable<FSD_BF16>& bt, Classed& out) {
     const uint32_t table = smem_u32(bt.e);
     const int u0 = share.first + (threadIdx.x & 31), u1 = min(share.first + share.iters * 32, share.units);
     Classed c = out;
@@ -790,9 +789,62 @@ __device__ __noinline__ void classed_pass_bf16(const void* a_row, const void* b_
         const uint4 va = na, vb = nb;
         if (u + 32 < u1) { na = ldg_vec(a_row, u + 32); nb = ldg_vec(b_row, u + 32); }
         const int k = u * 8;
+        if (!in_table(va, vb)) {                      // an entry of the vectors is small, large or -inf
+#pragma unroll 1
+            for (int e = 0; e < 8; ++e) {
+                const float xa = load_logit<FSD_BF16>(a_row, k + e), xb = load_logit<FSD_BF16>(b_row, k + e);
+                c.entry(k + e, xa, xb, exp_bf16(xa, bt), exp_bf16(xb, bt), hi, lo);
+            }
+            continue;
+        }
         const uint32_t wa[4] = {va.x, va.y, va.z, va.w}, wb[4] = {vb.x, vb.y, vb.z, vb.w};
         bool close = false;
-        const auto add = [&](float xa, float xb, double pa, double pb) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            double pa[2], pb[2];
+            table_exp2(wa[q], table, pa[0], pa[1]);
+            table_exp2(wb[q], table, pb[0], pb[1]);
+            const float d[2] = {bf16_lo(wa[q]) - bf16_lo(wb[q]), bf16_hi(wa[q]) - bf16_hi(wb[q])};
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const double one = __hiloint2double(d[e] > hi ? 0x3ff00000 : 0, 0);
+                c.za += pa[e];
+                c.zb += pb[e];
+                c.sa = fma(pa[e], one, c.sa);
+                c.sb = fma(pb[e], one, c.sb);
+                close = close || (d[e] >= lo && !(d[e] > hi));         // (as in Classed::entry: between the bounds, both included)
+            }
+        }
+        if (close) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const float xa = (e & 1) ? bf16_hi(wa[e >> 1]) : bf16_lo(wa[e >> 1]), xb = (e & 1) ? bf16_hi(wb[e >> 1]) : bf16_lo(wb[e >> 1]);
+                const float d = xa - xb;
+                if (d >= lo && !(d > hi)) c.close_call(k + e, d, exp_bf16(xa, bt), exp_bf16(xb, bt));
+            }
+        }
+    }
+    out = c;
+}
+// The same for rows whose logits lie so far off 0 that most are outside the table, or that they need a reference: every
+// exponential by the small table and the polynomial, in straight-line code (in the loop above, for the lanes that meet an entry
+// outside the table, it cost the other rows 9 %: 64 x 8 x 152064, strict rule, 133 -> 145 us).
+__device__ __noinline__ void classed_pass_far(const void* a_row, const void* b_row, const Share share, float hi, float lo,
+                                              const RowExp ea, const RowExp eb, const ResidualShared& rs, Classed& out) {
+    const int u0 = share.first + (threadIdx.x & 31), u1 = min(share.first + share.iters * 32, share.units);
+    Classed c = out;
+    uint4 na = make_uint4(0, 0, 0, 0), nb = na;       // the vectors after these, on their way
+    if (u0 < u1) { na = ldg_vec(a_row, u0); nb = ldg_vec(b_row, u0); }
+#pragma unroll 1
+    for (int u = u0; u < u1; u += 32) {
+        const uint4 va = na, vb = nb;
+        if (u + 32 < u1) { na = ldg_vec(a_row, u + 32); nb = ldg_vec(b_row, u + 32); }
+        const int k = u * 8;
+        const uint32_t wa[4] = {va.x, va.y, va.z, va.w}, wb[4] = {vb.x, vb.y, vb.z, vb.w};
+        const Exp2Consts ec = exp2_consts(rs.exp_consts);
+        bool close = false;
+        const auto add = [&](float xa, float xb) {
+            const double pa = ea(xa, rs.exp_table, ec), pb = eb(xb, rs.exp_table, ec);
             const float d = xa - xb;                  // (both -inf: NaN, no weight)
             const double one = __hiloint2double(d > hi ? 0x3ff00000 : 0, 0);
             c.za += pa;
@@ -801,28 +853,12 @@ __device__ __noinline__ void classed_pass_bf16(const void* a_row, const void* b_
             c.sb = fma(pb, one, c.sb);
             close = close || (d >= lo && !(d > hi));  // (as in Classed::entry: between the bounds, both included)
         };
-        if (tabled && in_table(va, vb)) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                double pa[2], pb[2];
-                table_exp2(wa[q], table, pa[0], pa[1]);
-                table_exp2(wb[q], table, pb[0], pb[1]);
-                add(bf16_lo(wa[q]), bf16_lo(wb[q]), pa[0], pb[0]);
-                add(bf16_hi(wa[q]), bf16_hi(wb[q]), pa[1], pb[1]);
-            }
-        } else {
-            const Exp2Consts ec = exp2_consts(rs.exp_consts);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                add(bf16_lo(wa[q]), bf16_lo(wb[q]), ea(bf16_lo(wa[q]), rs.exp_table, ec), eb(bf16_lo(wb[q]), rs.exp_table, ec));
-                add(bf16_hi(wa[q]), bf16_hi(wb[q]), ea(bf16_hi(wa[q]), rs.exp_table, ec), eb(bf16_hi(wb[q]), rs.exp_table, ec));
-            }
-        }
+        for (int q = 0; q < 4; ++q) { add(bf16_lo(wa[q]), bf16_lo(wb[q])); add(bf16_hi(wa[q]), bf16_hi(wb[q])); }
         if (close) {
 #pragma unroll 1
             for (int e = 0; e < 8; ++e) {
                 const float xa = load_logit<FSD_BF16>(a_row, k + e), xb = load_logit<FSD_BF16>(b_row, k + e), d = xa - xb;
-                const Exp2Consts ec = exp2_consts(rs.exp_consts);
                 if (d >= lo && !(d > hi)) c.close_call(k + e, d, ea(xa, rs.exp_table, ec), eb(xb, rs.exp_table, ec));
             }
         }
@@ -873,9 +909,10 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
             kra = ref.ka; krb = ref.kb; zea = ref.za; zeb = ref.zb;
             ln_rho = ref.ln_rho + (kra - krb) * kLn2D;
             common = true;
-            // bf16: plain e^x (no reference), by the table, as long as it neither overflows nor leaves the table for good: largest
-            // logits of about -64 to 64 (a record's reference can be 2^30 below its row's largest entry, no more)
-            tabled = DT == FSD_BF16 && fabsf(ref.ka) <= 92.f && fabsf(ref.kb) <= 92.f;
+            // bf16: plain e^x (no reference), by the table, as long as it does not overflow and most entries are in the table: largest
+            // logits of about -44 (rows reach some 20 below) to 64 (a record's reference can be 2^30 below its row's largest entry,
+            // no more).  16 x 5 x 50264, strict rule, logits 60 below 0: 48 us by the table
+            tabled = DT == FSD_BF16 && fminf(ref.ka, ref.kb) >= -64.f && fmaxf(ref.ka, ref.kb) <= 92.f;
             if (tabled) { zea *= pow2_any(static_cast<int>(ref.ka)); zeb *= pow2_any(static_cast<int>(ref.kb)); kra = 0.0; krb = 0.0; }
         }
     }
@@ -900,7 +937,7 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
     bool residual = true;
     // One pass instead of two, where it can be shown to give the same sums.  An entry has residual
     // weight iff e_a / Z_a > e_b / Z_b, i.e. e_a > rho * e_b with rho = Z_a / Z_b, which is known
-    // only after the pass -- but the record gives rho to about 1e-6.  Entries are classed against
+    // only after the pass -- but the record gives rho to about 2e-7.  Entries are classed against
     // rho_est * (1 +- margin): for those clearly above, e_a and e_b are summed separately, and their
     // residual weight is then sum e_a / Z_a - sum e_b / Z_b with the exact normalisers.
     // The few entries between the two bounds are settled with the exact normalisers afterwards: bf16 logits
@@ -921,9 +958,15 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
         const float hi = static_cast<float>(ln_rho + margin), lo = static_cast<float>(ln_rho - margin);
         bool done = false;
         if constexpr (DT == FSD_BF16) {
-            if (d.vec) { classed_pass_bf16(a_row, b_row, row_share(d.V / 8, cs, rank, warp), hi, lo, tabled, ea, eb, rs, bt, c); done = true; }
+            const Share share = row_share(d.V / 8, cs, rank, warp);
+            if (d.vec && tabled) classed_pass_bf16(a_row, b_row, share, hi, lo, bt, c);
+            else if (d.vec) classed_pass_far(a_row, b_row, share, hi, lo, ea, eb, rs, c);
+            done = d.vec;
         }
-        if (!done) for_units<DT>(d, warp, lane, true, [&](int k, float xa, float xb) { c.entry(k, xa, xb, exp_a(xa), exp_b(xb), hi, lo); });
+        if constexpr (DT == FSD_BF16) {               // (a loop of its own: with the choice inside it, 8 x 5 x 50257 28.7 -> 31.0 us)
+            if (!done && tabled) { for_units<DT>(d, warp, lane, true, [&](int k, float xa, float xb) { c.entry(k, xa, xb, exp_bf16(xa, bt), exp_bf16(xb, bt), hi, lo); }); done = true; }
+        }
+        if (!done) for_units<DT>(d, warp, lane, true, [&](int k, float xa, float xb) { c.entry(k, xa, xb, ea(xa, tab, ec), eb(xb, tab, ec), hi, lo); });
         if (!classify || c.close > 2) {
             atomicOr(&sh.amb, 1);
         } else if (c.qd == c.qd) {

@@ -118,8 +118,8 @@ int fsd_workspace_bytes(int B, int positions, int V, const fsd_opts *opts, size_
  *   workspace     device scratch, 256-byte aligned, at least fsd_workspace_bytes() bytes;
  *                 contents need not be initialised and are not preserved
  * Calls that share a workspace must be ordered on the stream(s) that use it.
- * The call enqueues two kernels (the first of at most one thread block per SM, both with
- * programmatic stream serialization) and nothing else, so it can be captured in a CUDA graph and replayed --
+ * The call enqueues one kernel (where all logits fit on chip at once: a thread-block cluster per row) or two (the first of at
+ * most one thread block per SM), with programmatic stream serialization, and nothing else, so it can be captured in a CUDA graph and replayed --
  * after one ordinary call with the same options on that device, which sets the kernels'
  * attributes (that cannot be done under capture). */
 int fsd_verify_chain(const void *target_logits, const void *draft_logits,
@@ -208,7 +208,7 @@ int fsd_version(void);
 /* Measurement aid (no counterpart in the paper).  While an event is set, every verify call
  * records it (cudaEventRecord) on the call's stream between its pair kernel and its finish
  * kernel, so a caller that brackets the call with two events of its own can time the two
- * kernels separately.  `event` is a cudaEvent_t passed as void*, owned by the caller; NULL
+ * kernels separately; calls that would take one kernel take the two.  `event` is a cudaEvent_t passed as void*, owned by the caller; NULL
  * clears the hook.  Process-wide and not synchronised with calls in flight on other host
  * threads: set it, make the calls to be measured, clear it.  The record between the two
  * kernels also keeps the finish kernel from being set up early, so timings taken with the hook
@@ -218,17 +218,19 @@ int fsd_set_stage_event(void *event);
 /* Test aid (no counterpart in the paper).  Every wait inside the streaming kernel is bounded; a
  * wait that runs out raises a flag in the workspace, the thread blocks that see it take no
  * further work, the call still returns, and every row's row_status carries FSD_ROW_TIMEOUT (its
- * other outputs are then not valid).  The finish kernel's waits within a cluster end the same way.
+ * other outputs are then not valid).  The finish kernel's waits within a cluster end the same way; where
+ * one kernel does the whole call, a row is marked when a wait of its own cluster runs out.
  * The flag is that call's own, and of a call in a graph that
  * replay's.  mode 1: the streaming kernel's first block raises that flag as it ends, which
  * exercises the reporting path alone.  mode 2: in the
  * streaming kernel one thread block keeps its first statistics message to itself and the limit
  * of the exchange wait is lowered to about a tenth of a second, so its partners' wait really
  * runs out and the kernel's own give-up path runs (every wait stays bounded; nothing faults).
+ * (Where one kernel does the call, one block of each cluster keeps its first sums to itself under a limit of 20 ms.)
  * mode 3, in a build with -DFSD_DEBUG_CHECKS only: the block keeps its message to itself and the
  * others do without, as they do when a block of a group is not running: they compute what it would
  * have sent after about a millisecond (ordinarily fifteen), and the call's results are the same.
- * mode 4, in such a build only: in the finish kernel and in the tuning kernels one block of each
+ * mode 4, in such a build only: in the finish kernel, the one kernel of a small call and the tuning kernels one block of each
  * cluster keeps its first values to itself, and the limit of their waits is lowered to 20 ms.
  * mode 0: off (the default).  Process-wide, read when a call is made.  Returns FSD_OK, or
  * FSD_ERR_ENUM for another mode. */
@@ -237,7 +239,7 @@ int fsd_set_timeout_injection(int mode);
 /* Test and tuning aid (no counterpart in the paper).  The streaming kernel splits every
  * (row, position) pair along the vocabulary over a group of 1..24 thread blocks; the library
  * picks the group size from the row length and the number of pairs.  A nonzero `group_size`
- * replaces that choice in later verify calls wherever it is possible (at least the smallest
+ * makes later verify calls take the streaming kernel and replaces that choice wherever it is possible (at least the smallest
  * size whose slice fits on chip, at most 16; otherwise the library's own choice stands); 0
  * restores the library's choice.  Results do not depend on the group size beyond the order of
  * floating-point additions.  Process-wide, read when a call is made.  Returns FSD_OK, or

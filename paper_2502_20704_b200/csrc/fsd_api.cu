@@ -13,6 +13,7 @@
 #include "fsd_finish.cuh"
 #include "fsd_pair_generic.cuh"
 #include "fsd_pair_stream.cuh"
+#include "fsd_row.cuh"
 #include "fsd_tuning.cuh"
 
 namespace {
@@ -75,7 +76,7 @@ int check_shape(int B, int G, int V) {
 // batch is large.
 int finish_cluster_size(int B, int G, int V) {
     int cs = 1;
-    while (cs < kMaxClusterSize && (static_cast<long long>(cs) * kFinishThreads * 8 < V || cs * kFinishWarps < G) &&
+    while (cs < kPortableCluster && (static_cast<long long>(cs) * kFinishThreads * 8 < V || cs * kFinishWarps < G) &&
            static_cast<long long>(B) * cs * 2 <= 2 * 148)
         cs <<= 1;
     return cs;
@@ -107,6 +108,50 @@ uint64_t next_nonce() {
 // ---- streaming kernel launch -----------------------------------------------------------
 constexpr int kMaxDev = 64;
 
+// Attributes of a kernel that takes all of an SM's shared memory, and how many clusters of each size from 1 to kMaxClusterSize the
+// device holds at once (0: none).  Puts nothing on a stream.
+template <typename K>
+bool prepare_clusters(K kernel, int threads, size_t smem, int* most) {
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess) return false;
+    const bool wide = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+    for (int cs = 1; cs <= kMaxClusterSize; ++cs) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(static_cast<unsigned>(256 * cs), 1, 1);
+        cfg.blockDim = dim3(static_cast<unsigned>(threads), 1, 1);
+        cfg.dynamicSmemBytes = smem;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = static_cast<unsigned>(cs); attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if ((cs <= kPortableCluster || wide) && cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) n = 0;
+        most[cs - 1] = n;
+    }
+    cudaGetLastError();                                                // (a size the device refuses is no error of this call's)
+    return true;
+}
+// How a kernel is launched in clusters, and set up while the kernel in front drains: it waits for that one's end itself.
+// (A kernel that stores into the shared memory of its cluster's blocks needs the attribute also where a cluster is one block:
+// without it the store is an illegal instruction.)  cs 0: no clusters, single blocks (with the attribute the streaming kernel
+// takes 0.3 us more).
+struct ClusterLaunch {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[2];
+    ClusterLaunch(int clusters, int cs, int threads, size_t smem, cudaStream_t s) {
+        cfg.gridDim = dim3(static_cast<unsigned>(cs > 0 ? clusters * cs : clusters), 1, 1);
+        cfg.blockDim = dim3(static_cast<unsigned>(threads), 1, 1);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = s;
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        attr[1].id = cudaLaunchAttributeClusterDimension;
+        attr[1].val.clusterDim.x = static_cast<unsigned>(cs > 0 ? cs : 1); attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = cs > 0 ? 2 : 1;
+    }
+};
+
 // One block per SM.  Puts nothing on a stream.
 template <int DT, int DIV, bool RAGGED>
 int prepare_stream(int dev) {
@@ -133,32 +178,18 @@ int launch_stream(const StreamParams& gp, int nsm, cudaStream_t s) {
     int grid = nsm < kMaxBlocks ? nsm : kMaxBlocks;
     if (want < grid) grid = static_cast<int>(want);
     if (grid < gp.C) return FSD_ERR_CUDA;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(grid), 1, 1);
-    cfg.blockDim = dim3(kStreamThreads, 1, 1);
-    cfg.dynamicSmemBytes = kStreamSmemBytes;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    // Set up while the kernel in front drains; the kernel waits for its end itself.  (A cooperative launch ignores this.)
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, fsd_pair_stream_kernel<DT, DIV, RAGGED>, gp) != cudaSuccess) return FSD_ERR_CUDA;
-    return FSD_OK;
+    const ClusterLaunch l(grid, 0, kStreamThreads, kStreamSmemBytes, s);
+    return cudaLaunchKernelEx(&l.cfg, fsd_pair_stream_kernel<DT, DIV, RAGGED>, gp) == cudaSuccess ? FSD_OK : FSD_ERR_CUDA;
 }
 
 using PrepareFn = int (*)(int);
 using LaunchFn = int (*)(const StreamParams&, int, cudaStream_t);
-template <int DT> PrepareFn stream_prepare(int div, bool ragged) {
-    if (div == FSD_DIV_JS) return ragged ? prepare_stream<DT, FSD_DIV_JS, true> : prepare_stream<DT, FSD_DIV_JS, false>;
-    if (div == FSD_DIV_KL) return ragged ? prepare_stream<DT, FSD_DIV_KL, true> : prepare_stream<DT, FSD_DIV_KL, false>;
-    return ragged ? prepare_stream<DT, FSD_DIV_TV, true> : prepare_stream<DT, FSD_DIV_TV, false>;
+struct StreamKernel { PrepareFn prepare; LaunchFn launch; };
+template <int DT, int DIV> StreamKernel stream_kernel(bool ragged) {
+    return ragged ? StreamKernel{prepare_stream<DT, DIV, true>, launch_stream<DT, DIV, true>} : StreamKernel{prepare_stream<DT, DIV, false>, launch_stream<DT, DIV, false>};
 }
-template <int DT> LaunchFn stream_launch(int div, bool ragged) {
-    if (div == FSD_DIV_JS) return ragged ? launch_stream<DT, FSD_DIV_JS, true> : launch_stream<DT, FSD_DIV_JS, false>;
-    if (div == FSD_DIV_KL) return ragged ? launch_stream<DT, FSD_DIV_KL, true> : launch_stream<DT, FSD_DIV_KL, false>;
-    return ragged ? launch_stream<DT, FSD_DIV_TV, true> : launch_stream<DT, FSD_DIV_TV, false>;
+template <int DT> StreamKernel stream_kernel(int div, bool ragged) {
+    return div == FSD_DIV_JS ? stream_kernel<DT, FSD_DIV_JS>(ragged) : div == FSD_DIV_KL ? stream_kernel<DT, FSD_DIV_KL>(ragged) : stream_kernel<DT, FSD_DIV_TV>(ragged);
 }
 
 // Blocks per pair for the streaming kernel; 0 if the row is too long for the largest group (the
@@ -179,13 +210,72 @@ int group_size(int nvec_row, int items, int nsm) {
         const int groups = blocks / C;
         const int rounds = (items + groups - 1) / groups;
         const int slice = (nvec_row + C - 1) / C;
-        const int warp_steps = (slice + 32 * S::kVecPerStep - 1) / (32 * S::kVecPerStep);     // of a block
-        double round = 0.3 + 0.4 * warp_steps / kComputeWarps;
+        const int block_steps = (slice + (32 * S::kVecPerStep) - 1) / (32 * S::kVecPerStep);
+        double round = 0.3 + 0.4 * block_steps / kComputeWarps;
         if (round < 0.5 * (round + 1.6)) round = 0.5 * (round + 1.6);
         const double cost = rounds * round;
         if (best == 0 || cost < best_cost) { best = C; best_cost = cost; }
     }
     return best;
+}
+
+// ---- row kernel launch -----------------------------------------------------------------
+// Attributes, and how many clusters of each size the device holds at once.  Puts nothing on a stream.
+template <int DT, int KIND, bool RAGGED>
+const int* prepare_row(int dev) {
+    static int most[kMaxDev][kMaxClusterSize] = {};
+    static bool ready[kMaxDev] = {};
+    static std::mutex mu;
+    if (dev < 0 || dev >= kMaxDev) return nullptr;
+    std::lock_guard<std::mutex> lock(mu);
+    if (!ready[dev]) {
+        if (!prepare_clusters(fsd_row_kernel<DT, KIND, RAGGED>, kFinishThreads, kRowSmemBytes, most[dev])) return nullptr;
+        ready[dev] = true;
+    }
+    return most[dev];
+}
+// Blocks per batch row: the largest cluster of which the GPU holds one for every row at once (a second wave would take as long
+// as the first), whose blocks have room for the row's logits and what is parked of them.  Larger was faster throughout, or
+// within 2 %: us on a B200 by the streaming and finish kernels / in clusters of half the size / of the size taken:
+//   1 x 4 x 32000 fp32 11.6 / 10.1 / 9.3 (16)    16 x 5 x 32000 16.0 / - / 12.6 (6)    8 x 5 x 50257 16.6 / - / 13.6 (10)
+//   8 x 3 x 64000 13.7 / - / 11.4 (10)    28 x 5 x 8192 12.8 / 11.7 / 10.8 (4)    4 x 16 x 8000 12.1 / 10.8 / 10.2 (16)
+struct RowPlan { int cs, span; };                                      // cs 0: not by the row kernel
+template <int DT, int KIND, bool RAGGED>
+RowPlan row_plan(int B, int G, size_t nvec_row, const int* most) {
+    constexpr int step = 32 * StreamShape<DT>::kVecPerStep;
+    const RowPlan none = {0, 0};
+    if (G > kRowMaxPairs || nvec_row > static_cast<size_t>(kMaxClusterSize) * kRowMaxItems * step) return none;
+    for (int cs = kMaxClusterSize; cs >= 1; --cs) {
+        if (most[cs - 1] < B) continue;
+        const int span = (static_cast<int>((nvec_row + cs - 1) / cs) + step - 1) / step * step, steps = span / step;
+        if (steps * G > kRowMaxItems || row_bytes_of(G, span, RAGGED) > row_smem_left<DT, KIND>()) continue;
+        return {cs, span};
+    }
+    return none;
+}
+template <int DT, int KIND, bool RAGGED>
+int launch_row(const FinishParams& fp, int cs, int span, size_t nvec_row, uint64_t nonce, int injection, cudaStream_t s) {
+    RowParams rp;
+    rp.fin = fp;
+    rp.nvec_row = static_cast<int>(nvec_row); rp.span = span; rp.nonce = nonce;
+    rp.silent = injection == 2 || injection == 4;
+    rp.limit_ns = rp.silent ? kInjectedWaitNs : kWaitNs;
+    rp.raise = injection == 1;
+    const ClusterLaunch l(fp.B, cs, kFinishThreads, kRowSmemBytes, s);
+    return cudaLaunchKernelEx(&l.cfg, fsd_row_kernel<DT, KIND, RAGGED>, rp) == cudaSuccess ? FSD_OK : FSD_ERR_CUDA;
+}
+// One launch if the row kernel takes the call; `taken` says so.
+template <int DT, int KIND, bool RAGGED>
+int try_row(const FinishParams& fp, size_t nvec_row, int dev, uint64_t nonce, int injection, cudaStream_t s, bool& taken) {
+    const int* most = prepare_row<DT, KIND, RAGGED>(dev);
+    if (most == nullptr) return FSD_ERR_CUDA;
+    const RowPlan plan = row_plan<DT, KIND, RAGGED>(fp.B, fp.G, nvec_row, most);
+    taken = plan.cs > 0;                                               // (a row kernel is ready for a later call all the same)
+    return taken ? launch_row<DT, KIND, RAGGED>(fp, plan.cs, plan.span, nvec_row, nonce, injection, s) : FSD_OK;
+}
+template <int DT, int KIND>
+int try_row(const FinishParams& fp, bool vec, size_t nvec_row, int dev, uint64_t nonce, int injection, cudaStream_t s, bool& taken) {
+    return vec ? try_row<DT, KIND, false>(fp, nvec_row, dev, nonce, injection, s, taken) : try_row<DT, KIND, true>(fp, nvec_row, dev, nonce, injection, s, taken);
 }
 
 template <int DT>
@@ -199,13 +289,29 @@ int launch_all(PairParams pp, FinishParams fp, bool vec, CallFlags* flags, Group
     // an unaligned row covers at most as many 16-byte granules as one that starts at a granule's last element
     const size_t nvec_row = vec ? row_bytes / 16 : (row_bytes + 16 - Logit<DT>::kBytes + 15) / 16;
     const int C = nvec_row <= static_cast<size_t>(kMaxGroupSize) * StreamShape<DT>::kBlockVecs ? group_size<DT>(static_cast<int>(nvec_row), items, nsm) : 0;
-#ifdef FSD_DEBUG_CHECKS
-    if (cudaMemsetAsync(&flags->debug, 0, sizeof(int), s) != cudaSuccess) return FSD_ERR_CUDA;   // the debug word starts at zero
-#endif
     pp.nonce = next_nonce(); pp.flags = flags;
     fp.flags = flags;
     const int injection = g_mark_timeout.load();
     fp.silent = injection == 4;
+    // everything that can fail without a launch (attributes, the occupancy queries) comes before the first thing put on the
+    // stream, of the streaming kernel also where this call does not need it: a later one, under capture, may
+    const StreamKernel kernel = stream_kernel<DT>(pp.div, !vec);
+    if (C > 0) {
+        const int rc = kernel.prepare(dev);
+        if (rc != FSD_OK) return rc;
+    }
+#ifdef FSD_DEBUG_CHECKS
+    if (cudaMemsetAsync(&flags->debug, 0, sizeof(int), s) != cudaSuccess) return FSD_ERR_CUDA;   // the debug word starts at zero
+#endif
+    // What fits on chip goes by the row kernel, unless a test or measurement aid asks for the streaming kernel.
+    bool row = g_group_size.load() == 0 && g_stage_event.load() == nullptr;
+    if (row) {
+        fp.records = records;
+        const int rc = fp.mode != FSD_MODE_FSD ? try_row<DT, kDrawResidual>(fp, vec, nvec_row, dev, pp.nonce, injection, s, row)
+                       : fp.sample == FSD_SAMPLE_GREEDY ? try_row<DT, kDrawGreedy>(fp, vec, nvec_row, dev, pp.nonce, injection, s, row)
+                                                        : try_row<DT, kDrawPt>(fp, vec, nvec_row, dev, pp.nonce, injection, s, row);
+        if (rc != FSD_OK || row) return rc;
+    }
     if (C > 0) {
         StreamParams sp;
         sp.target = pp.target; sp.draft = pp.draft; sp.parent = pp.parent; sp.G = pp.G;
@@ -230,11 +336,7 @@ int launch_all(PairParams pp, FinishParams fp, bool vec, CallFlags* flags, Group
         sp.help_after = injection == 2 ? 0xffffffffu : injection == 3 ? 1024 : 16384;
         sp.silent_rank = silent ? C - 1 : -1;
         sp.raise = injection == 1;                    // behave as if a bounded wait had run out
-        // everything that can fail without a launch (attributes, the occupancy query) comes before
-        // the first thing put on the stream
-        int rc = stream_prepare<DT>(pp.div, !vec)(dev);
-        if (rc != FSD_OK) return rc;
-        rc = stream_launch<DT>(pp.div, !vec)(sp, nsm, s);
+        const int rc = kernel.launch(sp, nsm, s);
         if (rc != FSD_OK) return rc;
         fp.records = records;
     } else {
@@ -248,26 +350,13 @@ int launch_all(PairParams pp, FinishParams fp, bool vec, CallFlags* flags, Group
         if (cudaEventRecord(static_cast<cudaEvent_t>(ev), s) != cudaSuccess) return FSD_ERR_CUDA;
     }
     const int cs = finish_cluster_size(fp.B, fp.G, fp.V);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(fp.B) * cs, 1, 1);
-    cfg.blockDim = dim3(kFinishThreads, 1, 1);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = cs;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
     // The finish kernel may be set up while the pair kernel drains: its CTAs take the SMs the
     // pair kernel's CTAs leave, build their tables, and wait (griddepcontrol.wait) for the pair
     // kernel to complete before they read anything it wrote.
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 2;
-    const auto kernel = fp.mode != FSD_MODE_FSD ? fsd_finish_kernel<DT, kDrawResidual>
+    const ClusterLaunch l(fp.B, cs, kFinishThreads, 0, s);
+    const auto finish = fp.mode != FSD_MODE_FSD ? fsd_finish_kernel<DT, kDrawResidual>
                         : fp.sample == FSD_SAMPLE_GREEDY ? fsd_finish_kernel<DT, kDrawGreedy> : fsd_finish_kernel<DT, kDrawPt>;
-    return cudaLaunchKernelEx(&cfg, kernel, fp) == cudaSuccess ? FSD_OK : FSD_ERR_CUDA;
+    return cudaLaunchKernelEx(&l.cfg, finish, fp) == cudaSuccess ? FSD_OK : FSD_ERR_CUDA;
 }
 
 int verify_common(const void* target, const void* draft, const int32_t* tokens, const float* u_accept,

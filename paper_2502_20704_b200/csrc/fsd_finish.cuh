@@ -205,21 +205,16 @@ struct PairTotals {
 __device__ __forceinline__ double pow2_int_d(double d) {
     return d < -1022.0 ? 0.0 : __hiloint2double((1023 + static_cast<int>(d)) << 20, 0);
 }
-// Called by all 32 lanes: lane r folds part r of the record; every lane returns the totals.
-__device__ inline PairTotals fold_record(const PairRecord* rec, int div) {
-    static_assert(kMaxGroupSize <= 32, "one lane per part");
-    const int r = threadIdx.x & 31;
-    PairTotals t;
-    t.state = 0;
+__device__ __forceinline__ Stats no_stats() {
     Stats c;
     c.ka = -INFINITY; c.kb = -INFINITY; c.za = 0.f; c.zb = 0.f; c.s0 = 0.f; c.sb = 0.f; c.x = 0.f; c.diff = 0;
-    float x = 0.f;
-    // every lane fetches its part at once with the count (one trip to L2); parts beyond the count are stale
-    const int rr = r < kMaxGroupSize ? r : 0;
-    const Stats cr = rec->part[rr];
-    const float xr = rec->x[rr];
-    t.state = rec->state;
-    if (r < static_cast<int>(rec->ncta) && r < kMaxGroupSize) { c = cr; x = xr; }
+    return c;
+}
+// Called by all 32 lanes, with a part of the pair each (no_stats() where there is none) and its second-sweep sum;
+// every lane returns the totals.
+__device__ __forceinline__ PairTotals fold_parts(const Stats& c, float x, uint32_t state, int div) {
+    PairTotals t;
+    t.state = state;
     const float ka = warp_redux_max_nan(c.ka), kb = warp_redux_max_nan(c.kb);      // NaN references win
     t.ka = ka; t.kb = kb;
     const double da = c.ka == -INFINITY ? 0.0 : static_cast<double>(c.ka) - ka;
@@ -241,39 +236,60 @@ __device__ inline PairTotals fold_record(const PairRecord* rec, int div) {
     t.differ = __any_sync(0xffffffffu, c.diff != 0) ? 1u : 0u;
     return t;
 }
+// Lane r folds part r of the record.
+__device__ inline PairTotals fold_record(const PairRecord* rec, int div) {
+    static_assert(kMaxGroupSize <= 32, "one lane per part");
+    const int r = threadIdx.x & 31;
+    Stats c = no_stats();
+    float x = 0.f;
+    // every lane fetches its part at once with the count (one trip to L2); parts beyond the count are stale
+    const int rr = r < kMaxGroupSize ? r : 0;
+    const Stats cr = rec->part[rr];
+    const float xr = rec->x[rr];
+    const uint32_t state = rec->state;
+    if (r < static_cast<int>(rec->ncta) && r < kMaxGroupSize) { c = cr; x = xr; }
+    return fold_parts(c, x, state, div);
+}
 
-// (x, ax, bx, ua: the candidate, its two logits and its uniform, for the ratio test)
-__device__ inline void judge_record(const FinishParams& P, const PairTotals& r, double lnZa, double lnZb,
-                                    int x, float ax, float bx, float ua, float& D_out, int& bit_out, int& st_out) {
-    if (r.state & kRecordBadTree) {
+// A candidate's token, logits and uniform, for the ratio test (residual draws alone)
+struct Candidate { int x; float ax, bx, ua; };
+// What of a pair's judgement does not need the second sweep's sum
+struct Judged {
+    bool bad_tree, finite, ratio_ok;
+    double base;               // KL: the divergence; JS: its part without the mixture's entropy
+};
+__device__ __forceinline__ Judged judge_early(const FinishParams& P, const PairTotals& r, double lnZa, double lnZb, const Candidate& c) {
+    Judged j;
+    j.bad_tree = (r.state & kRecordBadTree) != 0;
+    j.finite = isfinite(r.ka) && isfinite(r.kb) && r.Za > 0.0 && r.Zb > 0.0 && isfinite(r.Za) && isfinite(r.Zb);
+    j.base = divergence_base(P.div, r.Za, r.Zb, lnZa, lnZb, r.Sa, r.Sb, r.K);
+    j.ratio_ok = false;
+    if (P.mode != FSD_MODE_FSD && j.finite && c.x >= 0 && c.x < P.V) {
+        double pacc;                                                    // Eq. 1
+        if (c.bx == -INFINITY) {
+            pacc = (c.ax != -INFINITY) ? 1.0 : 0.0;
+        } else {
+            // ln P(x) = (x*log2e - k) ln2 - ln Z with the same float log2e the sums were built with
+            const double la = (static_cast<double>(c.ax) * static_cast<double>(kLog2e) - r.ka) * kLn2D - lnZa;
+            const double lb = (static_cast<double>(c.bx) * static_cast<double>(kLog2e) - r.kb) * kLn2D - lnZb;
+            pacc = exp(la - lb);
+            pacc = pacc < 1.0 ? pacc : 1.0;
+        }
+        j.ratio_ok = static_cast<double>(c.ua) < pacc;                 // Eq. 2
+    }
+    return j;
+}
+__device__ __forceinline__ void judge_late(const FinishParams& P, const PairTotals& r, const Judged& j, float& D_out, int& bit_out, int& st_out) {
+    if (j.bad_tree) {
         D_out = __int_as_float(0x7fc00000); bit_out = 0; st_out = FSD_ROW_BADTREE;
         return;
     }
-    const bool finite = isfinite(r.ka) && isfinite(r.kb) && r.Za > 0.0 && r.Zb > 0.0 && isfinite(r.Za) && isfinite(r.Zb);
     float D = __int_as_float(0x7fc00000);
-    if (finite) D = r.differ ? static_cast<float>(combine_divergence(P.div, r.Za, r.Zb, lnZa, lnZb, r.Sa, r.Sb, r.K, r.X)) : 0.0f;
-    const bool div_ok = finite && passes(D, P.T, P.cmp);
-    int bit = div_ok;
-    if (P.mode != FSD_MODE_FSD) {
-        bool ratio_ok = false;
-        if (finite) {
-            if (x >= 0 && x < P.V) {
-                double pacc;                                                    // Eq. 1
-                if (bx == -INFINITY) {
-                    pacc = (ax != -INFINITY) ? 1.0 : 0.0;
-                } else {
-                    // ln P(x) = (x*log2e - k) ln2 - ln Z with the same float log2e the sums were built with
-                    const double la = (static_cast<double>(ax) * static_cast<double>(kLog2e) - r.ka) * kLn2D - lnZa;
-                    const double lb = (static_cast<double>(bx) * static_cast<double>(kLog2e) - r.kb) * kLn2D - lnZb;
-                    pacc = exp(la - lb);
-                    pacc = pacc < 1.0 ? pacc : 1.0;
-                }
-                ratio_ok = static_cast<double>(ua) < pacc;        // Eq. 2
-            }
-        }
-        bit = P.mode == FSD_MODE_SD ? ratio_ok : (div_ok || ratio_ok);          // Eq. 6
-    }
-    D_out = D; bit_out = bit; st_out = finite ? 0 : FSD_ROW_NONFINITE;
+    if (j.finite) D = r.differ ? static_cast<float>(divergence_of(P.div, j.base, r.X)) : 0.0f;
+    const bool div_ok = j.finite && passes(D, P.T, P.cmp);
+    D_out = D;
+    bit_out = P.mode == FSD_MODE_FSD ? div_ok : P.mode == FSD_MODE_SD ? j.ratio_ok : (div_ok || j.ratio_ok);          // Eq. 6
+    st_out = j.finite ? 0 : FSD_ROW_NONFINITE;
 }
 
 // ---- how a row is shared out for the draw -------------------------------------------------------
@@ -288,30 +304,52 @@ struct Draw {
     bool shared_out;           // the cluster's CTAs have shared the judging: no pair's reference is at hand
     bool vec;                  // both rows are whole vectors on 16-byte boundaries
     double u;
+    int span;                  // LOCAL draws: granules of the target row that a CTA of the cluster holds in its shared memory ...
+    uint32_t local;            // ... and the address there at which granule 0 of the row would lie
 };
-struct Share { int units, iters, first; };            // units of the row, iterations of a warp, the warp's first unit
-__device__ __forceinline__ Share row_share(int units, int cs, int rank, int warp) {      // cs: a power of two
-    const int shift = 9 + 31 - __clz(cs);             // log2(cs * kFinishWarps * 32)
+struct Share { int units, iters, first; };            // where the run's row ends, iterations of a warp, the warp's first unit
+template <bool ANY_SIZE = false>                      // of the cluster; else a power of two
+__device__ __forceinline__ Share row_share(int units, int cs, int rank, int warp) {
     Share s;
     s.units = units;
-    s.iters = static_cast<int>((static_cast<uint32_t>(units) + (1u << shift) - 1) >> shift);
+    if constexpr (ANY_SIZE) {
+        const uint32_t all = static_cast<uint32_t>(cs) * kFinishThreads;
+        s.iters = static_cast<int>((static_cast<uint32_t>(units) + all - 1) / all);
+    } else {
+        const int shift = 9 + 31 - __clz(cs);         // log2(cs * kFinishWarps * 32)
+        s.iters = static_cast<int>((static_cast<uint32_t>(units) + (1u << shift) - 1) >> shift);
+    }
     const long long first = static_cast<long long>(rank * kFinishWarps + warp) * s.iters * 32;
     s.first = first < units ? static_cast<int>(first) : units;
     return s;
 }
+// The same for the granules of the target row, of which a CTA takes what it has at hand (LOCAL: a row in shared memory).
+template <bool LOCAL>
+__device__ __forceinline__ Share granule_share(const Draw& d, int granules, int warp) {
+    if constexpr (!LOCAL) return row_share(granules, d.cs, d.rank, warp);
+    Share s;
+    s.units = min(granules, (d.rank + 1) * d.span);
+    s.iters = (d.span + kFinishThreads - 1) / kFinishThreads;
+    s.first = min(d.rank * d.span + warp * s.iters * 32, s.units);
+    return s;
+}
 // The target row as granules: the granule that holds entry 0 starts `off` entries in front of it.
-template <int DT> struct Granules {
+template <int DT, bool LOCAL> struct Granules {
     const void* base;
+    uint32_t local;
     int off, count, V;
-    __device__ __forceinline__ Granules(const char* row, int v) : V(v) {
+    __device__ __forceinline__ explicit Granules(const Draw& d) : local(d.local), V(d.V) {
+        const char* const row = d.a_row;
+        const int v = d.V;
         const int bytes = static_cast<int>(reinterpret_cast<uintptr_t>(row) & 15);
         base = row - bytes;
         off = bytes / Logit<DT>::kBytes;
         count = (off + v + Logit<DT>::kPerVec - 1) / Logit<DT>::kPerVec;
     }
-    __device__ __forceinline__ uint4 fetch(int g) const {                // -inf where there is no entry
+    __device__ __forceinline__ uint4 fetch(int g, int end) const {       // -inf where there is no entry, and from granule `end` on
         constexpr uint32_t kNone = DT == FSD_BF16 ? 0xff80ff80u : 0xff800000u;
-        return g < count ? ldg_vec(base, g) : make_uint4(kNone, kNone, kNone, kNone);
+        if (g >= end) return make_uint4(kNone, kNone, kNone, kNone);
+        if constexpr (LOCAL) return ld_shared16(local + static_cast<uint32_t>(g) * 16); else return ldg_vec(base, g);
     }
     __device__ __forceinline__ uint4 cut(uint4 v, int g) const {         // the first and last granule's entries that are not the row's
         const int k0 = g * Logit<DT>::kPerVec - off;
@@ -319,10 +357,10 @@ template <int DT> struct Granules {
     }
 };
 // Calls f(k, a_k, b_k) for this warp's entries, unit by unit: vectors where `vec`, else single entries.
-template <int DT, typename F>
+template <int DT, bool ANY_SIZE, typename F>
 __device__ __forceinline__ void for_units(const Draw& d, int warp, int lane, bool with_b, F f) {
     constexpr int EPV = Logit<DT>::kPerVec;
-    const Share s = row_share(d.vec ? d.V / EPV : d.V, d.cs, d.rank, warp);
+    const Share s = row_share<ANY_SIZE>(d.vec ? d.V / EPV : d.V, d.cs, d.rank, warp);
     for (int it = 0; it < s.iters; ++it) {
         const int u = s.first + it * 32 + lane;
         if (u >= s.units) break;
@@ -520,13 +558,13 @@ template <int DT> __device__ __forceinline__ float vector_max(const uint4& v) { 
 }
 
 // Inverse CDF over P_T.  Writes the row's token, adds to its status (uniform over the cluster).
-template <int DT>
+template <int DT, bool LOCAL = false>
 __device__ __forceinline__ void draw_pt(const FinishParams& P, FinishShared& sh, const Draw& d, Link& link, int& status) {
     constexpr int EPV = Logit<DT>::kPerVec;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const Granules<DT> gr(d.a_row, d.V);
-    const Share mine = row_share(gr.count, d.cs, d.rank, warp);
-    FSD_CHECK(&P.flags->debug, mine.first >= 0 && mine.first <= gr.count && static_cast<long long>(mine.iters) * kFinishThreads * d.cs >= gr.count, kChkChunk);
+    const Granules<DT, LOCAL> gr(d);
+    const Share mine = granule_share<LOCAL>(d, gr.count, warp);
+    FSD_CHECK(&P.flags->debug, mine.first >= 0 && mine.first <= gr.count && (LOCAL || static_cast<long long>(mine.iters) * kFinishThreads * d.cs >= gr.count), kChkChunk);
     // ---- one pass: this thread's weights 2^(logit * log2e - kr) in double, kr the largest logit's exponent so far;
     //      four vectors are asked for before the first is used ----
     constexpr int BV = 4;
@@ -535,7 +573,7 @@ __device__ __forceinline__ void draw_pt(const FinishParams& P, FinishShared& sh,
     for (int it = 0; it < mine.iters; it += BV) {
         uint4 v[BV];
 #pragma unroll
-        for (int q = 0; q < BV; ++q) v[q] = gr.fetch(it + q < mine.iters ? mine.first + (it + q) * 32 + lane : INT_MAX);
+        for (int q = 0; q < BV; ++q) v[q] = gr.fetch(it + q < mine.iters ? mine.first + (it + q) * 32 + lane : INT_MAX, mine.units);
         float vm = -INFINITY;
 #pragma unroll
         for (int q = 0; q < BV; ++q) {
@@ -571,6 +609,7 @@ __device__ __forceinline__ void draw_pt(const FinishParams& P, FinishShared& sh,
     // ---- totals of warp, CTA and cluster, in a fixed order and on one scale: 2^0, or where a reference is out of a
     //      double's reach the largest reference of the cluster ----
     double K = 0.0, W, w_v, w_upto;
+    [[maybe_unused]] double blocks_upto = 0.0;        // LOCAL: the CTAs' running totals, a lane each
     const double (*all)[kExchangeDoubles];
 #pragma unroll 1
     for (bool scaled = false;; scaled = true) {
@@ -584,10 +623,18 @@ __device__ __forceinline__ void draw_pt(const FinishParams& P, FinishShared& sh,
         const double mine2[2] = {pre.total, scaled ? 0.0 : static_cast<double>(sh.far)};
         all = cluster_exchange(P, sh, d.cs, d.rank, link, mine2);
         if (link.lost) return;
-        double any = 0.0;
-        W = 0.0;
-        for (int r = 0; r < d.cs; ++r) { W += all[r][0]; any += all[r][1]; }
-        if (any == 0.0) break;
+        if constexpr (LOCAL) {                        // (clusters of up to sixteen: one scan is shorter than sixteen additions in a row)
+            const double (&its)[kExchangeDoubles] = all[lane < d.cs ? lane : 0];
+            const Prefix blocks(lane < d.cs ? its[0] : 0.0, lane);
+            blocks_upto = blocks.upto;
+            W = blocks.total;
+            if (!__any_sync(0xffffffffu, its[1] != 0.0)) break;
+        } else {
+            double any = 0.0;
+            W = 0.0;
+            for (int r = 0; r < d.cs; ++r) { W += all[r][0]; any += all[r][1]; }
+            if (any == 0.0) break;
+        }
         float m = -INFINITY;
         for (int w = 0; w < kFinishWarps; ++w) m = fmaxf(m, sh.warp_k[w]);
         __syncthreads();
@@ -603,21 +650,29 @@ __device__ __forceinline__ void draw_pt(const FinishParams& P, FinishShared& sh,
         return;
     }
     const double t = d.u * W;
-    double run = 0.0, cpre = 0.0;
+    double cpre = 0.0;
     int owner = -1;
-    for (int r = 0; r < d.cs && owner < 0; ++r) {
-        cpre = run;
-        run += all[r][0];
-        if (run > t) owner = r;
+    if constexpr (LOCAL) {
+        const unsigned past = __ballot_sync(0xffffffffu, blocks_upto > t);     // (lanes beyond the CTAs' have the total)
+        owner = past != 0 ? __ffs(past) - 1 : -1;
+        const double before_it = __shfl_sync(0xffffffffu, blocks_upto, owner > 0 ? owner - 1 : 0);
+        cpre = owner > 0 ? before_it : 0.0;
+    } else {
+        double run = 0.0;
+        for (int r = 0; r < d.cs && owner < 0; ++r) {
+            cpre = run;
+            run += all[r][0];
+            if (run > t) owner = r;
+        }
     }
     if (owner < 0) {                                  // t >= W after rounding (uniform): the last token that has weight
         int lastp = -1;
         const float nk = kr == -INFINITY ? 0.f : -kr;
         for (int it = 0; it < mine.iters; ++it) {
             const int g = mine.first + it * 32 + lane;
-            if (g >= gr.count) break;
+            if (g >= mine.units) break;
             float x[EPV];
-            unpack_vec<DT>(gr.cut(gr.fetch(g), g), x);
+            unpack_vec<DT>(gr.cut(gr.fetch(g, mine.units), g), x);
 #pragma unroll
             for (int e = 0; e < EPV; ++e) if (ex2(fmaf(x[e], kLog2e, nk)) > 0.f) lastp = g * EPV - gr.off + e;
         }
@@ -642,10 +697,11 @@ __device__ __forceinline__ void draw_pt(const FinishParams& P, FinishShared& sh,
     const double up = pow2_int_d(-fabs(static_cast<double>(ck) - K)), rest = t - cpre - before;
     const double target = static_cast<double>(ck) > K ? rest * up : rest / up;
     const float nk = -ck;
-    find_crossing<EPV>(P, sh, d, row_share(gr.count, d.cs, d.rank, cw), target,
+    const Share crossing = granule_share<LOCAL>(d, gr.count, cw);
+    find_crossing<EPV>(P, sh, d, crossing, target,
         [&](int g, double (&w)[EPV]) {
             float x[EPV];
-            unpack_vec<DT>(gr.cut(gr.fetch(g), g), x);
+            unpack_vec<DT>(gr.cut(gr.fetch(g, crossing.units), g), x);
 #pragma unroll
             for (int e = 0; e < EPV; ++e) w[e] = static_cast<double>(ex2(fmaf(x[e], kLog2e, nk)));
         },
@@ -654,19 +710,19 @@ __device__ __forceinline__ void draw_pt(const FinishParams& P, FinishShared& sh,
 
 // argmax of P_T == argmax of the logits, ties to the lowest index.  One pass: the largest logit, its index, and
 // whether the row is a valid distribution (no NaN, no +inf, something finite).
-template <int DT>
+template <int DT, bool LOCAL = false>
 __device__ __forceinline__ void draw_argmax(const FinishParams& P, FinishShared& sh, const Draw& d, Link& link, int& status) {
     constexpr int EPV = Logit<DT>::kPerVec;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const Granules<DT> gr(d.a_row, d.V);
-    const Share mine = row_share(gr.count, d.cs, d.rank, warp);
+    const Granules<DT, LOCAL> gr(d);
+    const Share mine = granule_share<LOCAL>(d, gr.count, warp);
     float best = -INFINITY;
     int idx = 0x7fffffff;
     bool bad = false;
 #pragma unroll 4
     for (int it = 0; it < mine.iters; ++it) {
         const int g = mine.first + it * 32 + lane;
-        const uint4 v = gr.cut(gr.fetch(g), g);
+        const uint4 v = gr.cut(gr.fetch(g, mine.units), g);
         const float vm = vector_max<DT>(v);
         bad = bad || !(vm < INFINITY);
         if (vm > best) {
@@ -882,7 +938,7 @@ __device__ __forceinline__ double fold_four(double v0, double v1, double v2, dou
 __device__ __forceinline__ float residual_margin(double ln_rho) { return fabs(ln_rho) < 8.0 ? 2e-6f : 2e-5f; }
 constexpr double kMostLnRho = 80.0;
 
-template <int DT>
+template <int DT, bool ANY_SIZE>
 __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShared& sh, ResidualShared& rs, const ExpTable<DT>& bt,
                                               const Draw& d, Link& link, int& status, bool greedy) {
     constexpr int EPV = Logit<DT>::kPerVec;
@@ -918,7 +974,7 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
     }
     float mx[2] = {-INFINITY, -INFINITY};
     if (!common) {
-        for_units<DT>(d, warp, lane, true, [&](int, float xa, float xb) {
+        for_units<DT, ANY_SIZE>(d, warp, lane, true, [&](int, float xa, float xb) {
             mx[0] = fmaxf(mx[0], xa);
             mx[1] = fmaxf(mx[1], xb);
         });
@@ -958,15 +1014,15 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
         const float hi = static_cast<float>(ln_rho + margin), lo = static_cast<float>(ln_rho - margin);
         bool done = false;
         if constexpr (DT == FSD_BF16) {
-            const Share share = row_share(d.V / 8, cs, rank, warp);
+            const Share share = row_share<ANY_SIZE>(d.V / 8, cs, rank, warp);
             if (d.vec && tabled) classed_pass_bf16(a_row, b_row, share, hi, lo, bt, c);
             else if (d.vec) classed_pass_far(a_row, b_row, share, hi, lo, ea, eb, rs, c);
             done = d.vec;
         }
         if constexpr (DT == FSD_BF16) {               // (a loop of its own: with the choice inside it, 8 x 5 x 50257 28.7 -> 31.0 us)
-            if (!done && tabled) { for_units<DT>(d, warp, lane, true, [&](int k, float xa, float xb) { c.entry(k, xa, xb, exp_bf16(xa, bt), exp_bf16(xb, bt), hi, lo); }); done = true; }
+            if (!done && tabled) { for_units<DT, ANY_SIZE>(d, warp, lane, true, [&](int k, float xa, float xb) { c.entry(k, xa, xb, exp_bf16(xa, bt), exp_bf16(xb, bt), hi, lo); }); done = true; }
         }
-        if (!done) for_units<DT>(d, warp, lane, true, [&](int k, float xa, float xb) { c.entry(k, xa, xb, ea(xa, tab, ec), eb(xb, tab, ec), hi, lo); });
+        if (!done) for_units<DT, ANY_SIZE>(d, warp, lane, true, [&](int k, float xa, float xb) { c.entry(k, xa, xb, ea(xa, tab, ec), eb(xb, tab, ec), hi, lo); });
         if (!classify || c.close > 2) {
             atomicOr(&sh.amb, 1);
         } else if (c.qd == c.qd) {
@@ -996,7 +1052,7 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
         for (int r = 0; r < cs; ++r) { Za += all[r][0]; Zb += all[r][1]; flags = all[r][4] == 1.0 || flags == 1.0 ? 1.0 : fmax(flags, all[r][4]); }
     } else {
         double z[2] = {0.0, 0.0};
-        for_units<DT>(d, warp, lane, true, [&](int, float xa, float xb) {
+        for_units<DT, ANY_SIZE>(d, warp, lane, true, [&](int, float xa, float xb) {
             if (Ra > -INFINITY) z[0] += exp2_table((static_cast<double>(xa) - Ra) * kLog2eD, tab);
             if (Rb > -INFINITY) z[1] += exp2_table((static_cast<double>(xb) - Rb) * kLog2eD, tab);
         });
@@ -1067,7 +1123,7 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
             const bool one = sh.n_close == 1 && rs.cq_warp == w;
             double before;
             const int cw = Prefix(residual_of(rs.wsum[w][2], rs.wsum[w][3], one ? rs.cq[0] : 0.0, one ? rs.cq[1] : 0.0), lane).crossing(t - cpre, before);
-            find_crossing<EPV>(P, sh, d, row_share(d.V / EPV, cs, rank, cw), t - cpre - before, vector_weights, [&](int u) { return u * EPV; });
+            find_crossing<EPV>(P, sh, d, row_share<ANY_SIZE>(d.V / EPV, cs, rank, cw), t - cpre - before, vector_weights, [&](int u) { return u * EPV; });
             return;
         }
     }
@@ -1099,7 +1155,7 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
                 if (r > 0.0) csum += r;
             }
         } else if (d.vec && common && residual) {
-            const Share share = row_share(d.V / EPV, cs, rank, warp);
+            const Share share = row_share<ANY_SIZE>(d.V / EPV, cs, rank, warp);
 #pragma unroll 1
             for (int u = share.first + lane; u < min(share.first + share.iters * 32, share.units); u += 32) {
                 double w[EPV];
@@ -1111,7 +1167,7 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
                 }
             }
         } else {
-            for_units<DT>(d, warp, lane, residual, [&](int k, float xa, float xb) {
+            for_units<DT, ANY_SIZE>(d, warp, lane, residual, [&](int k, float xa, float xb) {
                 const double w = weight(xa, xb);
                 csum += w;
                 if (greedy && w > wbest) { wbest = w; kbest = k; }
@@ -1183,7 +1239,7 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
         }
         if (owner < 0) {                                  // t >= W after rounding (uniform): the last token that has weight
             int lastp = -1;
-            for_units<DT>(d, warp, lane, residual, [&](int k, float xa, float xb) { if (weight(xa, xb) > 0.0) lastp = k; });
+            for_units<DT, ANY_SIZE>(d, warp, lane, residual, [&](int k, float xa, float xb) { if (weight(xa, xb) > 0.0) lastp = k; });
             lastp = __reduce_max_sync(0xffffffffu, lastp);
             if (lane == 0 && lastp >= 0) atomicMax(&sh.last_pos, lastp);
             __syncthreads();
@@ -1201,9 +1257,9 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
         const int cw = pre.crossing(t_local, before);
         const double target = t_local - before;
         if (d.vec && common && residual) {
-            find_crossing<EPV>(P, sh, d, row_share(d.V / EPV, cs, rank, cw), target, vector_weights, [&](int u) { return u * EPV; });
+            find_crossing<EPV>(P, sh, d, row_share<ANY_SIZE>(d.V / EPV, cs, rank, cw), target, vector_weights, [&](int u) { return u * EPV; });
         } else if (d.vec) {
-            find_crossing<EPV>(P, sh, d, row_share(d.V / EPV, cs, rank, cw), target,
+            find_crossing<EPV>(P, sh, d, row_share<ANY_SIZE>(d.V / EPV, cs, rank, cw), target,
                 [&](int u, double (&w)[EPV]) {
 #pragma unroll 1
                     for (int e = 0; e < EPV; ++e) {
@@ -1214,11 +1270,73 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
                 },
                 [&](int u) { return u * EPV; });
         } else {
-            find_crossing<1>(P, sh, d, row_share(d.V, cs, rank, cw), target,
+            find_crossing<1>(P, sh, d, row_share<ANY_SIZE>(d.V, cs, rank, cw), target,
                 [&](int u, double (&w)[1]) { w[0] = weight(load_logit<DT>(a_row, u), residual ? load_logit<DT>(b_row, u) : 0.f); },
                 [&](int u) { return u; });
         }
         return;
+    }
+}
+
+// ---- what the finish kernel and the row kernel share -------------------------------------------
+template <int DT, int KIND>
+__device__ __forceinline__ Candidate candidate(const FinishParams& P, int item, const char* a_row, const char* b_row) {
+    Candidate c = {-1, 0.f, 0.f, 0.f};
+    if constexpr (KIND == kDrawResidual) {
+        c.x = P.tokens[item];
+        if (c.x >= 0 && c.x < P.V) { c.ax = load_logit<DT>(a_row, c.x); c.bx = load_logit<DT>(b_row, c.x); }
+        c.ua = P.u_accept[item];
+    }
+    return c;
+}
+// (`rs` and `bt` below: of residual draws alone, else null.)
+// Position i of a row judged by a warp, as far as that goes without the second sweep's sum (its first lane returns that).
+template <int KIND>
+__device__ __forceinline__ Judged judge_pair_early(const FinishParams& P, ResidualShared* rs, const PairTotals& tot, int i, const Candidate& c, int lane) {
+    // the two logarithms the judgement needs, by two lanes at once
+    const double lz = log(lane == 1 ? tot.Zb : tot.Za);
+    const double lnZa = lz, lnZb = __shfl_down_sync(0xffffffffu, lz, 1);
+    Judged j = {false, false, false, 0.0};
+    if (lane == 0) {
+        j = judge_early(P, tot, lnZa, lnZb, c);
+        if constexpr (KIND == kDrawResidual) {
+            if (i < kPairRefs) {
+                PairRef ref;
+                ref.za = tot.Za; ref.zb = tot.Zb; ref.ln_rho = lnZa - lnZb; ref.ka = (tot.state & kRecordStats) ? tot.ka : __int_as_float(0x7fc00000); ref.kb = tot.kb;
+                rs->ref[i] = ref;
+            }
+        }
+    }
+    return j;
+}
+// What a residual draw's tables start from, by the block's first threads; a barrier before they are read.
+__device__ __forceinline__ void residual_tables(ResidualShared& rs, int tid) {
+    if (tid < kExpTable) rs.exp_table[tid] = exp2(static_cast<double>(tid) * (1.0 / kExpTable));
+    if (tid == 0) {
+        rs.exp_consts[0] = 6755399441055744.0; rs.exp_consts[1] = 256.0;
+        rs.exp_consts[2] = 2.239395190875157e-12; rs.exp_consts[3] = 3.308302680541371e-09;
+        rs.exp_consts[4] = 3.665565596910106e-06; rs.exp_consts[5] = 2.7076061740622863e-03;
+    }
+}
+// Entry i of the table of bf16 exponentials, of either sign
+__device__ __forceinline__ void bf16_table_entry(ExpTable<FSD_BF16>& bt, const ResidualShared& rs, int i) {
+    const double x = __uint_as_float(static_cast<uint32_t>(kBf16Lowest + i) << 16);
+    bt.e[i] = exp2_table(x * kLog2eD, rs.exp_table);
+    bt.e[kBf16Count + i] = exp2_table(-x * kLog2eD, rs.exp_table);
+}
+// The row's token.  `rejected`: drawn from the residual where the kind is.
+template <int DT, int KIND, bool LOCAL>
+__device__ __forceinline__ void draw_token(const FinishParams& P, FinishShared& sh, ResidualShared* rs, const ExpTable<DT>* bt, const Draw& d, Link& link, int& status, bool rejected) {
+    if constexpr (KIND == kDrawPt) {
+        draw_pt<DT, LOCAL>(P, sh, d, link, status);
+    } else if constexpr (KIND == kDrawGreedy) {
+        draw_argmax<DT, LOCAL>(P, sh, d, link, status);
+    } else {
+        const bool greedy = P.sample == FSD_SAMPLE_GREEDY;
+        if (!rejected) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        if (rejected) draw_residual<DT, LOCAL>(P, sh, *rs, *bt, d, link, status, greedy);
+        else if (greedy) draw_argmax<DT, LOCAL>(P, sh, d, link, status);
+        else draw_pt<DT, LOCAL>(P, sh, d, link, status);
     }
 }
 
@@ -1247,12 +1365,7 @@ __global__ void __launch_bounds__(kFinishThreads, 2) fsd_finish_kernel(const __g
     if (tid == 0) { sh.cand = -1; sh.last_pos = -1; sh.n_acc = G; sh.bad = 0; sh.row_sel = 0; sh.amb = 0; sh.n_close = 0; sh.next = 0; sh.far = 0; }
     if (tid < kJudgeWords) sh.bits[tid] = 0;
     if constexpr (KIND == kDrawResidual) {
-        if (tid < kExpTable) rs.exp_table[tid] = exp2(static_cast<double>(tid) * (1.0 / kExpTable));
-        if (tid == 0) {
-            rs.exp_consts[0] = 6755399441055744.0; rs.exp_consts[1] = 256.0;
-            rs.exp_consts[2] = 2.239395190875157e-12; rs.exp_consts[3] = 3.308302680541371e-09;
-            rs.exp_consts[4] = 3.665565596910106e-06; rs.exp_consts[5] = 2.7076061740622863e-03;
-        }
+        residual_tables(rs, tid);
     }
     __syncthreads();
     // What comes behind this kernel may be set up while it runs.  (A residual draw allows that when its pass is through:
@@ -1276,33 +1389,15 @@ __global__ void __launch_bounds__(kFinishThreads, 2) fsd_finish_kernel(const __g
         const int step = shared_out ? cs : 1, i0 = shared_out ? rank : 0;
         for (int i = warp * step + i0; i < G; i += kFinishWarps * step) {
             const int item = b * G + i;
-            int x = -1;
-            float ax = 0.f, bx = 0.f;
-            if constexpr (KIND == kDrawResidual) {       // the candidate's logits, on their way while the record is folded
-                x = P.tokens[item];
-                if (x >= 0 && x < V) {
-                    ax = load_logit<DT>(t_base + static_cast<size_t>(i) * rb, x);
-                    bx = load_logit<DT>(d_base + static_cast<size_t>(i) * rb, x);
-                }
-            }
-            float ua = 0.f;
-            if constexpr (KIND == kDrawResidual) ua = P.u_accept[item];
+            // (the candidate's logits are on their way while the record is folded)
+            const Candidate c = candidate<DT, KIND>(P, item, t_base + static_cast<size_t>(i) * rb, d_base + static_cast<size_t>(i) * rb);
             const PairTotals tot = fold_record(P.records + item, P.div);
-            // the two logarithms the judgement needs, by two lanes at once
-            const double lz = log(lane == 1 ? tot.Zb : tot.Za);
-            const double lnZa = lz, lnZb = __shfl_down_sync(0xffffffffu, lz, 1);
+            float D = 0.f;
+            int bit = 0, s = 0;
+            const Judged j = judge_pair_early<KIND>(P, &rs, tot, i, c, lane);
             if (lane == 0) {
-                float D;
-                int bit, s;
-                judge_record(P, tot, lnZa, lnZb, x, ax, bx, ua, D, bit, s);
+                judge_late(P, tot, j, D, bit, s);
                 if (shared_out || rank == 0) P.divergence[item] = D;
-                if constexpr (KIND == kDrawResidual) {
-                    if (i < kPairRefs) {
-                        PairRef ref;
-                        ref.za = tot.Za; ref.zb = tot.Zb; ref.ln_rho = lnZa - lnZb; ref.ka = (tot.state & kRecordStats) ? tot.ka : __int_as_float(0x7fc00000); ref.kb = tot.kb;
-                        rs.ref[i] = ref;
-                    }
-                }
                 st |= s;
                 if (tree) {
                     if constexpr (KIND != kDrawResidual) {
@@ -1331,10 +1426,7 @@ __global__ void __launch_bounds__(kFinishThreads, 2) fsd_finish_kernel(const __g
             if (lane == 0) part = atomicAdd(&sh.next, 1);
             part = __shfl_sync(0xffffffffu, part, 0);
             if (part >= kBf16Count / 32) break;
-            const int i = part * 32 + lane;
-            const double x = __uint_as_float(static_cast<uint32_t>(kBf16Lowest + i) << 16);
-            bt.e[i] = exp2_table(x * kLog2eD, rs.exp_table);
-            bt.e[kBf16Count + i] = exp2_table(-x * kLog2eD, rs.exp_table);
+            bf16_table_entry(bt, rs, part * 32 + lane);
         }
     }
     if (tid == 0) sh.u = u_mine;
@@ -1386,21 +1478,14 @@ __global__ void __launch_bounds__(kFinishThreads, 2) fsd_finish_kernel(const __g
     d.a_row = t_base + static_cast<size_t>(row_sel) * rb;
     d.b_row = d_base + static_cast<size_t>(residual ? n : 0) * rb;
     d.b = b; d.n = n; d.V = V; d.cs = cs; d.rank = rank; d.shared_out = shared_out; d.vec = P.vec != 0; d.u = static_cast<double>(sh.u);
+    d.span = 0; d.local = 0;
     if (link.lost) {
         n = 0;                                           // (nothing of the row is valid but its status)
     } else if (bad_tree) {
         n = 0;
         if (rank == 0 && tid == 0) P.next_token[b] = -1;
-    } else if constexpr (KIND == kDrawPt) {
-        draw_pt<DT>(P, sh, d, link, status);
-    } else if constexpr (KIND == kDrawGreedy) {
-        draw_argmax<DT>(P, sh, d, link, status);
     } else {
-        const bool greedy = P.sample == FSD_SAMPLE_GREEDY;
-        if (!residual) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-        if (residual) draw_residual<DT>(P, sh, rs, bt, d, link, status, greedy);
-        else if (greedy) draw_argmax<DT>(P, sh, d, link, status);
-        else draw_pt<DT>(P, sh, d, link, status);
+        draw_token<DT, KIND, false>(P, sh, &rs, &bt, d, link, status, residual);
     }
     if (rank == 0 && tid == 0) {
         P.accept_len[b] = n;

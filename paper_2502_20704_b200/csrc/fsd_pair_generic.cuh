@@ -34,22 +34,20 @@ struct PairParams {
 //   X        JS: sum_k s_k log2 s_k with s = p + q;  TV: sum_k |p_k - q_k|
 // Returns the divergence in nats (NaN when a row is not a valid distribution).
 // The variant with lnZa, lnZb takes the two logarithms from the caller (computed by two lanes at once).
-__device__ inline double combine_divergence(int div, double Za, double Zb, double lnZa, double lnZb, double Sa, double Sb, double K, double X) {
-    double D;
-    if (div == FSD_DIV_KL) {
-        D = kLn2D * K / Za - lnZa + lnZb;
-    } else if (div == FSD_DIV_JS) {
-        // sum p ln p = ln2 * Sa/Za - ln Za (the offset error in c cancels between the two terms);
-        // sum m ln m with m = s/2 and sum s = 2:  (ln2/2) * X - ln2
-        const double Pp = kLn2D * Sa / Za - lnZa, Pq = kLn2D * Sb / Zb - lnZb;
-        D = 0.5 * (Pp + Pq) - (0.5 * kLn2D * X - kLn2D);
-    } else {
-        D = 0.5 * X;
-    }
+__device__ __forceinline__ double divergence_base(int div, double Za, double Zb, double lnZa, double lnZb, double Sa, double Sb, double K) {
+    if (div == FSD_DIV_KL) return kLn2D * K / Za - lnZa + lnZb;
+    if (div == FSD_DIV_TV) return 0.0;
+    // sum p ln p = ln2 * Sa/Za - ln Za (the offset error in c cancels between the two terms)
+    const double Pp = kLn2D * Sa / Za - lnZa, Pq = kLn2D * Sb / Zb - lnZb;
+    return 0.5 * (Pp + Pq);
+}
+__device__ __forceinline__ double divergence_of(int div, double base, double X) {
+    // JS: sum m ln m with m = s/2 and sum s = 2:  (ln2/2) * X - ln2
+    const double D = div == FSD_DIV_KL ? base : div == FSD_DIV_JS ? base - (0.5 * kLn2D * X - kLn2D) : 0.5 * X;
     return D < 0.0 ? 0.0 : D;   // NaN stays NaN
 }
 __device__ inline double combine_divergence(int div, double Za, double Zb, double Sa, double Sb, double K, double X) {
-    return combine_divergence(div, Za, Zb, log(Za), log(Zb), Sa, Sb, K, X);
+    return divergence_of(div, divergence_base(div, Za, Zb, log(Za), log(Zb), Sa, Sb, K), X);
 }
 
 // ln P(x) of one token from its logit and the row's normaliser, in double.

@@ -60,7 +60,8 @@ constexpr int kMaxSteps = 4;                               // steps a warp parks
 constexpr int kStepEntries = 8;                            // vocabulary entries a lane handles per step
 constexpr int kTmemCols = 512;                             // all of the SM's columns: warp w owns 32 lanes x 128 columns
 constexpr int kParkCols = 2 * kStepEntries;                // e values a lane parks per step (both rows)
-constexpr int kMaxClusterSize = 8;                         // finish kernel (portable size)
+constexpr int kPortableCluster = 8;                        // most thread blocks of a cluster without asking for more (finish kernel)
+constexpr int kMaxClusterSize = 16;                        // and at all (row kernel)
 constexpr int kMaxGroupSize = 24;                          // most blocks in a group of the streaming kernel
 constexpr uint32_t kSpinLimit = 1u << 24;                  // polls before a wait gives up
 constexpr uint64_t kWaitNs = 4000000000ull;                // and its limit in time
@@ -144,10 +145,11 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
         : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
     return ok != 0;
 }
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint64_t* bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
+                 ::"r"(dst), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
 }
+__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) { bulk_g2s(smem_u32(dst), src, bytes, bar); }
 
 __device__ __forceinline__ uint64_t global_ns() {
     uint64_t t;

@@ -1,0 +1,108 @@
+"""Calls that one kernel does whole, a thread-block cluster per row, at the sizes where its shares can go wrong, against
+the oracle: rows shorter than a step, blocks without a granule, the last size that fits on chip and the first that does not,
+more pairs than warps; rows off a 16-byte boundary; logits whose first sweep has to be done over; invalid rows."""
+
+import numpy as np
+import pytest
+import torch
+
+import fsd_inputs as gi
+from tests import parity
+
+pytestmark = pytest.mark.gpu
+
+FORMS = [dict(T=0.2), dict(T=0.2, div="kl", sample="greedy"), dict(T=0.2, div="tv"), dict(mode="sd"), dict(mode="rfsd", T=0.05), dict(mode="sd", sample="greedy", div="kl")]
+
+
+def _chain(B, gamma, V, dtype, wid, **kw):
+    return gi.make_chain(B, gamma, V, dtype=dtype, recipe="zipf", sigma=(0.2, 1.5), sigma_mode="uniform", disjoint_frac=0.1, workload_id=wid, **kw)
+
+
+def _check(c, dev=None, **kw):
+    return parity.check_chain(c.target, c.draft, c.draft_tokens, c.u_accept, c.u_sample, c.dtype, dev=dev, **kw)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("B,gamma,V", [
+    (2, 2, 1), (3, 1, 7), (3, 3, 255), (3, 3, 257),    # less than a step, either side of one
+    (1, 2, 8800), (1, 3, 4484), (5, 2, 2056),          # blocks at the end without a granule or with one
+    (1, 8, 65536), (1, 8, 65544), (2, 16, 16392),      # as much as a warp parks, one step more, two pairs a warp
+    (1, 17, 6000), (2, 24, 3001), (1, 25, 3000),       # more pairs than warps, the most there may be, one more
+    (37, 3, 5000), (148, 1, 800),                      # clusters of a few blocks and of one
+])
+def test_sizes_at_an_edge(dtype, B, gamma, V):
+    c = _chain(B, gamma, V, dtype, 820)
+    for form in FORMS if B * gamma * V < 500000 else FORMS[:4]:
+        _check(c, **form)
+
+
+@pytest.mark.parametrize("dtype,offset", [("bf16", 1), ("bf16", 6), ("f32", 1), ("f32", 3)])
+@pytest.mark.parametrize("V", [5, 1001, 4096, 33003])
+def test_bases_and_rows_off_a_16_byte_boundary(dtype, offset, V):
+    c = _chain(3, 3, V, dtype, 821)
+
+    def shifted(a, off):
+        t = parity.to_device(a, dtype)
+        buf = torch.empty(t.numel() + off + 16, dtype=t.dtype, device="cuda")
+        v = buf[off:off + t.numel()].view(t.shape)
+        v.copy_(t)
+        return v
+
+    dev = dict(t=shifted(c.target, offset), d=shifted(c.draft, (3 * offset) % 8), tok=parity.to_device(c.draft_tokens, dtype),
+               ua=parity.to_device(c.u_accept, dtype), us=parity.to_device(c.u_sample, dtype))
+    for form in FORMS[:5]:
+        _check(c, dev=dev, **form)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("V", [40000, 40003])
+def test_sweeps_that_are_done_over_masked_entries_and_invalid_rows(dtype, V):
+    c = gi.make_chain(8, 3, V, dtype=dtype, recipe="spike", sigma=(0.5, 1.0), workload_id=822)
+    f32 = dtype == "f32"
+    t = (c.target if f32 else gi.bf16_bits_to_f32(c.target)).copy()
+    d = (c.draft if f32 else gi.bf16_bits_to_f32(c.draft)).copy()
+    t[0, :, V - 1] += 60.0                              # 86 binades above what a warp looks at first
+    d[0, :, 7000] += 45.0
+    t[1, 1, 9000:9300] = -np.inf
+    d[2, 2, ::97] = -np.inf
+    t[3, 0, : V // 2] = -np.inf                         # parts without a finite logit
+    t[4, :, 300:] = -np.inf
+    t[5, 2, 11] = np.nan
+    d[6, 0, 5] = np.inf
+    t[7, :3] = d[7]                                     # the same distribution
+    c.target[:] = t if f32 else gi.f32_to_bf16_bits(t)
+    c.draft[:] = d if f32 else gi.f32_to_bf16_bits(d)
+    for form in FORMS:
+        _check(c, **form)
+
+
+@pytest.mark.parametrize("dtype,V", [("bf16", 20000), ("bf16", 20003), ("f32", 15000)])
+@pytest.mark.parametrize("div", ["js", "kl", "tv"])
+def test_a_pairs_divergence_is_its_own_rows_alone(dtype, V, div):
+    c = gi.make_chain(7, 4, V, dtype=dtype, recipe="spike", sigma=(0.5, 1.0), workload_id=823)
+    t, d = (parity.to_device(x, dtype) for x in (c.target, c.draft))
+    us = parity.to_device(c.u_sample, dtype)
+
+    def divergences():
+        return parity.run_chain_gpu(c.target, c.draft, None, None, c.u_sample, dtype, div=div, T=0.25, dev=dict(t=t, d=d, tok=None, ua=None, us=us)).divergence
+
+    want = divergences()
+    t[0:3, :, ::53] = -float("inf")
+    t[3, 2, 11] = float("nan")
+    d[4, :, V - 5] += 60.0
+    d[5, 1, 9000:9400] = -float("inf")
+    got = divergences()
+    assert np.array_equal(got[6].view(np.uint32), want[6].view(np.uint32)) and np.array_equal(got[5, [0, 2, 3]].view(np.uint32), want[5, [0, 2, 3]].view(np.uint32))
+    assert not np.array_equal(got[:6].view(np.uint32), want[:6].view(np.uint32))
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("B,N,V", [(3, 5, 4096), (2, 17, 3001), (4, 24, 4100), (1, 25, 4096)])
+def test_small_trees(dtype, B, N, V):
+    t = gi.make_tree(B, N, V, dtype=dtype, sigma=0.5, max_depth=6, max_children=4, workload_id=824)
+    for T in (0.02, 0.05, 1.0):
+        parity.check_tree(t, T=T)
+    parity.check_tree(t, T=0.04, sample="greedy", div="kl")
+    t.parent[0, N - 1] = N - 1                          # not a tree
+    g, _ = parity.check_tree(t, T=0.05)
+    assert g.row_status[0] & 4 and g.next_token[0] == -1

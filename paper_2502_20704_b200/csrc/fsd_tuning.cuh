@@ -277,7 +277,7 @@ __device__ __forceinline__ void for_prefix_maxima(TuneRows& rows, F f) {
               [] { return false; }, [&] { f(key, run); });
 }
 
-constexpr int kTuneList = kTuneBins / kTuneCluster;                        // candidates that are ranked directly
+constexpr int kTuneList = kTuneBins / kTuneCluster;                        // candidates of a block that are ranked directly
 struct CalibrateShared {
     uint64_t bar[2];                                  // tiles
     uint64_t link[3][3];                              // [digit][parts of the histogram | sums | the digit found]
@@ -286,7 +286,7 @@ struct CalibrateShared {
     unsigned int recv[kTuneCluster][kTuneBins / kTuneCluster];   // this block's part of the peers' histograms; later, in block 0,
                                                       // everybody's candidates (sent when all have the first digit, so when all have read)
     uint64_t sums[kTuneCluster];
-    uint64_t found[2];                                // digit | keys equal to it << 32, keys below it
+    uint64_t found[2];                                // digit | keys equal to it << 32, keys below it | most of a block's equal to it << 32
     uint32_t list[kTuneList];                         // this block's candidates
     unsigned int warp_sum[kTuneThreads / 32];
     unsigned int n_list, count;
@@ -296,8 +296,11 @@ struct CalibrateShared {
 // A row's prefix maxima never fall, so a thread adds once per distinct value (two or three a row of
 // eight).  Per digit: every block pushes the eighth of its histogram that block r is to add up to
 // block r, then its sum over that eighth to everybody, and the block whose eighth holds the wanted
-// rank pushes the digit to everybody.  If no more than kTuneList keys share the first digit, they are
-// pushed to block 0, which ranks them by counting.  4096 x 8: 57 -> 11 us, 32768 x 20: 821 -> 74 us (one
+// rank pushes the digit to everybody.  If no block has more than kTuneList keys that share the first digit, they are
+// pushed to block 0, which goes on with them by itself, two more histograms (9 and 10 bits) of at most eight keys a thread: a digit
+// of the whole cluster's is a walk over all rows and three exchanges, 3 us.  (Some 800 keys of 4096 x 8 share it; as
+// long as all lists together had to fit in 512 that call went on by the cluster's digits: 12.3 us, now 10.0; 8192 x 10 16.2, now 13.2.)
+// 4096 x 8: 57 -> 11 us, 32768 x 20: 821 -> 74 us (one
 // block and four 8-bit digits before), of which the walks' shared-memory atomics are the larger part.
 template <int CS>
 __global__ void __launch_bounds__(kTuneThreads) fsd_calibrate_kernel(const float* __restrict__ D, int B, int G, float target,
@@ -399,7 +402,13 @@ __global__ void __launch_bounds__(kTuneThreads) fsd_calibrate_kernel(const float
 #pragma unroll
                 for (int q = 0; q < kMost; ++q) {
                     if (left > run && left <= run + c[q]) {
-                        const uint64_t w0 = static_cast<uint32_t>((CS > 1 ? rank * part : 0) + per * tid + q) | static_cast<uint64_t>(c[q]) << 32, w1 = run;
+                        unsigned int worst = c[q];
+                        if constexpr (CS > 1) {
+                            worst = 0;
+#pragma unroll
+                            for (int r = 0; r < CS; ++r) worst = max(worst, mine[r][tid]);
+                        }
+                        const uint64_t w0 = static_cast<uint32_t>((CS > 1 ? rank * part : 0) + per * tid + q) | static_cast<uint64_t>(c[q]) << 32, w1 = run | static_cast<uint64_t>(worst) << 32;
                         if constexpr (CS > 1) {
                             for (int r = 0; r < CS; ++r) {
                                 st_async(cluster_addr(&sh.found[0], r), w0, cluster_addr(&sh.link[digit][2], r));
@@ -421,7 +430,7 @@ __global__ void __launch_bounds__(kTuneThreads) fsd_calibrate_kernel(const float
             below += lower; left -= lower;
             if (__syncthreads_or(tune_wait.lost)) { found = false; break; }
             // everybody has read: the histogram and the rest may be written again
-            if (digit == 0 && equal <= kTuneList) { ranked = true; break; }
+            if (digit == 0 && (sh.found[1] >> 32) <= kTuneList) { ranked = true; break; }
         }
     }
     if (ranked) {
@@ -429,37 +438,55 @@ __global__ void __launch_bounds__(kTuneThreads) fsd_calibrate_kernel(const float
         for_prefix_maxima(rows, [&](uint32_t key, unsigned int count) {
             if ((key & 0xfff80000u) != prefix || key > kKeyInf) return;
             const unsigned int at = atomicAdd(&sh.n_list, count);
-            for (unsigned int q = 0; q < count && at + q < kTuneList; ++q) sh.list[at + q] = key;       // (at most `equal` <= kTuneList in all, unless a wait ran out)
+            for (unsigned int q = 0; q < count && at + q < kTuneList; ++q) sh.list[at + q] = key;       // (at most kTuneList of a block's, unless a wait ran out)
         });
         if constexpr (CS > 1) {
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             if (rank == 0 && tid == 0) mbar_arrive_expect_tx(&sh.list_link, CS * kTuneList * 4);
             __syncthreads();
             if (tid == 0) bulk_push(cluster_addr(&sh.recv[rank][0], 0), sh.list, kTuneList * 4, cluster_addr(&sh.list_link, 0));
-            if (rank == 0) {
-                tune_wait(&sh.list_link, 0);
-                if (tid == 0) sh.n_list = 0;
-                __syncthreads();
-                for (int i = tid; i < CS * kTuneList; i += kTuneThreads) {
-                    const uint32_t key = (&sh.recv[0][0])[i];
-                    if (key == 0xffffffffu) continue;
-                    const unsigned int at = atomicAdd(&sh.n_list, 1u);
-                    if (at < kTuneList) sh.list[at] = key;
-                }
-            }
-        }
-        __syncthreads();
-        if (rank == 0 && tid < static_cast<int>(equal)) {
-            const uint32_t key = sh.list[tid];
-            unsigned int less = 0, same = 0;
-            for (unsigned int q = 0; q < equal; ++q) { const uint32_t o = sh.list[q]; less += o < key; same += o == key; }
-            if (less < left && left <= less + same) { sh.found[0] = key | static_cast<uint64_t>(same) << 32; sh.found[1] = less; }   // (all that write, write this)
+            if (rank == 0) tune_wait(&sh.list_link, 0);
         }
         __syncthreads();
         if (rank == 0) {
-            prefix = static_cast<uint32_t>(sh.found[0]);
-            equal = static_cast<unsigned int>(sh.found[0] >> 32);
-            below += static_cast<unsigned int>(sh.found[1]);
+            // (where there is nothing, the lists hold 0xffffffff: no key, its upper bits are no prefix)
+            const uint32_t* const keys = CS > 1 ? reinterpret_cast<const uint32_t*>(&sh.recv[0][0]) : sh.list;
+#pragma unroll 1
+            for (int digit = 1; digit < 3; ++digit) {
+                const int shift = digit == 1 ? 10 : 0;
+                const uint32_t mask = digit == 1 ? 0xfff80000u : 0xfffffc00u, width = digit == 1 ? 511u : 1023u;
+                reinterpret_cast<uint2*>(sh.hist)[tid] = make_uint2(0, 0);      // 1024 bins, two a thread
+                __syncthreads();
+#pragma unroll
+                for (int q = 0; q < (CS > 1 ? CS * kTuneList / kTuneThreads : 1); ++q) {
+                    const uint32_t key = keys[tid + q * kTuneThreads];
+                    if ((key & mask) == prefix) atomicAdd(&sh.hist[(key >> shift) & width], 1u);
+                }
+                __syncthreads();
+                const uint2 c = reinterpret_cast<const uint2*>(sh.hist)[tid];
+                unsigned int incl = c.x + c.y;
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    const unsigned int up = __shfl_up_sync(0xffffffffu, incl, d);
+                    if (lane >= d) incl += up;
+                }
+                if (lane == 31) sh.warp_sum[warp] = incl;
+                __syncthreads();
+                unsigned int run = incl - c.x - c.y;
+#pragma unroll
+                for (int w = 0; w < kTuneThreads / 32; ++w) if (w < warp) run += sh.warp_sum[w];
+                if (left > run && left <= run + c.x + c.y) {                     // one thread
+                    const bool second = left > run + c.x;
+                    sh.found[0] = static_cast<uint32_t>(2 * tid + (second ? 1 : 0)) | static_cast<uint64_t>(second ? c.y : c.x) << 32;
+                    sh.found[1] = second ? run + c.x : run;
+                }
+                __syncthreads();
+                prefix |= static_cast<uint32_t>(sh.found[0]) << shift;
+                equal = static_cast<unsigned int>(sh.found[0] >> 32);
+                below += static_cast<unsigned int>(sh.found[1]);
+                left -= static_cast<unsigned int>(sh.found[1]);
+                __syncthreads();                      // (found and the histogram may be written again)
+            }
         }
     }
 

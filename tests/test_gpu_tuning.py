@@ -154,3 +154,30 @@ def test_long_rows_and_many_thresholds(B, G, K):
             need = int(np.ceil(np.float64(F(target)) * B))
             m, _ = tun.threshold_sweep(D, np.array([T, np.nextafter(F(T), F(-np.inf))], dtype=F), cmp)
             assert m[0] == got and round(float(np.float64(m[0]) * B)) >= need > round(float(np.float64(m[1]) * B))
+
+
+@pytest.mark.parametrize("B,G", [(520, 3), (600, 8), (4096, 8), (8192, 4)])
+@pytest.mark.parametrize("kind", ["spread", "narrow", "one_block", "ties", "inf"])
+def test_calibration_of_many_values_that_share_their_upper_bits(B, G, kind):
+    """The value looked for shares its upper twelve bits with hundreds or thousands of others: all in one block's rows, so
+    many in every block that they do not fit its list, equal to one another, or infinite."""
+    rng = np.random.default_rng(B + G)
+    D = (rng.random((B, G), dtype=F) ** 3 * F(0.6931)).astype(F)
+    if kind == "narrow":
+        D = (F(0.1251) + F(0.007) * rng.random((B, G), dtype=F)).astype(F)
+    elif kind == "one_block":
+        D[: B // 8] = F(0.1251) + F(0.007) * rng.random((B // 8, G), dtype=F)
+        D[B // 8:] *= rng.choice(np.array([1e-3, 100.0], dtype=F), size=(B - B // 8, 1))
+    elif kind == "ties":
+        D = rng.choice(np.array([0.126, 0.1261, 0.1262, 0.5], dtype=F), size=(B, G))
+    elif kind == "inf":
+        D[rng.random((B, G)) < 0.2] = np.inf
+        D[5, 1] = np.nan
+    for target in (0.3, 0.4 * G, 0.97 * G):
+        for cmp in ("lt", "le"):
+            # an order statistic of the prefix maxima (the oracle's search is quadratic); the mean it gives from the oracle
+            p = np.sort(np.maximum.accumulate(D, axis=1).ravel())           # (NaN propagates, and sorts last)
+            v = p[min(int(np.ceil(float(F(target)) * B)), D.size) - 1]
+            want = F(np.inf) if not v < np.inf else v if cmp == "le" else np.nextafter(v, F(np.inf))
+            T, got = _gpu_calibrate(D, target, cmp)
+            assert T == want and got == tun.threshold_sweep(D, [want], cmp)[0][0], (target, cmp, T, want)

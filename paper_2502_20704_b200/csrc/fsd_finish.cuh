@@ -1049,7 +1049,13 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
         all = cluster_exchange(P, sh, cs, rank, link, mine);
         if (link.lost) return;
         Ma = 0.0; Mb = 0.0; flags = 0.0;
-        for (int r = 0; r < cs; ++r) { Za += all[r][0]; Zb += all[r][1]; flags = all[r][4] == 1.0 || flags == 1.0 ? 1.0 : fmax(flags, all[r][4]); }
+        // (a CTA a lane, here and below: sums over eight of them in a row are a third of a microsecond each)
+        const double (&its)[kExchangeDoubles] = all[lane < cs ? lane : 0];
+        Za = lane < cs ? its[0] : 0.0; Zb = lane < cs ? its[1] : 0.0;
+#pragma unroll
+        for (int m = 8; m > 0; m >>= 1) { Za += shfl_xor_d(Za, m); Zb += shfl_xor_d(Zb, m); }
+        Za = __shfl_sync(0xffffffffu, Za, 0); Zb = __shfl_sync(0xffffffffu, Zb, 0);
+        flags = __any_sync(0xffffffffu, its[4] == 1.0) ? 1.0 : __any_sync(0xffffffffu, its[4] == 2.0) ? 2.0 : 0.0;
     } else {
         double z[2] = {0.0, 0.0};
         for_units<DT, ANY_SIZE>(d, warp, lane, true, [&](int, float xa, float xb) {
@@ -1107,15 +1113,14 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
     // are all there is to know.
     const auto residual_of = [&](double sa, double sb, double qa, double qb) { return fmax(sa * iZa - sb * iZb, 0.0) + fmax(qa * iZa - qb * iZb, 0.0); };
     if (one_pass && flags == 0.0 && d.vec) {
-        double W = 0.0, cpre = 0.0, run = 0.0;
-        for (int r = 0; r < cs; ++r) W += residual_of(all[r][2], all[r][3], all[r][5], all[r][6]);
-        const double t = d.u * W;
-        int owner = -1;
-        for (int r = 0; r < cs && owner < 0; ++r) {
-            cpre = run;
-            run += residual_of(all[r][2], all[r][3], all[r][5], all[r][6]);
-            if (run > t) owner = r;
-        }
+        // (With the sums of all CTAs taken one after another: 16 x 6 x 64000 fp32, strict rule, 32.1 us, now 30.0; 2 x 4 x 152064 22.9,
+        // now 21.8; 12 x 6 x 32000, relaxed rule, 20.5, now 18.6.)
+        const double (&its)[kExchangeDoubles] = all[lane < cs ? lane : 0];
+        const Prefix blocks(lane < cs ? residual_of(its[2], its[3], its[5], its[6]) : 0.0, lane);
+        const double t = d.u * blocks.total;
+        const unsigned past = __ballot_sync(0xffffffffu, blocks.upto > t);     // (lanes beyond the CTAs' have the total)
+        const int owner = past != 0 ? __ffs(past) - 1 : -1;
+        const double before_it = __shfl_sync(0xffffffffu, blocks.upto, owner > 0 ? owner - 1 : 0), cpre = owner > 0 ? before_it : 0.0;
         if (owner >= 0) {                                 // (no mass, or lost to rounding at the very end: the general way)
             if (owner != rank) return;
             asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

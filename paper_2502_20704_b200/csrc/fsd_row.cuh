@@ -10,13 +10,16 @@
 // A block's share of a row is `span` granules of 16 bytes.  Its sweeps are dealt out in items, a step (8 entries a lane) of a
 // pair each, pair by pair: a sixteenth of them, in one run, to every warp, so that a warp has to do with one or two pairs.
 //   1. First sweep of a warp's items of a pair, as in the streaming kernel but relative to their exact maxima: e = 2^(logit * log2e - k),
-//      Z, S (or the KL sum), "rows differ"; e parked in tensor memory (eight items a warp: all of the SM's).  The warp that
+//      Z, S (or the KL sum), "rows differ"; e parked in tensor memory.  The warp that
 //      is the last of a pair's folds what the pair's warps have posted and pushes the sums to all blocks of the cluster.
 //   2. A warp per pair folds what the blocks sent into 1/Z_a, 1/Z_b for its block.
 //   3. Second sweep of the items over the parked e, in the same order: JS sum (p+q) log2(p+q), TV sum |p - q|; folded and pushed
 //      likewise (KL has none).
 //   4. Every block judges all pairs from the sums of all blocks, in double precision, and draws as in the finish kernel.
 // A tree's nodes are pairs like any others, each against the target row of its parent.
+// What bounds it: latency.  16 x 5 x 32000 bf16 (16 clusters of 6), cycles from where the inputs may be read: first rows landed
+// 1400, first sweep 6900 (special functions 3400 of them), totals 9000, second sweep 12500 (1700), judged 15600, token 19900: 10.4 us of
+// 12.4 a call among others; 15.4 by the streaming and finish kernels.  1 x 4 x 32000 fp32 11.0 -> 9.1 us, 8 x 5 x 50257 16.1 -> 13.5.
 // All waits are for copies of the block's own or for pushes of its cluster's blocks, which run together by
 // the launch's terms; they are bounded all the same.
 #pragma once
@@ -25,10 +28,10 @@
 
 namespace fsd {
 
-constexpr int kRowMaxPairs = 24;                      // positions of a batch row
-constexpr int kRowItemsPerWarp = 8;                   // parked items: a warp's 128 columns of tensor memory
+constexpr int kRowMaxPairs = kFinishWarps;            // positions of a batch row: a warp judges one (3 x 20 x 16000 with two a warp: 14.9 us, the general path 12.9)
+constexpr int kRowItemsPerWarp = 7;                   // at most; a warp's 128 columns of tensor memory would park eight (26 x 5 x 31000: 19.3 us, the general path 17.4)
 constexpr int kRowMaxItems = kFinishWarps * kRowItemsPerWarp;
-static_assert(kRowMaxPairs < 32 && kRowMaxPairs <= kPairRefs, "a lane and a reference per pair");
+static_assert(kRowMaxPairs < 32 && kRowMaxPairs <= kPairRefs && kRowItemsPerWarp * kParkCols <= 128, "a lane and a reference per pair, columns");
 
 struct alignas(16) RowPost {                          // a warp's sums of a pair
     float z[4];                // za, zb, s0, sb
@@ -279,14 +282,9 @@ __global__ void __launch_bounds__(kFinishThreads, 1) fsd_row_kernel(const __grid
         if (bb != 0) bulk_g2s(d_dst, bsrc, bb, &ex.landed[p]);
     }
     // what the judgement wants from global memory, on its way meanwhile
-    static_assert(kRowMaxPairs <= 2 * kFinishWarps, "two pairs a warp at most");
-    Candidate cand[2] = {{-1, 0.f, 0.f, 0.f}, {-1, 0.f, 0.f, 0.f}};
+    Candidate cand = {-1, 0.f, 0.f, 0.f};
     if constexpr (KIND == kDrawResidual) {
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const int i = warp + k * kFinishWarps;
-            if (i < G) cand[k] = candidate<DT, KIND>(F, b * G + i, t_base + static_cast<size_t>(i) * rb, d_base + static_cast<size_t>(i) * rb);
-        }
+        if (warp < G) cand = candidate<DT, KIND>(F, b * G + warp, t_base + static_cast<size_t>(warp) * rb, d_base + static_cast<size_t>(warp) * rb);
         if constexpr (DT == FSD_BF16) {                   // (the copies take longer than the table)
             for (int i = tid; i < kBf16Count; i += kFinishThreads) bf16_table_entry(*bt, *rs, i);
         }
@@ -415,8 +413,8 @@ __global__ void __launch_bounds__(kFinishThreads, 1) fsd_row_kernel(const __grid
             __syncwarp();
             tmem_wait_st();
             // ---- 2. totals, a warp per pair ----
-#pragma unroll 1
-            for (int p = warp; p < G; p += kFinishWarps) {
+            if (warp < G) {
+                const int p = warp;
                 row_wait(&ex.sums_in[p], P.limit_ns, lost);
                 const float2 tot = pair_totals(ex.zsums[p], cs, lane);
                 if ((lane & 15) == 0) reinterpret_cast<float2*>(&ex.tot[p])[lane >> 4] = tot;
@@ -464,10 +462,8 @@ __global__ void __launch_bounds__(kFinishThreads, 1) fsd_row_kernel(const __grid
 
     // ---- 4. divergences, accept bits, status: a pair per warp; what does not need the second sweep's sums comes before they do ----
     int st = 0, first = G;
-#pragma unroll 1
-    for (int k = 0; k < 2; ++k) {
-        const int i = warp + k * kFinishWarps;
-        if (i >= G) break;
+    if (warp < G) {
+        const int i = warp;
         row_wait(&ex.sums_in[i], P.limit_ns, lost);
         Stats c = no_stats();
         if (lane < cs) {
@@ -475,7 +471,7 @@ __global__ void __launch_bounds__(kFinishThreads, 1) fsd_row_kernel(const __grid
             c.ka = z.x; c.za = z.y; c.kb = z.z; c.zb = z.w; c.s0 = r.x; c.sb = r.y; c.diff = __float_as_uint(r.z);
         }
         PairTotals tot = fold_parts(c, 0.f, __shfl_sync(0xffffffffu, my_bad, i) ? kRecordBadTree : kRecordStats, F.div);
-        const Judged early = judge_pair_early<KIND>(F, rs, tot, i, k == 0 ? cand[0] : cand[1], lane);
+        const Judged early = judge_pair_early<KIND>(F, rs, tot, i, cand, lane);
         if (second) {
             row_wait(&ex.x_in, P.limit_ns, lost);
             tot.X = warp_sum(lane < cs ? static_cast<double>(__uint_as_float(static_cast<uint32_t>(ex.x[i][lane]))) : 0.0);

@@ -359,7 +359,8 @@ def main():
     ws = torch.empty(wsb, dtype=torch.uint8, device="cuda")
     stream = torch.cuda.current_stream()
     sptr = stream.cuda_stream
-    launches_per_step = 2                              # pair kernel + finish kernel
+    # pair kernel + finish kernel; one kernel where a row's logits fit the shared memory of a cluster (counted as one wherever they may)
+    launches_per_step = 2 if (2 * P + 1) * V * (2 if c.dtype == "bf16" else 4) > 16 * 200 * 1024 else 1
 
     def call(t, d):
         if tree:

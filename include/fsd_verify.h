@@ -232,6 +232,8 @@ int fsd_set_stage_event(void *event);
  * have sent after about a millisecond (ordinarily fifteen), and the call's results are the same.
  * mode 4, in such a build only: in the finish kernel, the one kernel of a small call and the tuning kernels one block of each
  * cluster keeps its first values to itself, and the limit of their waits is lowered to 20 ms.
+ * mode 6, in such a build only: in the draw of both kernels one block of each cluster sends its first values after 60 ms, and
+ * one other, never the first, waits for no more than 20 ms: the rows are marked although the first block's own waits end well.
  * mode 0: off (the default).  Process-wide, read when a call is made.  Returns FSD_OK, or
  * FSD_ERR_ENUM for another mode. */
 int fsd_set_timeout_injection(int mode);

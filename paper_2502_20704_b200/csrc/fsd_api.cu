@@ -292,7 +292,7 @@ int launch_all(PairParams pp, FinishParams fp, bool vec, CallFlags* flags, Group
     pp.nonce = next_nonce(); pp.flags = flags;
     fp.flags = flags;
     const int injection = g_mark_timeout.load();
-    fp.silent = injection == 4;
+    fp.silent = injection == 4 ? 1 : injection == 6 ? 2 : 0;
     // everything that can fail without a launch (attributes, the occupancy queries) comes before the first thing put on the
     // stream, of the streaming kernel also where this call does not need it: a later one, under capture, may
     const StreamKernel kernel = stream_kernel<DT>(pp.div, !vec);
@@ -672,11 +672,11 @@ int fsd_debug_checks(int B, int positions, size_t* word_offset) {
 
 int fsd_set_timeout_injection(int mode) {
 #ifdef FSD_DEBUG_CHECKS
-    constexpr int kModes = 4;
+    const bool known = (mode >= 0 && mode <= 4) || mode == 6;
 #else
-    constexpr int kModes = 2;
+    const bool known = mode >= 0 && mode <= 2;
 #endif
-    if (mode < 0 || mode > kModes) return FSD_ERR_ENUM;
+    if (!known) return FSD_ERR_ENUM;
     g_mark_timeout.store(mode);
     return FSD_OK;
 }

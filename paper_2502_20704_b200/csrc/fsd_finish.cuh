@@ -58,7 +58,7 @@ struct FinishParams {
     int32_t* item_bits;        // [B, G] read when records == null
     int32_t* item_status;      // [B, G] read when records == null
     CallFlags* flags;
-    int silent;                // debug build, test aid: the last CTA of each cluster keeps its first exchange's values to itself
+    int silent;                // debug build, test aid: the last CTA of each cluster keeps its first exchange's values to itself (1) or sends them late (2)
     float* divergence;         // [B, G] written here when records != null
     int32_t* accept_len;       // [B]
     int32_t* path;             // [B, max_depth] (tree) or null
@@ -170,6 +170,7 @@ __device__ __forceinline__ double exp2_of_logit(float x, float xmin, double nk, 
 struct Link {
     int turn;                  // exchanges so far
     bool lost;                 // (the same for all of the CTA's threads)
+    const uint64_t* number;    // where the call's number is: what the first CTA of the cluster looks for in the flag
 };
 template <int N>
 __device__ __forceinline__ const double (*cluster_exchange(const FinishParams& P, FinishShared& sh, int cs, int rank, Link& link, const double (&v)[N]))[kExchangeDoubles] {
@@ -178,15 +179,22 @@ __device__ __forceinline__ const double (*cluster_exchange(const FinishParams& P
     if (threadIdx.x == 0) mbar_arrive_expect_tx(&sh.link[buf], static_cast<uint32_t>(cs) * N * 8);
     bool send = threadIdx.x < cs;
 #ifdef FSD_DEBUG_CHECKS
-    if (P.silent && link.turn == 0 && rank == cs - 1 && threadIdx.x != rank) send = false;
+    if (P.silent == 1 && link.turn == 0 && rank == cs - 1 && threadIdx.x != rank) send = false;
+    if (P.silent == 2 && link.turn == 0 && rank == cs - 1) {
+        const uint64_t t0 = global_ns();
+        for (int i = 0; i < 100000 && global_ns() - t0 < 3 * kInjectedWaitNs; ++i) __nanosleep(1000);
+    }
+    const uint64_t limit_ns = P.silent == 1 || (P.silent == 2 && rank == 1) ? kInjectedWaitNs : P.silent == 2 ? 10 * kInjectedWaitNs : 0;
+#else
+    constexpr uint64_t limit_ns = 0;
 #endif
     if (send) {
         const uint32_t dst = cluster_addr(&sh.got[buf][rank][0], threadIdx.x), bar = cluster_addr(&sh.link[buf], threadIdx.x);
 #pragma unroll
         for (int k = 0; k < N; ++k) st_async(dst + 8 * k, static_cast<uint64_t>(__double_as_longlong(v[k])), bar);
     }
-    link.lost = __syncthreads_or(!thread_wait(&sh.link[buf], (link.turn >> 1) & 1, P.silent != 0)) != 0;
-    if (link.lost && threadIdx.x == 0) raise_flag(P.flags, *reinterpret_cast<const volatile uint64_t*>(&P.flags->number));
+    link.lost = __syncthreads_or(!thread_wait(&sh.link[buf], (link.turn >> 1) & 1, limit_ns)) != 0;
+    if (link.lost && threadIdx.x == 0) raise_flag(P.flags, *const_cast<const volatile uint64_t*>(link.number));
     ++link.turn;
     return sh.got[buf];
 }
@@ -1379,7 +1387,7 @@ __global__ void __launch_bounds__(kFinishThreads, 2) fsd_finish_kernel(const __g
     // everything above touched no global memory; what follows reads what the pair kernel wrote
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");       // every CTA of the cluster runs: its shared memory may be written
-    Link link = {0, false};
+    Link link = {0, false, &P.flags->number};
     if (blockIdx.x == 0 && tid == 0) atomicAdd(reinterpret_cast<unsigned long long*>(&P.flags->epoch), 1ull);     // (nothing here reads it)
 
     // ---- 1. divergences, accept bits, status of this row's pairs ----

@@ -182,7 +182,7 @@ __device__ __noinline__ bool warp_wait_slow(uint64_t* bar, uint32_t parity, Call
 }
 // Bounded wait of a thread where nobody raises a flag meanwhile (the exchanges within a cluster, copies of its own).
 // (In one loop: with a function of its own for the waits that take longer, the finish kernel's draws were 1 to 4 % slower.)
-__device__ __forceinline__ bool thread_wait(uint64_t* bar, uint32_t parity, [[maybe_unused]] bool short_limit) {
+__device__ __forceinline__ bool thread_wait(uint64_t* bar, uint32_t parity, [[maybe_unused]] uint64_t limit_ns) {     // (a limit: debug build; 0: none)
 #ifdef FSD_DEBUG_CHECKS
     const uint64_t t0 = global_ns();
 #endif
@@ -190,7 +190,7 @@ __device__ __forceinline__ bool thread_wait(uint64_t* bar, uint32_t parity, [[ma
     for (uint32_t i = 0; i < kSpinLimit; ++i) {
         if (mbar_try_wait(bar, parity)) return true;
 #ifdef FSD_DEBUG_CHECKS
-        if (short_limit && global_ns() - t0 > kInjectedWaitNs) break;
+        if (limit_ns != 0 && global_ns() - t0 > limit_ns) break;
 #endif
     }
     return false;

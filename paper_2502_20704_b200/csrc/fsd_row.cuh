@@ -43,9 +43,10 @@ static_assert(sizeof(RowPost) == 32, "16-byte accesses");
 
 struct RowExchange {
     uint64_t landed[kRowMaxPairs + 1];                // a pair's rows; the bonus row
-    uint64_t sums_in[kRowMaxPairs];                   // all blocks' sums of a pair
+    uint64_t sums_in[kRowMaxPairs];                   // all blocks' sums of a pair (of the first: and the call's number)
     uint64_t ready[kRowMaxPairs];                     // its totals
     uint64_t x_in;                                    // all blocks' second-sweep sums of all pairs
+    uint64_t number;                                  // the call's, as the cluster's first block read it
     alignas(16) float4 zsums[kRowMaxPairs][kMaxClusterSize];      // ka, Za, kb, Zb of each block
     float4 rest[kRowMaxPairs][kMaxClusterSize];       // its s0, sb, "rows differ"
     uint64_t x[kRowMaxPairs][kMaxClusterSize];        // (a float's bits)
@@ -239,7 +240,7 @@ __global__ void __launch_bounds__(kFinishThreads, 1) fsd_row_kernel(const __grid
         mbar_init(&ex.landed[G], 1); mbar_init(&ex.x_in, 1);
         mbar_init(&sh.link[0], 1); mbar_init(&sh.link[1], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        for (int p = 0; p < G; ++p) mbar_arrive_expect_tx(&ex.sums_in[p], static_cast<uint32_t>(cs) * 32);
+        for (int p = 0; p < G; ++p) mbar_arrive_expect_tx(&ex.sums_in[p], static_cast<uint32_t>(cs) * 32 + (p == 0 ? 8 : 0));
         mbar_arrive_expect_tx(&ex.x_in, second ? static_cast<uint32_t>(cs * G) * 8 : 0);
         sh.cand = -1; sh.last_pos = -1; sh.n_acc = G; sh.bad = 0; sh.row_sel = 0; sh.amb = 0; sh.n_close = 0; sh.next = 0; sh.far = 0;
     }
@@ -306,6 +307,12 @@ __global__ void __launch_bounds__(kFinishThreads, 1) fsd_row_kernel(const __grid
     }
     __syncwarp();
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");       // every block of the cluster runs and its barriers are ready
+    // What a block raises where a wait of the draw's runs out is the number the first block of its cluster looks for: that block's
+    // own reading, to all of them.  (A row 0 that ends meanwhile moves the epoch on, and two blocks could read two numbers.)
+    if (rank == 0 && warp == 0) {
+        number = __shfl_sync(0xffffffffu, number, 0);
+        if (lane < cs) st_async(cluster_addr(&ex.number, lane), number, cluster_addr(&ex.sums_in[0], lane));
+    }
 
     bool lost = false;
     const uint32_t taddr = second ? ex.tmem_base + (static_cast<uint32_t>(32 * (warp & 3)) << 16) + static_cast<uint32_t>(128 * (warp >> 2)) : 0;
@@ -493,7 +500,7 @@ __global__ void __launch_bounds__(kFinishThreads, 1) fsd_row_kernel(const __grid
     }
     if (warp == kFinishWarps - 1) row_wait(&ex.landed[G], P.limit_ns, lost);      // (every pair's copies have been waited for by somebody; without them nobody has got here)
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    Link link = {0, __syncthreads_or(lost) != 0};
+    Link link = {0, __syncthreads_or(lost) != 0, &ex.number};
     if (second) {                                         // the second sweep is through with tensor memory
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(ex.tmem_base), "n"(kTmemCols) : "memory");
@@ -528,8 +535,9 @@ __global__ void __launch_bounds__(kFinishThreads, 1) fsd_row_kernel(const __grid
     if (rank == 0 && tid == 0) {
         F.accept_len[b] = n;
         F.row_status[b] = status | (link.lost || P.raise || timed_out(F.flags, number) ? FSD_ROW_TIMEOUT : 0);
-        // (The rows need nothing of one another, and a row is marked where a wait of its own cluster ran out.  The number is what a flag raised for this call carries;
-        // a cluster that starts after this one has ended, other kernels in its place until then, has another number, and no flag is raised for that.)
+        // (The rows need nothing of one another, and a row is marked where a wait of its own cluster ran out: a block that has lost one before the draw sends
+        // nothing there, so that this block's own wait runs out; one that loses one in the draw has raised the flag, see cluster_exchange.  A cluster that starts
+        // after row 0's has ended, other kernels in its place until then, has another number, which is raised and looked for by itself alone.)
         if (b == 0) { F.flags->number = number; atomicAdd(reinterpret_cast<unsigned long long*>(&F.flags->epoch), 1ull); }
     }
     leave_last(link.lost);

@@ -55,7 +55,7 @@ __device__ __forceinline__ void bulk_push(uint32_t dst, const void* src, uint32_
 struct TuneWait {
     bool lost;
     bool short_limit;                     // (test aid)
-    __device__ __forceinline__ void operator()(uint64_t* bar, uint32_t parity) { if (!lost && !thread_wait(bar, parity, short_limit)) lost = true; }
+    __device__ __forceinline__ void operator()(uint64_t* bar, uint32_t parity) { if (!lost && !thread_wait(bar, parity, short_limit ? kInjectedWaitNs : 0)) lost = true; }
 };
 #ifdef FSD_DEBUG_CHECKS
 #define FSD_TUNE_SILENT (silent != 0)

@@ -158,3 +158,43 @@ def test_waits_within_a_cluster_that_run_out_are_reported():
     env = dict(os.environ, FSD_VERIFY_LIB=lib_build.build(debug=True), PYTHONPATH=root + os.pathsep + os.environ.get("PYTHONPATH", ""))
     r = subprocess.run([sys.executable, "-c", _SCRIPT], cwd=root, env=env, capture_output=True, text=True, timeout=600)
     assert r.returncode == 0 and "reported" in r.stdout, r.stdout[-2000:] + r.stderr[-4000:]
+
+
+_LATE = r"""
+import numpy as np
+import fsd_inputs as gi
+from paper_2502_20704_b200 import binding as fsd
+from tests import parity
+assert fsd.fsd_debug_checks()[0], "this process must have loaded the debug build"
+c = gi.make_chain(6, 4, 36000, dtype="bf16", recipe="zipf", sigma=(0.3, 1.5), sigma_mode="uniform", workload_id=434)
+t = gi.make_tree(3, 9, 32000, dtype="bf16", sigma=0.6, max_depth=5, workload_id=446)
+
+def calls():
+    for mode, sample in (("fsd", "invcdf"), ("fsd", "greedy"), ("sd", "invcdf"), ("rfsd", "greedy")):
+        yield parity.run_chain_gpu(c.target, c.draft, c.draft_tokens, c.u_accept, c.u_sample, c.dtype, mode=mode, sample=sample, T=0.2)
+    yield parity.run_tree_gpu(t.target, t.draft, t.parent, t.u_sample, 5, t.dtype, T=0.05)
+
+for size in (0, 2):                                      # one kernel; the streaming and finish kernels
+    assert fsd.fsd_set_group_size(size) == 0
+    want = list(calls())
+    assert fsd.fsd_set_timeout_injection(6) == 0
+    for k, r in enumerate(calls()):
+        assert (r.row_status & fsd.FSD_ROW_TIMEOUT).all(), (size, k, r.row_status)
+    assert fsd.fsd_set_timeout_injection(0) == 0
+    for r, w in zip(calls(), want):
+        assert (r.row_status == 0).all() and np.array_equal(r.next_token, w.next_token) and np.array_equal(r.accept_len, w.accept_len)
+print("reported")
+"""
+
+
+def test_a_wait_that_runs_out_in_a_later_block_of_the_draw_is_reported():
+    """A block of the cluster other than the first gives up in the draw, while the first gets all it waits for (debug build,
+    in a process of its own).  The token may be the later block's to write, so the row has to be marked."""
+    import os
+    import subprocess
+    import sys
+    from paper_2502_20704_b200 import build as lib_build
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    env = dict(os.environ, FSD_VERIFY_LIB=lib_build.build(debug=True), PYTHONPATH=root + os.pathsep + os.environ.get("PYTHONPATH", ""))
+    r = subprocess.run([sys.executable, "-c", _LATE], cwd=root, env=env, capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0 and "reported" in r.stdout, r.stdout[-2000:] + r.stderr[-4000:]

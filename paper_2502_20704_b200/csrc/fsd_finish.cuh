@@ -617,7 +617,7 @@ __device__ __forceinline__ void draw_pt(const FinishParams& P, FinishShared& sh,
     // ---- totals of warp, CTA and cluster, in a fixed order and on one scale: 2^0, or where a reference is out of a
     //      double's reach the largest reference of the cluster ----
     double K = 0.0, W, w_v, w_upto;
-    [[maybe_unused]] double blocks_upto = 0.0;        // LOCAL: the CTAs' running totals, a lane each
+    [[maybe_unused]] double blocks_v = 0.0, blocks_upto = 0.0;      // LOCAL: the CTAs' totals and running totals, a lane each
     const double (*all)[kExchangeDoubles];
 #pragma unroll 1
     for (bool scaled = false;; scaled = true) {
@@ -634,7 +634,7 @@ __device__ __forceinline__ void draw_pt(const FinishParams& P, FinishShared& sh,
         if constexpr (LOCAL) {                        // (clusters of up to sixteen: one scan is shorter than sixteen additions in a row)
             const double (&its)[kExchangeDoubles] = all[lane < d.cs ? lane : 0];
             const Prefix blocks(lane < d.cs ? its[0] : 0.0, lane);
-            blocks_upto = blocks.upto;
+            blocks_v = blocks.v; blocks_upto = blocks.upto;
             W = blocks.total;
             if (!__any_sync(0xffffffffu, its[1] != 0.0)) break;
         } else {
@@ -661,7 +661,8 @@ __device__ __forceinline__ void draw_pt(const FinishParams& P, FinishShared& sh,
     double cpre = 0.0;
     int owner = -1;
     if constexpr (LOCAL) {
-        const unsigned past = __ballot_sync(0xffffffffu, blocks_upto > t);     // (lanes beyond the CTAs' have the total)
+        // (with weight: the scan's lanes add in different orders, and one without may be an ulp above the one before it)
+        const unsigned past = __ballot_sync(0xffffffffu, blocks_v > 0.0 && blocks_upto > t);
         owner = past != 0 ? __ffs(past) - 1 : -1;
         const double before_it = __shfl_sync(0xffffffffu, blocks_upto, owner > 0 ? owner - 1 : 0);
         cpre = owner > 0 ? before_it : 0.0;
@@ -1126,7 +1127,7 @@ __device__ __forceinline__ void draw_residual(const FinishParams& P, FinishShare
         const double (&its)[kExchangeDoubles] = all[lane < cs ? lane : 0];
         const Prefix blocks(lane < cs ? residual_of(its[2], its[3], its[5], its[6]) : 0.0, lane);
         const double t = d.u * blocks.total;
-        const unsigned past = __ballot_sync(0xffffffffu, blocks.upto > t);     // (lanes beyond the CTAs' have the total)
+        const unsigned past = __ballot_sync(0xffffffffu, blocks.v > 0.0 && blocks.upto > t);     // (with weight, as in draw_pt)
         const int owner = past != 0 ? __ffs(past) - 1 : -1;
         const double before_it = __shfl_sync(0xffffffffu, blocks.upto, owner > 0 ? owner - 1 : 0), cpre = owner > 0 ? before_it : 0.0;
         if (owner >= 0) {                                 // (no mass, or lost to rounding at the very end: the general way)

@@ -7,7 +7,9 @@ import numpy as np
 import pytest
 
 import fsd_inputs as gi
+import paper_2502_20704_b200 as fsd
 from tests import parity
+from tests.test_gpu_row_kernel import ULP_LOGITS, one_entry_a_block
 
 pytestmark = pytest.mark.gpu
 
@@ -173,3 +175,17 @@ def test_residual_of_bf16_rows_off_the_table_with_close_calls_and_masked_entries
     assert (r["accept_len"] < 2).any()
     _check(c, mode="sd", sample="greedy")
     _check(c, mode="rfsd", T=0.0)
+
+
+def test_a_thread_block_without_residual_draws_nothing():
+    """The finish kernel's residual draw, eight thread blocks of which each has 1024 vectors or what is left."""
+    V, span = 20000, 4096
+    t = one_entry_a_block(V, span, 1)
+    d = np.full((1, 1, V), -np.inf, np.float32)
+    d[0, 0, V - 1] = 0.0
+    assert fsd.fsd_set_group_size(2) == 0
+    try:
+        r = parity.run_chain_gpu(t, d, np.full((1, 1), V - 1, np.int32), np.zeros((1, 1), np.float32), np.full(1, 0.5, np.float32), "f32", mode="sd")
+    finally:
+        fsd.fsd_set_group_size(0)
+    assert r.row_status[0] == 0 and r.next_token[0] in [block * span for block in ULP_LOGITS]

@@ -106,3 +106,27 @@ def test_small_trees(dtype, B, N, V):
     t.parent[0, N - 1] = N - 1                          # not a tree
     g, _ = parity.check_tree(t, T=0.05)
     assert g.row_status[0] & 4 and g.next_token[0] == -1
+
+
+# Logits of weights 1, 0.75 ulp and 0.6 ulp, nothing, 1 (ulp: 2^-52) in blocks 0, 1, 2, 3, 4 of a cluster: a scan over the
+# blocks gives 1 + ulp up to block 2 and 1 + 2 ulp up to block 3, and half of the total is 1 + ulp.
+ULP_LOGITS = {0: 0.0, 1: float(np.log(0.75) - 52 * np.log(2.0)), 2: float(np.log(0.6) - 52 * np.log(2.0)), 4: 0.0}
+
+
+def one_entry_a_block(V, span, position_rows):
+    t = np.full((1, position_rows + 1, V), -np.inf, np.float32)
+    for block, x in ULP_LOGITS.items():
+        t[0, :, block * span] = x
+    return t
+
+
+@pytest.mark.parametrize("mode", ["fsd", "sd"])
+@pytest.mark.parametrize("V,span", [(32000, 2048), (32000, 2304), (32000, 2560), (32000, 2816), (24000, 2048), (32000, 3328), (32000, 4096)])
+def test_a_block_without_weight_draws_nothing(mode, V, span):
+    """What a block of the cluster holds depends on how many there are: spans of one to another number of blocks are tried."""
+    t = one_entry_a_block(V, span, 1)
+    d = np.full((1, 1, V), -np.inf, np.float32)
+    d[0, 0, V - 1] = 0.0
+    r = parity.run_chain_gpu(t, d, np.full((1, 1), V - 1, np.int32), np.zeros((1, 1), np.float32), np.full(1, 0.5, np.float32), "f32", mode=mode, T=0.0)
+    assert r.row_status[0] == 0 and r.accept_len[0] == 0
+    assert r.next_token[0] in [block * span for block in ULP_LOGITS]

@@ -21,7 +21,7 @@
 // 1400, first sweep 6900 (special functions 3400 of them), totals 9000, second sweep 12500 (1700), judged 15600, token 19900: 10.4 us of
 // 12.4 a call among others; 15.4 by the streaming and finish kernels.  1 x 4 x 32000 fp32 11.0 -> 9.1 us, 8 x 5 x 50257 16.1 -> 13.5.
 // All waits are for copies of the block's own or for pushes of its cluster's blocks, which run together by
-// the launch's terms; they are bounded all the same.
+// the launch's terms; they are bounded all the same.  A block that has lost one leaves when its copies have landed, and last.
 #pragma once
 
 #include "fsd_finish.cuh"
@@ -501,6 +501,7 @@ __global__ void __launch_bounds__(kFinishThreads, 1) fsd_row_kernel(const __grid
     if (warp == kFinishWarps - 1) row_wait(&ex.landed[G], P.limit_ns, lost);      // (every pair's copies have been waited for by somebody; without them nobody has got here)
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     Link link = {0, __syncthreads_or(lost) != 0, &ex.number};
+    if (link.lost && tid <= G) thread_wait(&ex.landed[tid], 0, 0);             // no copy may still be on its way into a block that leaves
     if (second) {                                         // the second sweep is through with tensor memory
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(ex.tmem_base), "n"(kTmemCols) : "memory");

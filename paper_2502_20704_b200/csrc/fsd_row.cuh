@@ -307,15 +307,18 @@ __global__ void __launch_bounds__(kFinishThreads, 1) fsd_row_kernel(const __grid
     }
     __syncwarp();
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");       // every block of the cluster runs and its barriers are ready
-    // What a block raises where a wait of the draw's runs out is the number the first block of its cluster looks for: that block's
-    // own reading, to all of them.  (A row 0 that ends meanwhile moves the epoch on, and two blocks could read two numbers.)
-    if (rank == 0 && warp == 0) {
-        number = __shfl_sync(0xffffffffu, number, 0);
-        if (lane < cs) st_async(cluster_addr(&ex.number, lane), number, cluster_addr(&ex.sums_in[0], lane));
-    }
 
     bool lost = false;
     const uint32_t taddr = second ? ex.tmem_base + (static_cast<uint32_t>(32 * (warp & 3)) << 16) + static_cast<uint32_t>(128 * (warp >> 2)) : 0;
+    // What a block raises where a wait of the draw's runs out is the number the first block of its cluster looks for: that block's
+    // own reading, to all of them.  (A row 0 that ends meanwhile moves the epoch on, and two blocks could read two numbers.
+    // Told in front of the first sweep, 16 x 5 x 32000 took 0.04 us more: the reading is a trip to L2.)
+    const auto tell_number = [&] {
+        if (rank == 0 && warp == 0) {
+            const uint64_t n = __shfl_sync(0xffffffffu, number, 0);
+            if (lane < cs) st_async(cluster_addr(&ex.number, lane), n, cluster_addr(&ex.sums_in[0], lane));
+        }
+    };
     const auto sweeps = [&](auto div_tag) {
         constexpr int DIV = decltype(div_tag)::value;
         // A vector of item (p, step)'s rows, target row `tr`
@@ -416,6 +419,7 @@ __global__ void __launch_bounds__(kFinishThreads, 1) fsd_row_kernel(const __grid
                 }
             }
         }
+        tell_number();
         if constexpr (DIV != FSD_DIV_KL) {
             __syncwarp();
             tmem_wait_st();

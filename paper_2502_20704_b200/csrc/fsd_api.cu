@@ -239,6 +239,10 @@ const int* prepare_row(int dev) {
 // within 2 %: us on a B200 by the streaming and finish kernels / in clusters of half the size / of the size taken:
 //   1 x 4 x 32000 fp32 11.6 / 10.1 / 9.3 (16)    16 x 5 x 32000 16.0 / - / 12.6 (6)    8 x 5 x 50257 16.6 / - / 13.6 (10)
 //   8 x 3 x 64000 13.7 / - / 11.4 (10)    28 x 5 x 8192 12.8 / 11.7 / 10.8 (4)    4 x 16 x 8000 12.1 / 10.8 / 10.2 (16)
+// At most twelve: a cluster's SMs are of one GPC, so the larger it is the sooner it waits for other kernels to end.  Beside a
+// kernel that has a block on 60 (74, 90, 100, 110, 120, 132) of the SMs for 1 ms, 1 x 4 x 32000 fp32 waits for its end in clusters of 16 (14, 12, 10,
+// 8 with 120, 6 with 132); the general path with 132.  Alone it takes 9.24 us in 16, 9.63 in 12, 10.1 in 8, 11.5 by the general path: twelve leave
+// a call its time beside kernels that hold half of the GPU.
 struct RowPlan { int cs, span; };                                      // cs 0: not by the row kernel
 template <int DT, int KIND, bool RAGGED>
 RowPlan row_plan(int B, int G, size_t nvec_row, const int* most) {

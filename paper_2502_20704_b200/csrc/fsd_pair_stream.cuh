@@ -61,7 +61,7 @@ constexpr int kStepEntries = 8;                            // vocabulary entries
 constexpr int kTmemCols = 512;                             // all of the SM's columns: warp w owns 32 lanes x 128 columns
 constexpr int kParkCols = 2 * kStepEntries;                // e values a lane parks per step (both rows)
 constexpr int kPortableCluster = 8;                        // most thread blocks of a cluster without asking for more (finish kernel)
-constexpr int kMaxClusterSize = 16;                        // and at all (row kernel)
+constexpr int kMaxClusterSize = 12;                        // and at all (row kernel, see row_plan)
 constexpr int kMaxGroupSize = 24;                          // most blocks in a group of the streaming kernel
 constexpr uint32_t kSpinLimit = 1u << 24;                  // polls before a wait gives up
 constexpr uint64_t kWaitNs = 4000000000ull;                // and its limit in time

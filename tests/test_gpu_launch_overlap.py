@@ -120,6 +120,42 @@ def test_calls_beside_kernels_that_hold_most_of_the_gpu():
     assert all(_same(c.out, want[0]) for c in calls)
 
 
+@pytest.mark.parametrize("B,gamma,V", [(1, 4, 32000), (1, 4, 8192), (4, 8, 16000), (7, 5, 32000)])
+def test_a_small_call_finds_room_beside_kernels_that_hold_half_of_the_gpu(B, gamma, V):
+    """74 of the 148 SMs have a block of another kernel for 0.2 s; a call of a few rows does not wait for these to end."""
+    import ctypes
+    import time
+    devs, want = _inputs(1, B, gamma, V, 0.2)
+    call, s = _Call(B, gamma, V, 0.2), torch.cuda.Stream()
+    call.load(devs[0])
+    call(torch.cuda.current_stream())
+    for o in call.out: o.zero_()
+    torch.cuda.synchronize()
+    raw = [ctypes.c_void_p() for _ in range(74)]         # (streams of torch's own are 32 in all)
+    for r in raw:
+        assert int(torch.cuda.cudart().cudaStreamCreate(ctypes.addressof(r))) == 0
+    holders, done, end = [torch.cuda.ExternalStream(r.value) for r in raw], torch.cuda.Event(), []
+    try:
+        for h in holders:
+            with torch.cuda.stream(h):
+                torch.cuda._sleep(400_000_000)
+                end.append(torch.cuda.Event())
+                end[-1].record(h)
+        time.sleep(0.01)
+        call(s)
+        done.record(s)
+        limit = time.time() + 0.08
+        while not done.query() and time.time() < limit:
+            time.sleep(0.001)
+        in_time, held = done.query(), sum(not e.query() for e in end)
+    finally:
+        torch.cuda.synchronize()
+        for r in raw:
+            torch.cuda.cudart().cudaStreamDestroy(r.value)
+    assert held == 74, f"only {held} SMs were held"
+    assert in_time and _same(call.out, want[0])
+
+
 _SCRIPT = r"""
 import fsd_inputs as gi
 import paper_2502_20704_b200 as fsd

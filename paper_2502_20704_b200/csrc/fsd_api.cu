@@ -250,7 +250,11 @@ RowPlan row_plan(int B, int G, size_t nvec_row, const int* most) {
     const RowPlan none = {0, 0};
     if (G > kRowMaxPairs || nvec_row > static_cast<size_t>(kMaxClusterSize) * kRowMaxItems * step) return none;
     for (int cs = kMaxClusterSize; cs >= 1; --cs) {
-        if (most[cs - 1] < B) continue;
+        // (A GPU that by the occupancy calculation holds 45 clusters of three, or 26 of five, does so where their places work out: 43 to
+        // 45 of three were 1.03, 1.24 and 1.38 times as long as clusters of two, 25 and 26 of five 1.19 and 1.37 times as long as clusters
+        // of four, as in a second wave; 42 and 24 were faster, and other sizes up to the last cluster.  25 x 8 x 16000 KL 11.2 -> 11.5 us in 25 of five.)
+        const int room = cs == 3 || cs == 5 ? most[cs - 1] * 15 / 16 : most[cs - 1];
+        if (room < B) continue;
         const int span = (static_cast<int>((nvec_row + cs - 1) / cs) + step - 1) / step * step, steps = span / step;
         if (steps * G > kRowMaxItems || row_bytes_of(G, span, RAGGED) > row_smem_left<DT, KIND>()) continue;
         return {cs, span};

@@ -201,3 +201,36 @@ def check_tree(c, T, div="js", cmp="lt", sample="invcdf"):
         assert g.next_token[b] == t_o or lo <= g.next_token[b] <= hi, f"row {b}: token {g.next_token[b]} vs {t_o}"
     assert np.array_equal(g.row_status, o.row_status)
     return g, o
+
+
+def kernels_of(call) -> int:
+    """Kernels that call() puts on the current stream, from the nodes of a captured graph."""
+    import ctypes
+    driver = ctypes.CDLL("libcuda.so.1")
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    call()                                               # (the kernels' attributes cannot be set under capture)
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        call()
+    raw, n, kind, kernels = ctypes.c_void_p(graph.raw_cuda_graph()), ctypes.c_size_t(0), ctypes.c_int(0), 0
+    assert driver.cuGraphGetNodes(raw, None, ctypes.byref(n)) == 0
+    nodes = (ctypes.c_void_p * n.value)()
+    assert driver.cuGraphGetNodes(raw, nodes, ctypes.byref(n)) == 0
+    for node in nodes:
+        assert driver.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
+        kernels += kind.value == 0                       # CU_GRAPH_NODE_TYPE_KERNEL
+    return kernels
+
+
+def chain_kernels(B, gamma, V, dtype="bf16", **opts) -> int:
+    """Kernels of a chain call of that shape: one where it is done whole in one, else two."""
+    o = fsd.make_opts(dtype=dtype, **opts)
+    t = torch.zeros(B, gamma + 1, V, dtype=torch.bfloat16 if dtype == "bf16" else torch.float32, device="cuda")
+    ints, floats = torch.zeros(3 * B + B * gamma, dtype=torch.int32, device="cuda"), torch.zeros(B + 2 * B * gamma, device="cuda")
+    n = fsd.fsd_workspace_bytes(B, gamma, V, o)
+    ws = torch.zeros(n, dtype=torch.uint8, device="cuda")
+
+    def call():
+        assert fsd.fsd_verify_chain(t, t, ints[3 * B:], floats[B:], floats, B, gamma, V, o, ints, ints[B:], floats[B + B * gamma:], ints[2 * B:], ws, n,
+                                    torch.cuda.current_stream().cuda_stream) == 0
+    return kernels_of(call)

@@ -130,3 +130,10 @@ def test_a_block_without_weight_draws_nothing(mode, V, span):
     r = parity.run_chain_gpu(t, d, np.full((1, 1), V - 1, np.int32), np.zeros((1, 1), np.float32), np.full(1, 0.5, np.float32), "f32", mode=mode, T=0.0)
     assert r.row_status[0] == 0 and r.accept_len[0] == 0
     assert r.next_token[0] in [block * span for block in ULP_LOGITS]
+
+
+@pytest.mark.parametrize("B,gamma,V,kernels", [(24, 8, 16000, 1), (25, 8, 16000, 2), (26, 3, 28544, 1), (42, 3, 19000, 1), (43, 3, 19000, 2), (45, 3, 8800, 1)])
+def test_no_call_is_shared_out_over_clusters_that_hardly_fit(B, gamma, V, kernels):
+    """More than 24 clusters of five, or 42 of three, take two waves: smaller clusters do the call, or where a row does not fit
+    those the streaming and finish kernels."""
+    assert parity.chain_kernels(B, gamma, V, T=0.2) == kernels

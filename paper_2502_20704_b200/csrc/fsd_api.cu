@@ -243,10 +243,20 @@ const int* prepare_row(int dev) {
 // kernel that has a block on 60 (74, 90, 100, 110, 120, 132) of the SMs for 1 ms, 1 x 4 x 32000 fp32 waits for its end in clusters of 16 (14, 12, 10,
 // 8 with 120, 6 with 132); the general path with 132.  Alone it takes 9.24 us in 16, 9.63 in 12, 10.1 in 8, 11.5 by the general path: twelve leave
 // a call its time beside kernels that hold half of the GPU.
+// A call whose clusters have less than half of the SMs is spread over more of them by the streaming kernel, and there the row kernel gains
+// only while a warp has little to do: at most five items, or four where there is no second sweep whose exchange it would save (KL), or one where
+// an argmax, the shortest draw, follows the sweeps of more than nine positions.  us on a B200 by the streaming and finish kernels / by this one:
+//   3 x 14 x 20352 KL greedy (7 items a warp) 8.2 / 9.0    4 x 15 x 21202 KL greedy (7) 9.3 / 10.5    1 x 14 x 19328 JS (7) 11.6 / 12.2
+//   2 x 11 x 10420 fp32 TV greedy (3) 9.5 / 10.2    5 x 10 x 5565 KL greedy (2) 8.4 / 8.7    but 10 x 16 x 8000 KL (4; 100 SMs) 11.3 / 9.5
+// (2000 random calls: 36 were slower by more than 1.5 % without these limits, 6 with them, of which 5 by less than 6 %; the mean gain 1.24 in both.)
+// One more: the argmax of a residual whose rows are not whole vectors is two passes entry by entry, which the finish kernel shares out over two
+// blocks where a row has more than 4096 entries (80 x 1 x 15580 TV rFSD greedy 35.7 / 45.8 in clusters of one).
 struct RowPlan { int cs, span; };                                      // cs 0: not by the row kernel
 template <int DT, int KIND, bool RAGGED>
-RowPlan row_plan(int B, int G, size_t nvec_row, const int* most) {
+RowPlan row_plan(const FinishParams& fp, int nsm, size_t nvec_row, const int* most) {
     constexpr int step = 32 * StreamShape<DT>::kVecPerStep;
+    const int B = fp.B, G = fp.G;
+    const bool greedy = fp.sample == FSD_SAMPLE_GREEDY;
     const RowPlan none = {0, 0};
     if (G > kRowMaxPairs || nvec_row > static_cast<size_t>(kMaxClusterSize) * kRowMaxItems * step) return none;
     for (int cs = kMaxClusterSize; cs >= 1; --cs) {
@@ -257,6 +267,9 @@ RowPlan row_plan(int B, int G, size_t nvec_row, const int* most) {
         if (room < B) continue;
         const int span = (static_cast<int>((nvec_row + cs - 1) / cs) + step - 1) / step * step, steps = span / step;
         if (steps * G > kRowMaxItems || row_bytes_of(G, span, RAGGED) > row_smem_left<DT, KIND>()) continue;
+        const int per_warp = (steps * G + kFinishWarps - 1) / kFinishWarps;
+        if (2 * B * cs < nsm && per_warp > (greedy && G > 9 ? 1 : fp.div == FSD_DIV_KL ? 4 : 5)) return none;
+        if (KIND == kDrawResidual && RAGGED && greedy && cs == 1 && fp.V > 8 * kFinishThreads) return none;
         return {cs, span};
     }
     return none;
@@ -274,16 +287,16 @@ int launch_row(const FinishParams& fp, int cs, int span, size_t nvec_row, uint64
 }
 // One launch if the row kernel takes the call; `taken` says so.
 template <int DT, int KIND, bool RAGGED>
-int try_row(const FinishParams& fp, size_t nvec_row, int dev, uint64_t nonce, int injection, cudaStream_t s, bool& taken) {
+int try_row(const FinishParams& fp, int nsm, size_t nvec_row, int dev, uint64_t nonce, int injection, cudaStream_t s, bool& taken) {
     const int* most = prepare_row<DT, KIND, RAGGED>(dev);
     if (most == nullptr) return FSD_ERR_CUDA;
-    const RowPlan plan = row_plan<DT, KIND, RAGGED>(fp.B, fp.G, nvec_row, most);
+    const RowPlan plan = row_plan<DT, KIND, RAGGED>(fp, nsm, nvec_row, most);
     taken = plan.cs > 0;                                               // (a row kernel is ready for a later call all the same)
     return taken ? launch_row<DT, KIND, RAGGED>(fp, plan.cs, plan.span, nvec_row, nonce, injection, s) : FSD_OK;
 }
 template <int DT, int KIND>
-int try_row(const FinishParams& fp, bool vec, size_t nvec_row, int dev, uint64_t nonce, int injection, cudaStream_t s, bool& taken) {
-    return vec ? try_row<DT, KIND, false>(fp, nvec_row, dev, nonce, injection, s, taken) : try_row<DT, KIND, true>(fp, nvec_row, dev, nonce, injection, s, taken);
+int try_row(const FinishParams& fp, int nsm, bool vec, size_t nvec_row, int dev, uint64_t nonce, int injection, cudaStream_t s, bool& taken) {
+    return vec ? try_row<DT, KIND, false>(fp, nsm, nvec_row, dev, nonce, injection, s, taken) : try_row<DT, KIND, true>(fp, nsm, nvec_row, dev, nonce, injection, s, taken);
 }
 
 template <int DT>
@@ -315,9 +328,9 @@ int launch_all(PairParams pp, FinishParams fp, bool vec, CallFlags* flags, Group
     bool row = g_group_size.load() == 0 && g_stage_event.load() == nullptr;
     if (row) {
         fp.records = records;
-        const int rc = fp.mode != FSD_MODE_FSD ? try_row<DT, kDrawResidual>(fp, vec, nvec_row, dev, pp.nonce, injection, s, row)
-                       : fp.sample == FSD_SAMPLE_GREEDY ? try_row<DT, kDrawGreedy>(fp, vec, nvec_row, dev, pp.nonce, injection, s, row)
-                                                        : try_row<DT, kDrawPt>(fp, vec, nvec_row, dev, pp.nonce, injection, s, row);
+        const int rc = fp.mode != FSD_MODE_FSD ? try_row<DT, kDrawResidual>(fp, nsm, vec, nvec_row, dev, pp.nonce, injection, s, row)
+                       : fp.sample == FSD_SAMPLE_GREEDY ? try_row<DT, kDrawGreedy>(fp, nsm, vec, nvec_row, dev, pp.nonce, injection, s, row)
+                                                        : try_row<DT, kDrawPt>(fp, nsm, vec, nvec_row, dev, pp.nonce, injection, s, row);
         if (rc != FSD_OK || row) return rc;
     }
     if (C > 0) {

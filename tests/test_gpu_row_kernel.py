@@ -137,3 +137,12 @@ def test_no_call_is_shared_out_over_clusters_that_hardly_fit(B, gamma, V, kernel
     """More than 24 clusters of five, or 42 of three, take two waves: smaller clusters do the call, or where a row does not fit
     those the streaming and finish kernels."""
     assert parity.chain_kernels(B, gamma, V, T=0.2) == kernels
+
+
+@pytest.mark.parametrize("B,gamma,V,kernels,form", [
+    (4, 15, 21202, 2, dict(div="kl", sample="greedy")), (1, 9, 48704, 2, dict(div="kl")), (1, 6, 30000, 1, dict(div="kl")), (10, 16, 8000, 1, dict(div="kl")),
+    (1, 12, 24672, 2, dict()), (4, 16, 8000, 1, dict()), (2, 10, 12000, 2, dict(div="tv", sample="greedy")), (2, 9, 12000, 1, dict(div="tv", sample="greedy")),
+    (4, 16, 2000, 1, dict(sample="greedy")), (24, 12, 4000, 1, dict(sample="greedy")), (80, 1, 15580, 2, dict(mode="rfsd", sample="greedy")), (80, 1, 15576, 1, dict(mode="rfsd", sample="greedy")),
+])
+def test_calls_of_few_rows_with_much_to_sweep_are_spread_over_the_gpu(B, gamma, V, kernels, form):
+    assert parity.chain_kernels(B, gamma, V, T=0.2, **form) == kernels

@@ -893,9 +893,11 @@ __device__ __noinline__ void classed_pass_bf16(const void* a_row, const void* b_
 }
 // The same for rows whose logits lie so far off 0 that most are outside the table, or that they need a reference: every
 // exponential by the small table and the polynomial, in straight-line code (in the loop above, for the lanes that meet an entry
-// outside the table, it cost the other rows 9 %: 64 x 8 x 152064, strict rule, 133 -> 145 us).
+// outside the table, it cost the other rows 9 %: 64 x 8 x 152064, strict rule, 133 -> 145 us).  It is called from two kernels, so that the
+// compiler has to be told that the table is in shared memory (64 x 8 x 152064 100 below 0, strict rule: 146 us by generic loads, now 142).
 __device__ __noinline__ void classed_pass_far(const void* a_row, const void* b_row, const Share share, float hi, float lo,
                                               const RowExp ea, const RowExp eb, const ResidualShared& rs, Classed& out) {
+    __builtin_assume(__isShared(&rs));
     const int u0 = share.first + (threadIdx.x & 31), u1 = min(share.first + share.iters * 32, share.units);
     Classed c = out;
     uint4 na = make_uint4(0, 0, 0, 0), nb = na;       // the vectors after these, on their way

@@ -24,3 +24,18 @@ def pytest_collection_modifyitems(config, items):
     for item in items:
         if "gpu" in item.keywords:
             item.add_marker(skip)
+
+
+@pytest.fixture
+def group_size(request):
+    """fsd_set_group_size for the test.  0: one kernel does a call whose logits fit on chip.  Else the streaming and finish kernels
+    do it, in groups of that size or, where a row is too long for these, of the library's choice."""
+    from paper_2502_20704_b200 import binding as fsd
+    assert fsd.fsd_set_group_size(request.param) == 0
+    yield request.param
+    fsd.fsd_set_group_size(0)
+
+
+def group_sizes(*sizes):
+    """Marks that run a test, or a file's tests, once per group size."""
+    return [pytest.mark.usefixtures("group_size"), pytest.mark.parametrize("group_size", sizes, indirect=True, ids=[f"groups{n}" for n in sizes])]

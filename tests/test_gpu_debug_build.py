@@ -1,5 +1,6 @@
 """The debug build of the library (the same kernels with their index and range checks compiled
-in) run on chain, tree, fp32, ragged and non-vector shapes in a process of its own: results must
+in) run on chain, tree, fp32, ragged and non-vector shapes in a process of its own, small ones in one kernel and by the
+streaming and finish kernels: results must
 still match the oracle and the workspace's debug word must stay zero."""
 
 import os
@@ -45,13 +46,15 @@ def run(c, tree=False, **kw):
     words.append(word)
     assert word == 0, f"range check failed: bits {word:#x}"
 
-run(gi.make_chain(6, 5, 36000, dtype="bf16", recipe="zipf", sigma=(0.3, 1.5), sigma_mode="uniform", workload_id=440), T=0.2)
-run(gi.make_chain(6, 5, 36000, dtype="bf16", recipe="zipf", sigma=(0.3, 1.5), sigma_mode="uniform", workload_id=440), T=0.2, mode="sd")
-run(gi.make_chain(3, 4, 152064, dtype="bf16", recipe="zipf", sigma=(0.2, 2.0), sigma_mode="uniform", workload_id=441), T=0.2, div="tv")
-run(gi.make_chain(3, 3, 32776, dtype="bf16", recipe="zipf", sigma=(0.5,), workload_id=442), T=0.1, div="kl")
-run(gi.make_chain(2, 3, 100000, dtype="f32", recipe="spike", sigma=(0.5,), workload_id=443), T=0.1)
-run(gi.make_chain(3, 2, 4099, dtype="f32", recipe="spike", sigma=(0.3, 1.0), workload_id=444), T=0.1, mode="rfsd")
-run(gi.make_tree(3, 40, 32000, dtype="bf16", sigma=0.6, max_depth=5, workload_id=445), tree=True, T=0.05)
+for size in (0, 1, 2):
+    assert fsd.fsd_set_group_size(size) == 0
+    run(gi.make_chain(6, 5, 36000, dtype="bf16", recipe="zipf", sigma=(0.3, 1.5), sigma_mode="uniform", workload_id=440), T=0.2)
+    run(gi.make_chain(6, 5, 36000, dtype="bf16", recipe="zipf", sigma=(0.3, 1.5), sigma_mode="uniform", workload_id=440), T=0.2, mode="sd")
+    run(gi.make_chain(3, 4, 152064, dtype="bf16", recipe="zipf", sigma=(0.2, 2.0), sigma_mode="uniform", workload_id=441), T=0.2, div="tv")
+    run(gi.make_chain(3, 3, 32776, dtype="bf16", recipe="zipf", sigma=(0.5,), workload_id=442), T=0.1, div="kl")
+    run(gi.make_chain(2, 3, 100000, dtype="f32", recipe="spike", sigma=(0.5,), workload_id=443), T=0.1)
+    run(gi.make_chain(3, 2, 4099, dtype="f32", recipe="spike", sigma=(0.3, 1.0), workload_id=444), T=0.1, mode="rfsd")
+    run(gi.make_tree(3, 40, 32000, dtype="bf16", sigma=0.6, max_depth=5, workload_id=445), tree=True, T=0.05)
 print("debug words", words)
 """
 

@@ -1,4 +1,4 @@
-"""The finish kernel where its forms part ways, against the oracle: residual draws between rows whose
+"""The finish kernel, and the draws it shares with the kernel of small calls, where their forms part ways, against the oracle: residual draws between rows whose
 normalisers are equal (every entry on which they agree is a close call) or far apart, logits outside the table of
 exponentials (tiny, beyond 64, of one sign, -inf), references out of a double's range, rows off a
 16-byte boundary, and trees and chains whose judging the cluster's thread blocks share."""
@@ -9,9 +9,10 @@ import pytest
 import fsd_inputs as gi
 import paper_2502_20704_b200 as fsd
 from tests import parity
+from tests.conftest import group_sizes
 from tests.test_gpu_row_kernel import ULP_LOGITS, one_entry_a_block
 
-pytestmark = pytest.mark.gpu
+pytestmark = [pytest.mark.gpu, *group_sizes(0, 2)]
 
 
 def _store(c, t, d):
@@ -189,3 +190,8 @@ def test_a_thread_block_without_residual_draws_nothing():
     finally:
         fsd.fsd_set_group_size(0)
     assert r.row_status[0] == 0 and r.next_token[0] in [block * span for block in ULP_LOGITS]
+
+
+def test_these_sizes_reach_the_finish_kernel(group_size):
+    for B, gamma, V, dtype, mode in ((5, 2, 24000, "bf16", "sd"), (6, 2, 32000, "f32", "sd"), (16, 1, 8200, "bf16", "sd"), (4, 2, 9001, "f32", "fsd"), (6, 2, 20011, "bf16", "rfsd")):
+        assert parity.chain_kernels(B, gamma, V, dtype, mode=mode, T=0.2) == (2 if group_size else 1)

@@ -1,7 +1,7 @@
-"""The streaming kernel may be set up before what precedes it in its stream has ended, and nothing makes
-its blocks resident together: inputs written just before the call, calls in a captured graph behind nodes
-of every kind, calls beside kernels that hold most of the GPU, and (in a process that loads the debug
-build) a group that has to do without one of its blocks' sums."""
+"""The first kernel of a call may be set up before what precedes it in its stream has ended, and nothing makes
+the streaming kernel's blocks resident together: inputs written just before the call, calls in a captured graph behind nodes
+of every kind, calls beside kernels that hold much of the GPU, and (in a process that loads the debug
+build) a group of the streaming kernel that has to do without one of its blocks' sums."""
 
 import os
 import subprocess
@@ -14,10 +14,18 @@ import torch
 import fsd_inputs as gi
 from paper_2502_20704_b200 import binding as fsd
 from tests import parity
+from tests.conftest import group_sizes
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 pytestmark = pytest.mark.gpu
+
+
+def both(f):
+    """Calls as the library does them (one kernel at these sizes), and by the streaming and finish kernels."""
+    for m in group_sizes(0, 1):
+        f = m(f)
+    return f
 
 
 class _Call:
@@ -53,6 +61,7 @@ def _same(out, want):
             and np.array_equal(D.view(np.uint32), want.divergence.view(np.uint32)))
 
 
+@both
 @pytest.mark.parametrize("B,gamma,V", [(1, 3, 4096), (6, 4, 36000)])
 def test_inputs_written_just_before_each_of_many_calls(B, gamma, V):
     devs, want = _inputs(3, B, gamma, V, 0.2)
@@ -66,8 +75,10 @@ def test_inputs_written_just_before_each_of_many_calls(B, gamma, V):
     assert all(_same(g, want[k % 3]) for k, g in enumerate(got))
 
 
-def test_calls_in_a_graph_behind_copies_memsets_kernels_and_a_join():
+@both
+def test_calls_in_a_graph_behind_copies_memsets_kernels_and_a_join(group_size):
     B, gamma, V = 6, 4, 36000
+    assert parity.chain_kernels(B, gamma, V, T=0.2) == (2 if group_size else 1)
     devs, want = _inputs(2, B, gamma, V, 0.2)
     a, b = _Call(B, gamma, V, 0.2), _Call(B, gamma, V, 0.2)
     side, other = torch.cuda.Stream(), torch.cuda.Stream()
@@ -162,6 +173,7 @@ import paper_2502_20704_b200 as fsd
 from tests import parity
 assert fsd.fsd_debug_checks()[0], "this process must have loaded the debug build"
 assert fsd.fsd_set_timeout_injection(3) == 0 and fsd.fsd_set_timeout_injection(5) != 0
+assert fsd.fsd_set_group_size(1) == 0                     # (no row below fits one block: groups of the library's choice, by the streaming kernel)
 def chain(*a, **k):
     kw = {x: k.pop(x) for x in ("div", "mode", "T") if x in k}
     c = gi.make_chain(*a, recipe="zipf", sigma=(0.3, 1.5), sigma_mode="uniform", workload_id=480, **k)
@@ -176,13 +188,14 @@ chain(4, 4, 152064, dtype="bf16", mode="sd", T=0.0)
 for size in (1, 2, 3, 16):
     assert fsd.fsd_set_group_size(size) == 0
     chain(5, 3, 16384 * min(size, 3) - 8, dtype="bf16", T=0.2)
-fsd.fsd_set_group_size(0)
+fsd.fsd_set_group_size(1)
 c = gi.make_tree(3, 40, 32000, dtype="bf16", sigma=0.6, max_depth=5, workload_id=445)
 parity.check_tree(c, T=0.05)
 
 # bit for bit what the same call gives when all blocks send: masked parts, late spikes, invalid rows among them
 import numpy as np
 def same(B, gamma, V, dtype, div, special):
+    assert parity.chain_kernels(B, gamma, V, dtype, div=div, T=0.2) == 2
     c = gi.make_chain(B, gamma, V, dtype=dtype, recipe="zipf", sigma=(0.3, 1.5), sigma_mode="uniform", workload_id=481)
     t, d, us = (parity.to_device(x, dtype) for x in (c.target, c.draft, c.u_sample))
     if special:

@@ -2,7 +2,8 @@
 
 The named workloads fix a handful of shapes; this sweep draws others (vocabulary sizes that are
 and are not multiples of the vector width, group sizes 1 to 16, one to five ring stages per
-pair, masked entries) so that every launch configuration of the pair kernels meets the oracle.
+pair, masked entries) so that every launch configuration of the kernels meets the oracle: as the library would do the
+call, and by the streaming and finish kernels whatever the size.
 The number of cases is small by default; FSD_SWEEP_CASES and FSD_SD_SWEEP_CASES in the environment
 extend the two chain sweeps (every case is seeded by its index, so a longer sweep repeats the
 shorter one and goes on).
@@ -15,8 +16,9 @@ import pytest
 
 import fsd_inputs as gi
 from tests import parity
+from tests.conftest import group_sizes
 
-pytestmark = pytest.mark.gpu
+pytestmark = [pytest.mark.gpu, *group_sizes(0, 2)]
 
 
 def _case(it: int):

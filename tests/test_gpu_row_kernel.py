@@ -26,7 +26,7 @@ def _check(c, dev=None, **kw):
 @pytest.mark.parametrize("B,gamma,V", [
     (2, 2, 1), (3, 1, 7), (3, 3, 255), (3, 3, 257),    # less than a step, either side of one
     (1, 2, 8800), (1, 3, 4484), (5, 2, 2056),          # blocks at the end without a granule or with one
-    (1, 8, 57344), (1, 8, 57352), (1, 7, 65536),       # as much as a warp takes, one step more, as much again
+    (1, 8, 57344), (1, 8, 57352), (1, 7, 65536),       # (clusters of sixteen would take these)
     (2, 16, 14000), (1, 16, 6000), (2, 17, 3001),      # a pair a warp, one more
     (37, 3, 5000), (148, 1, 800),                      # clusters of a few blocks and of one
 ])
@@ -146,3 +146,24 @@ def test_no_call_is_shared_out_over_clusters_that_hardly_fit(B, gamma, V, kernel
 ])
 def test_calls_of_few_rows_with_much_to_sweep_are_spread_over_the_gpu(B, gamma, V, kernels, form):
     assert parity.chain_kernels(B, gamma, V, T=0.2, **form) == kernels
+
+
+@pytest.mark.parametrize("B,gamma,V,kernels", [
+    (7, 8, 43008, 1), (7, 8, 43016, 2),                # seven items a warp, one step more
+    (1, 5, 49152, 1), (1, 5, 49160, 2),                # five where a call has few blocks, one step more
+    (1, 12, 3072, 1), (1, 12, 3080, 1),                # a step a block, one more
+])
+def test_as_much_as_a_warp_takes_and_one_step_more(B, gamma, V, kernels):
+    assert parity.chain_kernels(B, gamma, V, T=0.2) == kernels
+    c = _chain(B, gamma, V, "bf16", 825)
+    for form in FORMS[:2] + FORMS[3:4]:
+        _check(c, **form)
+
+
+@pytest.mark.parametrize("V,kernels", [(36864, 1), (36868, 2), (36861, 1), (36865, 2)])
+def test_as_much_as_shared_memory_takes_of_fp32_rows(V, kernels):
+    """Twelve blocks of twelve steps of seventeen rows: whole vectors, and rows that are shifted."""
+    assert parity.chain_kernels(7, 8, V, "f32", T=0.2) == kernels
+    c = _chain(7, 8, V, "f32", 826)
+    for form in FORMS[:4]:
+        _check(c, **form)

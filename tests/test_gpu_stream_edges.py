@@ -1,5 +1,5 @@
-"""The streaming kernel at the sizes where its partition can go wrong, against the oracle: rows of
-one entry to a few granules, either side of a step, of a block's slice and of the longest row it
+"""The streaming kernel at the sizes where its partition can go wrong (and what does a call of such sizes by itself), against
+the oracle: rows of one entry to a few granules, either side of a step, of a block's slice and of the longest row it
 takes; rows and bases that are not 16-byte aligned; logits its quick form has to notice (a late
 spike, masked entries in some parts only); fewer pairs than a round and many rounds."""
 
@@ -10,8 +10,9 @@ import torch
 import fsd_inputs as gi
 import paper_2502_20704_b200 as fsd
 from tests import parity
+from tests.conftest import group_sizes
 
-pytestmark = pytest.mark.gpu
+pytestmark = [pytest.mark.gpu, *group_sizes(0, 1, 2)]
 
 STEP = {"bf16": 256, "f32": 256}          # vocabulary entries of a step (32 lanes x 8)
 SLICE = {"bf16": 16384, "f32": 12288}     # of a block's largest slice
@@ -131,3 +132,9 @@ def test_a_pairs_divergence_is_its_own_rows_alone(dtype, V, div):
     got = divergences()
     assert np.array_equal(got[28:].view(np.uint32), want[28:].view(np.uint32))
     assert not np.array_equal(got[:28].view(np.uint32), want[:28].view(np.uint32))
+
+
+def test_these_sizes_reach_the_streaming_kernel(group_size):
+    for B, gamma, V, dtype in ((3, 2, 256, "bf16"), (3, 2, 16384, "bf16"), (3, 2, 24577, "f32"), (3, 3, 33003, "bf16"), (7, 4, 20003, "bf16")):
+        assert parity.chain_kernels(B, gamma, V, dtype, T=0.2) == (2 if group_size else 1)
+    assert parity.chain_kernels(40, 5, 40003, "bf16", T=0.2) == 2

@@ -1,9 +1,8 @@
-"""A device-side wait that runs out.  Two injections, neither of which faults or hangs anything:
-the library raises the flag itself on the host side of the call (the reporting path alone), and
-one thread block of the streaming kernel withholds a statistics message while the exchange wait's
-limit is lowered to about a tenth of a second, so that the wait of its partners really runs out
-and the kernel's own give-up path runs.  Either way the call must return, mark every row, and
-leave the next call untouched."""
+"""A device-side wait that runs out.  None of the injections faults or hangs anything: a kernel raises the
+flag itself (the reporting path alone), or one thread block withholds what others wait for, or sends it late, while
+the limits of these waits are lowered, so that they really run out and the kernel's own give-up path runs.  Either
+way the call must return, mark every row, and leave the next call untouched.  Small calls do so as the library does
+them, in one kernel, and by the streaming and finish kernels."""
 
 import numpy as np
 import pytest
@@ -12,10 +11,18 @@ import fsd_inputs as gi
 import paper_2502_20704_b200 as fsd
 from paper_2502_20704_b200 import binding
 from tests import parity
+from tests.conftest import group_sizes
 
 pytestmark = pytest.mark.gpu
 
 
+def both(f):
+    for m in group_sizes(0, 1):
+        f = m(f)
+    return f
+
+
+@both
 @pytest.mark.parametrize("mode", [1, 2])
 def test_injected_timeout_marks_every_row_and_the_next_call_is_clean(mode):
     c = gi.make_chain(6, 4, 36000, dtype="bf16", recipe="zipf", sigma=(0.3, 1.5), sigma_mode="uniform", workload_id=430)
@@ -47,11 +54,13 @@ def test_a_wait_that_runs_out_in_a_call_that_fills_the_gpu():
     assert fsd.fsd_set_timeout_injection(3) != 0
 
 
-def test_a_timeout_in_one_replay_of_a_graph_is_not_the_next_ones():
+@both
+def test_a_timeout_in_one_replay_of_a_graph_is_not_the_next_ones(group_size):
     """A captured call is replayed with the same parameters.  The number that marks its messages and its timeout flag is
     another one in every replay all the same: with the flag raised for one replay, that one is marked and
     the one after it is clean."""
     import torch
+    assert parity.chain_kernels(6, 4, 36000, T=0.2) == (2 if group_size else 1)
     c = gi.make_chain(6, 4, 36000, dtype="bf16", recipe="zipf", sigma=(0.3, 1.5), sigma_mode="uniform", workload_id=430)
     want = parity.run_chain_gpu(c.target, c.draft, None, None, c.u_sample, c.dtype, T=0.2)
     opts = fsd.make_opts(dtype="bf16", T=0.2)
@@ -86,6 +95,7 @@ def test_a_timeout_in_one_replay_of_a_graph_is_not_the_next_ones():
         assert clean()
 
 
+@both
 def test_an_injected_timeout_in_a_captured_call_is_reported_by_every_replay():
     import torch
     c = gi.make_chain(3, 2, 4096, dtype="bf16", recipe="zipf", sigma=(0.3, 1.5), sigma_mode="uniform", workload_id=432)
@@ -135,11 +145,14 @@ def statuses():
     yield parity.run_tree_gpu(t.target, t.draft, t.parent, t.u_sample, 5, t.dtype, T=0.05).row_status
 
 want = tuning()
-assert fsd.fsd_set_timeout_injection(4) == 0
-assert all((st & fsd.FSD_ROW_TIMEOUT).all() for st in statuses())
-assert np.isnan(tuning()).all()
-assert fsd.fsd_set_timeout_injection(0) == 0
-assert all((st == 0).all() for st in statuses())
+for size in (0, 1):                                      # the kernel of small calls; the finish kernel
+    assert fsd.fsd_set_group_size(size) == 0 and parity.chain_kernels(6, 4, 36000, T=0.2) == 1 + size
+    assert fsd.fsd_set_timeout_injection(4) == 0
+    assert all((st & fsd.FSD_ROW_TIMEOUT).all() for st in statuses())
+    assert np.isnan(tuning()).all()
+    assert fsd.fsd_set_timeout_injection(0) == 0
+    assert all((st == 0).all() for st in statuses())
+assert fsd.fsd_set_group_size(0) == 0
 assert np.array_equal(tuning(), want) and np.array_equal(want[:200], tun.threshold_sweep(D, Ts.cpu().numpy(), "lt")[0])
 for mode in ("fsd", "sd"):
     parity.check_chain(c.target, c.draft, c.draft_tokens, c.u_accept, c.u_sample, c.dtype, mode=mode, T=0.2)
@@ -148,8 +161,8 @@ print("reported")
 
 
 def test_waits_within_a_cluster_that_run_out_are_reported():
-    """One block of each cluster of the finish kernel and of the tuning kernels keeps its first values to itself (debug
-    build, in a process of its own): rows are marked, tuning results are NaN, and the next calls are clean."""
+    """One block of each cluster of the finish kernel, of the kernel of small calls and of the tuning kernels keeps its first values to
+    itself (debug build, in a process of its own): rows are marked, tuning results are NaN, and the next calls are clean."""
     import os
     import subprocess
     import sys

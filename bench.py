@@ -256,6 +256,27 @@ def run_reference(args, rank: int):
     print(json.dumps(line))
 
 
+def kernels_of(call) -> int:
+    """Kernels that call() puts on the current stream: the kernel nodes of a captured graph (after an ordinary call)."""
+    import ctypes
+    import torch
+    driver, graph = ctypes.CDLL("libcuda.so.1"), torch.cuda.CUDAGraph(keep_graph=True)
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        call()
+    raw, n, kind, kernels = ctypes.c_void_p(graph.raw_cuda_graph()), ctypes.c_size_t(0), ctypes.c_int(0), 0
+    if driver.cuGraphGetNodes(raw, None, ctypes.byref(n)) != 0:
+        raise RuntimeError("cuGraphGetNodes")
+    nodes = (ctypes.c_void_p * n.value)()
+    if driver.cuGraphGetNodes(raw, nodes, ctypes.byref(n)) != 0:
+        raise RuntimeError("cuGraphGetNodes")
+    for node in nodes:
+        if driver.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) != 0:
+            raise RuntimeError("cuGraphNodeGetType")
+        kernels += kind.value == 0                    # CU_GRAPH_NODE_TYPE_KERNEL
+    return kernels
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -359,14 +380,12 @@ def main():
     ws = torch.empty(wsb, dtype=torch.uint8, device="cuda")
     stream = torch.cuda.current_stream()
     sptr = stream.cuda_stream
-    # pair kernel + finish kernel; one kernel where a row's logits fit the shared memory of a cluster (counted as one wherever they may)
-    launches_per_step = 2 if (2 * P + 1) * V * (2 if c.dtype == "bf16" else 4) > 16 * 200 * 1024 else 1
 
-    def call(t, d):
+    def call(t, d, s=sptr):
         if tree:
-            rc = fsd.fsd_verify_tree(t, d, pard, us, B, P, V, c.max_depth, opts, acc, path, tok, D, st, ws, wsb, sptr)
+            rc = fsd.fsd_verify_tree(t, d, pard, us, B, P, V, c.max_depth, opts, acc, path, tok, D, st, ws, wsb, s)
         else:
-            rc = fsd.fsd_verify_chain(t, d, tokd, uad, us, B, P, V, opts, acc, tok, D, st, ws, wsb, sptr)
+            rc = fsd.fsd_verify_chain(t, d, tokd, uad, us, B, P, V, opts, acc, tok, D, st, ws, wsb, s)
         if rc != 0:
             raise RuntimeError(fsd.fsd_status_string(rc))
 
@@ -378,6 +397,7 @@ def main():
     n_ev = args.steps // chunk
     for i in range(args.warmup):
         step(i)
+    launches_per_step = kernels_of(lambda: call(*copies[0], torch.cuda.current_stream().cuda_stream))
     barrier()
     evs = [torch.cuda.Event(enable_timing=True) for _ in range(n_ev + 1)]
     ev_end = torch.cuda.Event(enable_timing=True)

@@ -235,10 +235,12 @@ const int* prepare_row(int dev) {
     return most[dev];
 }
 // Blocks per batch row: the largest cluster of which the GPU holds one for every row at once (a second wave would take as long
-// as the first), whose blocks have room for the row's logits and what is parked of them.  Larger was faster throughout, or
-// within 2 %: us on a B200 by the streaming and finish kernels / in clusters of half the size / of the size taken:
-//   1 x 4 x 32000 fp32 11.6 / 10.1 / 9.3 (16)    16 x 5 x 32000 16.0 / - / 12.6 (6)    8 x 5 x 50257 16.6 / - / 13.6 (10)
-//   8 x 3 x 64000 13.7 / - / 11.4 (10)    28 x 5 x 8192 12.8 / 11.7 / 10.8 (4)    4 x 16 x 8000 12.1 / 10.8 / 10.2 (16)
+// as the first), whose blocks have room for the row's logits and what is parked of them.  us on a B200 by the streaming and
+// finish kernels / in clusters of half the size / of the size taken:
+//   1 x 4 x 32000 fp32 11.5 / 11.2 / 9.6 (12)    16 x 5 x 32000 16.0 / - / 12.5 (6)    8 x 5 x 50257 16.6 / - / 13.5 (10)
+//   10 x 4 x 24000 12.5 / 10.9 / 9.8 (10)    28 x 5 x 8192 12.8 / 11.7 / 10.8 (4)    4 x 16 x 8000 11.4 / 11.7 / 10.2 (12)
+// (The largest is not always the fastest, 4 x 16 x 2000 9.34 in 12 and 9.40 in 8, 1 x 12 x 4000 10.7 in 12 and 10.4 in 6; over 700 random
+// shapes the fastest of up to twelve would be 1 % faster.)
 // At most twelve: a cluster's SMs are of one GPC, so the larger it is the sooner it waits for other kernels to end.  Beside a
 // kernel that has a block on 60 (74, 90, 100, 110, 120, 132) of the SMs for 1 ms, 1 x 4 x 32000 fp32 waits for its end in clusters of 16 (14, 12, 10,
 // 8 with 120, 6 with 132); the general path with 132.  Alone it takes 9.24 us in 16, 9.63 in 12, 10.1 in 8, 11.5 by the general path: twelve leave

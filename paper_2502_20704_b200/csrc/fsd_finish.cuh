@@ -631,7 +631,7 @@ __device__ __forceinline__ void draw_pt(const FinishParams& P, FinishShared& sh,
         const double mine2[2] = {pre.total, scaled ? 0.0 : static_cast<double>(sh.far)};
         all = cluster_exchange(P, sh, d.cs, d.rank, link, mine2);
         if (link.lost) return;
-        if constexpr (LOCAL) {                        // (clusters of up to sixteen: one scan is shorter than sixteen additions in a row)
+        if constexpr (LOCAL) {                        // (clusters of up to twelve: one scan is shorter than twelve additions in a row)
             const double (&its)[kExchangeDoubles] = all[lane < d.cs ? lane : 0];
             const Prefix blocks(lane < d.cs ? its[0] : 0.0, lane);
             blocks_v = blocks.v; blocks_upto = blocks.upto;

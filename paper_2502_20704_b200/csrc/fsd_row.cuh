@@ -9,17 +9,20 @@
 //
 // A block's share of a row is `span` granules of 16 bytes.  Its sweeps are dealt out in items, a step (8 entries a lane) of a
 // pair each, pair by pair: a sixteenth of them, in one run, to every warp, so that a warp has to do with one or two pairs.
-//   1. First sweep of a warp's items of a pair, as in the streaming kernel but relative to their exact maxima: e = 2^(logit * log2e - k),
-//      Z, S (or the KL sum), "rows differ"; e parked in tensor memory.  The warp that
+//   1. First sweep of a warp's items of a pair, as in the streaming kernel: e = 2^(logit * log2e - k),
+//      Z, S (or the KL sum), "rows differ"; e parked in tensor memory.  The references k come from the maxima of the first item; a warp that
+//      finds they were not near enough does its sweep over with those of all its items.  The warp that
 //      is the last of a pair's folds what the pair's warps have posted and pushes the sums to all blocks of the cluster.
 //   2. A warp per pair folds what the blocks sent into 1/Z_a, 1/Z_b for its block.
 //   3. Second sweep of the items over the parked e, in the same order: JS sum (p+q) log2(p+q), TV sum |p - q|; folded and pushed
 //      likewise (KL has none).
 //   4. Every block judges all pairs from the sums of all blocks, in double precision, and draws as in the finish kernel.
 // A tree's nodes are pairs like any others, each against the target row of its parent.
+// The sums of a pair are added up in an order that follows from its position and the call's shape, and from nothing that other pairs hold.
 // What bounds it: latency.  16 x 5 x 32000 bf16 (16 clusters of 6), cycles from where the inputs may be read: first rows landed
-// 1400, first sweep 6900 (special functions 3400 of them), totals 9000, second sweep 12500 (1700), judged 15600, token 19900: 10.4 us of
-// 12.4 a call among others; 15.4 by the streaming and finish kernels.  1 x 4 x 32000 fp32 11.0 -> 9.1 us, 8 x 5 x 50257 16.1 -> 13.5.
+// 1560, first sweep 7720 (special functions 3400 of them), totals 9460, second sweep 12890 (1700), judged 15940, token 20040: 10.4 us of
+// 12.5 a call among others; 15.4 by the streaming and finish kernels.  1 x 4 x 32000 fp32 11.0 -> 9.7 us, 8 x 5 x 50257 16.1 -> 13.5.
+// A residual draw: 12 x 6 x 32000 (clusters of 9), relaxed rule, judged 18100, token 30770 (the other rule 14890, 19030).
 // All waits are for copies of the block's own or for pushes of its cluster's blocks, which run together by
 // the launch's terms; they are bounded all the same.  A block that has lost one leaves when its copies have landed, and last.
 #pragma once
@@ -286,7 +289,7 @@ __global__ void __launch_bounds__(kFinishThreads, 1) fsd_row_kernel(const __grid
     Candidate cand = {-1, 0.f, 0.f, 0.f};
     if constexpr (KIND == kDrawResidual) {
         if (warp < G) cand = candidate<DT, KIND>(F, b * G + warp, t_base + static_cast<size_t>(warp) * rb, d_base + static_cast<size_t>(warp) * rb);
-        if constexpr (DT == FSD_BF16) {                   // (the copies take longer than the table)
+        if constexpr (DT == FSD_BF16) {                   // (longer than the copies take: 12 x 6 x 32000, the warps are through 2500 to 5000 cycles after the start, the first rows land after 1270)
             for (int i = tid; i < kBf16Count; i += kFinishThreads) bf16_table_entry(*bt, *rs, i);
         }
     }

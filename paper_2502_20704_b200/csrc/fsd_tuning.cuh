@@ -298,10 +298,9 @@ struct CalibrateShared {
 // block r, then its sum over that eighth to everybody, and the block whose eighth holds the wanted
 // rank pushes the digit to everybody.  If no block has more than kTuneList keys that share the first digit, they are
 // pushed to block 0, which goes on with them by itself, two more histograms (9 and 10 bits) of at most eight keys a thread: a digit
-// of the whole cluster's is a walk over all rows and three exchanges, 3 us.  (Some 800 keys of 4096 x 8 share it; as
-// long as all lists together had to fit in 512 that call went on by the cluster's digits: 12.3 us, now 10.0; 8192 x 10 16.2, now 13.2.)
-// 4096 x 8: 57 -> 11 us, 32768 x 20: 821 -> 74 us (one
-// block and four 8-bit digits before), of which the walks' shared-memory atomics are the larger part.
+// of the whole cluster's is a walk over all rows and three exchanges, 3 us.  us on a B200 by one block and four 8-bit digits / by the cluster's digits
+// where more than 512 keys in all share the first (some 800 of 4096 x 8 do) / now:
+//   4096 x 8 57 / 12.2 / 9.8    8192 x 10 - / 16.3 / 13.1    32768 x 20 821 / 73.8 / 73.9 (the walks' shared-memory atomics are the larger part)
 template <int CS>
 __global__ void __launch_bounds__(kTuneThreads) fsd_calibrate_kernel(const float* __restrict__ D, int B, int G, float target,
                                                                      int cmp, float* __restrict__ T_out,

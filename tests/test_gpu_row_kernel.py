@@ -1,12 +1,13 @@
 """Calls that one kernel does whole, a thread-block cluster per row, at the sizes where its shares can go wrong, against
 the oracle: rows shorter than a step, blocks without a granule, the last size that fits on chip and the first that does not,
-as many pairs as warps and more; rows off a 16-byte boundary; logits whose first sweep has to be done over; invalid rows."""
+as many pairs as warps and more, as much to sweep as the kernel takes; rows off a 16-byte boundary; logits whose first sweep has to be done over; invalid rows."""
 
 import numpy as np
 import pytest
 import torch
 
 import fsd_inputs as gi
+import paper_2502_20704_b200 as fsd
 from tests import parity
 
 pytestmark = pytest.mark.gpu
@@ -94,6 +95,23 @@ def test_a_pairs_divergence_is_its_own_rows_alone(dtype, V, div):
     got = divergences()
     assert np.array_equal(got[6].view(np.uint32), want[6].view(np.uint32)) and np.array_equal(got[5, [0, 2, 3]].view(np.uint32), want[5, [0, 2, 3]].view(np.uint32))
     assert not np.array_equal(got[:6].view(np.uint32), want[:6].view(np.uint32))
+
+
+@pytest.mark.parametrize("dtype,V", [("bf16", 20000), ("bf16", 20003), ("f32", 15000), ("f32", 15001)])
+@pytest.mark.parametrize("div", ["js", "kl", "tv"])
+def test_the_streaming_kernel_gives_the_same_divergences(dtype, V, div):
+    """The sweeps of the two kernels are written twice; their sums differ in the order of single-precision additions alone."""
+    c = _chain(7, 4, V, dtype, 827)
+    one = parity.run_chain_gpu(c.target, c.draft, None, None, c.u_sample, dtype, div=div, T=0.2)
+    assert fsd.fsd_set_group_size(2) == 0
+    try:
+        two = parity.run_chain_gpu(c.target, c.draft, None, None, c.u_sample, dtype, div=div, T=0.2)
+    finally:
+        fsd.fsd_set_group_size(0)
+    # sums of up to 28 terms a lane, then trees: 32 roundings of 6e-8 of terms whose sum is a few nats at most
+    assert np.allclose(one.divergence, two.divergence, rtol=4e-6, atol=4e-6)
+    clear = (np.abs(two.divergence - 0.2) > 1e-5).all(axis=1)
+    assert np.array_equal(one.accept_len[clear], two.accept_len[clear])
 
 
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])

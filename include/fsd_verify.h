@@ -118,7 +118,7 @@ int fsd_workspace_bytes(int B, int positions, int V, const fsd_opts *opts, size_
  *   workspace     device scratch, 256-byte aligned, at least fsd_workspace_bytes() bytes;
  *                 contents need not be initialised and are not preserved
  * Calls that share a workspace must be ordered on the stream(s) that use it.
- * The call enqueues one kernel (where all logits fit on chip at once: a thread-block cluster per row) or two (the first of at
+ * The call enqueues one kernel (where all logits fit on chip at once and it is the faster way: a thread-block cluster per row) or two (the first of at
  * most one thread block per SM), with programmatic stream serialization, and nothing else, so it can be captured in a CUDA graph and replayed --
  * after one ordinary call with the same options on that device, which sets the kernels'
  * attributes (that cannot be done under capture). */

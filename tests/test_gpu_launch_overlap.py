@@ -133,7 +133,7 @@ def test_calls_beside_kernels_that_hold_most_of_the_gpu():
 
 @pytest.mark.parametrize("B,gamma,V", [(1, 4, 32000), (1, 4, 8192), (4, 8, 16000), (7, 5, 32000)])
 def test_a_small_call_finds_room_beside_kernels_that_hold_half_of_the_gpu(B, gamma, V):
-    """74 of the 148 SMs have a block of another kernel for 0.2 s; a call of a few rows does not wait for these to end."""
+    """74 of the 148 SMs have a block of another kernel for half a second; a call of a few rows does not wait for these to end."""
     import ctypes
     import time
     devs, want = _inputs(1, B, gamma, V, 0.2)
@@ -149,7 +149,7 @@ def test_a_small_call_finds_room_beside_kernels_that_hold_half_of_the_gpu(B, gam
     try:
         for h in holders:
             with torch.cuda.stream(h):
-                torch.cuda._sleep(400_000_000)
+                torch.cuda._sleep(1_000_000_000)
                 end.append(torch.cuda.Event())
                 end[-1].record(h)
         time.sleep(0.01)
